@@ -49,15 +49,6 @@ struct Recs {
     __device__ __forceinline__ uint32_t &phi(int v) { return base[(4 * kMaxTree + v) * stride]; }
 };
 
-// The pair id of (u, v) (or kNone): a search of u's pairs, sorted by
-// destination; warp-cooperative from coop_min pairs on.
-__device__ __forceinline__ uint32_t pair_of_coop(const DevGraph &g, uint32_t u, uint32_t v, uint32_t coop_min)
-{
-    const uint32_t lo = __ldg(g.vpair_off + u), hi = __ldg(g.vpair_off + u + 1);
-    const uint32_t p = first_true_coop(ProbeGeU32{g.pair_dst, v}, lo, hi, coop_min);
-    return (p < hi && __ldg(g.pair_dst + p) == v) ? p : kNone;
-}
-
 // Multi-edge list range of pair (u, v), or an empty range.
 __device__ __forceinline__ void find_pair(const DevGraph &g, uint32_t u, uint32_t v, uint32_t &beg, uint32_t &end,
                                           uint32_t coop_min = 0xFFFFFFFFu)
@@ -271,9 +262,11 @@ __device__ uint64_t complete_count(const DevGraph &g, const DevPlan &P, const Wi
 
 // The first draws of sample j (Alg. 3): a window with probability W_i / W,
 // then its root edge through the window's guide table and CDF.  Sets the
-// layer p, the window's time range [wlo, whi] and the root edge id; 0, or -1
-// on an internal inconsistency (latched as ST_BADSTATE).
-__device__ __forceinline__ int sample_root(const DevPlan &P, const SampleJob &J, SampleRng &rng, uint32_t *status,
+// layer p, the window's time range [wlo, whi] and the root edge id.  On an
+// internal inconsistency (latched as ST_BADSTATE, the call then fails) it goes
+// on with values in range, as sample_child does: an early return would keep
+// the lanes of a warp apart for the rest of the sample.
+__device__ __forceinline__ void sample_root(const DevPlan &P, const SampleJob &J, SampleRng &rng, uint32_t *status,
                                            int &p, uint32_t &wlo, uint32_t &whi, uint32_t &root)
 {
     const u128 W = (u128)J.W_lo | ((u128)J.W_hi << 64);
@@ -281,7 +274,7 @@ __device__ __forceinline__ int sample_root(const DevPlan &P, const SampleJob &J,
     // window: last k with wcum[k] <= r, between the guide entries of r's bucket
     const uint32_t jb = (uint32_t)(r >> J.wshift);
     uint32_t lo = __ldg(J.wguide + jb), hi = __ldg(J.wguide + jb + 1) + 1;
-    if (lo >= hi || hi > J.nwtot) { latch(status, ST_BADSTATE); return -1; }
+    if (lo >= hi || hi > J.nwtot) { latch(status, ST_BADSTATE); lo = 0; hi = 1; r = 0; }
     while (hi - lo > 1) {
         uint32_t mid = (lo + hi) >> 1;
         u128 c = (u128)__ldg(J.wcum + 2 * (size_t)mid) | ((u128)__ldg(J.wcum + 2 * (size_t)mid + 1) << 64);
@@ -306,110 +299,202 @@ __device__ __forceinline__ int sample_root(const DevPlan &P, const SampleJob &J,
     // exceeds the bucket bounds below and above rr
     const uint32_t gsh = __ldg((p ? J.win_gshift1 : J.win_gshift0) + kk);
     const uint32_t *G = (p ? J.guide1 : J.guide0) + __ldg((p ? J.win_goff1 : J.win_goff0) + kk) + (rr >> gsh);
-    const uint32_t glo = __ldg(G), ghi = __ldg(G + 1);
-    if (glo < wbeg || ghi >= wend || glo > ghi) { latch(status, ST_BADSTATE); return -1; }
+    uint32_t glo = __ldg(G), ghi = __ldg(G + 1);
+    if (glo < wbeg || ghi >= wend || glo > ghi) { latch(status, ST_BADSTATE); glo = ghi = wbeg; }
     root = upper_idx64(cdf, glo, ghi + 1, rr);
-    if (root > ghi) { latch(status, ST_BADSTATE); return -1; }
-    return 0;
+    if (root > ghi) { latch(status, ST_BADSTATE); root = ghi; }
+}
+
+// Time range of the child edge q of a parent edge at time pt, inside the
+// window [wlo, whi] (Constraint 1); false when it is empty.
+__device__ __forceinline__ bool child_times(const DevPlan &P, int q, uint32_t pt, uint32_t wlo, uint32_t whi,
+                                            uint64_t &tlo, uint64_t &thi)
+{
+    const uint64_t d = (uint64_t)P.delta;
+    if (P.tlater[q]) { tlo = (uint64_t)pt + 1; thi = (uint64_t)pt + d; }
+    else {
+        if (pt == 0) return false;
+        tlo = (uint64_t)pt >= d ? (uint64_t)pt - d : 0;
+        thi = (uint64_t)pt - 1;
+    }
+    tlo = tlo < (uint64_t)wlo ? (uint64_t)wlo : tlo;
+    thi = thi > (uint64_t)whi ? (uint64_t)whi : thi;
+    return true;
+}
+
+// The candidate range of a parent edge whose range the weight pass did not
+// keep, found by the DP's searches.
+__device__ __noinline__ uint2 search_range(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t ppos,
+                                           uint32_t pt, uint32_t wlo, uint32_t whi)
+{
+    uint64_t tlo, thi;
+    uint32_t a = 0, b = 0, beg;
+    const uint32_t *tarr;
+    if (child_times(P, q, pt, wlo, whi, tlo, thi))
+        child_range(g, P.tzside[q] != 0 ? 1 : 0, P.tout[q] != 0, zg, ppos, pt, P.tlater[q] != 0, tlo, thi, a, b, beg,
+                    tarr);
+    return make_uint2(a, b);
+}
+
+// The excluded entries of such a range (Claim 3.1): the part [ea, eb) of the
+// multi-edge list from pb on - zg -> og for a child leaving the meeting
+// vertex, og -> zg for one entering it - in the child's time range.
+__device__ __noinline__ uint3 search_excluded(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t og,
+                                              uint32_t pt, uint32_t wlo, uint32_t whi)
+{
+    uint64_t tlo, thi;
+    const bool out = P.tout[q] != 0;
+    const uint32_t pe = pair_of(g, out ? zg : og, out ? og : zg);
+    if (pe == kNone || !child_times(P, q, pt, wlo, whi, tlo, thi)) return make_uint3(0, 0, 0);
+    const uint32_t pb = __ldg(g.pair_off + pe), pend = __ldg(g.pair_off + pe + 1);
+    const uint32_t ea = lower_idx(g.multi_t, pb, pend, tlo);
+    return make_uint3(pb, ea, gallop_idx(g.multi_t, ea, pend, thi + 1));
 }
 
 // One tree edge of Alg. 3: the edge of tree node q, drawn by weight from its
 // candidate list at the meeting vertex given its parent's edge (source ps,
 // destination pd, time pt, edge id pgid), in layer p whose
 // window spans [wlo, whi].  Sets the child's time, endpoints and, for a node
-// with children or when `ids` is set, its edge id; 0, or -1 on an
-// internal inconsistency (latched as ST_BADSTATE).
-__device__ __forceinline__ int sample_child(const DevGraph &g, const DevPlan &P, const SampleJob &J, int q, int p,
+// with children or when `ids` is set, its edge id.
+//
+// A sample is a chain of dependent loads and a warp waits for the longest of
+// its 32, so the chain is what is kept short: the candidate range and what is
+// excluded from it are read from what the DP kept; an excluded
+// weight is skipped by finding, once, how much of it lies before the pick (the
+// entries before the pick are those with at most rc of the remaining weight
+// before them), after which the pick is one plain search of the prefixes.
+// Against searching range, multi-edge list and pick anew for every sample:
+// 5-cycle + chord, 5e7 edges, 1e7 samples 6.80 -> 4.26 ms (near 3 TB/s of
+// random sectors); 4-cycle, 2e6 edges (in L2), 1e6 samples 361 -> 190 us, 1e4
+// samples 46 -> 25 us; 5-star over a day, 1e7 edges, 3e6 samples 1,785 -> 750 us.
+__device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P, const SampleJob &J, int q, int p,
                                             uint32_t wlo, uint32_t whi, SampleRng &rng, uint32_t *status,
                                             uint32_t ps, uint32_t pd, uint32_t pt, uint32_t pgid,
                                             bool ids, uint32_t &ct, uint32_t &cs, uint32_t &cd, uint32_t &cgid)
 {
-    const uint64_t d = (uint64_t)P.delta;
     const bool zs = P.tzside[q] != 0, out = P.tout[q] != 0, leaf = P.tleaf[q] != 0;
     const uint32_t zg = zs ? pd : ps;
     const uint32_t og = zs ? ps : pd;
-    uint64_t tlo, thi;
-    if (P.tlater[q]) { tlo = (uint64_t)pt + 1; thi = (uint64_t)pt + d; }
-    else {
-        if (pt == 0) { latch(status, ST_BADSTATE); return -1; }
-        tlo = (uint64_t)pt >= d ? (uint64_t)pt - d : 0;
-        thi = (uint64_t)pt - 1;
-    }
-    tlo = tlo < (uint64_t)wlo ? (uint64_t)wlo : tlo;
-    thi = thi > (uint64_t)whi ? (uint64_t)whi : thi;
     const uint32_t *nbr = out ? g.out_nbr : g.in_nbr;
-    const uint32_t *gids = out ? g.out_gid : g.in_gid;
+    const uint32_t *tarr = out ? g.out_t : g.in_t;
     // the parent edge's position in the meeting vertex's out-list (z is its
     // source) or in-list (z is its destination)
     const uint32_t ppos = __ldg((zs ? g.in_pos : g.out_pos) + pgid);
-    uint32_t a, b, beg;
-    const uint32_t *tarr;
-    child_range(g, zs ? 1 : 0, out, zg, ppos, pt, P.tlater[q] != 0, tlo, thi, a, b, beg, tarr);
-    // the excluded multi-edge list (Constraint 2): zg -> og for a child
-    // leaving the meeting vertex, og -> zg for one entering it (scanning a
-    // short range for such entries first measured slower than this lookup)
-    const uint32_t pe = !P.c2 ? kNone
-                      : out ? pair_of_coop(g, zg, og, J.coop_min) : pair_of_coop(g, og, zg, J.coop_min);
-    uint32_t ea = 0, eb = 0, pb = 0;
-    if (pe != kNone) {
-        pb = __ldg(g.pair_off + pe);
-        const uint32_t pend = __ldg(g.pair_off + pe + 1);
-        ea = lower_idx(g.multi_t, pb, pend, tlo);
-        eb = gallop_idx(g.multi_t, ea, pend, thi + 1);
-    }
-    const int slot = P.tslot[q];
-    const uint64_t *Pd = nullptr, *Pm = nullptr;
-    uint64_t base = 0, base_m = 0, total;
-    if (leaf) {
-        total = (uint64_t)(b - a) - (uint64_t)(eb - ea);
-    } else {
-        // layer p's lane of the slot's (layer 0, layer 1) prefix pairs
-        Pd = (const uint64_t *)J.pref_dir[slot] + p;
-        Pm = (const uint64_t *)J.pref_multi[slot] + p;
-        base = (a > beg && __ldg(tarr + a - 1) >= wlo) ? __ldg(Pd + 2 * (size_t)(a - 1)) : 0;
-        base_m = (ea > pb && __ldg(g.multi_t + ea - 1) >= wlo) ? __ldg(Pm + 2 * (size_t)(ea - 1)) : 0;
-        const uint64_t sr = b > a ? __ldg(Pd + 2 * (size_t)(b - 1)) - base : 0;
-        const uint64_t se = eb > ea ? __ldg(Pm + 2 * (size_t)(eb - 1)) - base_m : 0;
-        total = sr - se;
-    }
-    if (total == 0 || b <= a) { latch(status, ST_BADSTATE); return -1; }
-    const uint64_t rc = rng.below(total, status);
-    // smallest x in [a, b) with F(x) > rc, F(x) = weight of the
-    // non-excluded entries in [a, x]
-    uint32_t xl = a, xh = b - 1;
-    if (eb == ea) {
-        // nothing excluded: F(x) = x - a + 1 for a leaf (the pick is
-        // direct), the prefix difference otherwise
-        if (leaf) xl = a + (uint32_t)rc;
-        else xl = first_true_coop(ProbeGtU64S2{Pd, rc + base}, a, b, J.coop_min);
-    } else {
-        while (xl < xh) {
-            const uint32_t x = xl + ((xh - xl) >> 1);
-            const uint32_t tx = __ldg(tarr + x);
-            // excluded entries at or before x: those earlier in time, and
-            // the one at time tx if it sorts at or before x (the list
-            // orders equal times by the other endpoint)
-            uint32_t ce = lower_idx(g.multi_t, ea, eb, tx) - ea;
-            if (ea + ce < eb && __ldg(g.multi_t + ea + ce) == tx && og <= __ldg(nbr + x)) ++ce;
-            uint64_t F;
-            if (leaf) F = (uint64_t)(x - a + 1) - ce;
-            else F = (__ldg(Pd + 2 * (size_t)x) - base) - (ce ? __ldg(Pm + 2 * (size_t)(ea + ce - 1)) - base_m : 0);
-            if (F > rc) xh = x; else xl = x + 1;
+    // candidates [a, b) and the excluded ones among them: a bit set (bit i:
+    // entry a + i), or the entries [ea, ea + ne) of a multi-edge list (em: the
+    // entry before them is in the same prefix segment)
+    uint32_t a, b, ea = 0, ne = 0;
+    uint64_t hit = 0;
+    bool em = false;
+    uint2 r = make_uint2(0, kRangeLong | (kRangeLong << 16));
+    if (J.range.base) r = __ldg(J.range.base + (size_t)(q - 1) * J.range.stride + ppos);
+    uint4 ex = make_uint4(r.x, 0, 0, kExclBits);
+    if ((r.y & kRangeFlags) && r.x < J.range.excl_cap) ex = __ldg(J.range.excl + r.x);
+    const bool later = P.tlater[q] != 0;
+    const uint32_t half = (p ? r.y >> 16 : r.y) & 0xFFFFu, len = half & kRangeLong;
+    a = later ? ex.x : ex.x - len;
+    b = a + len;
+    if (len == kRangeLong) {
+        const uint2 ab = search_range(g, P, q, zg, ppos, pt, wlo, whi);
+        a = ab.x;
+        b = ab.y;
+        if (P.c2) {
+            const uint3 e = search_excluded(g, P, q, zg, og, pt, wlo, whi);
+            ea = e.y;
+            ne = e.z - e.y;
+            em = ea > e.x && __ldg(g.multi_t + ea - 1) >= wlo;
+        }
+    } else if (half & 0x8000u) {
+        if (ex.w == kExclBits) {
+            hit = (uint64_t)ex.y | ((uint64_t)ex.z << 32);
+            if (!later) hit = __brevll(hit) >> (64 - len);   // counted from a
+            else hit &= ~0ull >> (64 - len);
+        } else {
+            const uint32_t h = (p ? ex.z >> 16 : ex.z) & 0xFFFFu;
+            ne = h & kRangeLong;
+            ea = later ? ex.y : ex.y - ne;
+            em = (h & 0x8000u) != 0;
         }
     }
+    if (b <= a || b > g.m || ne > g.m || ea > g.m - ne) {
+        latch(status, ST_BADSTATE);
+        a = 0; b = 1; hit = 0; ne = 0;
+    }
+    // layer p's lane of the slot's (layer 0, layer 1) prefix pairs; base = the
+    // prefix before the range's first entry in its (vertex, window) segment
+    const uint64_t *Pd = nullptr;
+    uint64_t base = 0, total = b - a;
+    if (!leaf) {
+        Pd = (const uint64_t *)J.pref_dir[P.tslot[q]] + p;
+        const uint32_t beg = __ldg((out ? g.out_off : g.in_off) + zg);
+        const uint32_t tb = a > 0 ? __ldg(tarr + a - 1) : 0u;
+        const uint64_t pb = a > 0 ? __ldg(Pd + 2 * (size_t)(a - 1)) : 0;
+        base = (a > beg && tb >= wlo) ? pb : 0;
+        total = __ldg(Pd + 2 * (size_t)(b - 1)) - base;
+    }
+    auto before = [&](uint32_t x) -> uint64_t {   // weight of the range before entry x
+        return leaf ? x - a : x > a ? __ldg(Pd + 2 * (size_t)(x - 1)) - base : 0;
+    };
+    const uint64_t *Pm = nullptr;
+    uint64_t base_m = 0;
+    auto excluded = [&](uint32_t i) -> uint64_t {   // weight of the first i excluded entries
+        return leaf ? i : i ? __ldg(Pm + 2 * (size_t)(ea + i - 1)) - base_m : 0;
+    };
+    if (hit) {
+        if (leaf) total -= (uint32_t)__popcll((long long)hit);
+        else
+            for (uint64_t h = hit; h; h &= h - 1) {
+                const uint32_t x = a + (uint32_t)__ffsll((long long)h) - 1;
+                total -= before(x + 1) - before(x);
+            }
+    } else if (ne) {
+        if (!leaf) {
+            Pm = (const uint64_t *)J.pref_multi[P.tslot[q]] + p;
+            base_m = em && ea ? __ldg(Pm + 2 * (size_t)(ea - 1)) : 0;
+        }
+        total -= excluded(ne);
+    }
+    if (total == 0) latch(status, ST_BADSTATE);
+    uint64_t rc = rng.below(total, status);
+    // add the excluded weight that lies before the pick: the excluded entries
+    // with at most rc of the remaining weight before them
+    if (hit) {
+        uint64_t skip = 0;
+        do {
+            const uint32_t x = a + (uint32_t)__ffsll((long long)hit) - 1;
+            const uint64_t w0 = before(x);
+            if (w0 - skip > rc) break;
+            skip += before(x + 1) - w0;
+            hit &= hit - 1;
+        } while (hit);
+        rc += skip;
+    } else if (ne) {
+        uint32_t lo = 0, hi = ne;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            // the entry's place in the list of z: out-list position directly,
+            // in-list position through its edge id
+            uint32_t x = __ldg(g.multi_to_out + ea + mid);
+            if (!out) x = __ldg(g.in_pos + __ldg(g.out_gid + x));
+            if (before(x) - excluded(mid) <= rc) lo = mid + 1; else hi = mid;
+        }
+        rc += excluded(lo);
+    }
+    // the first entry whose weight up to and including itself exceeds rc
+    uint32_t xl = leaf ? (uint32_t)min((uint64_t)a + rc, (uint64_t)b)
+                       : first_true_coop(ProbeGtU64S2{Pd, rc + base}, a, b, J.coop_min);
+    if (xl >= b) { latch(status, ST_BADSTATE); xl = b - 1; }
     const uint32_t other = __ldg(nbr + xl);
     ct = __ldg(tarr + xl);
     cs = out ? zg : other;
     cd = out ? other : zg;
     // the edge id is read only for a node with children (or a trace)
-    if (!leaf || ids) cgid = __ldg(gids + xl);
-    return 0;
+    if (!leaf || ids) cgid = __ldg((out ? g.out_gid : g.in_gid) + xl);
 }
 
 // The tree of sample j (Alg. 3): the root, then every tree edge from its
-// candidate list.  Fills R; 0, or -1 on an internal inconsistency (latched
-// as ST_BADSTATE).
-__device__ int sample_tree(const DevGraph &g, const DevPlan &P, const SampleJob &J, uint64_t seed, uint64_t j,
+// candidate list.  Fills R.
+__device__ void sample_tree(const DevGraph &g, const DevPlan &P, const SampleJob &J, uint64_t seed, uint64_t j,
                            uint32_t *status, uint32_t *tg_out, Recs R)
 {
     SampleRng rng;
@@ -417,27 +502,23 @@ __device__ int sample_tree(const DevGraph &g, const DevPlan &P, const SampleJob 
     int p;
     uint32_t wlo, whi;
     uint32_t root;
-    if (sample_root(P, J, rng, status, p, wlo, whi, root)) return -1;
+    sample_root(P, J, rng, status, p, wlo, whi, root);
     load_edge(g, root, R, 0);
     for (int q = 1; q < P.ntree; ++q) {
         const int pq = P.tparent[q];
-        if (sample_child(g, P, J, q, p, wlo, whi, rng, status, R.src(pq), R.dst(pq), R.t(pq), R.gid(pq),
-                         tg_out != nullptr, R.t(q), R.src(q), R.dst(q), R.gid(q)))
-            return -1;
+        sample_child(g, P, J, q, p, wlo, whi, rng, status, R.src(pq), R.dst(pq), R.t(pq), R.gid(pq),
+                     tg_out != nullptr, R.t(q), R.src(q), R.dst(q), R.gid(q));
     }
     if (tg_out)
         for (int q = 0; q < P.ntree; ++q) tg_out[q] = R.gid(q);
-    return 0;
 }
 
-// One sample: returns 0 valid, 1/2/3 reject reasons, or -1 on an internal
-// inconsistency (latched as ST_BADSTATE).
+// One sample: returns 0 valid, 1/2/3 reject reasons.
 __device__ int sample_one(const DevGraph &g, const DevPlan &P, const SampleJob &J, uint64_t seed, uint64_t j,
                           uint32_t *status, uint64_t &contrib, uint32_t *tg_out, Recs R)
 {
     contrib = 0;
-    const int r = sample_tree(g, P, J, seed, j, status, tg_out, R);
-    if (r) return r;
+    sample_tree(g, P, J, seed, j, status, tg_out, R);
     uint32_t tmin, tmax;
     const int why = validate_tree(P, R, tmin, tmax);
     if (why) return why;
@@ -478,23 +559,26 @@ __device__ __forceinline__ int sample_one_reg(const DevGraph &g, const DevPlan &
     int p;
     uint32_t wlo, whi;
     uint32_t root;
-    if (sample_root(P, J, rng, status, p, wlo, whi, root)) return -1;
+    sample_root(P, J, rng, status, p, wlo, whi, root);
     // Alg. 3: the root edge, then each node from its parent (parents come first)
     uint32_t src[NT], dst[NT], t[NT], gid[NT];
+#pragma unroll
+    for (int q = 0; q < NT; ++q) { src[q] = dst[q] = t[q] = gid[q] = 0; }
     gid[0] = root;
     src[0] = __ldg(g.g_src + root);
     dst[0] = __ldg(g.g_dst + root);
     t[0] = __ldg(g.g_t + root);
-#pragma unroll
+    // one copy of the child step for all nodes (select chains read and write
+    // the records): unrolled it outgrows the instruction cache
+#pragma unroll 1
     for (int q = 1; q < NT; ++q) {
         const int pq = P.tparent[q];
-        uint32_t ps = src[0], pd = dst[0], pt = t[0], pg = gid[0];
+        uint32_t ct, cs, cd, cg = 0;
+        sample_child(g, P, J, q, p, wlo, whi, rng, status, rsel(src, pq), rsel(dst, pq), rsel(t, pq), rsel(gid, pq),
+                     false, ct, cs, cd, cg);
 #pragma unroll
-        for (int h = 1; h < q; ++h)
-            if (pq == h) { ps = src[h]; pd = dst[h]; pt = t[h]; pg = gid[h]; }
-        gid[q] = 0;
-        if (sample_child(g, P, J, q, p, wlo, whi, rng, status, ps, pd, pt, pg, false, t[q], src[q], dst[q], gid[q]))
-            return -1;
+        for (int h = 1; h < NT; ++h)
+            if (q == h) { src[h] = cs; dst[h] = cd; t[h] = ct; gid[h] = cg; }
     }
     // Alg. 4: the vertex map (1-1), the delta span, the pi order of tree edges
     uint32_t phi[NT + 1];
@@ -729,13 +813,12 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += stride) {
         uint64_t c = 0;
-        if (sample_tree(g, sp, J, seed, first + i, status, nullptr, R) == 0) {
-            uint32_t tmin, tmax;
-            if (validate_tree(sp, R, tmin, tmax) == 0) {
-                bool ovf = false;
-                c = derive_cnt(g, sp, R, tmin, tmax, ovf);
-                if (ovf) latch(status, ST_OVERFLOW);
-            }
+        sample_tree(g, sp, J, seed, first + i, status, nullptr, R);
+        uint32_t tmin, tmax;
+        if (validate_tree(sp, R, tmin, tmax) == 0) {
+            bool ovf = false;
+            c = derive_cnt(g, sp, R, tmin, tmax, ovf);
+            if (ovf) latch(status, ST_OVERFLOW);
         }
         cnt_out[i] = c;
     }
@@ -763,7 +846,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += stride) {
         const uint64_t o = offs[i], n = offs[i + 1] - o;
         if (n == 0 || o >= max_inst) continue;
-        if (sample_tree(g, sp, J, seed, first + i, status, tree_gids, R)) continue;
+        sample_tree(g, sp, J, seed, first + i, status, tree_gids, R);
         uint32_t tmin, tmax;
         if (validate_tree(sp, R, tmin, tmax)) { latch(status, ST_BADSTATE); continue; }
         const uint64_t got = enumerate_completions(g, sp, R, tmin, tmax, [&](uint64_t idx, const uint32_t *cur) {
@@ -803,7 +886,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
     unsigned long long nv = 0, nr1 = 0, nr2 = 0, nr3 = 0;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < k; i += stride) {
-        if (sample_tree(g, sp[0], J, seed, first + i, status, nullptr, R)) continue;
+        sample_tree(g, sp[0], J, seed, first + i, status, nullptr, R);
         uint32_t tmin, tmax;
         const int why = validate_tree(sp[0], R, tmin, tmax);
         if (why == 1) { ++nr1; continue; }
@@ -973,6 +1056,7 @@ void fill_job(tm_motif *mo, SampleJob &J, const DevPlan *dplan)
         J.pref_dir[s] = mo->pref_dir[s];
         J.pref_multi[s] = mo->pref_multi[s];
     }
+    J.range = mo->range;
     J.W_lo = mo->W.lo;
     J.W_hi = mo->W.hi;
 }

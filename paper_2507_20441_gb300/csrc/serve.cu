@@ -121,14 +121,16 @@ std::string make_key(uint32_t nv, uint32_t ne, const uint32_t *edges, const uint
 }
 
 // Device bytes a motif's resident weights will need (root CDF and its guide
-// table, prefix slots, window lists), before they are computed.
+// table, prefix slots, candidate ranges, window lists), before they are computed.
 size_t estimate_bytes(const tm_motif *mo, uint64_t m, uint64_t T)
 {
     uint64_t slots = (uint64_t)mo->plan.nslots;
     uint64_t nwin = T / (uint64_t)std::max<int64_t>(1, mo->plan.wdelta) + 2;
     nwin = std::min<uint64_t>(nwin, m + 2);
-    // root CDF 16 B and root-search guide about 2 B per edge, 32 B per prefix slot
-    return (size_t)((18 + 32 * slots) * std::max<uint64_t>(m, 1) + 96 * nwin + 4096);
+    // root CDF 16 B and root-search guide about 2 B per edge, 32 B per prefix
+    // slot, 12 B per non-root node's candidate ranges
+    const uint64_t ranges = (uint64_t)(mo->plan.ntree - 1);
+    return (size_t)((18 + 32 * slots + 12 * ranges) * std::max<uint64_t>(m, 1) + 96 * nwin + 4096);
 }
 
 void finish_locked(Server *S, Request *r)

@@ -77,13 +77,14 @@ struct SampleRng {
 };
 
 // First index in [lo, hi) with a[i] >= x (a sorted ascending); hi if none.
-__device__ __forceinline__ uint32_t lower_idx(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, uint64_t x)
+template <class Key>
+__device__ __forceinline__ uint32_t lower_idx(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, Key x)
 {
     uint32_t n = hi - lo;
     while (n > 0) {
         uint32_t half = n >> 1;
         uint32_t mid = lo + half;
-        if ((uint64_t)__ldg(a + mid) < x) { lo = mid + 1; n -= half + 1; }
+        if ((Key)__ldg(a + mid) < x) { lo = mid + 1; n -= half + 1; }
         else n = half;
     }
     return lo;
@@ -105,14 +106,39 @@ __device__ __forceinline__ uint32_t gallop_idx(const uint32_t *__restrict__ a, u
     return lower_idx(a, lo, probe, x);
 }
 
+// First index in [lo, hi) with a[i] > x; hi if none.
+__device__ __forceinline__ uint32_t above_idx(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, uint32_t x)
+{
+    uint32_t n = hi - lo;
+    while (n > 0) {
+        const uint32_t half = n >> 1, mid = lo + half;
+        if (__ldg(a + mid) <= x) { lo = mid + 1; n -= half + 1; }
+        else n = half;
+    }
+    return lo;
+}
+
+// The same, searching outward from lo first (1, 2, 4, ... entries ahead).
+__device__ __forceinline__ uint32_t gallop_above(const uint32_t *__restrict__ a, uint32_t lo, uint32_t hi, uint32_t x)
+{
+    uint32_t step = 1, probe = lo;
+    while (probe < hi && __ldg(a + probe) <= x) {
+        lo = probe + 1;
+        probe = (hi - probe > step) ? probe + step : hi;
+        step = step < 0x40000000u ? step << 1 : step;
+    }
+    return above_idx(a, lo, probe, x);
+}
+
 // First index in [beg, base] with a[i] >= x, when every index >= base is
 // known to hold a value >= x: searches backward from base (1, 2, 4, ...).
-__device__ __forceinline__ uint32_t gallop_back(const uint32_t *__restrict__ a, uint32_t beg, uint32_t base, uint64_t x)
+template <class Key>
+__device__ __forceinline__ uint32_t gallop_back(const uint32_t *__restrict__ a, uint32_t beg, uint32_t base, Key x)
 {
     uint32_t hi = base, step = 1;
     while (hi > beg) {
         const uint32_t probe = (hi - beg > step) ? hi - step : beg;
-        if ((uint64_t)__ldg(a + probe) < x) return lower_idx(a, probe + 1, hi, x);
+        if ((Key)__ldg(a + probe) < x) return lower_idx(a, probe + 1, hi, x);
         hi = probe;
         step = step < 0x40000000u ? step << 1 : step;
     }

@@ -28,30 +28,20 @@ constexpr int TB = 256;
 inline unsigned blocks_for(uint64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // Prefix arrays of the child nodes: per position the (layer 0, layer 1)
-// prefix pair, so one 16-byte load serves both layers.
+// prefix pair, so one 16-byte load serves both layers.  Slot i's prefix in the
+// out/in order starts at base + 2 i stride, its prefix in the multi-edge order
+// stride after that.
 struct ChildPrefix {
-    const ulonglong2 *pd[kMaxTree];    // [slot] prefix in the out/in order
-    const ulonglong2 *pm[kMaxTree];    // [slot] prefix in the multi-edge order
+    const ulonglong2 *base;
+    size_t stride;
 };
 
 __device__ __forceinline__ uint64_t lane_of(const ulonglong2 v, int p) { return p ? v.y : v.x; }
 
-// a[i] for a runtime slot i by a chain of selects: indexing a kernel
-// parameter array at a runtime index would copy it to local memory
-__device__ __forceinline__ const ulonglong2 *pick_slot(const ulonglong2 *const (&a)[kMaxTree], int i)
-{
-    const ulonglong2 *v = a[0];
-#pragma unroll
-    for (int s = 1; s < kMaxTree; ++s) v = (i == s) ? a[s] : v;
-    return v;
-}
-
 // Candidate ranges up to this many entries are scanned for the excluded
 // neighbour; longer ones search the excluded multi-edge list instead.
-#ifndef TM_DP_SCAN_LIMIT
-#define TM_DP_SCAN_LIMIT 96   // measured: 96 and 128 beat 48, 16 and 8 on the 5e7-edge workload
-#endif
-constexpr uint32_t kScanLimit = TM_DP_SCAN_LIMIT;
+constexpr uint32_t kScanLimit = 64;   // the bits of a RangeExcl
+constexpr int kScanStep = 8;          // independent loads per step (4 and 16 measured 0.2 - 1 % slower)
 
 // One side of tree node q (Claim 3.2): the product of the factors of q's
 // children that meet q at its tail (side 0) or head (side 1), for every edge
@@ -74,13 +64,26 @@ constexpr uint32_t kScanLimit = TM_DP_SCAN_LIMIT;
 // product through the out->in position map, and its pending-overflow bits
 // from two bit sets of m/32 words (one per layer; a warp of side 0 writes
 // the word of its 32 positions with a ballot), small enough to stay in L2.
+// Each child's ranges are also written out (8 bytes per edge, coalesced) for
+// the sampler, which would otherwise repeat the gallops and the search for
+// excluded entries, as one dependent load after another, for every sample.
+// The kernel is bound by the instructions it issues (about half of the issue
+// slots) and by occupancy, so empty ranges leave early, time bounds are 32-bit
+// compares and sides with leaf children only have a kernel without prefixes:
+// with these three and the ranges written 4.39 -> 4.21 ms for the three
+// launches of the 5-cycle + chord on 5e7 edges, 1,161 -> 1,125 us for the four
+// of a 6-path on 1e7 (without them the ranges cost 0.39 ms and 127 us).
 // Overflow rule: a factor >= 2^64, or an exact product >= 2^64 with no zero
 // factor.
+// LEAF: every child met on this side is a leaf, so no prefix sums are read and
+// the kernel needs few enough registers for 40 a thread almost without spills.
 #ifndef TM_DP_MINB
-#define TM_DP_MINB 5   // 48 registers, five blocks of 256 per SM (measured faster than 40 or 64 registers)
+#define TM_DP_MINB 6   // 40 registers, six blocks of 256 per SM (5 and 7 measured slower: 4355 and 4572 against 4206 us)
 #endif
+template <bool LEAF>
 __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, WinDiv wv, int q, int side, int first,
-                                                        int last, ChildPrefix cp, ulonglong2 *__restrict__ wout,
+                                                        int last, ChildPrefix cp, RangePtrs ranges,
+                                                        ulonglong2 *__restrict__ wout,
                                                         const uint32_t *__restrict__ scatter,
                                                         const ulonglong2 *__restrict__ in,
                                                         const uint32_t *__restrict__ pin, uint32_t *__restrict__ pout,
@@ -129,7 +132,7 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
         for (int ci = 0; ci < P.nchild[q] && !(zero[0] && zero[1]); ++ci) {
             const int c = P.child[q][ci];
             if (P.tzside[c] != side) continue;
-            const bool out = P.tout[c] != 0, later = P.tlater[c] != 0, leaf = P.tleaf[c] != 0;
+            const bool out = P.tout[c] != 0, later = P.tlater[c] != 0, leaf = LEAF || P.tleaf[c] != 0;
             // no earlier time than 0, no later one than the largest t'
             if ((!later && t == 0) || (later && t == 0xFFFFFFFFu)) { zero[0] = zero[1] = true; break; }
             const uint32_t *off = out ? g.out_off : g.in_off;
@@ -143,19 +146,21 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
             if (later) {
                 const uint64_t hu64 = (uint64_t)t + d;
                 const uint32_t l0 = t + 1, hu = hu64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)hu64;
-                const uint32_t a0 = gallop_idx(tarr, base, end, l0);
-                const uint32_t bu = gallop_idx(tarr, a0, end, (uint64_t)hu + 1);
+                const uint32_t a0 = gallop_above(tarr, base, end, t);
+                const uint32_t bu = gallop_above(tarr, a0, end, hu);
+                if (bu == a0) { zero[0] = zero[1] = true; break; }
 #pragma unroll
                 for (int p = 0; p < 2; ++p) {
                     lo[p] = l0;
                     hi[p] = hu < whi[p] ? hu : whi[p];
                     a[p] = a0;
-                    b[p] = (zero[p] || hi[p] == hu) ? bu : lower_idx(tarr, a0, bu, (uint64_t)hi[p] + 1);
+                    b[p] = (zero[p] || hi[p] == hu) ? bu : above_idx(tarr, a0, bu, hi[p]);
                     if (lo[p] > hi[p]) zero[p] = true;
                 }
             } else {
                 const uint32_t h0 = t - 1, lu = (uint64_t)t >= d ? (uint32_t)((uint64_t)t - d) : 0u;
                 const uint32_t au = gallop_back(tarr, beg, base, lu);
+                if (au == base) { zero[0] = zero[1] = true; break; }
 #pragma unroll
                 for (int p = 0; p < 2; ++p) {
                     hi[p] = h0;
@@ -166,7 +171,7 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
                 }
             }
             if (zero[0] && zero[1]) break;
-            const ulonglong2 *Pd = leaf ? nullptr : pick_slot(cp.pd, P.tslot[c]);
+            const ulonglong2 *Pd = leaf ? nullptr : cp.base + 2 * P.tslot[c] * cp.stride;
             uint64_t excl[2] = {0, 0};
             // the union of the live layers' ranges
             uint32_t ua = 0xFFFFFFFFu, ub = 0;
@@ -175,7 +180,13 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
                 if (!zero[p]) { ua = min(ua, a[p]); ub = max(ub, b[p]); }
             // an excluded entry x (other endpoint o) of the range: its weight,
             // in each layer whose range holds it
+            // what the sampler is told of them: a bit each (short ranges), or
+            // their list positions and per-layer numbers
+            uint32_t ex_y = 0, ex_z = 0;
+            const bool scanned = ub <= ua || ub - ua <= kScanLimit;
             auto add_excl = [&](uint32_t x) {
+                const uint32_t bit = later ? x - ua : ub - 1 - x;
+                if (bit < 32) ex_y |= 1u << bit; else ex_z |= 1u << (bit - 32);
                 ulonglong2 wx2 = make_ulonglong2(1, 1);
                 if (!leaf) {
                     // the entry's weight: its prefix minus the previous entry's in
@@ -192,10 +203,17 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
             };
             if (!P.c2) {
                 // without Constraint 2 nothing is excluded
-            } else if (ub <= ua || ub - ua <= kScanLimit) {
-                // (reading four neighbours per 16-byte load measured no faster)
-                for (uint32_t x = ua; x < ub; ++x)
-                    if (__ldg(nbr + x) == o) add_excl(x);
+            } else if (scanned) {
+                for (uint32_t x0 = ua; x0 < ub; x0 += kScanStep) {
+                    uint32_t hit = 0;
+#pragma unroll
+                    for (int i = 0; i < kScanStep; ++i)
+                        hit |= (x0 + i < ub && __ldg(nbr + x0 + i) == o) ? 1u << i : 0u;
+                    while (hit) {
+                        add_excl(x0 + (uint32_t)__ffs((int)hit) - 1);
+                        hit &= hit - 1;
+                    }
+                }
             } else {
                 // the excluded multi-edge list: z -> o for a child leaving z, o -> z
                 // for one entering it
@@ -208,16 +226,41 @@ __global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, W
                         const uint32_t ea = lower_idx(g.multi_t, xb, xe, lo[p]);
                         const uint32_t eb = gallop_idx(g.multi_t, ea, xe, (uint64_t)hi[p] + 1);
                         if (eb <= ea) continue;
+                        // a later child's lists start together, an earlier one's end together
+                        ex_y = later ? ea : eb;
+                        ex_z |= min(eb - ea, kRangeLong) << (16 * p);
                         if (leaf) {
                             excl[p] = eb - ea;
                         } else {
-                            const ulonglong2 *Pm = pick_slot(cp.pm, P.tslot[c]);
-                            const uint64_t bs = (ea > xb && __ldg(g.multi_t + ea - 1) >= wlo[p])
-                                                    ? lane_of(__ldg(Pm + ea - 1), p) : 0;
-                            excl[p] = lane_of(__ldg(Pm + eb - 1), p) - bs;
+                            const ulonglong2 *Pm = cp.base + (2 * P.tslot[c] + 1) * cp.stride;
+                            const bool same = ea > xb && __ldg(g.multi_t + ea - 1) >= wlo[p];
+                            ex_z |= same ? 0x8000u << (16 * p) : 0u;
+                            excl[p] = lane_of(__ldg(Pm + eb - 1), p) - (same ? lane_of(__ldg(Pm + ea - 1), p) : 0);
                         }
                     }
                 }
+            }
+            // the sampler draws this child from the same ranges
+            if (ranges.base) {
+                uint2 *rg = ranges.base + (size_t)(c - 1) * ranges.stride;
+                const uint32_t near = later ? a[0] : b[0];
+                uint32_t len0 = min(b[0] - a[0], kRangeLong), len1 = min(b[1] - a[1], kRangeLong);
+                uint2 rec = make_uint2(near, 0);
+                if (excl[0] | excl[1]) {
+                    const unsigned long long i = atomicAdd(ranges.excl_n, 1ull);
+                    if (i < ranges.excl_cap) {
+                        ranges.excl[i] = make_uint4(near, ex_y, ex_z, scanned ? kExclBits : kExclList);
+                        rec = make_uint2((uint32_t)i, (excl[0] ? 0x8000u : 0u) | (excl[1] ? 0x80000000u : 0u));
+                        if (!scanned) {   // more excluded entries than a half holds: searched
+                            if ((ex_z & kRangeLong) == kRangeLong) len0 = kRangeLong;
+                            if (((ex_z >> 16) & kRangeLong) == kRangeLong) len1 = kRangeLong;
+                        }
+                    } else {
+                        len0 = len1 = kRangeLong;
+                    }
+                }
+                rec.y |= len0 | (len1 << 16);
+                rg[pos] = rec;
             }
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
@@ -647,6 +690,7 @@ static void free_motif_weights(tm_ctx *ctx, tm_motif *mo)
     mo->bytes = 0;
     for (int p = 0; p < 2; ++p) mo->layer[p] = LayerData();
     for (int sl = 0; sl < kMaxTree; ++sl) mo->pref_dir[sl] = mo->pref_multi[sl] = nullptr;
+    mo->range = RangePtrs{};
     mo->wcum = nullptr;
     mo->wguide = nullptr;
     mo->have_weights = false;
@@ -697,7 +741,18 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
         size_t total = al(((size_t)nwh[0] + 1) * 4) * 4 + al(((size_t)nwh[1] + 1) * 4) * 4 + 2 * al(mm * 8) +
                        (size_t)P.nslots * 2 * al(mm * 16) + al(((size_t)nwh[0] + nwh[1] + 1) * 16) +
                        al(guide_n(nwh[0]) * 4) + al(guide_n(nwh[1]) * 4) + al((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
-        char *blk = (char *)malloc_motif(ctx, mo, total);
+        // the candidate ranges come last: a block this large that does not fit
+        // with them is tried without (the sampler then searches the ranges)
+        // (room for excluded entries at a quarter of the edges per node: with
+        // bursts of repeated pairs a star's nodes have them at 0.2 - 0.3)
+        const size_t excl_cap = (size_t)(P.ntree - 1) * (mm / 4);
+        const size_t range_bytes = (size_t)(P.ntree - 1) * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl)) + al(8);
+        bool with_ranges = true;
+        char *blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
+        if (!blk && total >= ((size_t)4 << 30)) {
+            with_ranges = false;
+            blk = (char *)malloc_motif(ctx, mo, total);
+        }
         if (!blk) return TM_E_NOMEM;
         size_t off = 0;
         auto take = [&](size_t bytes) { char *q = blk + off; off += al(bytes); return (void *)q; };
@@ -711,12 +766,20 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
             L.win_goff = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
             L.guide = (uint32_t *)take(guide_n(nwh[p]) * 4);
         }
-        for (int sl = 0; sl < P.nslots; ++sl) {
+        for (int sl = 0; sl < P.nslots; ++sl) {   // one after the other (ChildPrefix)
             mo->pref_dir[sl] = (ulonglong2 *)take(mm * 16);
             mo->pref_multi[sl] = (ulonglong2 *)take(mm * 16);
         }
         mo->wcum = (uint64_t *)take(((size_t)nwh[0] + nwh[1] + 1) * 16);
         mo->wguide = (uint32_t *)take((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
+        if (with_ranges) {
+            mo->range.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
+            mo->range.base = (uint2 *)take((size_t)(P.ntree - 1) * mo->range.stride * sizeof(uint2));
+            mo->range.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
+            mo->range.excl_n = (unsigned long long *)take(8);
+            mo->range.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
+            cudaMemsetAsync(mo->range.excl_n, 0, 8, st);
+        }
     }
     {
         PhaseScope ph(ctx, TM_PH_WINDOWS);
@@ -734,7 +797,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
     uint32_t *pend = nullptr;                 // per layer a bit set: pending overflow of a side-0 partial
     w = (ulonglong2 *)salloc(ctx, (size_t)(m ? m : 1) * 16);
     if (!w) return TM_E_NOMEM;
-    ChildPrefix cp{};
+    const ChildPrefix cp{P.nslots ? mo->pref_dir[0] : nullptr, (size_t)((m ? m : 1) * (uint64_t)16 + 255) / 256 * 16};
     int maxh = 0;
     for (int q = 0; q < P.ntree; ++q) maxh = std::max(maxh, (int)P.height[q]);
     std::vector<int> order;
@@ -746,7 +809,12 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
         // sides of q that children meet; the weights come out in the order of
         // the last side run (out-list order for side 0, in-list for side 1)
         bool has[2] = {false, false};
-        for (int ci = 0; ci < P.nchild[q]; ++ci) has[P.tzside[P.child[q][ci]]] = true;
+        bool inner[2] = {false, false};   // a child with children meets this side
+        for (int ci = 0; ci < P.nchild[q]; ++ci) {
+            const int c = P.child[q][ci];
+            has[P.tzside[c]] = true;
+            if (!P.tleaf[c]) inner[P.tzside[c]] = true;
+        }
         const bool in_order = has[1];
         {
             PhaseScope ph(ctx, TM_PH_DP);
@@ -756,19 +824,26 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
                 if (!pw || !pend) return TM_E_NOMEM;
             }
             if (m) {
+                const uint32_t *none = nullptr;
+                const ulonglong2 *no_in = nullptr;
+                auto dp = [&](int side, int first, int last, ulonglong2 *wout, const uint32_t *scatter,
+                              const ulonglong2 *in, const uint32_t *pin, uint32_t *pout) {
+                    auto go = [&](auto kernel) {
+                        launch(ctx, kernel, blocks_for(m, TB), TB, g, P, wv, q, side, first, last, cp, mo->range, wout,
+                               scatter, in, pin, pout, ctx->status);
+                    };
+                    if (inner[side]) go(k_dp<false>);
+                    else go(k_dp<true>);
+                };
                 if (has[0] && has[1]) {
-                    launch(ctx, k_dp, blocks_for(m, TB), TB, g, P, wv, q, 0, 1, 0, cp, pw, (const uint32_t *)nullptr,
-                           (const ulonglong2 *)nullptr, (const uint32_t *)nullptr, pend, ctx->status);
-                    launch(ctx, k_dp, blocks_for(m, TB), TB, g, P, wv, q, 1, 0, 1, cp, w, (const uint32_t *)nullptr,
-                           (const ulonglong2 *)pw, (const uint32_t *)pend, (uint32_t *)nullptr, ctx->status);
+                    dp(0, 1, 0, pw, none, no_in, none, pend);
+                    dp(1, 0, 1, w, none, pw, pend, nullptr);
                 } else {
                     // a non-root node leaving its parent's meeting vertex runs in
                     // in-list order and is scanned by its parent in out-list
                     // order: it writes through the in -> out map
                     const bool to_out = q != 0 && P.tout[q] != 0 && in_order;
-                    launch(ctx, k_dp, blocks_for(m, TB), TB, g, P, wv, q, in_order ? 1 : 0, 1, 1, cp, w,
-                           to_out ? (const uint32_t *)g.in_to_out : (const uint32_t *)nullptr,
-                           (const ulonglong2 *)nullptr, (const uint32_t *)nullptr, (uint32_t *)nullptr, ctx->status);
+                    dp(in_order ? 1 : 0, 1, 1, w, to_out ? g.in_to_out : none, no_in, none, nullptr);
                 }
             }
         }
@@ -809,8 +884,6 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
             DirScan2 fm{w, g.multi_to_out, g.multi_t, ob.multi, wv};
             rc = segmented_scan2_u64(ctx, fm, m, nullptr, nullptr, mo->pref_multi[slot]);
             if (rc) return rc;
-            cp.pd[slot] = mo->pref_dir[slot];
-            cp.pm[slot] = mo->pref_multi[slot];
         }
     }
     // ---- window totals and their 128-bit running sum (K5)
