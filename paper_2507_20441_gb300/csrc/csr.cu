@@ -36,97 +36,253 @@ namespace {
 
 // ---- radix sort --------------------------------------------------------
 // Keys are sorted least significant digit first, with up to 7-bit digits
-// (a 21-bit vertex id takes three passes, a 27-bit time four).  A pass is
-//   1. per-tile digit counts (4096 keys per tile), stored digit-major;
-//   2. an exclusive scan of those counts, which gives, for every (digit,
-//      tile), where the tile's run of that digit starts in the output;
-//   3. the scatter: each tile ranks its keys stably (per warp, by one ballot
-//      per digit bit, or at once when the warp's digits agree; then across
-//      warps), reorders them by digit in shared memory and writes each
-//      digit's run out contiguously.
-// No block waits on another.
+// (a 21-bit vertex id takes three passes, a 27-bit time four; 9-bit digits,
+// fewer passes of shorter runs, measured 6.2 against 5.4 ms for the sorts of
+// 5e7 edges and the same at 2e6).  The digit counts of every pass of a sort are made once,
+// before its first pass (for the build's sorts by the kernel that compacts the
+// input, which reads the keys anyway), and a pass is one kernel: a tile of
+// keys is ranked stably, the tile finds where its digits start in the output
+// by looking back over the counts that the tiles before it have published, and
+// writes its digit runs out.
 #ifndef TM_RS_ITEMS
 #define TM_RS_ITEMS 16   // keys per thread (8 and 12 measured slower)
-#endif
-#ifndef TM_RS_MATCH
-#define TM_RS_MATCH 0    // 1: peers of a digit by one match-any instead of a ballot per digit bit
 #endif
 constexpr int OS_THREADS = 256;
 constexpr int OS_ITEMS = TM_RS_ITEMS;
 constexpr int OS_TILE = OS_THREADS * OS_ITEMS;     // 4096 keys per tile
 constexpr int OS_WARPS = OS_THREADS / 32;
-constexpr int OS_WCHUNK = OS_ITEMS * 32;           // keys per warp chunk
-#ifndef TM_RS_MAXBITS
-#define TM_RS_MAXBITS 7   // measured: 7-bit digits beat 9 (a 27-bit time in four passes instead of three)
-#endif
-constexpr int OS_MAXBITS = TM_RS_MAXBITS;
+constexpr int OS_MAXBITS = 7;
 constexpr int OS_MAXRADIX = 1 << OS_MAXBITS;
-constexpr int OS_SCAN = 512;   // entries of the block scan of the digit totals (two per thread)
-static_assert(OS_MAXRADIX <= OS_SCAN && OS_THREADS * 2 == OS_SCAN, "digit scan layout");
+constexpr int OS_SCAN = 512;   // entries of the block scan of bucket counts (two per thread)
+static_assert(OS_MAXRADIX <= OS_SCAN && OS_THREADS * 2 == OS_SCAN, "bucket scan layout");
 constexpr int OS_MAXPASS = (32 + OS_MAXBITS - 1) / OS_MAXBITS;   // any 32-bit key
-// dynamic shared memory of a scatter pass with np payload arrays
-[[maybe_unused]] constexpr size_t os_smem(int np)
+// Sorts of up to kSmallSort keys take tiles of 1024: a tile of 4096 would leave
+// most SMs without one (20,000 keys: 5 tiles against 20).
+constexpr int OS_SMALL_ITEMS = 4;
+constexpr uint32_t kSmallSort = 300000;
+
+// The digits of a key's passes: bits [sh, sh + bits) each.
+struct DigitPlan {
+    int npass = 0;
+    int sh[OS_MAXPASS] = {}, bits[OS_MAXPASS] = {};
+};
+// counts[pass * OS_MAXRADIX + digit] of one key array
+constexpr int OS_HIST = OS_MAXPASS * OS_MAXRADIX;
+
+__device__ __forceinline__ void hist_key(const DigitPlan &D, uint32_t key, uint32_t *__restrict__ h)
 {
-    return (size_t)OS_TILE * 4 * (1 + np) + (size_t)OS_TILE * 2 + (size_t)OS_WARPS * OS_MAXRADIX * 2 +
-           (size_t)(OS_SCAN + OS_MAXRADIX) * 4;
+#pragma unroll
+    for (int p = 0; p < OS_MAXPASS; ++p)
+        if (p < D.npass) atomicAdd(h + p * OS_MAXRADIX + ((key >> D.sh[p]) & ((1u << D.bits[p]) - 1u)), 1u);
 }
 
-// per-tile digit counts, written to counts[d * ntiles + tile].  Each warp
-// counts into its own histogram with shared atomics; a warp whose 32 digits
-// agree (sorted or nearly sorted input) adds once.
-// Up to two independent arrays of the same length sorted by the same passes:
-// blocks [0, ntiles) work on set 0, blocks [ntiles, 2 ntiles) on set 1.  The
-// counts of set 1 follow those of set 0, so after one exclusive scan over
-// both, set 1's output offsets are shifted by exactly n.
+__device__ __forceinline__ void hist_flush(const uint32_t *__restrict__ h, int n, uint32_t *__restrict__ out)
+{
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (h[i]) atomicAdd(out + i, h[i]);
+}
+
+// Digit counts of every pass over one key array.
+__global__ void __launch_bounds__(OS_THREADS) k_rs_hist(const uint32_t *__restrict__ key, uint32_t n, DigitPlan D,
+                                                        uint32_t *__restrict__ hist)
+{
+    __shared__ uint32_t h[OS_HIST];
+    for (int i = threadIdx.x; i < OS_HIST; i += OS_THREADS) h[i] = 0;
+    __syncthreads();
+    for (uint64_t i = (uint64_t)blockIdx.x * OS_THREADS + threadIdx.x; i < n; i += (uint64_t)gridDim.x * OS_THREADS)
+        hist_key(D, __ldg(key + i), h);
+    __syncthreads();
+    hist_flush(h, OS_HIST, hist);
+}
+
+// Inputs and outputs of a sort's pass: the key and up to four payloads.
 struct RsSet {
-    const uint32_t *kin, *p0in, *p1in;
-    uint32_t *kout, *p0out, *p1out;
-    const uint32_t *p2in = nullptr;
-    uint32_t *p2out = nullptr;
-    const uint32_t *p3in = nullptr;
-    uint32_t *p3out = nullptr;
+    const uint32_t *kin = nullptr, *pin[4] = {};
+    uint32_t *kout = nullptr, *pout[4] = {};
     uint32_t *inv = nullptr;   // when set: inv[payload 0] = output position (the inverse permutation)
 };
-struct RsJobs {
-    RsSet s[2];
-};
 
-__global__ void __launch_bounds__(OS_THREADS, 6) k_rs_count(RsJobs J, uint32_t n, int shift, int bits, uint32_t ntiles,
-                                                             uint32_t *__restrict__ counts_all)
+// What a tile has published of a digit: its count, or the count of it and of
+// every tile before it.
+enum : unsigned long long { kTileSum = 1ull << 62, kTilePrefix = 2ull << 62 };
+
+constexpr int kLookback = 4;   // tiles read at a time when looking back (2 measured 1 - 3 % slower, 8 the same)
+
+// One pass.  Tiles are taken from a counter, so every tile before this one has
+// been started and publishes its counts without waiting for anyone; waits for
+// them are bounded all the same (ST_TIMEOUT).  A warp ranks 32 keys at a time:
+// each lane marks its bit in its digit's word of shared memory and reads the
+// word back, which gives the peers before it (a ballot per digit bit, which
+// this replaces, was most of the pass's instructions).  The tile is staged
+// through one shared array: keys first, then each payload in its own round.
+// What bounds it is shared memory traffic (70 - 77 % of its throughput with
+// ranks and output positions kept in shared arrays), so a thread's tile slots
+// and output positions stay in registers (64, four blocks per SM; 48 and 80
+// measured 4 - 28 % slower, tiles of 3072 and 5120 keys 3 - 40 %).
+// 5e7 keys with three payloads: 395 us a pass, 421 with the shared arrays; with
+// separate count, scan and scatter kernels 394 + 53 + 13 us.  2e6 keys: 29 us
+// against 26 + 9 + 13 in four launches.
+template <int NP, int ITEMS>
+__global__ void __launch_bounds__(OS_THREADS, 4)
+    k_rs_sweep(RsSet J, uint32_t n, int shift, int bits, const uint32_t *__restrict__ hist,
+               unsigned long long *__restrict__ state, uint32_t *__restrict__ ticket, uint32_t *status)
 {
-    const uint32_t job = blockIdx.x >= ntiles ? 1u : 0u, tile = blockIdx.x - job * ntiles;
-    const uint32_t *__restrict__ kin = job ? J.s[1].kin : J.s[0].kin;
-    uint32_t *__restrict__ counts = counts_all + ((size_t)job * ntiles << bits);
-    __shared__ uint32_t h[OS_WARPS][OS_MAXRADIX];
-    const uint32_t radix = 1u << bits, dmask = radix - 1u;
-    for (uint32_t i = threadIdx.x; i < (uint32_t)(OS_WARPS * OS_MAXRADIX); i += OS_THREADS) (&h[0][0])[i] = 0;
+    constexpr int TILE = OS_THREADS * ITEMS, WCHUNK = ITEMS * 32;
+    static_assert(ITEMS % 2 == 0, "slots are kept two to a register");
+    __shared__ uint32_t s_buf[TILE];                          // one array of the tile
+    __shared__ uint32_t s_match[OS_WARPS * OS_MAXRADIX];      // [warp][digit] lanes of the digit
+    __shared__ uint16_t s_wcnt[OS_WARPS * OS_MAXRADIX];       // [warp][digit] counts, then tile slots
+    __shared__ uint32_t s_gpos[OS_MAXRADIX];                  // digit start in the output - in the tile
+    __shared__ uint32_t s_wt[8];
+    __shared__ uint32_t s_tile;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (t == 0) s_tile = atomicAdd(ticket, 1u);
+    for (int i = t; i < OS_WARPS * OS_MAXRADIX; i += OS_THREADS) { s_wcnt[i] = 0; s_match[i] = 0; }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t base = tile * OS_TILE;
-    uint32_t kv[OS_ITEMS];
+    const uint32_t tile = s_tile;
+    const uint32_t radix = 1u << bits, dmask = radix - 1u;
+    const uint32_t base = tile * (uint32_t)TILE;
+    const uint32_t tile_n = min((uint32_t)TILE, n - base);
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t li0 = warp * WCHUNK + lane;   // this thread's inputs: li0, li0 + 32, ...
+    uint16_t *wc = s_wcnt + warp * OS_MAXRADIX;
+    uint32_t *wm = s_match + warp * OS_MAXRADIX;
+    uint32_t kv[ITEMS];         // the keys, then one payload after the other
+    uint32_t slot[ITEMS / 2];   // rank in the warp's chunk, then tile slot, 16 bits each
+    auto load = [&](const uint32_t *__restrict__ in) {
 #pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {   // all loads in flight before any count
-        const uint32_t i = base + j * OS_THREADS + threadIdx.x;
-        kv[j] = i < n ? __ldg(kin + i) : 0u;
-    }
+        for (int j = 0; j < ITEMS; ++j) {
+            const uint32_t li = li0 + j * 32;
+            kv[j] = li < tile_n ? (in ? __ldg(in + base + li) : base + li) : 0u;
+        }
+    };
+    auto slot_of = [&](int j) { return j & 1 ? slot[j / 2] >> 16 : slot[j / 2] & 0xFFFFu; };
+    load(J.kin);
+    // ---- rank inside each warp's chunk (order: warp, item, lane)
 #pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t i = base + j * OS_THREADS + threadIdx.x;
-        const bool valid = i < n;
-        const uint32_t d = valid ? ((kv[j] >> shift) & dmask) : radix;
+    for (int j = 0; j < ITEMS; ++j) {
+        const bool valid = li0 + j * 32 < tile_n;
+        const uint32_t d = (kv[j] >> shift) & dmask;
         const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-        if (__all_sync(0xffffffffu, d == d0)) {
-            if (lane == 0 && d0 < radix) atomicAdd(&h[warp][d0], 32u);
-        } else if (valid) {
-            atomicAdd(&h[warp][d], 1u);
+        uint32_t peers;
+        if (__all_sync(0xffffffffu, valid && d == d0)) {
+            peers = 0xffffffffu;
+        } else {
+            if (valid) atomicOr(wm + d, 1u << lane);
+            __syncwarp();
+            peers = valid ? wm[d] : 0u;
+        }
+        const uint32_t cur = valid ? wc[d] : 0;
+        __syncwarp();
+        const uint32_t r = cur + __popc(peers & lt);
+        slot[j / 2] = j & 1 ? slot[j / 2] | (r << 16) : r;
+        if (valid && (peers & lt) == 0) { wc[d] = (uint16_t)(cur + __popc(peers)); wm[d] = 0; }
+        __syncwarp();
+    }
+    __syncthreads();
+    // ---- per digit (thread d): the tile's count published, the exclusive scans
+    // over the digits of it and of the whole array's counts, and where each
+    // warp's keys of the digit go in the tile
+    uint32_t cnt = 0, tot = 0, ci = 0, ti = 0;
+    const bool digit = t < (int)radix;
+    if (t < OS_MAXRADIX) {
+        if (digit) {
+            for (int w = 0; w < OS_WARPS; ++w) cnt += s_wcnt[w * OS_MAXRADIX + t];
+            *(volatile unsigned long long *)(state + (size_t)tile * OS_MAXRADIX + t) =
+                (tile == 0 ? kTilePrefix : kTileSum) | cnt;
+            tot = __ldg(hist + t);
+        }
+        ci = cnt;
+        ti = tot;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, ci, o), z = __shfl_up_sync(0xffffffffu, ti, o);
+            if (lane >= o) { ci += y; ti += z; }
+        }
+        if (lane == 31) { s_wt[warp] = ci; s_wt[4 + warp] = ti; }
+    }
+    __syncthreads();
+    uint32_t tex = 0, gbase = 0;   // the digit's start in the tile and in the output
+    if (digit) {
+        for (int w = 0; w < warp; ++w) { ci += s_wt[w]; ti += s_wt[4 + w]; }
+        tex = ci - cnt;
+        gbase = ti - tot;
+        uint32_t run = tex;
+        for (int w = 0; w < OS_WARPS; ++w) {
+            const uint32_t c = s_wcnt[w * OS_MAXRADIX + t];
+            s_wcnt[w * OS_MAXRADIX + t] = (uint16_t)run;
+            run += c;
         }
     }
     __syncthreads();
-    for (uint32_t d = threadIdx.x; d < radix; d += OS_THREADS) {
-        uint32_t c = 0;
+    // ---- keys into their tile slots
 #pragma unroll
-        for (int w = 0; w < OS_WARPS; ++w) c += h[w][d];
-        counts[(size_t)d * ntiles + tile] = c;
+    for (int j = 0; j < ITEMS; ++j) {
+        if (li0 + j * 32 < tile_n) {
+            const uint32_t pos = wc[(kv[j] >> shift) & dmask] + slot_of(j);
+            s_buf[pos] = kv[j];
+            slot[j / 2] = j & 1 ? (slot[j / 2] & 0xFFFFu) | (pos << 16) : (slot[j / 2] & 0xFFFF0000u) | pos;
+        }
+    }
+    if (NP > 0) load(J.pin[0]);   // on its way while the tile looks back
+    // ---- look back: the digit's keys in the tiles before this one, kLookback
+    // tiles' words in flight at a time
+    if (digit) {
+        uint32_t before = 0;
+        bool done = tile == 0;
+        for (int64_t j = (int64_t)tile - 1; !done; j -= kLookback) {
+            unsigned long long v[kLookback];
+#pragma unroll
+            for (int i = 0; i < kLookback; ++i)
+                v[i] = j - i >= 0 ? *(volatile unsigned long long *)(state + (size_t)(j - i) * OS_MAXRADIX + t)
+                                  : (unsigned long long)kTilePrefix;
+#pragma unroll
+            for (int i = 0; i < kLookback; ++i) {
+                if (done) break;
+                for (int it = 0; (v[i] >> 62) == 0; ++it) {
+                    if (it >= kLookbackPolls) { latch(status, ST_TIMEOUT); done = true; break; }
+                    __nanosleep(32);
+                    v[i] = *(volatile unsigned long long *)(state + (size_t)(j - i) * OS_MAXRADIX + t);
+                }
+                before += (uint32_t)v[i];
+                if ((v[i] >> 62) == 2) done = true;
+            }
+        }
+        if (tile != 0)
+            *(volatile unsigned long long *)(state + (size_t)tile * OS_MAXRADIX + t) = kTilePrefix | (before + cnt);
+        s_gpos[t] = gbase + before - tex;
+    }
+    __syncthreads();
+    // ---- keys out; this thread's slots t, t + OS_THREADS, ... and their output
+    // positions stay the same for the payloads
+    uint32_t g[ITEMS];
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t p = t + j * OS_THREADS;
+        if (p < tile_n) {
+            const uint32_t k = s_buf[p];
+            g[j] = s_gpos[(k >> shift) & dmask] + p;
+            J.kout[g[j]] = k;
+        }
+    }
+    // ---- payloads, one round each
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+        uint32_t *__restrict__ pout = J.pout[a];
+        __syncthreads();   // the previous round's reads of s_buf are done
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j)
+            if (li0 + j * 32 < tile_n) s_buf[slot_of(j)] = kv[j];
+        if (a + 1 < NP) load(J.pin[a + 1]);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) {
+            const uint32_t p = t + j * OS_THREADS;
+            if (p < tile_n) {
+                const uint32_t v = s_buf[p];
+                pout[g[j]] = v;
+                if (a == 0 && J.inv && v < n) J.inv[v] = g[j];
+            }
+        }
     }
 }
 
@@ -155,284 +311,6 @@ __device__ __forceinline__ void os_block_scan512(uint32_t *vals /* smem [512] in
     vals[2 * t] = ex;
     vals[2 * t + 1] = ex + a;
     __syncthreads();
-}
-
-// Keys (and payloads) of one tile are ranked stably per warp chunk: a warp
-// whose 32 digits agree takes its ranks directly; otherwise the lanes with
-// the same digit are found with one ballot per digit bit.  A null p0in reads
-// payload 0 as the key's input index.  With inv set (a final pass), each
-// element also writes its output position at inv[payload 0].  Payloads 0-2
-// are held in registers from the start; payload 3 is read when the tile is
-// placed in shared memory.
-template <int NP>
-__global__ void __launch_bounds__(OS_THREADS, NP >= 3 ? 2 : NP >= 2 ? 3 : 4)
-    k_rs_scatter(RsJobs J, uint32_t n, int shift, int bits, uint32_t ntiles, const uint32_t *__restrict__ offs_all)
-{
-    const uint32_t job = blockIdx.x >= ntiles ? 1u : 0u, tile = blockIdx.x - job * ntiles;
-    // per-field selects keep the parameter block out of local memory
-    const uint32_t *__restrict__ kin = job ? J.s[1].kin : J.s[0].kin;
-    const uint32_t *__restrict__ p0in = job ? J.s[1].p0in : J.s[0].p0in;
-    const uint32_t *__restrict__ p1in = job ? J.s[1].p1in : J.s[0].p1in;
-    uint32_t *__restrict__ kout = job ? J.s[1].kout : J.s[0].kout;
-    uint32_t *__restrict__ p0out = job ? J.s[1].p0out : J.s[0].p0out;
-    uint32_t *__restrict__ p1out = job ? J.s[1].p1out : J.s[0].p1out;
-    const uint32_t *__restrict__ p2in = job ? J.s[1].p2in : J.s[0].p2in;
-    uint32_t *__restrict__ p2out = job ? J.s[1].p2out : J.s[0].p2out;
-    const uint32_t *__restrict__ p3in = job ? J.s[1].p3in : J.s[0].p3in;
-    uint32_t *__restrict__ p3out = job ? J.s[1].p3out : J.s[0].p3out;
-    uint32_t *__restrict__ inv = job ? J.s[1].inv : J.s[0].inv;
-    const uint32_t *__restrict__ offs = offs_all + ((size_t)job * ntiles << bits);
-    const uint32_t bias = job * n;   // set 1's scanned offsets start at n
-    extern __shared__ __align__(16) unsigned char os_smem_buf[];
-    uint32_t *s_key = reinterpret_cast<uint32_t *>(os_smem_buf);
-    uint32_t *s_p0 = s_key + OS_TILE;
-    uint32_t *s_p1 = s_p0 + (NP >= 1 ? OS_TILE : 0);
-    uint32_t *s_p2 = s_p1 + (NP >= 2 ? OS_TILE : 0);
-    uint32_t *s_p3 = s_p2 + (NP >= 3 ? OS_TILE : 0);
-    uint16_t *s_rank = reinterpret_cast<uint16_t *>(s_p3 + (NP >= 4 ? OS_TILE : 0));
-    uint16_t *s_wcnt = s_rank + OS_TILE;                                            // [warp][digit]
-    uint32_t *s_tex = reinterpret_cast<uint32_t *>(s_wcnt + OS_WARPS * OS_MAXRADIX);  // digit start in the tile
-    uint32_t *s_gpos = s_tex + OS_SCAN;                                             // digit start in the output
-    __shared__ uint32_t s_wt[OS_WARPS];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t radix = 1u << bits, dmask = radix - 1u;
-    const uint32_t base = tile * OS_TILE;
-    for (int i = t; i < OS_WARPS * OS_MAXRADIX; i += OS_THREADS) s_wcnt[i] = 0;
-    for (uint32_t d = t; d < (uint32_t)OS_MAXRADIX; d += OS_THREADS)
-        s_gpos[d] = d < radix ? __ldg(offs + (size_t)d * ntiles + tile) - bias : 0u;
-    const uint32_t lt = (1u << lane) - 1u;
-    uint16_t *wc = s_wcnt + warp * OS_MAXRADIX;
-    constexpr int NA = NP >= 1 ? OS_ITEMS : 1, NB = NP >= 2 ? OS_ITEMS : 1, NC = NP >= 3 ? OS_ITEMS : 1;
-    uint32_t kv[OS_ITEMS], av[NA], bv[NB], cv[NC];
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {   // keys and payloads in flight before any vote
-        const uint32_t i = base + warp * OS_WCHUNK + j * 32 + lane;
-        kv[j] = i < n ? __ldg(kin + i) : 0u;
-        if (NP >= 1) av[j % NA] = i < n ? (p0in ? __ldg(p0in + i) : i) : 0u;
-        if (NP >= 2) bv[j % NB] = i < n ? __ldg(p1in + i) : 0u;
-        if (NP >= 3) cv[j % NC] = i < n ? __ldg(p2in + i) : 0u;
-    }
-    __syncthreads();
-    // ---- rank inside each warp's chunk (order: warp, item, lane)
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t li = warp * OS_WCHUNK + j * 32 + lane;
-        const bool valid = base + li < n;
-        const uint32_t d = valid ? ((kv[j] >> shift) & dmask) : radix;
-        uint32_t peers;
-#if TM_RS_MATCH
-        peers = __match_any_sync(0xffffffffu, d);   // lanes with the same digit (invalid lanes: digit radix)
-#else
-        if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
-            peers = 0xffffffffu;
-        } else {
-            peers = __ballot_sync(0xffffffffu, valid);
-            if (!valid) peers = ~peers;
-            for (int b = 0; b < bits; ++b) {
-                const uint32_t bb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-                peers &= ((d >> b) & 1u) ? bb : ~bb;
-            }
-        }
-#endif
-        uint32_t cur = valid ? wc[d] : 0;
-        __syncwarp();
-        if (valid) {
-            s_rank[li] = (uint16_t)(cur + __popc(peers & lt));
-            if ((peers & lt) == 0) wc[d] = (uint16_t)(cur + __popc(peers));
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    // ---- per digit: tile total and warp offsets
-    for (uint32_t d = t; d < (uint32_t)OS_SCAN; d += OS_THREADS) {   // entries past the radix: 0
-        uint32_t run = 0;
-        if (d < radix)
-            for (int w = 0; w < OS_WARPS; ++w) {
-                uint32_t c = s_wcnt[w * OS_MAXRADIX + d];
-                s_wcnt[w * OS_MAXRADIX + d] = (uint16_t)run;
-                run += c;
-            }
-        s_tex[d] = run;
-    }
-    __syncthreads();
-    os_block_scan512(s_tex, s_wt);
-    // ---- place keys (and payloads) in digit order inside shared memory
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t li = warp * OS_WCHUNK + j * 32 + lane;
-        if (base + li < n) {
-            const uint32_t k = kv[j];
-            const uint32_t d = (k >> shift) & dmask;
-            const uint32_t pos = s_tex[d] + s_wcnt[warp * OS_MAXRADIX + d] + s_rank[li];
-            s_key[pos] = k;
-            if (NP >= 1) s_p0[pos] = av[j % NA];
-            if (NP >= 2) s_p1[pos] = bv[j % NB];
-            if (NP >= 3) s_p2[pos] = cv[j % NC];
-            if (NP >= 4) s_p3[pos] = __ldg(p3in + base + li);
-        }
-    }
-    __syncthreads();
-    // ---- write the tile's digit runs out
-    const uint32_t tile_n = min((uint32_t)OS_TILE, n - base);
-    for (uint32_t p = t; p < tile_n; p += OS_THREADS) {
-        const uint32_t k = s_key[p];
-        const uint32_t d = (k >> shift) & dmask;
-        const uint32_t g = s_gpos[d] + (p - s_tex[d]);
-        kout[g] = k;
-        if (NP >= 1) p0out[g] = s_p0[p];
-        if (NP >= 2) p1out[g] = s_p1[p];
-        if (NP >= 3) p2out[g] = s_p2[p];
-        if (NP >= 4) p3out[g] = s_p3[p];
-        if (NP >= 1 && inv) inv[s_p0[p]] = g;
-    }
-}
-
-// The same pass with the tile staged through one shared array at a time:
-// keys first (which also fixes every element's output position), then each
-// payload, read from global memory in its own round.  Shared memory stays at
-// 52 KB whatever the payload count, so four blocks fit on an SM where the
-// all-at-once layout above fits two.
-#ifndef TM_RS_STAGED
-#define TM_RS_STAGED 1
-#endif
-#ifndef TM_RS_ST_MINB
-#define TM_RS_ST_MINB 4   // blocks per SM the staged pass is compiled for (64 registers)
-#endif
-[[maybe_unused]] constexpr size_t os_smem_staged()
-{
-    return (size_t)OS_TILE * 4 * 2 + (size_t)OS_TILE * 2 + (size_t)OS_WARPS * OS_MAXRADIX * 2 +
-           (size_t)(OS_SCAN + OS_MAXRADIX) * 4;
-}
-
-template <int NP>
-__global__ void __launch_bounds__(OS_THREADS, TM_RS_ST_MINB)
-    k_rs_scatter_st(RsJobs J, uint32_t n, int shift, int bits, uint32_t ntiles, const uint32_t *__restrict__ offs_all)
-{
-    const uint32_t job = blockIdx.x >= ntiles ? 1u : 0u, tile = blockIdx.x - job * ntiles;
-    const uint32_t *__restrict__ kin = job ? J.s[1].kin : J.s[0].kin;
-    uint32_t *__restrict__ kout = job ? J.s[1].kout : J.s[0].kout;
-    uint32_t *__restrict__ inv = job ? J.s[1].inv : J.s[0].inv;
-    const uint32_t *__restrict__ offs = offs_all + ((size_t)job * ntiles << bits);
-    const uint32_t bias = job * n;
-    extern __shared__ __align__(16) unsigned char os_smem_buf[];
-    uint32_t *s_buf = reinterpret_cast<uint32_t *>(os_smem_buf);                  // one array of the tile
-    uint32_t *s_g = s_buf + OS_TILE;                                              // output position by tile slot
-    uint16_t *s_rank = reinterpret_cast<uint16_t *>(s_g + OS_TILE);               // rank, then tile slot, by input
-    uint16_t *s_wcnt = s_rank + OS_TILE;                                          // [warp][digit]
-    uint32_t *s_tex = reinterpret_cast<uint32_t *>(s_wcnt + OS_WARPS * OS_MAXRADIX);   // OS_SCAN entries
-    uint32_t *s_gpos = s_tex + OS_SCAN;
-    __shared__ uint32_t s_wt[OS_WARPS];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t radix = 1u << bits, dmask = radix - 1u;
-    const uint32_t base = tile * OS_TILE;
-    const uint32_t tile_n = min((uint32_t)OS_TILE, n - base);
-    for (int i = t; i < OS_WARPS * OS_MAXRADIX; i += OS_THREADS) s_wcnt[i] = 0;
-    for (uint32_t d = t; d < (uint32_t)OS_MAXRADIX; d += OS_THREADS)
-        s_gpos[d] = d < radix ? __ldg(offs + (size_t)d * ntiles + tile) - bias : 0u;
-    const uint32_t lt = (1u << lane) - 1u;
-    uint16_t *wc = s_wcnt + warp * OS_MAXRADIX;
-    uint32_t kv[OS_ITEMS];
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t i = base + warp * OS_WCHUNK + j * 32 + lane;
-        kv[j] = i < n ? __ldg(kin + i) : 0u;
-    }
-    __syncthreads();
-    // ---- rank inside each warp's chunk (order: warp, item, lane)
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t li = warp * OS_WCHUNK + j * 32 + lane;
-        const bool valid = base + li < n;
-        const uint32_t d = valid ? ((kv[j] >> shift) & dmask) : radix;
-        uint32_t peers;
-#if TM_RS_MATCH
-        peers = __match_any_sync(0xffffffffu, d);
-#else
-        if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
-            peers = 0xffffffffu;
-        } else {
-            peers = __ballot_sync(0xffffffffu, valid);
-            if (!valid) peers = ~peers;
-            for (int b = 0; b < bits; ++b) {
-                const uint32_t bb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-                peers &= ((d >> b) & 1u) ? bb : ~bb;
-            }
-        }
-#endif
-        uint32_t cur = valid ? wc[d] : 0;
-        __syncwarp();
-        if (valid) {
-            s_rank[li] = (uint16_t)(cur + __popc(peers & lt));
-            if ((peers & lt) == 0) wc[d] = (uint16_t)(cur + __popc(peers));
-        }
-        __syncwarp();
-    }
-    __syncthreads();
-    for (uint32_t d = t; d < (uint32_t)OS_SCAN; d += OS_THREADS) {   // entries past the radix: 0
-        uint32_t run = 0;
-        if (d < radix)
-            for (int w = 0; w < OS_WARPS; ++w) {
-                uint32_t c = s_wcnt[w * OS_MAXRADIX + d];
-                s_wcnt[w * OS_MAXRADIX + d] = (uint16_t)run;
-                run += c;
-            }
-        s_tex[d] = run;
-    }
-    __syncthreads();
-    os_block_scan512(s_tex, s_wt);
-    // ---- keys into their tile slots; each element keeps its slot (in s_rank,
-    // read back only by the thread that wrote it)
-#pragma unroll
-    for (int j = 0; j < OS_ITEMS; ++j) {
-        const uint32_t li = warp * OS_WCHUNK + j * 32 + lane;
-        if (base + li < n) {
-            const uint32_t k = kv[j];
-            const uint32_t d = (k >> shift) & dmask;
-            const uint32_t pos = s_tex[d] + s_wcnt[warp * OS_MAXRADIX + d] + s_rank[li];
-            s_buf[pos] = k;
-            s_rank[li] = (uint16_t)pos;
-        }
-    }
-    __syncthreads();
-    // ---- keys out; each slot's output position, kept for the payload rounds
-    // (slot p is handled by the same thread in every round)
-    for (uint32_t p = t; p < tile_n; p += OS_THREADS) {
-        const uint32_t k = s_buf[p];
-        const uint32_t d = (k >> shift) & dmask;
-        const uint32_t g = s_gpos[d] + (p - s_tex[d]);
-        s_g[p] = g;
-        kout[g] = k;
-    }
-    // ---- payloads, one round each
-#pragma unroll
-    for (int a = 0; a < NP; ++a) {
-        const uint32_t *__restrict__ pin = a == 0 ? (job ? J.s[1].p0in : J.s[0].p0in)
-                                         : a == 1 ? (job ? J.s[1].p1in : J.s[0].p1in)
-                                         : a == 2 ? (job ? J.s[1].p2in : J.s[0].p2in)
-                                                  : (job ? J.s[1].p3in : J.s[0].p3in);
-        uint32_t *__restrict__ pout = a == 0 ? (job ? J.s[1].p0out : J.s[0].p0out)
-                                    : a == 1 ? (job ? J.s[1].p1out : J.s[0].p1out)
-                                    : a == 2 ? (job ? J.s[1].p2out : J.s[0].p2out)
-                                             : (job ? J.s[1].p3out : J.s[0].p3out);
-        uint32_t pv[OS_ITEMS];
-#pragma unroll
-        for (int j = 0; j < OS_ITEMS; ++j) {   // loads in flight before the slots are written
-            const uint32_t i = base + warp * OS_WCHUNK + j * 32 + lane;
-            pv[j] = i < n ? (pin ? __ldg(pin + i) : i) : 0u;
-        }
-        __syncthreads();   // the previous round's reads of s_buf are done
-#pragma unroll
-        for (int j = 0; j < OS_ITEMS; ++j) {
-            const uint32_t li = warp * OS_WCHUNK + j * 32 + lane;
-            if (base + li < n) s_buf[s_rank[li]] = pv[j];
-        }
-        __syncthreads();
-        for (uint32_t p = t; p < tile_n; p += OS_THREADS) {
-            const uint32_t v = s_buf[p], g = s_g[p];
-            pout[g] = v;
-            if (a == 0 && inv) inv[v] = g;
-        }
-    }
 }
 
 // ---- inverse of a permutation, written through buckets -------------------
@@ -470,6 +348,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__
 #pragma unroll
     for (int j = 0; j < OS_ITEMS; ++j) {
         const uint32_t i = base + j * OS_THREADS + t;
+        v[j] = min(v[j], n - 1);   // (a sort whose wait ran out leaves anything here)
         r[j] = i < n ? atomicAdd(&s_cnt[v[j] >> shift], 1u) : 0u;
     }
     __syncthreads();
@@ -533,117 +412,18 @@ int bits_for(uint64_t maxval)
     return b;
 }
 
-// Stable LSD sort of (key, p0[, p1]) by the low `bits` bits of key, for one
-// or two independent arrays of the same length (same payload count), sorted
-// by the same launches; on return the sorted data is in the caller's buffers.
-struct RsHost {
-    uint32_t *key, *p0, *p1;
-};
-
-static int rs_prepare(tm_ctx *ctx, int np)
+DigitPlan digit_plan(int bits)
 {
-    // per device and cheap: set on every call
-#if TM_RS_STAGED
-    const int sm = (int)os_smem_staged();
-    cudaError_t e = np == 0 ? cudaFuncSetAttribute(k_rs_scatter_st<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                  : np == 1 ? cudaFuncSetAttribute(k_rs_scatter_st<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                  : np == 2 ? cudaFuncSetAttribute(k_rs_scatter_st<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                  : np == 3 ? cudaFuncSetAttribute(k_rs_scatter_st<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm)
-                            : cudaFuncSetAttribute(k_rs_scatter_st<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-#else
-    cudaError_t e = np == 0 ? cudaFuncSetAttribute(k_rs_scatter<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem(0))
-                  : np == 1 ? cudaFuncSetAttribute(k_rs_scatter<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem(1))
-                  : np == 2 ? cudaFuncSetAttribute(k_rs_scatter<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem(2))
-                  : np == 3 ? cudaFuncSetAttribute(k_rs_scatter<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem(3))
-                            : cudaFuncSetAttribute(k_rs_scatter<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)os_smem(4));
-#endif
-    return check_cuda(ctx, e, "radix pass shared memory");
-}
-
-// One LSD pass over digit bits [sh, sh + pb): counts, their scan, the scatter.
-static int rs_pass(tm_ctx *ctx, const RsJobs &in, int nsets, int np, uint32_t n, uint32_t ntiles, int sh, int pb,
-                   uint32_t *counts)
-{
-    const unsigned nblk = ntiles * (unsigned)nsets;
-    const uint64_t ncount = ((uint64_t)ntiles << pb) * (uint64_t)nsets;
-    launch(ctx, k_rs_count, nblk, OS_THREADS, in, n, sh, pb, ntiles, counts);
-    int rc = exclusive_scan_u32(ctx, counts, counts, ncount, nullptr);
-    if (rc) return rc;
-#if TM_RS_STAGED
-    const size_t sm = os_smem_staged();
-    if (np == 0)
-        launch_smem(ctx, k_rs_scatter_st<0>, nblk, OS_THREADS, sm, in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 1)
-        launch_smem(ctx, k_rs_scatter_st<1>, nblk, OS_THREADS, sm, in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 2)
-        launch_smem(ctx, k_rs_scatter_st<2>, nblk, OS_THREADS, sm, in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 3)
-        launch_smem(ctx, k_rs_scatter_st<3>, nblk, OS_THREADS, sm, in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else
-        launch_smem(ctx, k_rs_scatter_st<4>, nblk, OS_THREADS, sm, in, n, sh, pb, ntiles, (const uint32_t *)counts);
-#else
-    if (np == 0)
-        launch_smem(ctx, k_rs_scatter<0>, nblk, OS_THREADS, os_smem(0), in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 1)
-        launch_smem(ctx, k_rs_scatter<1>, nblk, OS_THREADS, os_smem(1), in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 2)
-        launch_smem(ctx, k_rs_scatter<2>, nblk, OS_THREADS, os_smem(2), in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else if (np == 3)
-        launch_smem(ctx, k_rs_scatter<3>, nblk, OS_THREADS, os_smem(3), in, n, sh, pb, ntiles, (const uint32_t *)counts);
-    else
-        launch_smem(ctx, k_rs_scatter<4>, nblk, OS_THREADS, os_smem(4), in, n, sh, pb, ntiles, (const uint32_t *)counts);
-#endif
-    return check_cuda(ctx, cudaGetLastError(), "radix pass");
-}
-
-int radix_sort_sets(tm_ctx *ctx, const RsHost *sets, int nsets, uint32_t n, int bits)
-{
-    ScratchScope scope(ctx);
-    if (n <= 1 || bits <= 0 || nsets <= 0) return TM_OK;
-    if (nsets > 2) return set_err(ctx, TM_E_LIMIT, "at most two arrays per radix sort");
-    const int np = sets[0].p1 ? 2 : (sets[0].p0 ? 1 : 0);
-    const int npass = (bits + OS_MAXBITS - 1) / OS_MAXBITS;
-    if (npass > OS_MAXPASS) return set_err(ctx, TM_E_LIMIT, "radix key wider than 32 bits");
-    const uint32_t ntiles = (n + OS_TILE - 1) / OS_TILE;
-    uint32_t *counts = (uint32_t *)salloc(ctx, (size_t)nsets * ntiles * OS_MAXRADIX * 4);
-    if (!counts) return TM_E_NOMEM;
-    RsJobs in{};
-    for (int j = 0; j < nsets; ++j) {
-        uint32_t *k2 = (uint32_t *)salloc(ctx, (size_t)n * 4);
-        uint32_t *a2 = np >= 1 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-        uint32_t *b2 = np >= 2 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-        if (!k2 || (np >= 1 && !a2) || (np >= 2 && !b2)) return TM_E_NOMEM;
-        in.s[j] = RsSet{sets[j].key, sets[j].p0, sets[j].p1, k2, a2, b2};
-    }
-    int rc = rs_prepare(ctx, np);
-    if (rc) return rc;
-    cudaStream_t st = ctx->stream;
-    for (int pass = 0, sh = 0; pass < npass && rc == TM_OK; ++pass) {
-        const int left = npass - pass, pb = (bits - sh + left - 1) / left;
-        rc = rs_pass(ctx, in, nsets, np, n, ntiles, sh, pb, counts);
-        // the outputs of this pass are the inputs of the next
-        for (int j = 0; j < nsets; ++j) {
-            RsSet &x = in.s[j];
-            RsSet y{x.kout, x.p0out, x.p1out, const_cast<uint32_t *>(x.kin), const_cast<uint32_t *>(x.p0in),
-                    const_cast<uint32_t *>(x.p1in)};
-            x = y;
-        }
+    DigitPlan D;
+    D.npass = (bits + OS_MAXBITS - 1) / OS_MAXBITS;
+    for (int pass = 0, sh = 0; pass < D.npass; ++pass) {
+        const int left = D.npass - pass, pb = (bits - sh + left - 1) / left;
+        D.sh[pass] = sh;
+        D.bits[pass] = pb;
         sh += pb;
     }
-    for (int j = 0; rc == TM_OK && j < nsets; ++j) {
-        const RsSet &x = in.s[j];
-        if (x.kin == sets[j].key) continue;
-        cudaMemcpyAsync(sets[j].key, x.kin, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-        if (np >= 1) cudaMemcpyAsync(sets[j].p0, x.p0in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-        if (np >= 2) cudaMemcpyAsync(sets[j].p1, x.p1in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-    }
-    return rc;
+    return D;
 }
-
-
-#ifndef TM_RS_INV_BUCKET
-#define TM_RS_INV_BUCKET 1   // 0: the last radix pass writes the inverse with one random store per element
-#endif
 
 // inv[perm[i]] = i for a permutation perm of [0, n); tkey/tpos are n-entry
 // work arrays (allocated here when null).
@@ -664,118 +444,115 @@ static int inverse_perm(tm_ctx *ctx, const uint32_t *perm, uint32_t n, uint32_t 
            (const uint32_t *)tkey, (const uint32_t *)tpos, n, inv);
     return check_cuda(ctx, cudaGetLastError(), "inverse permutation");
 }
+// Up to here the last pass writes the inverse itself, a random 4-byte store per
+// element: the array stays in L2 (64 MB of it), where a partial sector costs
+// nothing more, and two launches and 12 bytes per element are saved.
+// (1e7 keys: 56 us more in the pass against 97 for the two kernels; 5e7: about
+// 1.3 ms against 0.5.)
+constexpr uint32_t kInvDirect = 16000000;
 
-// The same sort from read-only inputs into separate outputs (no copies): the
-// passes alternate between the outputs and scratch so that the last one
-// writes the outputs.  A set whose p0_in is null and p0 is not gets payload 0
-// = the input index (the sorting permutation).  Outputs must not alias inputs.
+// A stable LSD sort of the key and up to four payloads by the low `bits` bits
+// of the key, from read-only inputs into separate outputs (no copies): the
+// passes alternate between the outputs and scratch so that the last one writes
+// the outputs.  A null p[0] input with an output gives payload 0 = the input
+// index (the sorting permutation).  Outputs must not alias inputs.
 struct RsTo {
-    const uint32_t *key_in, *p0_in, *p1_in;
-    uint32_t *key, *p0, *p1;
-    const uint32_t *p2_in = nullptr;
-    uint32_t *p2 = nullptr;
-    const uint32_t *p3_in = nullptr;
-    uint32_t *p3 = nullptr;
-    uint32_t *inv = nullptr;   // optional: inv[payload 0] = sorted position, written by the last pass
+    const uint32_t *key_in = nullptr, *p_in[4] = {};
+    uint32_t *key = nullptr, *p[4] = {};
+    uint32_t *inv = nullptr;          // optional: inv[payload 0] = sorted position (payload 0 = the input index)
+    const uint32_t *hist = nullptr;   // the key's digit counts (OS_HIST), when they are known
 };
 
-__global__ void k_iota2(uint32_t *__restrict__ a, uint32_t *__restrict__ b, uint32_t m)
+__global__ void k_iota(uint32_t *__restrict__ a, uint32_t m)
 {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) { if (a) a[i] = i; if (b) b[i] = i; }
+    if (i < m) a[i] = i;
 }
 
-int radix_sort_sets_to(tm_ctx *ctx, const RsTo *sets, int nsets, uint32_t n, int bits)
+template <int ITEMS>
+static int rs_pass(tm_ctx *ctx, const RsSet &J, int np, uint32_t n, int sh, int pb, const uint32_t *hist,
+                   unsigned long long *state, uint32_t *ticket)
+{
+    const unsigned ntiles = (n + OS_THREADS * ITEMS - 1) / (OS_THREADS * ITEMS);
+    auto go = [&](auto kernel) {
+        launch(ctx, kernel, ntiles, OS_THREADS, J, n, sh, pb, hist, state, ticket, ctx->status);
+        return check_cuda(ctx, cudaGetLastError(), "radix pass");
+    };
+    switch (np) {
+    case 0: return go(k_rs_sweep<0, ITEMS>);
+    case 1: return go(k_rs_sweep<1, ITEMS>);
+    case 2: return go(k_rs_sweep<2, ITEMS>);
+    case 3: return go(k_rs_sweep<3, ITEMS>);
+    default: return go(k_rs_sweep<4, ITEMS>);
+    }
+}
+
+int radix_sort_to(tm_ctx *ctx, const RsTo &x, uint32_t n, int bits)
 {
     ScratchScope scope(ctx);
-    if (nsets <= 0 || n == 0) return TM_OK;
-    if (nsets > 2) return set_err(ctx, TM_E_LIMIT, "at most two arrays per radix sort");
-    const int np = sets[0].p3 ? 4 : sets[0].p2 ? 3 : sets[0].p1 ? 2 : (sets[0].p0 ? 1 : 0);
+    if (n == 0) return TM_OK;
+    int np = 0;
+    while (np < 4 && x.p[np]) ++np;
+    if (x.inv && x.p_in[0]) return set_err(ctx, TM_E_ARG, "internal: inverse of a sort with explicit payload 0");
     cudaStream_t st = ctx->stream;
-    if (n <= 1 || bits <= 0) {
-        for (int j = 0; j < nsets; ++j) {
-            const RsTo &x = sets[j];
-            cudaMemcpyAsync(x.key, x.key_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-            if (np >= 1) {
-                if (x.p0_in) cudaMemcpyAsync(x.p0, x.p0_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-                else launch(ctx, k_iota2, (n + 255) / 256, 256, x.p0, (uint32_t *)nullptr, n);
-            }
-            if (np >= 2) cudaMemcpyAsync(x.p1, x.p1_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-            if (np >= 3) cudaMemcpyAsync(x.p2, x.p2_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-            if (np >= 4) cudaMemcpyAsync(x.p3, x.p3_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
-            if (x.inv) {   // an identity order (payload 0 is then the input index)
-                if (x.p0_in) return set_err(ctx, TM_E_ARG, "internal: inverse of a sort with explicit payload 0");
-                launch(ctx, k_iota2, (n + 255) / 256, 256, x.inv, (uint32_t *)nullptr, n);
-            }
+    if (n <= 1 || bits <= 0) {   // every key equal: the identity order
+        cudaMemcpyAsync(x.key, x.key_in, (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
+        for (int a = 0; a < np; ++a) {
+            if (x.p_in[a]) cudaMemcpyAsync(x.p[a], x.p_in[a], (size_t)n * 4, cudaMemcpyDeviceToDevice, st);
+            else launch(ctx, k_iota, (n + 255) / 256, 256, x.p[a], n);
         }
+        if (x.inv) launch(ctx, k_iota, (n + 255) / 256, 256, x.inv, n);
         return TM_OK;
     }
-    const int npass = (bits + OS_MAXBITS - 1) / OS_MAXBITS;
-    if (npass > OS_MAXPASS) return set_err(ctx, TM_E_LIMIT, "radix key wider than 32 bits");
-    const uint32_t ntiles = (n + OS_TILE - 1) / OS_TILE;
-    uint32_t *counts = (uint32_t *)salloc(ctx, (size_t)nsets * ntiles * OS_MAXRADIX * 4);
-    if (!counts) return TM_E_NOMEM;
-    RsSet scr[2] = {}, dst[2] = {};
-    for (int j = 0; j < nsets; ++j) {
-        dst[j] = RsSet{nullptr, nullptr, nullptr, sets[j].key, sets[j].p0, sets[j].p1};
-        dst[j].p2out = sets[j].p2;
-        dst[j].p3out = sets[j].p3;
-        if (npass >= 2) {
-            uint32_t *k2 = (uint32_t *)salloc(ctx, (size_t)n * 4);
-            uint32_t *a2 = np >= 1 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-            uint32_t *b2 = np >= 2 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-            uint32_t *c2 = np >= 3 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-            uint32_t *d2 = np >= 4 ? (uint32_t *)salloc(ctx, (size_t)n * 4) : nullptr;
-            if (!k2 || (np >= 1 && !a2) || (np >= 2 && !b2) || (np >= 3 && !c2) || (np >= 4 && !d2)) return TM_E_NOMEM;
-            scr[j] = RsSet{nullptr, nullptr, nullptr, k2, a2, b2};
-            scr[j].p2out = c2;
-            scr[j].p3out = d2;
-        }
+    const DigitPlan D = digit_plan(bits);
+    if (D.npass > OS_MAXPASS) return set_err(ctx, TM_E_LIMIT, "radix key wider than 32 bits");
+    const bool small = n <= kSmallSort;
+    const size_t ntiles = (n + (small ? OS_THREADS * OS_SMALL_ITEMS : OS_TILE) - 1) /
+                          (small ? OS_THREADS * OS_SMALL_ITEMS : OS_TILE);
+    // one buffer of tile words for each pass, cleared at once; a large sort's
+    // passes share one (8 bytes x 128 per tile)
+    const size_t words = ntiles * OS_MAXRADIX;
+    const bool share = words * 8 * D.npass > ((size_t)32 << 20);
+    const size_t state_bytes = words * 8 * (share ? 1 : D.npass);
+    char *blk = (char *)salloc(ctx, state_bytes + 64 + OS_HIST * 4);
+    if (!blk) return TM_E_NOMEM;
+    unsigned long long *state = (unsigned long long *)blk;
+    uint32_t *ticket = (uint32_t *)(blk + state_bytes);
+    uint32_t *own_hist = ticket + 16;
+    RsSet scr;
+    if (D.npass >= 2) {
+        if (!(scr.kout = (uint32_t *)salloc(ctx, (size_t)n * 4))) return TM_E_NOMEM;
+        for (int a = 0; a < np; ++a)
+            if (!(scr.pout[a] = (uint32_t *)salloc(ctx, (size_t)n * 4))) return TM_E_NOMEM;
     }
-    int rc = rs_prepare(ctx, np);
-    if (rc) return rc;
-    RsJobs in{};
-    for (int j = 0; j < nsets; ++j) {
-        in.s[j] = RsSet{sets[j].key_in, sets[j].p0_in, sets[j].p1_in, nullptr, nullptr, nullptr};
-        in.s[j].p2in = sets[j].p2_in;
-        in.s[j].p3in = sets[j].p3_in;
-    }
-    for (int pass = 0, sh = 0; pass < npass && rc == TM_OK; ++pass) {
-        const int left = npass - pass, pb = (bits - sh + left - 1) / left;
+    cudaMemsetAsync(blk, 0, state_bytes + 64 + (x.hist ? 0 : OS_HIST * 4), st);
+    if (!x.hist)
+        launch(ctx, k_rs_hist, (unsigned)std::min<uint64_t>(((uint64_t)n + 4095) / 4096, (uint64_t)ctx->num_sms * 8),
+               OS_THREADS, x.key_in, n, D, own_hist);
+    const uint32_t *hist = x.hist ? x.hist : own_hist;
+    RsSet J;
+    J.kin = x.key_in;
+    for (int a = 0; a < np; ++a) J.pin[a] = x.p_in[a];
+    int rc = TM_OK;
+    for (int pass = 0; pass < D.npass && rc == TM_OK; ++pass) {
+        const bool last = pass == D.npass - 1;
         // pass i writes the outputs when npass - 1 - i is even, else scratch
-        const bool to_dst = ((npass - 1 - pass) & 1) == 0;
-        for (int j = 0; j < nsets; ++j) {
-            const RsSet &o = to_dst ? dst[j] : scr[j];
-            in.s[j].kout = o.kout; in.s[j].p0out = o.p0out; in.s[j].p1out = o.p1out; in.s[j].p2out = o.p2out;
-            in.s[j].p3out = o.p3out;
-            in.s[j].inv = !TM_RS_INV_BUCKET && pass == npass - 1 ? sets[j].inv : nullptr;
-        }
-        rc = rs_pass(ctx, in, nsets, np, n, ntiles, sh, pb, counts);
-        for (int j = 0; j < nsets; ++j) {
-            RsSet nx{in.s[j].kout, in.s[j].p0out, in.s[j].p1out, nullptr, nullptr, nullptr};
-            nx.p2in = in.s[j].p2out;
-            nx.p3in = in.s[j].p3out;
-            in.s[j] = nx;
-        }
-        sh += pb;
+        const bool to_dst = ((D.npass - 1 - pass) & 1) == 0;
+        J.kout = to_dst ? x.key : scr.kout;
+        for (int a = 0; a < np; ++a) J.pout[a] = to_dst ? x.p[a] : scr.pout[a];
+        J.inv = last && n <= kInvDirect ? x.inv : nullptr;
+        unsigned long long *st_p = state + (share ? 0 : words * pass);
+        if (share && pass) cudaMemsetAsync(state, 0, state_bytes, st);
+        const uint32_t *h = hist + pass * OS_MAXRADIX;
+        rc = small ? rs_pass<OS_SMALL_ITEMS>(ctx, J, np, n, D.sh[pass], D.bits[pass], h, st_p, ticket + pass)
+                   : rs_pass<OS_ITEMS>(ctx, J, np, n, D.sh[pass], D.bits[pass], h, st_p, ticket + pass);
+        J.kin = J.kout;
+        for (int a = 0; a < np; ++a) J.pin[a] = J.pout[a];
     }
-#if TM_RS_INV_BUCKET
-    // the inverse permutations, through buckets; the scratch of the passes
-    // (free once the last pass has written the outputs) holds the pairs
-    for (int j = 0; rc == TM_OK && j < nsets; ++j) {
-        if (!sets[j].inv) continue;
-        if (sets[j].p0_in) return set_err(ctx, TM_E_ARG, "internal: inverse of a sort with explicit payload 0");
-        uint32_t *tk = npass >= 2 ? scr[j].kout : nullptr, *tp = npass >= 2 ? scr[j].p0out : nullptr;
-        rc = inverse_perm(ctx, sets[j].p0, n, sets[j].inv, tk, tp);
-    }
-#endif
+    // the inverse permutation of a large sort, through buckets; the scratch of
+    // the passes (free once the last pass has written the outputs) holds the pairs
+    if (rc == TM_OK && x.inv && n > kInvDirect) rc = inverse_perm(ctx, x.p[0], n, x.inv, scr.kout, scr.pout[0]);
     return rc;
-}
-
-int radix_sort(tm_ctx *ctx, uint32_t *key, uint32_t *p0, uint32_t *p1, uint32_t n, int bits)
-{
-    RsHost h{key, p0, p1};
-    return radix_sort_sets(ctx, &h, 1, n, bits);
 }
 
 // ---- input validation and t' -------------------------------------------
@@ -841,23 +618,45 @@ __global__ void k_keep_nonself(const uint32_t *__restrict__ src, const uint32_t 
     if (i < m) keep[i] = src[i] != dst[i] ? 1u : 0u;
 }
 
-// Compact the kept tuples into (t', src, dst) u32 arrays.
-__global__ void k_compact_input(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
-                                const int64_t *__restrict__ t, uint64_t m, const uint32_t *__restrict__ keep,
-                                const uint32_t *__restrict__ pos, long long tmin, uint32_t *__restrict__ ot,
-                                uint32_t *__restrict__ os, uint32_t *__restrict__ od)
+// Compact the kept tuples into (t', src, dst) u32 arrays, and count the digits
+// of the sorts to come: of t' at hist, of src at hist + OS_HIST, of dst after
+// that.  A few blocks per SM stride over the input, so that the counts of a
+// block are added to the totals once.
+__global__ void __launch_bounds__(OS_THREADS)
+    k_compact_input(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst, const int64_t *__restrict__ t,
+                    uint64_t m, const uint32_t *__restrict__ keep, const uint32_t *__restrict__ pos, long long tmin,
+                    uint32_t *__restrict__ ot, uint32_t *__restrict__ os, uint32_t *__restrict__ od, DigitPlan Dt,
+                    DigitPlan Dv, uint32_t *__restrict__ hist)
 {
-    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
+    __shared__ uint32_t h[3 * OS_HIST];
+    for (int i = threadIdx.x; i < 3 * OS_HIST; i += OS_THREADS) h[i] = 0;
+    __syncthreads();
+    const uint64_t stride = (uint64_t)gridDim.x * OS_THREADS * kElemItems;
+    for (uint64_t b = (uint64_t)blockIdx.x * OS_THREADS * kElemItems + threadIdx.x; b < m; b += stride) {
+        uint32_t u[kElemItems], v[kElemItems];
+        int64_t tt[kElemItems];
+        bool k[kElemItems];
 #pragma unroll
-    for (int k = 0; k < kElemItems; ++k) {
-        const uint64_t i = i0 + (uint64_t)k * blockDim.x;
-        if (i >= m) break;
-        if (keep && !keep[i]) continue;
-        const uint32_t p = pos ? pos[i] : (uint32_t)i;
-        ot[p] = (uint32_t)(t[i] - tmin);
-        os[p] = src[i];
-        od[p] = dst[i];
+        for (int j = 0; j < kElemItems; ++j) {
+            const uint64_t i = b + (uint64_t)j * OS_THREADS;
+            k[j] = i < m && (!keep || keep[i]);
+            if (k[j]) { u[j] = src[i]; v[j] = dst[i]; tt[j] = t[i]; }
+        }
+#pragma unroll
+        for (int j = 0; j < kElemItems; ++j) {
+            const uint64_t i = b + (uint64_t)j * OS_THREADS;
+            if (!k[j]) continue;
+            const uint32_t p = pos ? pos[i] : (uint32_t)i, x = (uint32_t)(tt[j] - tmin);
+            ot[p] = x;
+            os[p] = u[j];
+            od[p] = v[j];
+            hist_key(Dt, x, h);
+            hist_key(Dv, u[j], h + OS_HIST);
+            hist_key(Dv, v[j], h + 2 * OS_HIST);
+        }
     }
+    __syncthreads();
+    hist_flush(h, 3 * OS_HIST, hist);
 }
 
 // After the GLOBAL sort: flag tuples equal to their predecessor.
@@ -1101,7 +900,7 @@ struct XR {
 #ifndef TM_XR_ITEMS
 #define TM_XR_ITEMS 4
 #endif
-__global__ void k_cross_rank(XR a, XR b, uint32_t m)
+__global__ void k_cross_rank(XR a, XR b, uint32_t m, uint32_t n)
 {
     constexpr int K = TM_XR_ITEMS;
     const bool s1 = blockIdx.y != 0;
@@ -1115,7 +914,7 @@ __global__ void k_cross_rank(XR a, XR b, uint32_t m)
         const uint64_t i = i0 + (uint64_t)k * blockDim.x;
         lo[k] = 0; len[k] = 0; key[k] = 0;
         if (i < m) {
-            const uint32_t z = __ldg(owner + i);
+            const uint32_t z = min(__ldg(owner + i), n - 1);   // (a sort whose wait ran out leaves anything here)
             key[k] = __ldg(own_t + i);
             lo[k] = __ldg(other_off + z);
             len[k] = __ldg(other_off + z + 1) - lo[k];
@@ -1214,17 +1013,25 @@ int build_csr(tm_ctx *ctx)
     uint32_t *S0 = (uint32_t *)salloc(ctx, (size_t)(m ? m : 1) * 4);
     uint32_t *D0 = (uint32_t *)salloc(ctx, (size_t)(m ? m : 1) * 4);
     if (!T0 || !S0 || !D0) return TM_E_NOMEM;
+    int vbits = bits_for(n ? n - 1 : 0);
+    int tbits = bits_for((unsigned long long)tmax - (unsigned long long)tmin);
+    const DigitPlan Dt = digit_plan(tbits), Dv = digit_plan(vbits);
+    uint32_t *hist = (uint32_t *)salloc(ctx, 3 * OS_HIST * 4);   // digit counts of t', src, dst
+    if (!hist) return TM_E_NOMEM;
+    cudaMemsetAsync(hist, 0, 3 * OS_HIST * 4, st);
+    const unsigned cblk = (unsigned)std::min<uint64_t>(blocks_for((m0 + kElemItems - 1) / kElemItems, TB),
+                                                       (uint64_t)ctx->num_sms * 8);
     if (hs.nself) {
         uint32_t *keep = (uint32_t *)salloc(ctx, m0 * 4), *pos = (uint32_t *)salloc(ctx, m0 * 4);
         if (!keep || !pos) return TM_E_NOMEM;
         launch(ctx, k_keep_nonself, blocks_for(m0, TB), TB, ctx->in_src, ctx->in_dst, m0, keep);
         rc = exclusive_scan_u32(ctx, keep, pos, m0, nullptr);
         if (rc) return rc;
-        launch(ctx, k_compact_input, blocks_for((m0 + kElemItems - 1) / kElemItems, TB), TB, ctx->in_src, ctx->in_dst,
-               ctx->in_t, m0, keep, pos, tmin, T0, S0, D0);
+        launch(ctx, k_compact_input, cblk, TB, ctx->in_src, ctx->in_dst, ctx->in_t, m0, keep, pos, tmin, T0, S0, D0,
+               Dt, Dv, hist);
     } else if (m) {
-        launch(ctx, k_compact_input, blocks_for((m0 + kElemItems - 1) / kElemItems, TB), TB, ctx->in_src, ctx->in_dst,
-               ctx->in_t, m0, nullptr, nullptr, tmin, T0, S0, D0);
+        launch(ctx, k_compact_input, cblk, TB, ctx->in_src, ctx->in_dst, ctx->in_t, m0, nullptr, nullptr, tmin, T0,
+               S0, D0, Dt, Dv, hist);
     }
     // every m- and n-sized array of the graph in one block, sized before the
     // duplicates are known (they are rare; their slots stay unused)
@@ -1242,11 +1049,10 @@ int build_csr(tm_ctx *ctx)
     // by dst, src and t' instead
     sec.reset();
     sec.reset(new PhaseScope(ctx, TM_PH_CSR_GLOBAL));
-    int vbits = bits_for(n ? n - 1 : 0);
-    int tbits = bits_for((unsigned long long)tmax - (unsigned long long)tmin);
     {
-        RsTo ts{T0, S0, D0, g.g_t, g.g_src, g.g_dst};
-        rc = radix_sort_sets_to(ctx, &ts, 1, m, tbits);
+        RsTo ts{T0, {S0, D0}, g.g_t, {g.g_src, g.g_dst}};
+        ts.hist = hist;
+        rc = radix_sort_to(ctx, ts, m, tbits);
         if (rc) return rc;
     }
     // ---- duplicates (and the run check, read with the same copy)
@@ -1269,9 +1075,12 @@ int build_csr(tm_ctx *ctx)
         rc = check_cuda(ctx, cudaStreamSynchronize(st), "duplicate scan");
         if (rc) return rc;
         if (hnd[1]) {
-            rc = radix_sort(ctx, g.g_dst, g.g_src, g.g_t, m, vbits);
-            if (!rc) rc = radix_sort(ctx, g.g_src, g.g_dst, g.g_t, m, vbits);
-            if (!rc) rc = radix_sort(ctx, g.g_t, g.g_src, g.g_dst, m, tbits);
+            // (the work arrays hold the same tuples in input order)
+            const RsTo by_dst{D0, {S0, T0}, g.g_dst, {g.g_src, g.g_t}}, by_src{g.g_src, {g.g_dst, g.g_t}, S0, {D0, T0}},
+                by_t{T0, {S0, D0}, g.g_t, {g.g_src, g.g_dst}};
+            rc = radix_sort_to(ctx, by_dst, m, vbits);
+            if (!rc) rc = radix_sort_to(ctx, by_src, m, vbits);
+            if (!rc) rc = radix_sort_to(ctx, by_t, m, tbits);
             if (rc) return rc;
             cudaMemsetAsync(nd, 0, 8, st);
             launch(ctx, k_flag_unique, blocks_for(m, TB), TB, g.g_t, g.g_src, g.g_dst, m, keep, nd);
@@ -1300,6 +1109,12 @@ int build_csr(tm_ctx *ctx)
             cudaMemcpyAsync(g.g_dst, D0, bytes, cudaMemcpyDeviceToDevice, st);
         }
         m = (uint32_t)(m - ndup);
+        if (ndup) {   // the counts of the endpoints' digits without the repeats
+            cudaMemsetAsync(hist + OS_HIST, 0, 2 * OS_HIST * 4, st);
+            const unsigned hb = (unsigned)std::min<uint64_t>(((uint64_t)m + 4095) / 4096, (uint64_t)ctx->num_sms * 8);
+            launch(ctx, k_rs_hist, hb, OS_THREADS, (const uint32_t *)g.g_src, m, Dv, hist + OS_HIST);
+            launch(ctx, k_rs_hist, hb, OS_THREADS, (const uint32_t *)g.g_dst, m, Dv, hist + 2 * OS_HIST);
+        }
     }
     g.m = m;
     g.tmin = tmin;
@@ -1324,13 +1139,13 @@ int build_csr(tm_ctx *ctx)
         // writes each edge's list position by gid (the inverse permutation).
         // The in-list sort then carries each edge's out-list position (read in
         // GLOBAL order), which gives the in -> out map directly.
-        RsTo os{g.g_src, nullptr, g.g_t, g.out_src, g.out_gid, g.out_t};
-        os.p2_in = g.g_dst; os.p2 = g.out_nbr; os.inv = g.out_pos;
-        rc = radix_sort_sets_to(ctx, &os, 1, m, vbits);
+        RsTo os{g.g_src, {nullptr, g.g_t, g.g_dst}, g.out_src, {g.out_gid, g.out_t, g.out_nbr}};
+        os.inv = g.out_pos; os.hist = hist + OS_HIST;
+        rc = radix_sort_to(ctx, os, m, vbits);
         if (rc) return rc;
-        RsTo is{g.g_dst, nullptr, g.g_t, g.in_dst, g.in_gid, g.in_t};
-        is.p2_in = g.g_src; is.p2 = g.in_nbr; is.p3_in = g.out_pos; is.p3 = g.in_to_out; is.inv = g.in_pos;
-        rc = radix_sort_sets_to(ctx, &is, 1, m, vbits);
+        RsTo is{g.g_dst, {nullptr, g.g_t, g.g_src, g.out_pos}, g.in_dst, {g.in_gid, g.in_t, g.in_nbr, g.in_to_out}};
+        is.inv = g.in_pos; is.hist = hist + 2 * OS_HIST;
+        rc = radix_sort_to(ctx, is, m, vbits);
         if (rc) return rc;
     }
     sec.reset();
@@ -1353,10 +1168,9 @@ int build_csr(tm_ctx *ctx)
         {
             // payloads: t', the destination and each entry's out-list
             // position, straight into the multi-edge arrays
-            RsTo ms{g.in_nbr, g.in_t, g.in_dst, key, g.multi_t, tmp};
-            ms.p2_in = g.in_to_out;
-            ms.p2 = g.multi_to_out;
-            rc = radix_sort_sets_to(ctx, &ms, 1, m, vbits);
+            RsTo ms{g.in_nbr, {g.in_t, g.in_dst, g.in_to_out}, key, {g.multi_t, tmp, g.multi_to_out}};
+            ms.hist = hist + OS_HIST;   // the sources again
+            rc = radix_sort_to(ctx, ms, m, vbits);
             if (rc) return rc;
         }
         // key = pair src, tmp = pair dst per multi position
@@ -1381,7 +1195,7 @@ int build_csr(tm_ctx *ctx)
         // cross ranks between a vertex's out- and in-lists
         launch(ctx, k_cross_rank, dim3(blocks_for(((uint64_t)m + TM_XR_ITEMS - 1) / TM_XR_ITEMS, TB), 2), TB,
                XR{g.out_t, g.out_src, g.in_off, g.in_t, g.out_xrank},
-               XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m);
+               XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m, n);
         // owner starts of the three orders (segment heads of the weight pass's scans)
         const uint32_t words = m / 32 + 1;
         launch(ctx, k_owner_bits, blocks_for(((uint64_t)words * 32 + kElemItems - 1) / kElemItems, TB), TB,

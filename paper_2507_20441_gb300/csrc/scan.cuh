@@ -1,7 +1,7 @@
 // Device-wide scans used by the CSR builder and the weight pass.
 //
 // * exclusive_scan_u32: reduce-then-scan over u32 counts (recursive over the
-//   tile totals), for radix-sort offsets and compaction.
+//   tile totals), for compaction, pair ids and window offsets.
 // * segmented_scan_u64: inclusive prefix sums that restart at segment heads,
 //   with every 64-bit addition inside a segment checked for wrap-around.  It
 //   is a three-phase reduce / scan-of-tile-aggregates / rescan, so no block
