@@ -669,8 +669,13 @@ constexpr int kSampleThreads = TM_SAMPLE_THREADS;
 #define TM_RECS_SMEM 0   // per-sample records in local memory: L1 stays large for the searches
 #endif
 
+// Blocks per SM of the samplers with their records in local memory: the trace
+// measured 122 us at five against 134 at four and 136 at six (5e5 samples, 2e6
+// edges), a group of five motifs 431 at six against 466 at four (1e6 samples).
+constexpr int kTraceMinB = 5, kGroupMinB = 6;
+
 template <bool TRACE>
-__global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB) k_sample(DevGraph g, const DevPlan *__restrict__ plan,
+__global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph g, const DevPlan *__restrict__ plan,
                                                               SampleJob J, uint64_t seed, uint64_t first, uint64_t k,
                                                               Acc *acc, uint32_t *status, uint32_t *tr_gid,
                                                               uint64_t *tr_contrib, int32_t *tr_reason)
@@ -867,7 +872,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
 // pass and one stream of sampled trees: each sample is drawn and validated
 // once with the first plan and completed (Alg. 5) once per motif.
 template <int NM>
-__global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
+__global__ void __launch_bounds__(kSampleThreads, kGroupMinB)
     k_sample_group(DevGraph g, const DevPlan *__restrict__ plans, SampleJob J, uint64_t seed, uint64_t first,
                    uint64_t k, Acc *acc, uint32_t *status)
 {
@@ -940,8 +945,12 @@ struct BatchQuery {
     uint64_t seed, first, k;   // sample ids first .. first+k-1
 };
 
+// 64 registers, 1024 threads per SM: 7,200 us for 5.3e7 samples of 32 queries on
+// 2e6 edges; 1536 threads at 40 registers 8,326, 1280 7,722, 768 8,088 (all
+// seven tree sizes with their records in registers: 7,071 at 1.4 KB of spills).
+constexpr int kBatchThreads = 1024;
 template <int THREADS, int SMEM_RECS>
-__global__ void __launch_bounds__(THREADS, 1536 / THREADS) k_batch(DevGraph g, const BatchQuery *__restrict__ qs,
+__global__ void __launch_bounds__(THREADS, kBatchThreads / THREADS) k_batch(DevGraph g, const BatchQuery *__restrict__ qs,
                                                   const uint32_t *__restrict__ tile_base, uint32_t nq, uint32_t tile,
                                                   uint32_t *counter, Acc *accs, uint32_t *status)
 {
@@ -1076,13 +1085,16 @@ static void finish_result(tm_motif *mo, uint64_t k, const Acc &a, tm_result *out
     out->estimate = k ? W * h / (2.0 * (double)k) : 0.0;
 }
 
-// The register-record sampler for this plan's tree size; false when the plan
-// is not a spanning tree of nv - 1 nodes or needs the general DeriveCnt (the
-// caller launches k_sample).
+// Whether a plan's samples can be drawn with their records in registers: a
+// spanning tree of nv - 1 nodes that does not need the general DeriveCnt.
+static bool reg_plan(const DevPlan &P) { return P.nv == P.ntree + 1 && (P.nnt == 0 || P.derive_simple); }
+
+// The register-record sampler for this plan's tree size; false when there is
+// none (the caller launches k_sample).
 static bool launch_sample_reg(tm_ctx *ctx, const DevPlan &P, unsigned blocks, int threads, const DevPlan *dplan,
                               const SampleJob &J, uint64_t seed, uint64_t first, uint64_t k, Acc *dacc)
 {
-    if (P.nv != P.ntree + 1 || (P.nnt > 0 && !P.derive_simple)) return false;
+    if (!reg_plan(P)) return false;
     switch (P.ntree) {
 #define TM_REG_CASE(N) \
     case N: launch(ctx, k_sample_reg<N>, blocks, threads, ctx->g, dplan, J, seed, first, k, dacc, ctx->status); return true;
@@ -1115,7 +1127,8 @@ int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t f
     fill_job(mo, J, dplan);
     const int threads = kSampleThreads;
     uint64_t want = (k + threads - 1) / threads;
-    uint64_t cap = (uint64_t)ctx->num_sms * TM_SAMPLE_GRID_PER_SM;
+    const bool local = trace || !reg_plan(mo->plan);   // records in local memory: k_sample
+    uint64_t cap = (uint64_t)ctx->num_sms * (local ? kTraceMinB : TM_SAMPLE_GRID_PER_SM);
     unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min(want, cap));
     if (k / ((uint64_t)blocks * threads) >= 0xFFFFFFFFull)
         return set_err(ctx, TM_E_LIMIT, "too many samples in one call (split the range with first_index)");
