@@ -829,6 +829,80 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
     }
 }
 
+// Row offsets of the samples: the exclusive prefix of their counts in place,
+// and the total after them, in three launches over tiles of kListTile counts
+// (sums per tile, one block over the sums, the tiles again).  Taking the
+// counts to the host for it and the offsets back cost 640 of 830 us at 3e5
+// samples.  A sum past 2^64 latches ST_OVERFLOW.
+constexpr int kListItems = 8, kListTile = kSampleThreads * kListItems;
+
+// Exclusive prefix of v over the block and the block's total (u64, checked).
+__device__ __forceinline__ uint64_t list_block_scan(uint64_t v, uint64_t &total, bool &ovf)
+{
+    __shared__ uint64_t s_w[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint64_t incl = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl = add_chk(y, incl, ovf);
+    }
+    __syncthreads();   // an earlier scan's reads are done
+    if (lane == 31) s_w[warp] = incl;
+    __syncthreads();
+    uint64_t before = 0;
+    total = 0;
+    for (int w = 0; w < nw; ++w) {
+        if (w == warp) before = total;
+        total = add_chk(total, s_w[w], ovf);
+    }
+    return add_chk(before, incl - v, ovf);
+}
+
+__global__ void __launch_bounds__(kSampleThreads) k_list_sums(const uint64_t *__restrict__ cnt, uint64_t k,
+                                                              uint64_t *__restrict__ sums, uint32_t *status)
+{
+    const uint64_t i0 = (uint64_t)blockIdx.x * kListTile + (uint64_t)threadIdx.x * kListItems;
+    uint64_t s = 0, total;
+    bool ovf = false;
+#pragma unroll
+    for (int j = 0; j < kListItems; ++j) s = add_chk(s, i0 + j < k ? cnt[i0 + j] : 0, ovf);
+    list_block_scan(s, total, ovf);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
+    if (ovf) latch(status, ST_OVERFLOW);
+}
+
+__global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums, uint64_t n, uint64_t *__restrict__ total,
+                                                    uint32_t *status)
+{
+    uint64_t carry = 0;
+    bool ovf = false;
+    for (uint64_t b = 0; b < n; b += blockDim.x) {
+        const uint64_t i = b + threadIdx.x;
+        uint64_t t;
+        const uint64_t before = list_block_scan(i < n ? sums[i] : 0, t, ovf);
+        if (i < n) sums[i] = add_chk(carry, before, ovf);
+        carry = add_chk(carry, t, ovf);
+    }
+    if (threadIdx.x == 0) *total = carry;
+    if (ovf) latch(status, ST_OVERFLOW);
+}
+
+__global__ void __launch_bounds__(kSampleThreads) k_list_offsets(uint64_t *__restrict__ cnt, uint64_t k,
+                                                                 const uint64_t *__restrict__ sums)
+{
+    const uint64_t i0 = (uint64_t)blockIdx.x * kListTile + (uint64_t)threadIdx.x * kListItems;
+    uint64_t v[kListItems], s = 0, total;
+    bool ovf = false;   // a wrap was latched by the sums
+#pragma unroll
+    for (int j = 0; j < kListItems; ++j) { v[j] = i0 + j < k ? cnt[i0 + j] : 0; s += v[j]; }
+    uint64_t run = sums[blockIdx.x] + list_block_scan(s, total, ovf);
+#pragma unroll
+    for (int j = 0; j < kListItems; ++j) {
+        if (i0 + j < k) cnt[i0 + j] = run;
+        run += v[j];
+    }
+}
+
 // Pass 2: each sample's instances at rows offs[i] .. offs[i+1]-1 (rows at or
 // beyond max_inst are not written): ne edge ids per row, motif edge e in
 // column e, and the sample id.
@@ -1192,37 +1266,36 @@ int run_list(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t firs
         launch(ctx, k_list_count, blocks, kSampleThreads, ctx->g, (const DevPlan *)dplan, J, seed, first, k, dcnt,
                ctx->status);
     }
+    // row offsets of every sample, in place; their end is the number of instances
+    const uint64_t tiles = (k + kListTile - 1) / kListTile;
+    uint64_t *sums = (uint64_t *)salloc(ctx, (size_t)tiles * 8);
+    if (!sums) return TM_E_NOMEM;
+    {
+        PhaseScope ph(ctx, TM_PH_SAMPLE);
+        launch(ctx, k_list_sums, (unsigned)tiles, kSampleThreads, (const uint64_t *)dcnt, k, sums, ctx->status);
+        launch(ctx, k_list_scan, 1, 1024, sums, tiles, dcnt + k, ctx->status);
+        launch(ctx, k_list_offsets, (unsigned)tiles, kSampleThreads, dcnt, k, (const uint64_t *)sums);
+    }
     int rc = check_cuda(ctx, cudaGetLastError(), "listing count");
     if (rc) return rc;
-    // row offsets of every sample (exclusive prefix of the counts, on the host)
-    std::vector<uint64_t> offs((size_t)k + 1);
-    copy_d2h(ctx, offs.data() + 1, dcnt, (size_t)k * 8);
-    rc = check_cuda(ctx, cudaStreamSynchronize(st), "listing count copy");
-    if (rc) return rc;
+    copy_d2h(ctx, ctx->status_host + 4, dcnt + k, 8);   // pinned: read with the status
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
-    if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a completion count exceeds 2^64");
+    if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a completion count or the instance count exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "listing reached an inconsistent state");
-    offs[0] = 0;
-    for (uint64_t i = 1; i <= k; ++i) {
-        if (offs[i] > ~0ull - offs[i - 1]) return set_err(ctx, TM_E_OVERFLOW, "instance count exceeds 2^64");
-        offs[i] += offs[i - 1];
-    }
-    *n_inst = offs[k];
-    const uint64_t rows = std::min(max_inst, offs[k]);
+    memcpy(n_inst, ctx->status_host + 4, 8);
+    const uint64_t rows = std::min<uint64_t>(max_inst, *n_inst);
     if (rows == 0 || !inst_gids || !inst_sample) return TM_OK;
     const size_t ne = mo->ne;
-    uint64_t *doffs = dcnt;   // reuse: k + 1 entries
     uint32_t *dg = (uint32_t *)salloc(ctx, (size_t)rows * ne * 4);
     uint64_t *ds = (uint64_t *)salloc(ctx, (size_t)rows * 8);
     if (!dg || !ds) return TM_E_NOMEM;
-    copy_h2d(ctx, doffs, offs.data(), (size_t)(k + 1) * 8);
     cudaMemsetAsync(ctx->status, 0, 4, st);
     {
         PhaseScope ph(ctx, TM_PH_SAMPLE);
         launch(ctx, k_list_emit, blocks, kSampleThreads, ctx->g, (const DevPlan *)dplan, J, seed, first, k,
-               (const uint64_t *)doffs, rows, dg, ds, ctx->status);
+               (const uint64_t *)dcnt, rows, dg, ds, ctx->status);
     }
     rc = check_cuda(ctx, cudaGetLastError(), "listing emit");
     if (rc) return rc;
