@@ -762,6 +762,17 @@ int tm_tree_candidates(uint32_t nv, uint32_t ne, const uint32_t *edges, const ui
 
 static bool u128_less(const tm_u128 &a, const tm_u128 &b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 
+// tm_weights without the samplers' guide tables: a candidate is asked for its W
+// (the tables are 30 of a pass's 465 us on 2e6 edges, plus two launches).
+static int candidate_weights(tm_ctx *ctx, tm_motif *mo, tm_u128 *W)
+{
+    cudaSetDevice(ctx->device);
+    const int rc = compute_weights(ctx, mo, false);
+    if (rc) { release_weights(ctx, mo); return rc; }
+    *W = mo->W;
+    return TM_OK;
+}
+
 int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges, const uint32_t *order, int64_t delta,
                    uint32_t n_c, int all_roots, tm_motif **out, tm_tree_cand *cands, uint32_t max_cand, uint32_t *n_cand)
 {
@@ -791,7 +802,7 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
                 return set_err(ctx, rc, "internal: candidate tree did not compile");
             }
             tm_u128 W{0, 0};
-            const int crc = tm_weights(ctx, mo, &W);
+            const int crc = candidate_weights(ctx, mo, &W);
             if (cands && evaluated < max_cand) {
                 tm_tree_cand &c = cands[evaluated];
                 c.tree_mask = R[t].mask;
@@ -817,6 +828,8 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
     }
     if (n_cand) *n_cand = evaluated;
     if (!best) return set_err(ctx, TM_E_OVERFLOW, "every candidate's weight pass overflowed");
+    rc = fill_guides(ctx, best);
+    if (rc) { tm_motif_free(best); return rc; }
     *out = best;
     return TM_OK;
 }

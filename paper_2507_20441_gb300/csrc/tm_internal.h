@@ -291,7 +291,10 @@ void spare_free(tm_ctx *ctx);
 int build_csr(tm_ctx *ctx);
 
 // ---- weights (weights.cu) ----
-int compute_weights(tm_ctx *ctx, tm_motif *mo);
+// guides = false leaves the samplers' guide tables to a later fill_guides (tree
+// selection needs them for the winner only)
+int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true);
+int fill_guides(tm_ctx *ctx, tm_motif *mo);
 int export_weights(tm_ctx *ctx, tm_motif *mo, int q, int layer, uint64_t *host_out);
 
 // ---- sampler (sampler.cu) ----

@@ -12,6 +12,7 @@
 // window and the sums are differences of segmented prefix sums.
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -473,74 +474,6 @@ __global__ void __launch_bounds__(TB) k_win_fill(const uint32_t *__restrict__ t,
     }
 }
 
-// Window totals W_i (last root-CDF entry of each window) and their 128-bit
-// running sum over (layer 0 windows, layer 1 windows).  One block; each
-// thread scans a contiguous chunk.
-__global__ void k_window_cum(const uint64_t *__restrict__ cdf0, const uint32_t *__restrict__ beg0, uint32_t nw0,
-                             const uint64_t *__restrict__ cdf1, const uint32_t *__restrict__ beg1, uint32_t nw1,
-                             uint64_t *__restrict__ wcum)
-{
-    __shared__ u128 warp_tot[32];
-    const uint32_t n = nw0 + nw1;
-    const uint32_t per = (n + blockDim.x - 1) / blockDim.x;
-    uint32_t lo = threadIdx.x * per, hi = min(n, lo + per);
-    if (lo > n) lo = n;
-    auto total = [&](uint32_t k) -> uint64_t {
-        if (k < nw0) return cdf0[beg0[k + 1] - 1];
-        k -= nw0;
-        return cdf1[beg1[k + 1] - 1];
-    };
-    u128 s = 0;
-    for (uint32_t k = lo; k < hi; ++k) s += total(k);
-    // exclusive scan of the chunk sums (128-bit) across the block
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    u128 incl = s;
-    for (int o = 1; o < 32; o <<= 1) {
-        uint64_t yl = __shfl_up_sync(0xffffffffu, (uint64_t)incl, o);
-        uint64_t yh = __shfl_up_sync(0xffffffffu, (uint64_t)(incl >> 64), o);
-        if (lane >= o) incl += (u128)yl | ((u128)yh << 64);
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        u128 run = 0;
-        const int nw = (blockDim.x + 31) / 32;
-        for (int w = 0; w < nw; ++w) { u128 c = warp_tot[w]; warp_tot[w] = run; run += c; }
-        wcum[2 * (size_t)n] = (uint64_t)run;
-        wcum[2 * (size_t)n + 1] = (uint64_t)(run >> 64);
-    }
-    __syncthreads();
-    u128 run = warp_tot[warp] + incl - s;
-    for (uint32_t k = lo; k < hi; ++k) {
-        wcum[2 * (size_t)k] = (uint64_t)run;
-        wcum[2 * (size_t)k + 1] = (uint64_t)(run >> 64);
-        run += total(k);
-    }
-}
-
-// Guide table of the window pick: entry j is the window holding draw j 2^s
-// (the last k with wcum[k] <= j 2^s), for the ceil(W / 2^s) buckets, then a
-// sentinel (the last window).  One thread per bucket, a binary search each;
-// W is read on the device (the last cumulative entry).
-__global__ void k_wguide(const uint64_t *__restrict__ wcum, uint32_t nw, uint32_t *__restrict__ guide)
-{
-    const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    const u128 W = (u128)wcum[2 * (size_t)nw] | ((u128)wcum[2 * (size_t)nw + 1] << 64);
-    if (W == 0) return;
-    const uint32_t s = wguide_shift((uint64_t)W, (uint64_t)(W >> 64), nw);
-    const uint64_t nb = (uint64_t)((W + ((u128)1 << s) - 1) >> s);
-    if (j > nb) return;
-    if (j == nb) { guide[j] = nw - 1; return; }
-    const u128 x = (u128)j << s;
-    uint32_t lo = 0, hi = nw;   // wcum[0] = 0 <= x; find the last k with wcum[k] <= x
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        const u128 c = (u128)wcum[2 * (size_t)mid] | ((u128)wcum[2 * (size_t)mid + 1] << 64);
-        if (c <= x) lo = mid; else hi = mid;
-    }
-    guide[j] = lo;
-}
-
 // ---- guide table of the root search --------------------------------------
 // Window kk of a layer gets about n/4 buckets of width 2^s over its draws
 // [0, W_kk); the table holds, per bucket j, the first edge whose in-window
@@ -557,45 +490,109 @@ struct GuideArgs {
     GuideLayer L[2];
 };
 
-// One block per layer: each thread sizes a contiguous run of windows, then
-// the block turns the counts into the windows' table offsets.
-__global__ void __launch_bounds__(1024) k_guide_setup(GuideArgs A)
+// Window totals W_i (last root-CDF entry of each window) and their 128-bit
+// running sum over (layer 0 windows, layer 1 windows) by block 0; the guide
+// table's bucket width and offset of each window by block 1 + p for layer p.
+// A block takes kTotItems windows per thread at a time, whose loads are
+// independent (a contiguous run of windows per thread is one load after the
+// other: 82 + 38 us in two launches for 5.6e4 windows, 36 us like this).
+constexpr int kTotItems = 8;
+__global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *__restrict__ wcum)
 {
-    __shared__ uint32_t warp_tot[32];
-    const GuideLayer &L = blockIdx.x ? A.L[1] : A.L[0];
-    const uint32_t nw = L.nwin, per = (nw + blockDim.x - 1) / blockDim.x;
-    const uint32_t lo = min(nw, threadIdx.x * per), hi = min(nw, lo + per);
-    uint32_t sum = 0;
-    for (uint32_t kk = lo; kk < hi; ++kk) {
-        const uint32_t n = L.win_beg[kk + 1] - L.win_beg[kk];
-        const uint64_t W = L.cdf[L.win_beg[kk + 1] - 1];
-        const uint64_t target = n >> 2 ? n >> 2 : 1;
-        uint32_t sh = 0;
-        while (sh < 63 && W && ((W - 1) >> sh) + 1 > target) ++sh;
-        L.gshift[kk] = sh;
-        const uint32_t c = (uint32_t)(W ? ((W - 1) >> sh) + 1 : 0) + 1;
-        L.goff[kk] = c;   // count for now, offset below
-        sum += c;
-    }
+    __shared__ u128 s_tot[32];
+    __shared__ u128 s_carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t incl = sum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
+    const uint32_t nw0 = A.L[0].nwin, nw1 = A.L[1].nwin;
+    const int b = blockIdx.x;
+    const uint32_t n = b == 0 ? nw0 + nw1 : b == 1 ? nw0 : nw1;
+    if (threadIdx.x == 0) s_carry = 0;
+    for (uint32_t base = 0; base < n || base == 0; base += 1024 * kTotItems) {
+        const uint32_t k0 = base + threadIdx.x * kTotItems;
+        uint64_t v[kTotItems];
+        u128 sum = 0;
+#pragma unroll
+        for (int j = 0; j < kTotItems; ++j) {
+            const uint32_t k = k0 + j;
+            v[j] = 0;
+            if (k < n) {
+                const bool second = b == 2 || (b == 0 && k >= nw0);
+                const uint32_t *win_beg = second ? A.L[1].win_beg : A.L[0].win_beg;
+                const uint32_t kk = b == 0 && second ? k - nw0 : k, wend = win_beg[kk + 1];
+                const uint64_t W = (second ? A.L[1].cdf : A.L[0].cdf)[wend - 1];
+                if (b == 0) {
+                    v[j] = W;
+                } else {
+                    // about n / 4 buckets of 2^sh draws each over the window's W
+                    const uint32_t ne = wend - win_beg[kk], target = ne >> 2 ? ne >> 2 : 1;
+                    uint32_t sh = 0;
+                    if (W) {
+                        const int d = __clz((int)target) - 32 + 64 - __clzll((long long)(W - 1));
+                        sh = d > 1 ? d - 1 : 0;   // not above the least width, then stepped up to it
+                        while (sh < 63 && ((W - 1) >> sh) + 1 > target) ++sh;
+                    }
+                    (second ? A.L[1].gshift : A.L[0].gshift)[kk] = sh;
+                    v[j] = (W ? ((W - 1) >> sh) + 1 : 0) + 1;
+                }
+            }
+            sum += v[j];
+        }
+        // exclusive scan of the threads' sums (128-bit) across the block
+        u128 incl = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t yl = __shfl_up_sync(0xffffffffu, (uint64_t)incl, o);
+            const uint64_t yh = __shfl_up_sync(0xffffffffu, (uint64_t)(incl >> 64), o);
+            if (lane >= o) incl += (u128)yl | ((u128)yh << 64);
+        }
+        if (lane == 31) s_tot[warp] = incl;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            u128 run = s_carry;
+            for (int w = 0; w < 32; ++w) { const u128 c = s_tot[w]; s_tot[w] = run; run += c; }
+            s_carry = run;
+        }
+        __syncthreads();
+        u128 run = s_tot[warp] + incl - sum;
+#pragma unroll
+        for (int j = 0; j < kTotItems; ++j) {
+            const uint32_t k = k0 + j;
+            if (k < n) {
+                if (b == 0) {
+                    wcum[2 * (size_t)k] = (uint64_t)run;
+                    wcum[2 * (size_t)k + 1] = (uint64_t)(run >> 64);
+                } else {
+                    (b == 2 ? A.L[1].goff : A.L[0].goff)[k] = (uint32_t)run;
+                }
+            }
+            run += v[j];
+        }
+        __syncthreads();   // s_tot is written again
     }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) { const uint32_t c = warp_tot[w]; warp_tot[w] = run; run += c; }
+    if (b == 0 && threadIdx.x == 0) {
+        wcum[2 * (size_t)n] = (uint64_t)s_carry;
+        wcum[2 * (size_t)n + 1] = (uint64_t)(s_carry >> 64);
     }
-    __syncthreads();
-    uint32_t run = warp_tot[warp] + incl - sum;
-    for (uint32_t kk = lo; kk < hi; ++kk) {
-        const uint32_t c = L.goff[kk];
-        L.goff[kk] = run;
-        run += c;
+}
+
+// Guide table of the window pick: entry j is the window holding draw j 2^s
+// (the last k with wcum[k] <= j 2^s), for the ceil(W / 2^s) buckets, then a
+// sentinel (the last window).  A binary search per bucket j; W is read on the
+// device (the last cumulative entry).
+__device__ void wguide_entry(const uint64_t *__restrict__ wcum, uint32_t nw, uint32_t *__restrict__ guide, uint32_t j)
+{
+    const u128 W = (u128)wcum[2 * (size_t)nw] | ((u128)wcum[2 * (size_t)nw + 1] << 64);
+    if (W == 0) return;
+    const uint32_t s = wguide_shift((uint64_t)W, (uint64_t)(W >> 64), nw);
+    const uint64_t nb = (uint64_t)((W + ((u128)1 << s) - 1) >> s);
+    if (j > nb) return;
+    if (j == nb) { guide[j] = nw - 1; return; }
+    const u128 x = (u128)j << s;
+    uint32_t lo = 0, hi = nw;   // wcum[0] = 0 <= x; find the last k with wcum[k] <= x
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        const u128 c = (u128)wcum[2 * (size_t)mid] | ((u128)wcum[2 * (size_t)mid + 1] << 64);
+        if (c <= x) lo = mid; else hi = mid;
     }
+    guide[j] = lo;
 }
 
 // Edges in GLOBAL order, kGuideItems consecutive ones per thread, layer p =
@@ -604,26 +601,41 @@ __global__ void __launch_bounds__(1024) k_guide_setup(GuideArgs A)
 // edges l, l + 32, ... of them (coalesced CDF reads); the warp finds the
 // window of its first edge by a binary search over the window starts, and a
 // lane steps to the next window as its edges cross one, so a window of any
-// size is spread over many threads.
+// size is spread over many threads.  blockIdx.y = 2: the window pick's guide,
+// a bucket per thread.
 #ifndef TM_GUIDE_ITEMS
 #define TM_GUIDE_ITEMS 32   // measured: 32 edges per lane beat 8 (1.77 against 1.81 ms for the root phase) and 2
 #endif
 constexpr int kGuideItems = TM_GUIDE_ITEMS;
-__global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m)
+__global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m, const uint64_t *__restrict__ wcum,
+                                                   uint32_t *__restrict__ wguide)
 {
     const int p = blockIdx.y;
-    const GuideLayer &L = p ? A.L[1] : A.L[0];
+    if (p == 2) {
+        const uint32_t nw = A.L[0].nwin + A.L[1].nwin;
+        for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= 4 * (uint64_t)nw;
+             j += (uint64_t)gridDim.x * blockDim.x)
+            wguide_entry(wcum, nw, wguide, (uint32_t)j);
+        return;
+    }
+    // per-field selects keep the parameter block out of local memory
+    const uint32_t nwin = p ? A.L[1].nwin : A.L[0].nwin;
+    const uint64_t *__restrict__ cdf = p ? A.L[1].cdf : A.L[0].cdf;
+    const uint32_t *__restrict__ win_beg = p ? A.L[1].win_beg : A.L[0].win_beg;
+    const uint32_t *__restrict__ gshift = p ? A.L[1].gshift : A.L[0].gshift;
+    const uint32_t *__restrict__ goff = p ? A.L[1].goff : A.L[0].goff;
+    uint32_t *__restrict__ guide = p ? A.L[1].guide : A.L[0].guide;
     const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t xs = (gt >> 5) * (32u * kGuideItems) + (gt & 31u);
-    if (xs >= m || L.nwin == 0) return;
+    if (xs >= m || nwin == 0) return;
     // kk = the last window starting at or before the warp's first edge x0
     // (none: x0 precedes every window); the same search in every lane, so
     // each probe is one broadcast load
     const uint32_t x0 = (uint32_t)(xs - (gt & 31u));
-    uint32_t lo = 0, hi = L.nwin;
+    uint32_t lo = 0, hi = nwin;
     while (lo < hi) {
         const uint32_t mid = (lo + hi) >> 1;
-        if (L.win_beg[mid] <= x0) lo = mid + 1; else hi = mid;
+        if (win_beg[mid] <= x0) lo = mid + 1; else hi = mid;
     }
     int64_t kk = (int64_t)lo - 1;
     const uint64_t xe = min((uint64_t)m, (uint64_t)(xs + 32u * kGuideItems));
@@ -635,19 +647,19 @@ __global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m)
 #pragma unroll
         for (int u = 0; u < kGuideBatch; ++u) {
             const uint64_t xx = xb + 32u * u;
-            c1v[u] = xx < xe ? L.cdf[xx] : 0;
-            c0v[u] = (xx < xe && xx > 0) ? L.cdf[xx - 1] : 0;
+            c1v[u] = xx < xe ? cdf[xx] : 0;
+            c0v[u] = (xx < xe && xx > 0) ? cdf[xx - 1] : 0;
         }
 #pragma unroll
         for (int u = 0; u < kGuideBatch; ++u) {
             const uint64_t xx = xb + 32u * u;
             if (xx >= xe) break;
             const uint32_t x = (uint32_t)xx;
-            while (kk + 1 < (int64_t)L.nwin && L.win_beg[kk + 1] <= x) ++kk;
+            while (kk + 1 < (int64_t)nwin && win_beg[kk + 1] <= x) ++kk;
             if (kk < 0) continue;   // before the layer's first window
-            const uint32_t wbeg = L.win_beg[kk], wend = L.win_beg[kk + 1];
-            const uint32_t sh = L.gshift[kk];
-            uint32_t *G = L.guide + L.goff[kk];
+            const uint32_t wbeg = win_beg[kk], wend = win_beg[kk + 1];
+            const uint32_t sh = gshift[kk];
+            uint32_t *G = guide + goff[kk];
             const uint64_t c1 = c1v[u], c0 = x > wbeg ? c0v[u] : 0;
             const uint64_t j1 = ceil_shift(c1, sh);
             for (uint64_t j = ceil_shift(c0, sh); j < j1; ++j) G[j] = x;
@@ -699,7 +711,27 @@ static void free_motif_weights(tm_ctx *ctx, tm_motif *mo)
 // Owner bit sets of the out-, in- and multi-edge orders (built with the graph).
 struct OwnerBits { const uint32_t *out, *in, *multi; };
 
-int compute_weights(tm_ctx *ctx, tm_motif *mo)
+static GuideArgs guide_args(const tm_motif *mo)
+{
+    GuideArgs ga{};
+    for (int p = 0; p < 2; ++p) {
+        const LayerData &L = mo->layer[p];
+        ga.L[p] = GuideLayer{L.root_cdf, L.win_beg, L.nwin, L.win_gshift, L.win_goff, L.guide};
+    }
+    return ga;
+}
+
+int fill_guides(tm_ctx *ctx, tm_motif *mo)
+{
+    const uint64_t m = ctx->g.m;
+    if (m == 0 || mo->nwtot == 0) return TM_OK;
+    const uint64_t gwarps = (m + 32 * kGuideItems - 1) / (32 * kGuideItems);
+    launch(ctx, k_guide_fill, dim3(blocks_for(gwarps * 32, TB), 3), TB, guide_args(mo), (uint32_t)m,
+           (const uint64_t *)mo->wcum, mo->wguide);
+    return check_cuda(ctx, cudaGetLastError(), "guide tables");
+}
+
+int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
 {
     ScratchScope scope(ctx);
     free_motif_weights(ctx, mo);
@@ -851,20 +883,9 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
         if (rc) return rc;
         if (q == 0) {
             PhaseScope ph(ctx, TM_PH_ROOT);
-            GuideArgs ga{};
             RootScan2 f{w, g.g_t, wv, in_order ? g.in_pos : g.out_pos};
             rc = segmented_scan2_u64(ctx, f, m, mo->layer[0].root_cdf, mo->layer[1].root_cdf);
             if (rc) return rc;
-            for (int p = 0; p < 2; ++p) {
-                LayerData &L = mo->layer[p];
-                ga.L[p] = GuideLayer{L.root_cdf, L.win_beg, L.nwin, L.win_gshift, L.win_goff, L.guide};
-            }
-            // guide tables of the root search, both layers (edge-parallel)
-            if (m && nwh[0] + nwh[1]) {
-                launch(ctx, k_guide_setup, 2, 1024, ga);
-                const uint64_t gwarps = ((uint64_t)m + 32 * kGuideItems - 1) / (32 * kGuideItems);
-                launch(ctx, k_guide_fill, dim3(blocks_for(gwarps * 32, TB), 2), TB, ga, m);
-            }
         } else {
             PhaseScope ph(ctx, TM_PH_PREFIX);
             const int slot = P.tslot[q];
@@ -889,23 +910,21 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo)
     // ---- window totals and their 128-bit running sum (K5)
     uint32_t nw0 = mo->layer[0].nwin, nw1 = mo->layer[1].nwin;
     mo->nwtot = nw0 + nw1;
-    uint64_t Wh[2] = {0, 0};
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
-        launch(ctx, k_window_cum, 1, 1024, mo->layer[0].root_cdf, mo->layer[0].win_beg, nw0, mo->layer[1].root_cdf,
-                                         mo->layer[1].win_beg, nw1, mo->wcum);
-        if (mo->nwtot)
-            launch(ctx, k_wguide, blocks_for(4 * (uint64_t)mo->nwtot + 1, TB), TB, (const uint64_t *)mo->wcum,
-                   mo->nwtot, mo->wguide);
-        copy_d2h(ctx, Wh, mo->wcum + 2 * (size_t)mo->nwtot, 16);
+        launch(ctx, k_window_totals, 3, 1024, guide_args(mo), mo->wcum);
+        if (guides) {
+            rc = fill_guides(ctx, mo);
+            if (rc) return rc;
+        }
+        copy_d2h(ctx, ctx->status_host + 4, mo->wcum + 2 * (size_t)mo->nwtot, 16);   // pinned: read with the status
     }
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a weight, prefix sum or window total exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "device status error in weight pass");
-    mo->W.lo = Wh[0];
-    mo->W.hi = Wh[1];
+    memcpy(&mo->W, ctx->status_host + 4, 16);
     mo->have_weights = true;
     mo->graph_epoch = ctx->epoch;
     return TM_OK;
