@@ -2,10 +2,9 @@
 //
 // * exclusive_scan_u32: reduce-then-scan over u32 counts (recursive over the
 //   tile totals), for compaction, pair ids and window offsets.
-// * segmented_scan_u64: inclusive prefix sums that restart at segment heads,
-//   with every 64-bit addition inside a segment checked for wrap-around.  It
-//   is a three-phase reduce / scan-of-tile-aggregates / rescan, so no block
-//   ever waits on another block.
+// * segmented_scan2_u64: inclusive prefix sums that restart at segment heads,
+//   with every 64-bit addition inside a segment checked for wrap-around, in one
+//   pass with a bounded look-back between tiles.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -140,9 +139,10 @@ inline int exclusive_scan_u32(tm_ctx *ctx, const uint32_t *in, uint32_t *out, ui
 // Inclusive prefix sums that restart at segment heads, with every 64-bit
 // addition inside a segment checked for wrap-around, over pairs (layer 0,
 // layer 1) that share their positions (one gather of a 16-byte pair serves
-// both layers).  Heads may differ per layer (bit p of head2()).  Functor
-// interface: value2(pos) -> ulonglong2, head2(pos) -> bits, and
-// kGathered (value2 is a gather).
+// both layers).  A segment of layer p starts where the window of layer p
+// changes or, in both layers, where a new owner starts.  Functor interface:
+// value2(pos) -> ulonglong2, tarr (position -> t'), wv (the window divider) and
+// owner_word(w) -> the owner-start bits of positions 32 w .. 32 w + 31.
 struct SegAgg2 {
     uint64_t v0, v1;
     uint32_t f;     // bit p: the range contains a head of layer p
@@ -157,156 +157,6 @@ __device__ __forceinline__ SegAgg2 seg_combine2(SegAgg2 a, SegAgg2 b, bool &ovf)
     r.v1 = (b.f & 2u) ? b.v1 : add_chk(a.v1, b.v1, ovf);
     r.pad = 0;
     return r;
-}
-
-__device__ __forceinline__ SegAgg2 seg_shfl_up2(SegAgg2 a, int o)
-{
-    SegAgg2 y;
-    y.v0 = __shfl_up_sync(0xffffffffu, a.v0, o);
-    y.v1 = __shfl_up_sync(0xffffffffu, a.v1, o);
-    y.f = __shfl_up_sync(0xffffffffu, a.f, o);
-    y.pad = 0;
-    return y;
-}
-
-template <class F>
-__global__ void k_segscan2_reduce(F f, uint64_t n, SegAgg2 *__restrict__ aggs, ulonglong2 *__restrict__ stash,
-                                  uint32_t *status)
-{
-    __shared__ SegAgg2 warp_agg[SCAN_THREADS / 32];
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
-    bool ovf = false;
-    SegAgg2 a{0, 0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-        const uint64_t i = base + j;
-        if (i < n) {
-            const ulonglong2 v = f.value2(i);
-            if (stash) stash[i] = v;          // gathered once; the rescan reads it back in order
-            SegAgg2 x{v.x, v.y, f.head2(i), 0};
-            a = seg_combine2(a, x, ovf);
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 1; o < 32; o <<= 1) {
-        const SegAgg2 y = seg_shfl_up2(a, o);
-        if (lane >= o) a = seg_combine2(y, a, ovf);
-    }
-    if (lane == 31) warp_agg[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        SegAgg2 t = warp_agg[0];
-        for (int w = 1; w < SCAN_THREADS / 32; ++w) t = seg_combine2(t, warp_agg[w], ovf);
-        aggs[blockIdx.x] = t;
-    }
-    if (ovf) latch(status, ST_OVERFLOW);
-}
-
-__global__ void k_segscan2_carries(SegAgg2 *__restrict__ aggs, uint64_t ntiles, uint32_t *status)
-{
-    __shared__ SegAgg2 warp_tot[32];
-    bool ovf = false;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t per = (ntiles + blockDim.x - 1) / blockDim.x;
-    uint64_t lo = (uint64_t)threadIdx.x * per, hi = lo + per;
-    if (hi > ntiles) hi = ntiles;
-    if (lo > ntiles) lo = ntiles;
-    SegAgg2 a{0, 0, 0, 0};
-    for (uint64_t i = lo; i < hi; ++i) a = seg_combine2(a, aggs[i], ovf);
-    SegAgg2 incl = a;
-    for (int o = 1; o < 32; o <<= 1) {
-        const SegAgg2 y = seg_shfl_up2(incl, o);
-        if (lane >= o) incl = seg_combine2(y, incl, ovf);
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int nw = (blockDim.x + 31) / 32;
-        const SegAgg2 w = lane < nw ? warp_tot[lane] : SegAgg2{0, 0, 0, 0};
-        SegAgg2 wi = w;
-        for (int o = 1; o < 32; o <<= 1) {
-            const SegAgg2 y = seg_shfl_up2(wi, o);
-            if (lane >= o) wi = seg_combine2(y, wi, ovf);
-        }
-        SegAgg2 ex = seg_shfl_up2(wi, 1);
-        if (lane == 0) ex = SegAgg2{0, 0, 0, 0};
-        if (lane < nw) warp_tot[lane] = ex;
-    }
-    __syncthreads();
-    const SegAgg2 ex_lane = seg_shfl_up2(incl, 1);
-    SegAgg2 run = warp_tot[warp];
-    if (lane > 0) run = seg_combine2(run, ex_lane, ovf);
-    for (uint64_t i = lo; i < hi; ++i) {
-        const SegAgg2 c = aggs[i];
-        aggs[i] = run;
-        run = seg_combine2(run, c, ovf);
-    }
-    if (ovf) latch(status, ST_OVERFLOW);
-}
-
-#ifndef TM_SCAN2_MINB
-#define TM_SCAN2_MINB 4   // four blocks of 256 per SM (measured faster than two)
-#endif
-template <class F>
-__global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN2_MINB) k_segscan2_final(F f, uint64_t n, const SegAgg2 *__restrict__ carries,
-                                 const ulonglong2 *__restrict__ stash, uint64_t *__restrict__ out0,
-                                 uint64_t *__restrict__ out1, ulonglong2 *__restrict__ outp, uint32_t *status)
-{
-    __shared__ SegAgg2 warp_agg[SCAN_THREADS / 32];
-    const uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
-    bool ovf = false;
-    ulonglong2 v[SCAN_ITEMS];
-    uint32_t hbits = 0;
-    SegAgg2 a{0, 0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-        const uint64_t i = base + j;
-        v[j] = make_ulonglong2(0, 0);
-        if (i < n) {
-            v[j] = stash ? stash[i] : f.value2(i);
-            const uint32_t h = f.head2(i);
-            hbits |= h << (2 * j);
-            SegAgg2 x{v[j].x, v[j].y, h, 0};
-            a = seg_combine2(a, x, ovf);
-        }
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    SegAgg2 incl = a;
-    for (int o = 1; o < 32; o <<= 1) {
-        const SegAgg2 y = seg_shfl_up2(incl, o);
-        if (lane >= o) incl = seg_combine2(y, incl, ovf);
-    }
-    if (lane == 31) warp_agg[warp] = incl;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        SegAgg2 run = carries[blockIdx.x];
-        for (int w = 0; w < SCAN_THREADS / 32; ++w) {
-            const SegAgg2 c = warp_agg[w];
-            warp_agg[w] = run;
-            run = seg_combine2(run, c, ovf);
-        }
-    }
-    __syncthreads();
-    const SegAgg2 excl_lane = seg_shfl_up2(incl, 1);
-    SegAgg2 pre = warp_agg[warp];
-    if (lane > 0) pre = seg_combine2(pre, excl_lane, ovf);
-    uint64_t r0 = pre.v0, r1 = pre.v1;
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-        const uint64_t i = base + j;
-        if (i < n) {
-            const uint32_t h = (hbits >> (2 * j)) & 3u;
-            r0 = (h & 1u) ? v[j].x : add_chk(r0, v[j].x, ovf);
-            r1 = (h & 2u) ? v[j].y : add_chk(r1, v[j].y, ovf);
-            if (outp) {
-                outp[i] = make_ulonglong2(r0, r1);
-            } else {
-                out0[i] = r0;
-                out1[i] = r1;
-            }
-        }
-    }
-    if (ovf) latch(status, ST_OVERFLOW);
 }
 
 // ---- one pass with decoupled look-back -------------------------------
@@ -335,16 +185,21 @@ __device__ __forceinline__ void seg_publish(SegTile *t, const SegAgg2 &v, uint32
     vt->status = st;
 }
 
-// (Staging each tile through shared memory so that the global loads and
-// stores are striped across lanes measured slower: 1.82 against 1.51 ms for
-// the two list-order scans on 5e7 edges.)
+// A warp takes kScanRows rows of 32 consecutive positions, a lane one position
+// of each, so that every load and store but a gather is coalesced, an owner
+// word serves a row as it is, and a row is scanned with four shuffles a step (a
+// lane knows from the head bits how far back its segment reaches).  With eight
+// consecutive positions per thread instead, 16-byte accesses at a stride of 128
+// bytes kept the L1 busiest (62 % of its throughput) and the two scans of a
+// node took 356 us on 1e7 edges.
+constexpr int kScanRows = 8;   // (4 and 6 rows at more blocks per SM measured 2 - 6 % slower)
+constexpr int kScan2Tile = SCAN_THREADS * kScanRows;
 #ifndef TM_SCAN_MINB
-#define TM_SCAN_MINB 4   // 64 registers, four blocks per SM: measured 1.50 against 1.71 ms uncapped (76 registers)
+#define TM_SCAN_MINB 4   // 64 registers, four blocks per SM
 #endif
 template <class F>
 __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass(F f, uint64_t n, SegTile *__restrict__ tiles,
                                                                    uint32_t *__restrict__ counter,
-                                                                   ulonglong2 *__restrict__ keep,
                                                                    uint64_t *__restrict__ out0,
                                                                    uint64_t *__restrict__ out1,
                                                                    ulonglong2 *__restrict__ outp, uint32_t *status)
@@ -354,31 +209,60 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
     if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
-    const uint64_t base = (uint64_t)tile * SCAN_TILE + (uint64_t)threadIdx.x * SCAN_ITEMS;
-    bool ovf = false;
-    ulonglong2 v[SCAN_ITEMS];
-    uint32_t hbits = 0;
-    SegAgg2 a{0, 0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-        const uint64_t i = base + j;
-        v[j] = make_ulonglong2(0, 0);
-        if (i < n) {
-            v[j] = f.value2(i);
-            if (keep) keep[i] = v[j];
-            const uint32_t h = f.head2(i);
-            hbits |= h << (2 * j);
-            SegAgg2 x{v[j].x, v[j].y, h, 0};
-            a = seg_combine2(a, x, ovf);
-        }
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    SegAgg2 incl = a;
-    for (int o = 1; o < 32; o <<= 1) {
-        const SegAgg2 y = seg_shfl_up2(incl, o);
-        if (lane >= o) incl = seg_combine2(y, incl, ovf);
+    const uint64_t base = (uint64_t)tile * kScan2Tile + (uint64_t)warp * (32 * kScanRows);   // the warp's first position
+    const uint32_t le = 0xffffffffu >> (31 - lane);                                         // lanes up to this one
+    bool ovf = false;
+    ulonglong2 v[kScanRows];
+    uint32_t t[kScanRows];
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) {
+        const uint64_t i = base + r * 32 + lane;
+        t[r] = i < n ? __ldg(f.tarr + i) : 0u;
     }
-    if (lane == 31) warp_agg[warp] = incl;
+    uint32_t tb = base > 0 && base < n ? __ldg(f.tarr + base - 1) : 0u;   // the time before the warp's first
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) {
+        const uint64_t i = base + r * 32 + lane;
+        v[r] = i < n ? f.value2(i) : make_ulonglong2(0, 0);
+    }
+    uint32_t qb = f.wv.quot(tb);    // the quotient before the row's first
+    uint32_t need0 = 0, need1 = 0;  // bit r: no head of the layer in the chunk up to row r's position
+    bool seen0 = false, seen1 = false;
+    uint64_t c0 = 0, c1 = 0;        // the sums at the row before's last position
+#pragma unroll
+    for (int r = 0; r < kScanRows; ++r) {
+        const uint64_t row = base + r * 32;
+        const uint32_t q = f.wv.quot(t[r]);
+        uint32_t qp = __shfl_up_sync(0xffffffffu, q, 1);
+        if (lane == 0) qp = qb;
+        qb = __shfl_sync(0xffffffffu, q, 31);
+        const bool in = row + lane < n;
+        // the window of layer p is that of q with parity p: q / 2 and (q + 1) / 2 tell it
+        uint32_t h0 = __ballot_sync(0xffffffffu, in && (q >> 1) != (qp >> 1));
+        uint32_t h1 = __ballot_sync(0xffffffffu, in && ((q + 1) >> 1) != ((qp + 1) >> 1));
+        uint32_t own = row < n ? f.owner_word(row >> 5) : 0u;
+        if (row == 0) own |= 1u;
+        h0 |= own;
+        h1 |= own;
+        const uint32_t b0 = h0 & le, b1 = h1 & le;
+        const int reach0 = b0 ? lane - (31 - __clz((int)b0)) : lane, reach1 = b1 ? lane - (31 - __clz((int)b1)) : lane;
+        uint64_t x0 = v[r].x, x1 = v[r].y;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t y0 = __shfl_up_sync(0xffffffffu, x0, o), y1 = __shfl_up_sync(0xffffffffu, x1, o);
+            if (o <= reach0) x0 = add_chk(y0, x0, ovf);
+            if (o <= reach1) x1 = add_chk(y1, x1, ovf);
+        }
+        if (!b0) { x0 = add_chk(c0, x0, ovf); need0 |= seen0 ? 0u : 1u << r; }
+        if (!b1) { x1 = add_chk(c1, x1, ovf); need1 |= seen1 ? 0u : 1u << r; }
+        c0 = __shfl_sync(0xffffffffu, x0, 31);
+        c1 = __shfl_sync(0xffffffffu, x1, 31);
+        seen0 |= h0 != 0;
+        seen1 |= h1 != 0;
+        v[r] = make_ulonglong2(x0, x1);
+    }
+    if (lane == 0) warp_agg[warp] = SegAgg2{c0, c1, (seen0 ? 1u : 0u) | (seen1 ? 2u : 0u), 0};
     __syncthreads();
     if (warp == 0) {
         // the tile's aggregate (every lane of warp 0 folds the warp totals)
@@ -442,17 +326,15 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
         }
     }
     __syncthreads();
-    const SegAgg2 excl_lane = seg_shfl_up2(incl, 1);
-    SegAgg2 pre = warp_agg[warp];
-    if (lane > 0) pre = seg_combine2(pre, excl_lane, ovf);
-    uint64_t r0 = pre.v0, r1 = pre.v1;
+    // (storing what needs no carry before the look-back measured 5 - 10 % slower)
+    const SegAgg2 pre = warp_agg[warp];
 #pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-        const uint64_t i = base + j;
+    for (int r = 0; r < kScanRows; ++r) {
+        const uint64_t i = base + r * 32 + lane;
         if (i < n) {
-            const uint32_t h = (hbits >> (2 * j)) & 3u;
-            r0 = (h & 1u) ? v[j].x : add_chk(r0, v[j].x, ovf);
-            r1 = (h & 2u) ? v[j].y : add_chk(r1, v[j].y, ovf);
+            uint64_t r0 = v[r].x, r1 = v[r].y;
+            if ((need0 >> r) & 1u) r0 = add_chk(pre.v0, r0, ovf);
+            if ((need1 >> r) & 1u) r1 = add_chk(pre.v1, r1, ovf);
             if (outp) {
                 outp[i] = make_ulonglong2(r0, r1);
             } else {
@@ -465,36 +347,21 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
 }
 
 // Outputs: out0 / out1 (one array per layer), or outp (the (layer 0,
-// layer 1) pairs interleaved) when it is non-null.  A gathering functor's
-// values are stashed in scan order; with `keep` non-null the stash is that
-// caller-owned array (n pairs), which then holds the gathered values.
-#ifndef TM_SCAN_ONEPASS
-#define TM_SCAN_ONEPASS 1   // 1: one pass with look-back; 0: reduce, carries, rescan
-#endif
+// layer 1) pairs interleaved) when it is non-null.
 template <class F>
 int segmented_scan2_u64(tm_ctx *ctx, const F &f, uint64_t n, uint64_t *out0, uint64_t *out1,
-                        ulonglong2 *outp = nullptr, ulonglong2 *keep = nullptr)
+                        ulonglong2 *outp = nullptr)
 {
     if (n == 0) return TM_OK;
-    const uint64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
+    const uint64_t tiles = (n + kScan2Tile - 1) / kScan2Tile;
     ScratchScope scope(ctx);
-#if TM_SCAN_ONEPASS
     if (tiles >= 0xFFFFFFFFull) return set_err(ctx, TM_E_LIMIT, "scan of more than 2^32 tiles");
     char *st = (char *)salloc(ctx, tiles * sizeof(SegTile) + 256);
     if (!st) return TM_E_NOMEM;
     uint32_t *counter = (uint32_t *)(st + tiles * sizeof(SegTile));
     cudaMemsetAsync(st, 0, tiles * sizeof(SegTile) + 4, ctx->stream);
-    launch(ctx, k_segscan2_onepass<F>, (unsigned)tiles, SCAN_THREADS, f, n, (SegTile *)st, counter, keep, out0, out1,
-           outp, ctx->status);
-    return check_cuda(ctx, cudaGetLastError(), "segmented scan");
-#endif
-    SegAgg2 *aggs = (SegAgg2 *)salloc(ctx, tiles * sizeof(SegAgg2));
-    ulonglong2 *stash = !F::kGathered ? nullptr : keep ? keep : (ulonglong2 *)salloc(ctx, n * sizeof(ulonglong2));
-    if (!aggs || (F::kGathered && !stash)) return TM_E_NOMEM;
-    launch(ctx, k_segscan2_reduce<F>, (unsigned)tiles, SCAN_THREADS, f, n, aggs, stash, ctx->status);
-    launch(ctx, k_segscan2_carries, 1, 1024, aggs, tiles, ctx->status);
-    launch(ctx, k_segscan2_final<F>, (unsigned)tiles, SCAN_THREADS, f, n, aggs, (const ulonglong2 *)stash, out0,
-           out1, outp, ctx->status);
+    launch(ctx, k_segscan2_onepass<F>, (unsigned)tiles, SCAN_THREADS, f, n, (SegTile *)st, counter, out0, out1, outp,
+           ctx->status);
     return check_cuda(ctx, cudaGetLastError(), "segmented scan");
 }
 

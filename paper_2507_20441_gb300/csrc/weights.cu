@@ -335,32 +335,22 @@ struct RootHead {
 // Both layers at once (two-lane scans): the pair of weights of a position is
 // one 16-byte gather; heads are per layer (bit p).
 struct DirScan2 {
-    static constexpr bool kGathered = true;
     const ulonglong2 *w;        // (layer 0, layer 1) weights
     const uint32_t *perm;       // scan position -> weight position (null: same order)
     const uint32_t *tarr;       // position -> t'
     const uint32_t *ownbits;    // bit set: position starts a new owner
     WinDiv wv;
     __device__ ulonglong2 value2(uint64_t i) const { return __ldg(w + (perm ? __ldg(perm + i) : i)); }
-    __device__ uint32_t head2(uint64_t i) const
-    {
-        if (i == 0 || ((__ldg(ownbits + (i >> 5)) >> (i & 31)) & 1u)) return 3u;
-        return win_change(wv, __ldg(tarr + i), __ldg(tarr + i - 1));
-    }
+    __device__ uint32_t owner_word(uint64_t w32) const { return __ldg(ownbits + w32); }
 };
 
 struct RootScan2 {
-    static constexpr bool kGathered = true;
     const ulonglong2 *w;        // root weight pairs in list order
     const uint32_t *tarr;       // g_t
     WinDiv wv;
     const uint32_t *perm;       // gid -> weight position
     __device__ ulonglong2 value2(uint64_t i) const { return __ldg(w + (perm ? __ldg(perm + i) : i)); }
-    __device__ uint32_t head2(uint64_t i) const
-    {
-        if (i == 0) return 3u;
-        return win_change(wv, __ldg(tarr + i), __ldg(tarr + i - 1));
-    }
+    __device__ uint32_t owner_word(uint64_t) const { return 0u; }
 };
 
 // ---- windows of both layers (Constraint 3, Alg. 1) ------------------------
