@@ -159,7 +159,7 @@ void copy_d2h(tm_ctx *ctx, void *dst, const void *src, size_t bytes)
 
 int read_status(tm_ctx *ctx, uint32_t *bits)
 {
-    copy_d2h(ctx, ctx->status_host, ctx->status, 4);
+    copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
     int rc = check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronize");
     *bits = rc ? 0 : *ctx->status_host;
     if (!rc) prof_collect(ctx);
@@ -538,11 +538,11 @@ int tm_create(tm_ctx **out, const tm_config *cfg, void *cuda_stream)
         if (cuda_stream) ctx->stream = (cudaStream_t)cuda_stream;
         else { rc = check_cuda(ctx, cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking), "stream"); ctx->own_stream = true; }
     }
-    if (!rc) rc = check_cuda(ctx, cudaMallocHost((void **)&ctx->status_host, 64), "pinned status");
+    if (!rc) rc = check_cuda(ctx, cudaMallocHost((void **)&ctx->status_host, kStatusBytes), "pinned status");
     if (!rc) {
-        ctx->status = (uint32_t *)dalloc(ctx, 64);
+        ctx->status = (uint32_t *)dalloc(ctx, kStatusBytes);
         if (!ctx->status) rc = TM_E_NOMEM;
-        else cudaMemsetAsync(ctx->status, 0, 64, ctx->stream);
+        else cudaMemsetAsync(ctx->status, 0, kStatusBytes, ctx->stream);
     }
     if (rc) { tm_destroy(ctx); return rc; }
     *out = ctx;
@@ -562,7 +562,7 @@ void tm_destroy(tm_ctx *ctx)
     free_graph(ctx);
     arena_free(ctx);
     spare_free(ctx);
-    if (ctx->status) dfree(ctx, ctx->status, 64);
+    if (ctx->status) dfree(ctx, ctx->status, kStatusBytes);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     if (ctx->status_host) cudaFreeHost(ctx->status_host);
     if (ctx->pinned_acc) cudaFreeHost(ctx->pinned_acc);

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
     uint16_t *wc = s_wcnt + warp * OS_MAXRADIX;
     uint32_t *wm = s_match + warp * OS_MAXRADIX;
     uint32_t kv[ITEMS];         // the keys, then one payload after the other
-    uint32_t slot[ITEMS / 2];   // rank in the warp's chunk, then tile slot, 16 bits each
+    uint32_t slot[ITEMS / 2] = {};   // rank in the warp's chunk, then tile slot, 16 bits each
     auto load = [&](const uint32_t *__restrict__ in) {
 #pragma unroll
         for (int j = 0; j < ITEMS; ++j) {
@@ -603,8 +603,7 @@ __global__ void k_input_stats(const uint32_t *__restrict__ src, const uint32_t *
 }
 
 // Elementwise kernels below take kElemItems elements per thread (i, i +
-// blockDim, ...): with one element per thread the list offsets kernel
-// measured twice as slow.
+// blockDim, ...); one element per thread measured up to twice as slow.
 #ifndef TM_ELEM_ITEMS
 #define TM_ELEM_ITEMS 4
 #endif
@@ -793,94 +792,172 @@ __global__ void k_compact3(const uint32_t *__restrict__ a, const uint32_t *__res
 }
 
 
-// Owner-start bit sets of the out-, in- and multi-edge orders: position x
-// starts a new owner when its source (out-lists) or destination (in-lists)
-// differs from position x-1's, or when it heads a pair (multi-edge lists,
-// from the pair-head flags).  One thread per position; each warp's ballots
-// are one word of each set.
-__global__ void k_owner_bits(const uint32_t *__restrict__ out_src, const uint32_t *__restrict__ in_dst,
-                             const uint32_t *__restrict__ pair_head, uint32_t m, uint32_t words,
-                             uint32_t *__restrict__ own_out, uint32_t *__restrict__ own_in,
-                             uint32_t *__restrict__ own_multi)
+// The list offsets of a sorted key array, by the position at which a new key
+// starts: off[v] = x for every v after the key before it and up to its own.
+__device__ __forceinline__ void fill_offsets(uint32_t *__restrict__ off, uint32_t after, uint32_t upto, uint32_t n,
+                                             uint32_t x)
 {
+    for (uint32_t v = after; v <= upto && v <= n; ++v) off[v] = x;
+}
+
+// Vertex lists of the out and in orders: the offsets of each vertex's list, and
+// the owner-start bit sets (position x starts a new owner when its source
+// (out) or destination (in) differs from position x - 1's).  A warp takes 32
+// positions, whose ballots are one word of each set, and reads each key once
+// (offsets and bit sets by separate kernels: 250 us on 5e7 edges, 164 like
+// this; instructions bound it).
+__global__ void k_owners(const uint32_t *__restrict__ out_src, const uint32_t *__restrict__ in_dst, uint32_t m,
+                         uint32_t n, uint32_t words, uint32_t *__restrict__ out_off, uint32_t *__restrict__ in_off,
+                         uint32_t *__restrict__ own_out, uint32_t *__restrict__ own_in,
+                         const uint32_t *__restrict__ status)
+{
+    if (*status & ST_TIMEOUT) return;   // a sort whose wait ran out: its keys are anything
+    const int lane = threadIdx.x & 31;
     const uint64_t x0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
+    uint32_t k[2][kElemItems], kp[2][kElemItems];
 #pragma unroll
-    for (int k = 0; k < kElemItems; ++k) {
+    for (int r = 0; r < kElemItems; ++r) {
+        const uint64_t x = x0 + (uint64_t)r * blockDim.x;
+        k[0][r] = x < m ? __ldg(out_src + x) : 0u;
+        k[1][r] = x < m ? __ldg(in_dst + x) : 0u;
+        kp[0][r] = lane == 0 && x > 0 && x <= m ? __ldg(out_src + x - 1) : 0u;
+        kp[1][r] = lane == 0 && x > 0 && x <= m ? __ldg(in_dst + x - 1) : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < kElemItems; ++r) {
         // a warp's 32 positions are consecutive and start at a multiple of 32,
         // and words * 32 is a multiple of 32: whole warps leave together
-        const uint64_t x = x0 + (uint64_t)k * blockDim.x;
+        const uint64_t x = x0 + (uint64_t)r * blockDim.x;
         if (x >= (uint64_t)words * 32) break;
-        const bool in = x < m, first = x == 0;
-        const bool bo = in && (first || out_src[x] != out_src[x - 1]);
-        const bool bi = in && (first || in_dst[x] != in_dst[x - 1]);
-        const bool bm = in && pair_head[x] != 0;
-        const uint32_t wo = __ballot_sync(0xffffffffu, bo), wi = __ballot_sync(0xffffffffu, bi),
-                       wm = __ballot_sync(0xffffffffu, bm);
-        if ((threadIdx.x & 31) == 0) {
-            own_out[x >> 5] = wo;
-            own_in[x >> 5] = wi;
-            own_multi[x >> 5] = wm;
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const uint32_t up = __shfl_up_sync(0xffffffffu, k[s][r], 1);
+            const uint32_t prev = lane == 0 ? kp[s][r] : up;
+            const bool head = x < m && (x == 0 || k[s][r] != prev);
+            const uint32_t w = __ballot_sync(0xffffffffu, head);
+            if (lane == 0) (s ? own_in : own_out)[x >> 5] = w;
+            if (head || x == m) fill_offsets(s ? in_off : out_off, x == 0 ? 0u : prev + 1u, x == m ? n : k[s][r], n, (uint32_t)x);
         }
     }
 }
 
-// off[v] = first position whose sorted key is >= v, for v in [0, n].  With
-// m_dev set, the key count is min(m, *m_dev) (a count known only on the
-// device; m bounds the grid).
-#ifndef TM_OFF_ITEMS
-#define TM_OFF_ITEMS 8   // positions per thread (1: one per thread)
-#endif
-__global__ void k_offsets(const uint32_t *__restrict__ keys, uint32_t m, uint32_t n, uint32_t *__restrict__ off,
-                          const uint32_t *__restrict__ m_dev)
+// The pairs of the multi-edge order (msrc, mdst: sorted source and destination
+// of each position) in one pass: a position that starts a new pair is counted
+// over the rows of its warp, the warps of its tile and, by look-back, the tiles
+// before it, which numbers the pairs; their list starts, destinations, each
+// source's first pair and the owner bits follow.  The number of pairs goes to
+// *npairs.  The prefix moves through the tiles at about 32 per round trip to
+// L2, so large arrays take tiles of 64 rows per warp and read the keys, which
+// L2 still holds, again behind the look-back: 246 us on 5e7 edges (8 rows kept
+// in registers 457; flags, their scan, fill and source offsets as separate
+// kernels about 560).
+constexpr int kPairChunk = 8;   // rows whose loads are in flight together
+template <int ROWS>
+__global__ void __launch_bounds__(256) k_pairs(const uint32_t *__restrict__ msrc, const uint32_t *__restrict__ mdst,
+                                               uint32_t m, uint32_t n, unsigned long long *__restrict__ state,
+                                               uint32_t *__restrict__ ticket, uint32_t *__restrict__ pair_off,
+                                               uint32_t *__restrict__ pair_dst, uint32_t *__restrict__ vpair_off,
+                                               uint32_t *__restrict__ own_multi, uint32_t *__restrict__ npairs,
+                                               uint32_t *status)
 {
-    // positions [i0, i0 + TM_OFF_ITEMS) of this thread, the previous key carried
-    const uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * TM_OFF_ITEMS;
-    if (m_dev) m = min(m, *m_dev);
-    if (i0 > m) return;
-    uint32_t prev = i0 == 0 ? 0u : __ldg(keys + i0 - 1) + 1u;
+    __shared__ uint32_t s_w[8], s_tile, s_before, s_h[8][ROWS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0)   // a sort whose wait ran out: its keys are anything
+        s_tile = (*(volatile uint32_t *)status & ST_TIMEOUT) ? 0xFFFFFFFFu : atomicAdd(ticket, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile;
+    if (tile == 0xFFFFFFFFu) return;
+    const uint64_t base = ((uint64_t)tile * 8 + warp) * (32 * ROWS);
+    uint32_t u[kPairChunk], v[kPairChunk], pu, pv;   // a chunk of rows, and the keys before it
+    auto load = [&](uint64_t x0) {
 #pragma unroll
-    for (int j = 0; j < TM_OFF_ITEMS; ++j) {
-        const uint64_t i = i0 + j;
-        if (i > m) break;
-        const uint32_t lo = prev;
-        const uint32_t hi = (i == m) ? n : __ldg(keys + i);
-        for (uint32_t v = lo; v <= hi && v <= n; ++v) off[v] = (uint32_t)i;
-        prev = hi + 1u;
-    }
-}
-
-// Pair heads in the multi-edge order (src from the sorted keys, dst gathered).
-__global__ void k_pair_heads(const uint32_t *__restrict__ msrc, const uint32_t *__restrict__ mdst, uint32_t m,
-                             uint32_t *__restrict__ head)
-{
-    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < kElemItems; ++k) {
-        const uint64_t i = i0 + (uint64_t)k * blockDim.x;
-        if (i >= m) break;
-        head[i] = (i == 0 || msrc[i] != msrc[i - 1] || mdst[i] != mdst[i - 1]) ? 1u : 0u;
-    }
-}
-
-__global__ void k_pair_fill(const uint32_t *__restrict__ msrc, const uint32_t *__restrict__ mdst,
-                            const uint32_t *__restrict__ head, const uint32_t *__restrict__ pid_excl, uint32_t m,
-                            uint32_t *__restrict__ pair_off, uint32_t *__restrict__ pair_src,
-                            uint32_t *__restrict__ pair_dst)
-{
-    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < kElemItems; ++k) {
-        const uint32_t i = (uint32_t)(i0 + (uint64_t)k * blockDim.x);
-        if (i0 + (uint64_t)k * blockDim.x >= m) break;
-        if (head[i]) {
-            const uint32_t pid = pid_excl[i];
-            pair_off[pid] = i;
-            pair_src[pid] = msrc[i];
-            pair_dst[pid] = mdst[i];
+        for (int r = 0; r < kPairChunk; ++r) {
+            const uint64_t x = x0 + r * 32 + lane;
+            u[r] = x < m ? __ldg(msrc + x) : 0u;
+            v[r] = x < m ? __ldg(mdst + x) : 0u;
         }
-        if (i == m - 1) pair_off[pid_excl[i] + head[i]] = m;   // the end of the last pair's list
+        pu = x0 > 0 && x0 <= m ? __ldg(msrc + x0 - 1) : 0u;
+        pv = x0 > 0 && x0 <= m ? __ldg(mdst + x0 - 1) : 0u;
+    };
+    uint32_t mine = 0;
+    for (int c = 0; c < ROWS; c += kPairChunk) {
+        load(base + c * 32);
+#pragma unroll
+        for (int r = 0; r < kPairChunk; ++r) {
+            const uint64_t x = base + (c + r) * 32 + lane;
+            uint32_t a = __shfl_up_sync(0xffffffffu, u[r], 1), b = __shfl_up_sync(0xffffffffu, v[r], 1);
+            if (lane == 0) { a = pu; b = pv; }
+            pu = __shfl_sync(0xffffffffu, u[r], 31);
+            pv = __shfl_sync(0xffffffffu, v[r], 31);
+            const uint32_t h = __ballot_sync(0xffffffffu, x < m && (x == 0 || u[r] != a || v[r] != b));
+            mine += __popc(h);
+            if (lane == 0) {
+                s_h[warp][c + r] = h;
+                if (x <= m) own_multi[x >> 5] = h;
+            }
+        }
+    }
+    if (lane == 0) s_w[warp] = mine;
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t sum = 0;
+        for (int w = 0; w < 8; ++w) sum += s_w[w];
+        if (lane == 0) *(volatile unsigned long long *)(state + tile) = (tile == 0 ? kTilePrefix : kTileSum) | sum;
+        uint32_t before = 0;
+        for (int64_t j = (int64_t)tile - 1 - lane; tile != 0; j -= 32) {   // lane i at the i-th tile before
+            unsigned long long x = kTilePrefix;
+            if (j >= 0) {
+                x = *(volatile unsigned long long *)(state + j);
+                for (int it = 0; (x >> 62) == 0 && it < kLookbackPolls; ++it) {
+                    __nanosleep(32);
+                    x = *(volatile unsigned long long *)(state + j);
+                }
+                if ((x >> 62) == 0) { latch(status, ST_TIMEOUT); x = kTilePrefix; }
+            }
+            const unsigned end = __ballot_sync(0xffffffffu, (x >> 62) == 2);
+            const int last = end ? __ffs((int)end) - 1 : 31;
+            before += __reduce_add_sync(0xffffffffu, lane <= last ? (uint32_t)x : 0u);
+            if (end) break;
+        }
+        if (lane == 0) {
+            if (tile != 0) *(volatile unsigned long long *)(state + tile) = kTilePrefix | (before + sum);
+            s_before = before;
+        }
+    }
+    __syncthreads();
+    uint32_t pid = s_before;   // pairs before the row
+    for (int w = 0; w < warp; ++w) pid += s_w[w];
+    for (int c = 0; c < ROWS; c += kPairChunk) {
+        if (ROWS > kPairChunk || c > 0) load(base + c * 32);
+        else pu = base > 0 && base <= m ? __ldg(msrc + base - 1) : 0u;
+#pragma unroll
+        for (int r = 0; r < kPairChunk; ++r) {
+            const uint64_t x = base + (c + r) * 32 + lane;
+            uint32_t a = __shfl_up_sync(0xffffffffu, u[r], 1);
+            if (lane == 0) a = pu;
+            pu = __shfl_sync(0xffffffffu, u[r], 31);
+            const uint32_t h = s_h[warp][c + r];
+            const uint32_t id = pid + __popc(h & ((1u << lane) - 1u));
+            const bool head = (h >> lane) & 1u;
+            if (head) {
+                pair_off[id] = (uint32_t)x;
+                pair_dst[id] = v[r];
+                if (x == 0 || u[r] != a) fill_offsets(vpair_off, x == 0 ? 0u : a + 1u, u[r], n, id);
+            }
+            if (x == m - 1) {   // after the last pair
+                const uint32_t end = id + (head ? 1u : 0u);
+                pair_off[end] = m;
+                *npairs = end;
+                fill_offsets(vpair_off, u[r] + 1u, n, n, end);
+            }
+            pid += __popc(h);
+        }
     }
 }
+// rows per warp: small arrays need the blocks more than the fewer tiles
+constexpr int kPairRowsSmall = 8, kPairRowsLarge = 64;
+constexpr uint32_t kPairSmall = 4000000;   // 244 tiles of the larger size: about one for each SM
+inline uint32_t pair_tiles(uint32_t m) { return m / (256 * (m <= kPairSmall ? kPairRowsSmall : kPairRowsLarge)) + 1; }
 
 // where each list time falls in the same vertex's other list
 // Cross ranks of both lists (blockIdx.y = 0: out-list entries into the
@@ -1016,9 +1093,12 @@ int build_csr(tm_ctx *ctx)
     int vbits = bits_for(n ? n - 1 : 0);
     int tbits = bits_for((unsigned long long)tmax - (unsigned long long)tmin);
     const DigitPlan Dt = digit_plan(tbits), Dv = digit_plan(vbits);
-    uint32_t *hist = (uint32_t *)salloc(ctx, 3 * OS_HIST * 4);   // digit counts of t', src, dst
+    // cleared together: digit counts of t', src, dst; the pair kernel's ticket
+    // (16 words) and tile words
+    uint32_t *hist = (uint32_t *)salloc(ctx, (3 * OS_HIST + 16) * 4 + ((size_t)m + 2047) / 2048 * 8 + 64);
     if (!hist) return TM_E_NOMEM;
-    cudaMemsetAsync(hist, 0, 3 * OS_HIST * 4, st);
+    unsigned long long *pair_state = (unsigned long long *)(hist + 3 * OS_HIST + 16);
+    cudaMemsetAsync(hist, 0, (3 * OS_HIST + 16) * 4 + ((size_t)m + 2047) / 2048 * 8 + 64, st);
     const unsigned cblk = (unsigned)std::min<uint64_t>(blocks_for((m0 + kElemItems - 1) / kElemItems, TB),
                                                        (uint64_t)ctx->num_sms * 8);
     if (hs.nself) {
@@ -1150,8 +1230,12 @@ int build_csr(tm_ctx *ctx)
     }
     sec.reset();
     sec.reset(new PhaseScope(ctx, TM_PH_CSR_IN));
-    launch(ctx, k_offsets, blocks_for(((uint64_t)m + TM_OFF_ITEMS) / TM_OFF_ITEMS, TB), TB, g.out_src, m, n, g.out_off, nullptr);
-    launch(ctx, k_offsets, blocks_for(((uint64_t)m + TM_OFF_ITEMS) / TM_OFF_ITEMS, TB), TB, g.in_dst, m, n, g.in_off, nullptr);
+    g.own_out = gtake(gb, (size_t)m / 32 + 1); g.own_in = gtake(gb, (size_t)m / 32 + 1);
+    g.own_multi = gtake(gb, (size_t)m / 32 + 1);
+    if (!g.own_out || !g.own_in || !g.own_multi) return TM_E_NOMEM;
+    const uint32_t words = m / 32 + 1;
+    launch(ctx, k_owners, blocks_for(((uint64_t)words * 32 + kElemItems - 1) / kElemItems, TB), TB, g.out_src, g.in_dst,
+           m, n, words, g.out_off, g.in_off, g.own_out, g.own_in, ctx->status);
     uint32_t *key = S0, *tmp = D0;
     // ---- multi-edge order: stable re-sort of the IN order by source
     sec.reset();
@@ -1159,10 +1243,7 @@ int build_csr(tm_ctx *ctx)
     g.multi_t = gtake(gb, m);
     g.multi_to_out = gtake(gb, m);
     g.vpair_off = gtake(gb, (size_t)n + 1);
-    g.own_out = gtake(gb, (size_t)m / 32 + 1); g.own_in = gtake(gb, (size_t)m / 32 + 1);
-    g.own_multi = gtake(gb, (size_t)m / 32 + 1);
-    if (!g.multi_t || !g.vpair_off || !g.multi_to_out || !g.own_out || !g.own_in || !g.own_multi)
-        return TM_E_NOMEM;
+    if (!g.multi_t || !g.vpair_off || !g.multi_to_out) return TM_E_NOMEM;
     uint32_t np = 0;
     if (m) {
         {
@@ -1173,46 +1254,31 @@ int build_csr(tm_ctx *ctx)
             rc = radix_sort_to(ctx, ms, m, vbits);
             if (rc) return rc;
         }
-        // key = pair src, tmp = pair dst per multi position
-        uint32_t *head = T0;
-        uint32_t *pid = (uint32_t *)salloc(ctx, (size_t)m * 4);
-        uint32_t *dnp = (uint32_t *)salloc(ctx, 4);
-        if (!pid || !dnp) return TM_E_NOMEM;
-        launch(ctx, k_pair_heads, blocks_for(((uint64_t)m + kElemItems - 1) / kElemItems, TB), TB, key, tmp, m, head);
-        rc = exclusive_scan_u32(ctx, head, pid, m, dnp);
-        if (rc) return rc;
-        // dnp = the number of pairs (the scan's total), used on the device;
-        // the pair tables are m-sized slots of the graph block
+        // key = pair src, tmp = pair dst per multi position; the pair tables
+        // are m-sized slots of the graph block, the pair count stays on the
+        // device until the closing synchronize
         g.pair_off = gtake(gb, (size_t)m + 1);
         g.pair_dst = gtake(gb, m);
-        uint32_t *pair_src = (uint32_t *)salloc(ctx, (size_t)m * 4);
-        if (!g.pair_off || !g.pair_dst || !pair_src) return TM_E_NOMEM;
-        launch(ctx, k_pair_fill, blocks_for(((uint64_t)m + kElemItems - 1) / kElemItems, TB), TB, (const uint32_t *)key,
-               (const uint32_t *)tmp,
-               (const uint32_t *)head, (const uint32_t *)pid, m, g.pair_off, pair_src, g.pair_dst);
-        launch(ctx, k_offsets, blocks_for(((uint64_t)m + TM_OFF_ITEMS) / TM_OFF_ITEMS, TB), TB, pair_src, m, n, g.vpair_off, (const uint32_t *)dnp);
-        copy_d2h(ctx, ctx->status_host + 1, dnp, 4);   // pinned: read after the closing synchronize
+        if (!g.pair_off || !g.pair_dst) return TM_E_NOMEM;
+        launch(ctx, m <= kPairSmall ? k_pairs<kPairRowsSmall> : k_pairs<kPairRowsLarge>, pair_tiles(m), 256,
+               (const uint32_t *)key, (const uint32_t *)tmp, m, n, pair_state, hist + 3 * OS_HIST, g.pair_off,
+               g.pair_dst, g.vpair_off, g.own_multi, ctx->status + 1, ctx->status);
         // cross ranks between a vertex's out- and in-lists
         launch(ctx, k_cross_rank, dim3(blocks_for(((uint64_t)m + TM_XR_ITEMS - 1) / TM_XR_ITEMS, TB), 2), TB,
                XR{g.out_t, g.out_src, g.in_off, g.in_t, g.out_xrank},
                XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m, n);
-        // owner starts of the three orders (segment heads of the weight pass's scans)
-        const uint32_t words = m / 32 + 1;
-        launch(ctx, k_owner_bits, blocks_for(((uint64_t)words * 32 + kElemItems - 1) / kElemItems, TB), TB,
-               (const uint32_t *)g.out_src, (const uint32_t *)g.in_dst,
-               (const uint32_t *)head, m, words, g.own_out, g.own_in, g.own_multi);
     } else {
         GraphBlock pbk;
         if (!gblock_open(ctx, pbk, 3 * 256)) return TM_E_NOMEM;
         g.pair_off = gtake(pbk, 1);
         g.pair_dst = gtake(pbk, 1);
         cudaMemsetAsync(g.pair_off, 0, 4, st);
-        launch(ctx, k_offsets, 1, TB, key, 0, n, g.vpair_off, nullptr);
+        cudaMemsetAsync(g.vpair_off, 0, ((size_t)n + 1) * 4, st);
     }
     uint32_t bits = 0;
     int rc2 = read_status(ctx, &bits);   // the build's one closing synchronize
     if (rc2) return rc2;
-    if (m) np = ctx->status_host[1];
+    if (m) np = ctx->status_host[1];   // copied with the status
     g.npairs = np;
     if (bits) return set_err(ctx, TM_E_CUDA, "CSR build: device status " + std::to_string(bits));
     return TM_OK;

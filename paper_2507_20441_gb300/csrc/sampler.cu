@@ -871,8 +871,8 @@ __global__ void __launch_bounds__(kSampleThreads) k_list_sums(const uint64_t *__
     if (ovf) latch(status, ST_OVERFLOW);
 }
 
-__global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums, uint64_t n, uint64_t *__restrict__ total,
-                                                    uint32_t *status)
+__global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums, uint64_t n, uint64_t *__restrict__ end,
+                                                    uint64_t *__restrict__ total, uint32_t *status)
 {
     uint64_t carry = 0;
     bool ovf = false;
@@ -883,7 +883,7 @@ __global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums,
         if (i < n) sums[i] = add_chk(carry, before, ovf);
         carry = add_chk(carry, t, ovf);
     }
-    if (threadIdx.x == 0) *total = carry;
+    if (threadIdx.x == 0) *end = *total = carry;
     if (ovf) latch(status, ST_OVERFLOW);
 }
 
@@ -1273,18 +1273,17 @@ int run_list(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t firs
     {
         PhaseScope ph(ctx, TM_PH_SAMPLE);
         launch(ctx, k_list_sums, (unsigned)tiles, kSampleThreads, (const uint64_t *)dcnt, k, sums, ctx->status);
-        launch(ctx, k_list_scan, 1, 1024, sums, tiles, dcnt + k, ctx->status);
+        launch(ctx, k_list_scan, 1, 1024, sums, tiles, dcnt + k, (uint64_t *)(ctx->status + 4), ctx->status);
         launch(ctx, k_list_offsets, (unsigned)tiles, kSampleThreads, dcnt, k, (const uint64_t *)sums);
     }
     int rc = check_cuda(ctx, cudaGetLastError(), "listing count");
     if (rc) return rc;
-    copy_d2h(ctx, ctx->status_host + 4, dcnt + k, 8);   // pinned: read with the status
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a completion count or the instance count exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "listing reached an inconsistent state");
-    memcpy(n_inst, ctx->status_host + 4, 8);
+    memcpy(n_inst, ctx->status_host + 4, 8);   // copied with the status
     const uint64_t rows = std::min<uint64_t>(max_inst, *n_inst);
     if (rows == 0 || !inst_gids || !inst_sample) return TM_OK;
     const size_t ne = mo->ne;

@@ -27,6 +27,8 @@ enum : uint32_t {
     ST_RANGE = 32u         // an id out of range
 };
 
+constexpr size_t kStatusBytes = 64;   // tm_ctx::status
+
 // Guide table of the window pick: draws r in [j 2^s, (j+1) 2^s) fall in a
 // window between wguide[j] and wguide[j+1].  s = max(0, bitlen(W) -
 // bitlen(nw) - 1), so there are at most 4 nw buckets; the same function
@@ -237,8 +239,9 @@ struct tm_ctx {
     bool in_borrowed = false;                        // in_* point at the caller's arrays
     timest::DevGraph g;
     std::vector<std::pair<void *, size_t>> graph_bufs;
-    uint32_t *status = nullptr;          // device status word
-    uint32_t *status_host = nullptr;     // pinned: [0] status mirror, [1] the CSR build's pair count
+    uint32_t *status = nullptr;          // device block, copied as a whole (kStatusBytes): [0] status bits,
+                                         // [1] the CSR build's pair count, [4] on: a call's small results
+    uint32_t *status_host = nullptr;     // its pinned mirror
     int num_sms = 0;
     // phase timing (cfg.profile)
     struct PendingPhase { int phase; cudaEvent_t a, b; uint64_t launches; };

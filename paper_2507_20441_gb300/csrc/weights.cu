@@ -481,13 +481,15 @@ struct GuideArgs {
 };
 
 // Window totals W_i (last root-CDF entry of each window) and their 128-bit
-// running sum over (layer 0 windows, layer 1 windows) by block 0; the guide
+// running sum over (layer 0 windows, layer 1 windows) by block 0, which also
+// puts their total at W; the guide
 // table's bucket width and offset of each window by block 1 + p for layer p.
 // A block takes kTotItems windows per thread at a time, whose loads are
 // independent (a contiguous run of windows per thread is one load after the
 // other: 82 + 38 us in two launches for 5.6e4 windows, 36 us like this).
 constexpr int kTotItems = 8;
-__global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *__restrict__ wcum)
+__global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *__restrict__ wcum,
+                                                        uint64_t *__restrict__ W)
 {
     __shared__ u128 s_tot[32];
     __shared__ u128 s_carry;
@@ -558,8 +560,8 @@ __global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *_
         __syncthreads();   // s_tot is written again
     }
     if (b == 0 && threadIdx.x == 0) {
-        wcum[2 * (size_t)n] = (uint64_t)s_carry;
-        wcum[2 * (size_t)n + 1] = (uint64_t)(s_carry >> 64);
+        W[0] = wcum[2 * (size_t)n] = (uint64_t)s_carry;
+        W[1] = wcum[2 * (size_t)n + 1] = (uint64_t)(s_carry >> 64);
     }
 }
 
@@ -902,19 +904,18 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     mo->nwtot = nw0 + nw1;
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
-        launch(ctx, k_window_totals, 3, 1024, guide_args(mo), mo->wcum);
+        launch(ctx, k_window_totals, 3, 1024, guide_args(mo), mo->wcum, (uint64_t *)(ctx->status + 4));
         if (guides) {
             rc = fill_guides(ctx, mo);
             if (rc) return rc;
         }
-        copy_d2h(ctx, ctx->status_host + 4, mo->wcum + 2 * (size_t)mo->nwtot, 16);   // pinned: read with the status
     }
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a weight, prefix sum or window total exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "device status error in weight pass");
-    memcpy(&mo->W, ctx->status_host + 4, 16);
+    memcpy(&mo->W, ctx->status_host + 4, 16);   // copied with the status
     mo->have_weights = true;
     mo->graph_epoch = ctx->epoch;
     return TM_OK;

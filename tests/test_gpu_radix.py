@@ -2,7 +2,8 @@
 1024 and of 4096 keys, the size from which a sort takes the larger tile, sorts
 of one to five passes, digit counts made anew after repeats are dropped, a run
 of equal times too long to order in place (the sort by all three keys), and an
-inverse permutation past the size up to which the last pass writes it.  Every
+inverse permutation past the size up to which the last pass writes it, where the
+pair tables take their larger tiles too.  Every
 array of the temporal CSR equals the oracle's definition; for the last, that
 definition's properties (whole numbers, no tolerance)."""
 import numpy as np
@@ -62,4 +63,13 @@ def test_inverse_of_a_large_sort(tg):
         assert np.array_equal(pos[gid], at)
         assert np.array_equal(owner, g_owner[gid])
         assert np.all((owner[1:] > owner[:-1]) | ((owner[1:] == owner[:-1]) & (gid[1:] > gid[:-1])))
+    # the pair tables (larger tiles than a small array's)
+    pairs, count = np.unique(g_src.astype(np.int64) * n + g_dst, return_counts=True)
+    start = np.concatenate([[0], np.cumsum(count)])
+    assert np.array_equal(ctx.csr("pair_dst"), pairs % n)
+    assert np.array_equal(ctx.csr("pair_off"), start)
+    assert np.array_equal(ctx.csr("vpair_off"), np.searchsorted(pairs // n, np.arange(n + 1)))
+    own = np.zeros((m // 32 + 1) * 32, np.uint8)
+    own[start[:-1]] = 1
+    assert np.array_equal(ctx.csr("own_multi"), np.packbits(own, bitorder="little").view(np.uint32))
     ctx.close()
