@@ -21,6 +21,7 @@
 // per thread in lockstep).
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <algorithm>
 #include <memory>
@@ -1053,7 +1054,6 @@ int build_csr(tm_ctx *ctx)
 {
     ScratchScope scope(ctx);
     GraphBlock gb;
-    cudaMemsetAsync(ctx->status, 0, 4, ctx->stream);
     const int TB = 256;
     cudaStream_t st = ctx->stream;
     uint64_t m0 = ctx->m_in;
@@ -1064,17 +1064,21 @@ int build_csr(tm_ctx *ctx)
     int rc = TM_OK;
     // ---- statistics: t range, self loops, bad ids
     std::unique_ptr<PhaseScope> sec(new PhaseScope(ctx, TM_PH_CSR_STATS));
+    // (in the status block, which the copy clears: pinned both ways)
+    static_assert(16 + sizeof(Stats) <= kStatusBytes, "the statistics fit the status block");
     Stats hs{LLONG_MAX, LLONG_MIN, 0, 0};
-    Stats *ds = (Stats *)salloc(ctx, sizeof(Stats));
-    if (!ds) return TM_E_NOMEM;
-    copy_h2d(ctx, ds, &hs, sizeof(Stats));
+    Stats *ds = (Stats *)(ctx->status + 4);
+    memset(ctx->status_host, 0, kStatusBytes);
+    memcpy(ctx->status_host + 4, &hs, sizeof(Stats));
+    copy_h2d(ctx, ctx->status, ctx->status_host, kStatusBytes);
     if (m0) {
         unsigned nb = std::min<uint64_t>(blocks_for(m0, TB), (uint64_t)ctx->num_sms * 8);
         launch(ctx, k_input_stats, nb, TB, ctx->in_src, ctx->in_dst, ctx->in_t, m0, n, ds);
     }
-    copy_d2h(ctx, &hs, ds, sizeof(Stats));
+    copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
     rc = check_cuda(ctx, cudaStreamSynchronize(st), "input statistics");
     if (rc) return rc;
+    memcpy(&hs, ctx->status_host + 4, sizeof(Stats));
     if (hs.nbad) return set_err(ctx, TM_E_ARG, "vertex id >= n in input");
     if (hs.nself && !(ctx->load_flags & TM_DROP_SELF))
         return set_err(ctx, TM_E_SELFLOOP, "input has self loops (pass TM_DROP_SELF to drop them)");
@@ -1139,9 +1143,9 @@ int build_csr(tm_ctx *ctx)
     {
         uint32_t *keep = (uint32_t *)salloc(ctx, (size_t)(m ? m : 1) * 4);
         // [0] duplicates, [1] a run too long, [2] number of listed runs
-        unsigned long long *nd = (unsigned long long *)salloc(ctx, 24);
+        unsigned long long *nd = (unsigned long long *)(ctx->status + 4);
         uint2 *long_runs = (uint2 *)salloc(ctx, ((size_t)m / (kRunMax + 1) + 1) * sizeof(uint2));
-        if (!keep || !nd || !long_runs) return TM_E_NOMEM;
+        if (!keep || !long_runs) return TM_E_NOMEM;
         cudaMemsetAsync(nd, 0, 24, st);
         if (m) {
             launch(ctx, k_order_runs, blocks_for(((uint64_t)m + kElemItems - 1) / kElemItems, TB), TB,
@@ -1151,9 +1155,10 @@ int build_csr(tm_ctx *ctx)
                    (const uint32_t *)(nd + 2), nd);
         }
         unsigned long long hnd[2] = {0, 0};
-        copy_d2h(ctx, hnd, nd, 16);
+        copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
         rc = check_cuda(ctx, cudaStreamSynchronize(st), "duplicate scan");
         if (rc) return rc;
+        memcpy(hnd, ctx->status_host + 4, 16);
         if (hnd[1]) {
             // (the work arrays hold the same tuples in input order)
             const RsTo by_dst{D0, {S0, T0}, g.g_dst, {g.g_src, g.g_t}}, by_src{g.g_src, {g.g_dst, g.g_t}, S0, {D0, T0}},
@@ -1164,9 +1169,10 @@ int build_csr(tm_ctx *ctx)
             if (rc) return rc;
             cudaMemsetAsync(nd, 0, 8, st);
             launch(ctx, k_flag_unique, blocks_for(m, TB), TB, g.g_t, g.g_src, g.g_dst, m, keep, nd);
-            copy_d2h(ctx, hnd, nd, 8);
+            copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
             rc = check_cuda(ctx, cudaStreamSynchronize(st), "duplicate scan");
             if (rc) return rc;
+            memcpy(hnd, ctx->status_host + 4, 8);
         }
         const unsigned long long ndup = hnd[0];
         if (ndup && !(ctx->load_flags & TM_DEDUP)) {

@@ -675,7 +675,7 @@ constexpr int kSampleThreads = TM_SAMPLE_THREADS;
 constexpr int kTraceMinB = 5, kGroupMinB = 6;
 
 template <bool TRACE>
-__global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph g, const DevPlan *__restrict__ plan,
+__global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph g, const __grid_constant__ DevPlan plan,
                                                               SampleJob J, uint64_t seed, uint64_t first, uint64_t k,
                                                               Acc *acc, uint32_t *status, uint32_t *tr_gid,
                                                               uint64_t *tr_contrib, int32_t *tr_reason)
@@ -685,7 +685,7 @@ __global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph 
     __shared__ uint32_t recs[kRecRows * kSampleThreads];
 #endif
     {
-        const int *src = reinterpret_cast<const int *>(plan);
+        const int *src = reinterpret_cast<const int *>(&plan);
         int *dst = reinterpret_cast<int *>(&sp);
         for (int i = threadIdx.x; i < (int)(sizeof(DevPlan) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
     }
@@ -713,13 +713,13 @@ __global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph 
 
 // k_sample without a trace for a tree of NT nodes, records in registers.
 template <int NT>
-__global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB) k_sample_reg(DevGraph g, const DevPlan *__restrict__ plan,
+__global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB) k_sample_reg(DevGraph g, const __grid_constant__ DevPlan plan,
                                                               SampleJob J, uint64_t seed, uint64_t first, uint64_t k,
                                                               Acc *acc, uint32_t *status)
 {
     __shared__ DevPlan sp;
     {
-        const int *src = reinterpret_cast<const int *>(plan);
+        const int *src = reinterpret_cast<const int *>(&plan);
         int *dst = reinterpret_cast<int *>(&sp);
         for (int i = threadIdx.x; i < (int)(sizeof(DevPlan) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
     }
@@ -1165,13 +1165,13 @@ static bool reg_plan(const DevPlan &P) { return P.nv == P.ntree + 1 && (P.nnt ==
 
 // The register-record sampler for this plan's tree size; false when there is
 // none (the caller launches k_sample).
-static bool launch_sample_reg(tm_ctx *ctx, const DevPlan &P, unsigned blocks, int threads, const DevPlan *dplan,
-                              const SampleJob &J, uint64_t seed, uint64_t first, uint64_t k, Acc *dacc)
+static bool launch_sample_reg(tm_ctx *ctx, const DevPlan &P, unsigned blocks, int threads, const SampleJob &J,
+                              uint64_t seed, uint64_t first, uint64_t k, Acc *dacc)
 {
     if (!reg_plan(P)) return false;
     switch (P.ntree) {
 #define TM_REG_CASE(N) \
-    case N: launch(ctx, k_sample_reg<N>, blocks, threads, ctx->g, dplan, J, seed, first, k, dacc, ctx->status); return true;
+    case N: launch(ctx, k_sample_reg<N>, blocks, threads, ctx->g, P, J, seed, first, k, dacc, ctx->status); return true;
         TM_REG_CASE(1) TM_REG_CASE(2) TM_REG_CASE(3) TM_REG_CASE(4) TM_REG_CASE(5) TM_REG_CASE(6) TM_REG_CASE(7)
 #undef TM_REG_CASE
     default: return false;
@@ -1189,16 +1189,14 @@ int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t f
         return TM_OK;
     }
     const bool trace = trace_gids || trace_contrib || trace_reason;
-    size_t plan_bytes = sizeof(DevPlan), acc_bytes = sizeof(Acc);
-    char *scratch = (char *)salloc(ctx, plan_bytes + acc_bytes + 64);
-    if (!scratch) return TM_E_NOMEM;
-    DevPlan *dplan = (DevPlan *)scratch;
-    Acc *dacc = (Acc *)(scratch + ((plan_bytes + 15) / 16) * 16);
-    copy_h2d(ctx, dplan, &mo->plan, plan_bytes);
-    cudaMemsetAsync(dacc, 0, acc_bytes, st);
-    cudaMemsetAsync(ctx->status, 0, 4, st);
+    // the plan goes with the launch, the sums come back with the status: one
+    // clear, one kernel, one copy (a plan copied before and sums copied after
+    // were 9 of the 53 us of a call of 1e4 samples)
+    static_assert(16 + sizeof(Acc) <= kStatusBytes, "the sums fit the status block");
+    Acc *dacc = (Acc *)(ctx->status + 4);
+    cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
     SampleJob J;
-    fill_job(mo, J, dplan);
+    fill_job(mo, J, nullptr);
     const int threads = kSampleThreads;
     uint64_t want = (k + threads - 1) / threads;
     const bool local = trace || !reg_plan(mo->plan);   // records in local memory: k_sample
@@ -1218,15 +1216,13 @@ int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t f
             dc = (uint64_t *)t;
             dr = (int32_t *)(t + (size_t)k * 8);
             dg = (uint32_t *)(t + (size_t)k * 12);
-            launch(ctx, k_sample<true>, blocks, threads, ctx->g, dplan, J, seed, first, k, dacc, ctx->status, dg, dc, dr);
-        } else if (!launch_sample_reg(ctx, mo->plan, blocks, threads, dplan, J, seed, first, k, dacc)) {
-            launch(ctx, k_sample<false>, blocks, threads, ctx->g, dplan, J, seed, first, k, dacc, ctx->status, nullptr,
-                                                        nullptr, nullptr);
+            launch(ctx, k_sample<true>, blocks, threads, ctx->g, mo->plan, J, seed, first, k, dacc, ctx->status, dg, dc, dr);
+        } else if (!launch_sample_reg(ctx, mo->plan, blocks, threads, J, seed, first, k, dacc)) {
+            launch(ctx, k_sample<false>, blocks, threads, ctx->g, mo->plan, J, seed, first, k, dacc, ctx->status,
+                   nullptr, nullptr, nullptr);
         }
         rc = check_cuda(ctx, cudaGetLastError(), "sampler launch");
     }
-    Acc h{};
-    copy_d2h(ctx, &h, dacc, acc_bytes);
     if (trace && rc == TM_OK) {
         if (trace_gids) copy_d2h(ctx, trace_gids, dg, (size_t)k * 4 * mo->plan.ntree);
         if (trace_contrib) copy_d2h(ctx, trace_contrib, dc, (size_t)k * 8);
@@ -1236,6 +1232,8 @@ int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t f
     int rc2 = read_status(ctx, &bits);
     if (rc) return rc;
     if (rc2) return rc2;
+    Acc h;
+    memcpy(&h, ctx->status_host + 4, sizeof(Acc));   // copied with the status
     finish_result(mo, k, h, out);
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a completion count exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "sampler reached an inconsistent state (status " + std::to_string(bits) + ")");
@@ -1532,9 +1530,9 @@ int run_batch(tm_ctx *ctx, uint32_t nq, tm_motif *const *motifs, const uint64_t 
 // framework that owns the allocator and forbids allocations from plug-ins,
 // or a latency-bound loop that cannot afford an allocator call (which may
 // synchronise the device).  tm_sample_noalloc runs the same sampling kernel
-// as tm_sample, but its scratch -- the device copy of the motif plan and the
-// result accumulators -- lives in the fixed array below instead of memory
-// obtained from the allocator.
+// as tm_sample (the motif plan goes with the launch), but its scratch -- the
+// result accumulators behind room for a plan -- lives in the fixed array below
+// instead of memory obtained from the allocator.
 // ---------------------------------------------------------------------------
 namespace timest {
 namespace {
@@ -1591,20 +1589,18 @@ extern "C" int tm_sample_noalloc(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t
         finish_result(mo, k, zero, out);
         return TM_OK;
     }
-    DevPlan *dplan = (DevPlan *)scratch;
     Acc *dacc = (Acc *)(scratch + plan_bytes);
     cudaStream_t st = ctx->stream;
-    copy_h2d(ctx, dplan, &mo->plan, sizeof(DevPlan));
     cudaMemsetAsync(dacc, 0, sizeof(Acc), st);   // the array keeps the previous call's sums
     cudaMemsetAsync(ctx->status, 0, 4, st);
     SampleJob J;
-    fill_job(mo, J, dplan);
+    fill_job(mo, J, nullptr);
     const int threads = kSampleThreads;
     uint64_t want = (k + threads - 1) / threads;
     uint64_t cap = (uint64_t)ctx->num_sms * 16;
     unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min(want, cap));
-    launch(ctx, k_sample<false>, blocks, threads, ctx->g, dplan, J, seed, first_index, k, dacc, ctx->status, nullptr,
-           nullptr, nullptr);
+    launch(ctx, k_sample<false>, blocks, threads, ctx->g, mo->plan, J, seed, first_index, k, dacc, ctx->status,
+           nullptr, nullptr, nullptr);
     rc = check_cuda(ctx, cudaGetLastError(), "sampler launch");
     Acc h{};
     copy_d2h(ctx, &h, dacc, sizeof(Acc));

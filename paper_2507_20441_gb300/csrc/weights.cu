@@ -749,7 +749,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
             launch(ctx, k_win_count, ntile, TB, g.g_t, m, wv, ntile, wcount);
             rc = exclusive_scan_u32(ctx, wcount, woffs, 2 * (uint64_t)ntile, woffs + 2 * (size_t)ntile);
             if (rc) return rc;
-            uint32_t both[2] = {0, 0};
+            uint32_t *both = ctx->status_host + 4;   // pinned
             copy_d2h(ctx, &both[0], woffs + ntile, 4);                  // layer 0's windows
             copy_d2h(ctx, &both[1], woffs + 2 * (size_t)ntile, 4);      // all windows
             rc = check_cuda(ctx, cudaStreamSynchronize(st), "window count");
