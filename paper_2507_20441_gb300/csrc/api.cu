@@ -457,6 +457,18 @@ static int compile_plan(const MotifDesc &M, const int *tree, int root, int64_t d
     }
     for (int q = 0; q < P.ntree; ++q) P.tslot[q] = (q > 0 && !P.tleaf[q]) ? slot++ : -1;
     P.nslots = slot;
+    P.nkinds = 0;
+    P.tkind[0] = -1;
+    for (int q = 1; q < P.ntree; ++q) {
+        int k = 0;
+        while (k < P.nkinds && (P.kside[k] != P.tzside[q] || P.kout[k] != P.tout[q] || P.klater[k] != P.tlater[q])) ++k;
+        if (k == P.nkinds) {
+            ++P.nkinds;
+            P.kside[k] = P.tzside[q]; P.kout[k] = P.tout[q]; P.klater[k] = P.tlater[q];
+        }
+        P.tkind[q] = k;
+        if (!P.tleaf[q]) P.kinner[k] = 1;
+    }
     // non-tree edges along pi and their neighbouring tree positions
     for (int e = 0; e < M.ne; ++e) P.tnode_of_edge[e] = -1;
     for (int q = 0; q < P.ntree; ++q) P.tnode_of_edge[P.tedge[q]] = q;

@@ -305,52 +305,6 @@ __device__ __forceinline__ void sample_root(const DevPlan &P, const SampleJob &J
     if (root > ghi) { latch(status, ST_BADSTATE); root = ghi; }
 }
 
-// Time range of the child edge q of a parent edge at time pt, inside the
-// window [wlo, whi] (Constraint 1); false when it is empty.
-__device__ __forceinline__ bool child_times(const DevPlan &P, int q, uint32_t pt, uint32_t wlo, uint32_t whi,
-                                            uint64_t &tlo, uint64_t &thi)
-{
-    const uint64_t d = (uint64_t)P.delta;
-    if (P.tlater[q]) { tlo = (uint64_t)pt + 1; thi = (uint64_t)pt + d; }
-    else {
-        if (pt == 0) return false;
-        tlo = (uint64_t)pt >= d ? (uint64_t)pt - d : 0;
-        thi = (uint64_t)pt - 1;
-    }
-    tlo = tlo < (uint64_t)wlo ? (uint64_t)wlo : tlo;
-    thi = thi > (uint64_t)whi ? (uint64_t)whi : thi;
-    return true;
-}
-
-// The candidate range of a parent edge whose range the weight pass did not
-// keep, found by the DP's searches.
-__device__ __noinline__ uint2 search_range(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t ppos,
-                                           uint32_t pt, uint32_t wlo, uint32_t whi)
-{
-    uint64_t tlo, thi;
-    uint32_t a = 0, b = 0, beg;
-    const uint32_t *tarr;
-    if (child_times(P, q, pt, wlo, whi, tlo, thi))
-        child_range(g, P.tzside[q] != 0 ? 1 : 0, P.tout[q] != 0, zg, ppos, pt, P.tlater[q] != 0, tlo, thi, a, b, beg,
-                    tarr);
-    return make_uint2(a, b);
-}
-
-// The excluded entries of such a range (Claim 3.1): the part [ea, eb) of the
-// multi-edge list from pb on - zg -> og for a child leaving the meeting
-// vertex, og -> zg for one entering it - in the child's time range.
-__device__ __noinline__ uint3 search_excluded(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t og,
-                                              uint32_t pt, uint32_t wlo, uint32_t whi)
-{
-    uint64_t tlo, thi;
-    const bool out = P.tout[q] != 0;
-    const uint32_t pe = pair_of(g, out ? zg : og, out ? og : zg);
-    if (pe == kNone || !child_times(P, q, pt, wlo, whi, tlo, thi)) return make_uint3(0, 0, 0);
-    const uint32_t pb = __ldg(g.pair_off + pe), pend = __ldg(g.pair_off + pe + 1);
-    const uint32_t ea = lower_idx(g.multi_t, pb, pend, tlo);
-    return make_uint3(pb, ea, gallop_idx(g.multi_t, ea, pend, thi + 1));
-}
-
 // One tree edge of Alg. 3: the edge of tree node q, drawn by weight from its
 // candidate list at the meeting vertex given its parent's edge (source ps,
 // destination pd, time pt, edge id pgid), in layer p whose
@@ -387,31 +341,33 @@ __device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P
     uint64_t hit = 0;
     bool em = false;
     uint2 r = make_uint2(0, kRangeLong | (kRangeLong << 16));
-    if (J.range.base) r = __ldg(J.range.base + (size_t)(q - 1) * J.range.stride + ppos);
+    if (J.range.base) r = __ldg(J.range.base + (size_t)P.tkind[q] * J.range.stride + ppos);
     uint4 ex = make_uint4(r.x, 0, 0, kExclBits);
     if ((r.y & kRangeFlags) && r.x < J.range.excl_cap) ex = __ldg(J.range.excl + r.x);
     const bool later = P.tlater[q] != 0;
     const uint32_t half = (p ? r.y >> 16 : r.y) & 0xFFFFu, len = half & kRangeLong;
     a = later ? ex.x : ex.x - len;
     b = a + len;
+    bool same = (half & kRangeSame) != 0;   // the entry before a is in a's segment of the prefixes
     if (len == kRangeLong) {
         const uint2 ab = search_range(g, P, q, zg, ppos, pt, wlo, whi);
         a = ab.x;
         b = ab.y;
+        same = !leaf && a > __ldg((out ? g.out_off : g.in_off) + zg) && __ldg(tarr + a - 1) >= wlo;
         if (P.c2) {
             const uint3 e = search_excluded(g, P, q, zg, og, pt, wlo, whi);
             ea = e.y;
             ne = e.z - e.y;
             em = ea > e.x && __ldg(g.multi_t + ea - 1) >= wlo;
         }
-    } else if (half & 0x8000u) {
+    } else if (half & kRangeHasExcl) {
         if (ex.w == kExclBits) {
             hit = (uint64_t)ex.y | ((uint64_t)ex.z << 32);
             if (!later) hit = __brevll(hit) >> (64 - len);   // counted from a
             else hit &= ~0ull >> (64 - len);
         } else {
             const uint32_t h = (p ? ex.z >> 16 : ex.z) & 0xFFFFu;
-            ne = h & kRangeLong;
+            ne = h & kExclMany;
             ea = later ? ex.y : ex.y - ne;
             em = (h & 0x8000u) != 0;
         }
@@ -426,10 +382,7 @@ __device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P
     uint64_t base = 0, total = b - a;
     if (!leaf) {
         Pd = (const uint64_t *)J.pref_dir[P.tslot[q]] + p;
-        const uint32_t beg = __ldg((out ? g.out_off : g.in_off) + zg);
-        const uint32_t tb = a > 0 ? __ldg(tarr + a - 1) : 0u;
-        const uint64_t pb = a > 0 ? __ldg(Pd + 2 * (size_t)(a - 1)) : 0;
-        base = (a > beg && tb >= wlo) ? pb : 0;
+        base = same && a > 0 ? __ldg(Pd + 2 * (size_t)(a - 1)) : 0;
         total = __ldg(Pd + 2 * (size_t)(b - 1)) - base;
     }
     auto before = [&](uint32_t x) -> uint64_t {   // weight of the range before entry x

@@ -140,9 +140,12 @@ inline int exclusive_scan_u32(tm_ctx *ctx, const uint32_t *in, uint32_t *out, ui
 // addition inside a segment checked for wrap-around, over pairs (layer 0,
 // layer 1) that share their positions (one gather of a 16-byte pair serves
 // both layers).  A segment of layer p starts where the window of layer p
-// changes or, in both layers, where a new owner starts.  Functor interface:
-// value2(pos) -> ulonglong2, tarr (position -> t'), wv (the window divider) and
-// owner_word(w) -> the owner-start bits of positions 32 w .. 32 w + 31.
+// changes or, in both layers, where a new owner starts.  Functor interface: w
+// (the pairs), perm (position -> place in w; null: the same), nz (null, or a bit
+// set of the non-zero pairs by place in w), tarr (position -> t'), wv (the
+// window divider) and owner_word(w) -> the owner-start bits of positions 32 w ..
+// 32 w + 31.  A pair behind a map is a random sector of memory and most are
+// zero, which the bit set, small enough for L2, tells first.
 struct SegAgg2 {
     uint64_t v0, v1;
     uint32_t f;     // bit p: the range contains a head of layer p
@@ -221,10 +224,24 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
         t[r] = i < n ? __ldg(f.tarr + i) : 0u;
     }
     uint32_t tb = base > 0 && base < n ? __ldg(f.tarr + base - 1) : 0u;   // the time before the warp's first
+    {
+        uint32_t x[kScanRows];
 #pragma unroll
-    for (int r = 0; r < kScanRows; ++r) {
-        const uint64_t i = base + r * 32 + lane;
-        v[r] = i < n ? f.value2(i) : make_ulonglong2(0, 0);
+        for (int r = 0; r < kScanRows; ++r) {
+            const uint64_t i = base + r * 32 + lane;
+            x[r] = i < n ? (f.perm ? __ldg(f.perm + i) : (uint32_t)i) : 0u;
+        }
+        uint32_t on = 0xffffffffu;   // bit r: row r's pair is read
+        if (f.perm && f.nz) {
+            on = 0;
+#pragma unroll
+            for (int r = 0; r < kScanRows; ++r) on |= ((__ldg(f.nz + (x[r] >> 5)) >> (x[r] & 31)) & 1u) << r;
+        }
+#pragma unroll
+        for (int r = 0; r < kScanRows; ++r) {
+            const uint64_t i = base + r * 32 + lane;
+            v[r] = i < n && ((on >> r) & 1u) ? __ldg(f.w + x[r]) : make_ulonglong2(0, 0);
+        }
     }
     uint32_t qb = f.wv.quot(tb);    // the quotient before the row's first
     uint32_t need0 = 0, need1 = 0;  // bit r: no head of the layer in the chunk up to row r's position

@@ -128,8 +128,8 @@ size_t estimate_bytes(const tm_motif *mo, uint64_t m, uint64_t T)
     uint64_t nwin = T / (uint64_t)std::max<int64_t>(1, mo->plan.wdelta) + 2;
     nwin = std::min<uint64_t>(nwin, m + 2);
     // root CDF 16 B and root-search guide about 2 B per edge, 32 B per prefix
-    // slot, 12 B per non-root node's candidate ranges
-    const uint64_t ranges = (uint64_t)(mo->plan.ntree - 1);
+    // slot, 12 B per kind of candidate range
+    const uint64_t ranges = (uint64_t)mo->plan.nkinds;
     return (size_t)((18 + 32 * slots + 12 * ranges) * std::max<uint64_t>(m, 1) + 96 * nwin + 4096);
 }
 

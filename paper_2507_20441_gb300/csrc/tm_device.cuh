@@ -181,6 +181,52 @@ __device__ __forceinline__ uint32_t pair_of(const DevGraph &g, uint32_t u, uint3
     return (p < hi && __ldg(g.pair_dst + p) == v) ? p : kNone;
 }
 
+// Time range of the child edge q of a parent edge at time pt, inside the
+// window [wlo, whi] (Constraint 1); false when it is empty.
+__device__ __forceinline__ bool child_times(const DevPlan &P, int q, uint32_t pt, uint32_t wlo, uint32_t whi,
+                                            uint64_t &tlo, uint64_t &thi)
+{
+    const uint64_t d = (uint64_t)P.delta;
+    if (P.tlater[q]) { tlo = (uint64_t)pt + 1; thi = (uint64_t)pt + d; }
+    else {
+        if (pt == 0) return false;
+        tlo = (uint64_t)pt >= d ? (uint64_t)pt - d : 0;
+        thi = (uint64_t)pt - 1;
+    }
+    tlo = tlo < (uint64_t)wlo ? (uint64_t)wlo : tlo;
+    thi = thi > (uint64_t)whi ? (uint64_t)whi : thi;
+    return tlo <= thi;
+}
+
+// A candidate range that the weight pass did not keep, found by searches from
+// the parent edge's position ppos in the list of its meeting vertex zg.
+[[maybe_unused]] static __device__ __noinline__ uint2 search_range(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t ppos,
+                                           uint32_t pt, uint32_t wlo, uint32_t whi)
+{
+    uint64_t tlo, thi;
+    uint32_t a = 0, b = 0, beg;
+    const uint32_t *tarr;
+    if (child_times(P, q, pt, wlo, whi, tlo, thi))
+        child_range(g, P.tzside[q] != 0 ? 1 : 0, P.tout[q] != 0, zg, ppos, pt, P.tlater[q] != 0, tlo, thi, a, b, beg,
+                    tarr);
+    return make_uint2(a, b);
+}
+
+// The excluded entries of such a range (Claim 3.1): the part [ea, eb) of the
+// multi-edge list from pb on - zg -> og for a child leaving the meeting
+// vertex, og -> zg for one entering it - in the child's time range.
+[[maybe_unused]] static __device__ __noinline__ uint3 search_excluded(const DevGraph &g, const DevPlan &P, int q, uint32_t zg, uint32_t og,
+                                              uint32_t pt, uint32_t wlo, uint32_t whi)
+{
+    uint64_t tlo, thi;
+    const bool out = P.tout[q] != 0;
+    const uint32_t pe = pair_of(g, out ? zg : og, out ? og : zg);
+    if (pe == kNone || !child_times(P, q, pt, wlo, whi, tlo, thi)) return make_uint3(0, 0, 0);
+    const uint32_t pb = __ldg(g.pair_off + pe), pend = __ldg(g.pair_off + pe + 1);
+    const uint32_t ea = lower_idx(g.multi_t, pb, pend, tlo);
+    return make_uint3(pb, ea, gallop_idx(g.multi_t, ea, pend, thi + 1));
+}
+
 // ---- warp-cooperative search ----------------------------------------------
 // A lane whose search range holds at least coop_min entries is served by all
 // active lanes of its warp together: with n lanes, each step probes n evenly

@@ -143,6 +143,13 @@ struct DevPlan {
     int32_t child[kMaxTree][kMaxTree];
     int32_t height[kMaxTree];
     int32_t nslots;
+    // kinds of candidate range: a child's range for a parent edge depends only
+    // on the side it meets the parent at, its direction and its pi relation to
+    // the parent, so children that agree in these share one
+    int32_t nkinds;
+    int32_t tkind[kMaxTree];             // kind of tree node q's candidate ranges (-1 for the root)
+    int32_t kside[kMaxTree], kout[kMaxTree], klater[kMaxTree];
+    int32_t kinner[kMaxTree];            // 1: some child of the kind has children
     // DeriveCnt layout (Alg. 5): non-tree edges by pi position
     int32_t tnode_of_edge[kMaxE];        // tree node of a motif edge, -1 if non-tree
     int32_t nnt;                         // number of non-tree edges
@@ -167,28 +174,30 @@ struct LayerData {
     uint32_t *guide = nullptr;           // [m/4 + 3 nwin + 1]
 };
 
-// Candidate range of a child node for one parent edge (Claim 3.1), as the
-// weight DP found it, kept for the sampler.  y holds per layer p, in bits
-// 16p .. 16p + 15, the number of entries (bits 0-14; kRangeLong: not held, the
-// range is searched) and whether an excluded entry of non-zero weight is among
-// them (bit 15).  x is the bound next to the parent edge's time - the first
-// entry of a later child, the end of an earlier one's - or, when either layer
-// has excluded entries, the index of a RangeExcl.
-constexpr uint32_t kRangeLong = 0x7FFFu;
-constexpr uint32_t kRangeFlags = 0x80008000u;
+// Candidate range of a child for one parent edge (Claim 3.1), found once per
+// kind by the weight pass and read by its DP and by the sampler.  y holds per
+// layer p, in bits 16p .. 16p + 15, the number of entries (bits 0-13;
+// kRangeLong: not held, the range is searched), whether the entry before the
+// range is in the same (vertex, window) segment of the prefixes (bit 14; kinds
+// with an inner child) and whether excluded entries are among them (bit 15).
+// x is the bound next to the parent edge's time - the first entry of a later
+// child, the end of an earlier one's - or, when either layer has excluded
+// entries, the index of a RangeExcl.
+constexpr uint32_t kRangeLong = 0x3FFFu, kRangeSame = 0x4000u, kRangeHasExcl = 0x8000u;
+constexpr uint32_t kRangeFlags = kRangeHasExcl | (kRangeHasExcl << 16);
 // The excluded entries of such a range (16 bytes): x = the bound above.
 // w = kExclBits: y, z = a bit per entry counted from that bound (bit i: entry
 // x + i of a later child, x - 1 - i of an earlier one's), set for an excluded
-// one; the DP scans ranges of up to 64 entries.  w = kExclList: z holds per
-// layer the number of excluded entries (bits 0-14 of each half) and whether
+// one; ranges of up to 64 entries are scanned for them.  w = kExclList: z holds
+// per layer the number of excluded entries (bits 0-14 of each half) and whether
 // the entry before them is in the same segment of the prefixes (bit 15), y the
 // first of them in multi-edge order (later child) or their end (earlier).
-constexpr uint32_t kExclBits = 0, kExclList = 1;
+constexpr uint32_t kExclBits = 0, kExclList = 1, kExclMany = 0x7FFFu;
 typedef uint4 RangeExcl;
 struct RangePtrs {
-    uint2 *base;             // node q's at base + (q - 1) stride, by the parent edge's position in the
+    uint2 *base;             // kind k's at base + k stride, by the parent edge's position in the
     size_t stride;           // meeting vertex's list; null: ranges not kept
-    RangeExcl *excl;         // shared by the nodes, in no order
+    RangeExcl *excl;         // shared by the kinds, in no order
     unsigned long long *excl_n;   // entries asked for (beyond the capacity: such ranges are searched)
     uint32_t excl_cap;
 };
@@ -213,7 +222,7 @@ struct tm_motif {
     // multi-edge order, as (layer 0, layer 1) pairs per position
     ulonglong2 *pref_dir[timest::kMaxTree] = {};
     ulonglong2 *pref_multi[timest::kMaxTree] = {};
-    timest::RangePtrs range{};           // candidate ranges per non-root tree node (null: kept without them)
+    timest::RangePtrs range{};           // candidate ranges per kind (null: kept without them)
     uint64_t *wcum = nullptr;            // [2*(nw0+nw1+1)] u128 window cumulative (lo,hi)
     uint32_t *wguide = nullptr;          // [4*(nw0+nw1)+2] guide table of the window pick
     uint32_t nwtot = 0;
@@ -314,7 +323,7 @@ struct SampleJob {
     const uint32_t *win_gshift0, *win_gshift1, *win_goff0, *win_goff1, *guide0, *guide1;
     const ulonglong2 *pref_dir[kMaxTree];     // (layer 0, layer 1) prefix pairs per slot
     const ulonglong2 *pref_multi[kMaxTree];
-    RangePtrs range;                          // candidate ranges per node (null: searched)
+    RangePtrs range;                          // candidate ranges per kind (null: searched)
     uint64_t W_lo, W_hi;
 };
 int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t first,

@@ -44,20 +44,176 @@ __device__ __forceinline__ uint64_t lane_of(const ulonglong2 v, int p) { return 
 constexpr uint32_t kScanLimit = 64;   // the bits of a RangeExcl
 constexpr int kScanStep = 8;          // independent loads per step (4 and 16 measured 0.2 - 1 % slower)
 
+// The candidate ranges of one kind (Claim 3.1) for every edge as the parent, in
+// both layers.  Threads walk the meeting vertex's own list (out-list order for
+// side 0, in-list order for side 1), so the lanes of a warp share the vertex,
+// its candidate lists and nearby positions in them.  A range is galloped to
+// from the parent edge's position in that list (or its cross rank into the
+// vertex's other list).  Both layers share the unclipped range: the edge's
+// windows of the two layers both contain t, so the bound on the side of the
+// edge itself is common and only the far bound is clipped, in at most one
+// layer, by a search inside the unclipped range.  The excluded entries are
+// exactly the entries of the range whose other endpoint is the parent's other
+// endpoint: short ranges are scanned for them in place (one pass serves both
+// layers); long ones search the excluded multi-edge list.
+// The instructions issued bound it, so time bounds are 32-bit compares, empty
+// ranges (two thirds of a power-law graph's) leave early, and 32 registers let
+// eight blocks run on an SM.  Kept, a range serves every tree node of its kind
+// in the DP and every sample: 0.61 ms per kind on 5e7 edges, two kinds for the
+// 5-cycle + chord, against 4.2 ms for the DP that searched them in each node.
+__global__ void __launch_bounds__(256, 8) k_ranges(DevGraph g, int c2, int64_t delta, WinDiv wv, int side, int out,
+                                                   int later, int inner, uint2 *__restrict__ rec, RangePtrs R)
+{
+    const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
+    if (pos >= g.m) return;
+    const uint32_t t = __ldg((side ? g.in_t : g.out_t) + pos);
+    const uint32_t z = __ldg((side ? g.in_dst : g.out_src) + pos);
+    // no earlier time than 0, no later one than the largest t'
+    if (t == (later ? 0xFFFFFFFFu : 0u)) { rec[pos] = make_uint2(0, 0); return; }
+    const uint32_t *off = out ? g.out_off : g.in_off;
+    const uint32_t *tarr = out ? g.out_t : g.in_t;
+    const uint32_t *nbr = out ? g.out_nbr : g.in_nbr;
+    const uint32_t beg = __ldg(off + z), end = __ldg(off + z + 1);
+    const uint32_t base = ((side == 0) == (out != 0)) ? gallop_back(tarr, beg, pos, t)
+                                                      : __ldg((side == 0 ? g.out_xrank : g.in_xrank) + pos);
+    // the unclipped range, [near, far) or [far, near)
+    const uint64_t d = (uint64_t)delta;
+    uint32_t near, far, lim;   // lim: the far end's time
+    if (later) {
+        const uint64_t hu = (uint64_t)t + d;
+        lim = hu > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)hu;
+        near = gallop_above(tarr, base, end, t);
+        far = gallop_above(tarr, near, end, lim);
+    } else {
+        lim = (uint64_t)t >= d ? (uint32_t)((uint64_t)t - d) : 0u;
+        near = base;
+        far = gallop_back(tarr, beg, base, lim);
+    }
+    if (near == far) { rec[pos] = make_uint2(near, 0); return; }
+    // window bounds as 32-bit times: wlo <= t fits, whi is clamped to the
+    // largest t' (no time lies beyond it), which leaves every comparison
+    // unchanged and keeps the bounds in half the registers
+    const uint64_t wd = (uint64_t)wv.d;
+    const uint32_t qt = wv.quot(t);
+    uint32_t wlo[2], n[2];   // n: entries of the layer's range
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const int64_t wi = WinDiv::win_of(qt, p);
+        const uint64_t whi64 = ((uint64_t)wi + 2) * wd - 1;
+        const uint32_t whi = whi64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)whi64;
+        wlo[p] = wi < 0 ? 0u : (uint32_t)((uint64_t)wi * wd);
+        if (wi < 0) n[p] = 0;
+        else if (later) n[p] = (whi >= lim ? far : above_idx(tarr, near, far, whi)) - near;
+        else n[p] = near - (wlo[p] <= lim ? far : lower_idx(tarr, far, near, wlo[p]));
+    }
+    const uint32_t most = max(n[0], n[1]);
+    if (most == 0) { rec[pos] = make_uint2(near, 0); return; }
+    uint32_t y = 0;
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        y |= min(n[p], kRangeLong) << (16 * p);
+        if (inner && n[p]) {
+            const uint32_t a = later ? near : near - n[p];
+            if (a > beg && __ldg(tarr + a - 1) >= wlo[p]) y |= kRangeSame << (16 * p);
+        }
+    }
+    // the excluded entries; without Constraint 2 nothing is
+    uint4 ex = make_uint4(near, 0, 0, kExclBits);
+    uint32_t has = 0;
+    if (c2) {
+        const uint32_t o = __ldg((side ? g.in_nbr : g.out_nbr) + pos);   // the parent's other endpoint
+        if (most <= kScanLimit) {
+            const uint32_t a = later ? near : near - most;
+            for (uint32_t i0 = 0; i0 < most; i0 += kScanStep) {
+                uint32_t hit = 0;   // entry a + i0 + i
+#pragma unroll
+                for (int i = 0; i < kScanStep; ++i)
+                    hit |= (i0 + i < most && __ldg(nbr + a + i0 + i) == o) ? 1u << i : 0u;
+                while (hit) {
+                    const uint32_t i = i0 + (uint32_t)__ffs((int)hit) - 1, bit = later ? i : most - 1 - i;
+                    if (bit < 32) ex.y |= 1u << bit; else ex.z |= 1u << (bit - 32);
+                    has |= (bit < n[0] ? kRangeHasExcl : 0u) | (bit < n[1] ? kRangeHasExcl << 16 : 0u);
+                    hit &= hit - 1;
+                }
+            }
+        } else {
+            // z -> o for a child leaving z, o -> z for one entering it
+            const uint32_t pe = out ? pair_of(g, z, o) : pair_of(g, o, z);
+            if (pe != kNone) {
+                const uint32_t xb = __ldg(g.pair_off + pe), xe = __ldg(g.pair_off + pe + 1);
+                ex.w = kExclList;
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    if (n[p] == 0) continue;
+                    // the times of the layer's range: (t, hi] or [lo, t)
+                    uint32_t ea, eb;
+                    if (later) {
+                        const int64_t wi = WinDiv::win_of(qt, p);
+                        const uint64_t whi64 = ((uint64_t)wi + 2) * wd - 1;
+                        ea = above_idx(g.multi_t, xb, xe, t);
+                        eb = gallop_above(g.multi_t, ea, xe, whi64 < lim ? (uint32_t)whi64 : lim);
+                        ex.y = ea;
+                    } else {
+                        ea = lower_idx(g.multi_t, xb, xe, max(lim, wlo[p]));
+                        eb = gallop_idx(g.multi_t, ea, xe, t);
+                        ex.y = eb;   // both layers' lists end together, a later child's start together
+                    }
+                    if (eb <= ea) continue;
+                    has |= kRangeHasExcl << (16 * p);
+                    ex.z |= min(eb - ea, kExclMany) << (16 * p);
+                    if (inner && ea > xb && __ldg(g.multi_t + ea - 1) >= wlo[p]) ex.z |= 0x8000u << (16 * p);
+                    if (eb - ea >= kExclMany) y |= kRangeLong << (16 * p);   // more than a half holds: searched
+                }
+            }
+        }
+    }
+    uint32_t x = near;
+    if (has) {
+        const unsigned long long i = atomicAdd(R.excl_n, 1ull);
+        if (i < R.excl_cap) {
+            R.excl[i] = ex;
+            x = (uint32_t)i;
+            y |= has;
+        } else {
+            y = kRangeLong | (kRangeLong << 16);
+        }
+    }
+    rec[pos] = make_uint2(x, y);
+}
+
+// The sum of child c's candidates for the edge at `pos` of the list of side
+// `side`, in layer p, when the range is not kept.
+static __device__ __noinline__ uint64_t search_sum(const DevGraph &g, const DevPlan &P, const WinDiv &wv, const ChildPrefix &cp,
+                                            int c, uint32_t pos, int p)
+{
+    const bool side = P.tzside[c] != 0, out = P.tout[c] != 0, leaf = P.tleaf[c] != 0;
+    const uint32_t t = __ldg((side ? g.in_t : g.out_t) + pos), z = __ldg((side ? g.in_dst : g.out_src) + pos);
+    const int64_t wi = wv.win(t, p);
+    if (wi < 0) return 0;
+    const uint64_t whi64 = ((uint64_t)wi + 2) * (uint64_t)wv.d - 1;
+    const uint32_t wlo = (uint32_t)((uint64_t)wi * (uint64_t)wv.d), whi = whi64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)whi64;
+    const uint2 ab = search_range(g, P, c, z, pos, t, wlo, whi);
+    if (ab.y <= ab.x) return 0;
+    uint3 e = make_uint3(0, 0, 0);
+    if (P.c2) e = search_excluded(g, P, c, z, __ldg((side ? g.in_nbr : g.out_nbr) + pos), t, wlo, whi);
+    if (leaf) return (uint64_t)(ab.y - ab.x) - (e.z - e.y);
+    const uint64_t *Pd = (const uint64_t *)(cp.base + 2 * P.tslot[c] * cp.stride) + p;
+    const uint64_t *Pm = (const uint64_t *)(cp.base + (2 * P.tslot[c] + 1) * cp.stride) + p;
+    const uint32_t beg = __ldg((out ? g.out_off : g.in_off) + z);
+    uint64_t sum = __ldg(Pd + 2 * (size_t)(ab.y - 1));
+    if (ab.x > beg && __ldg((out ? g.out_t : g.in_t) + ab.x - 1) >= wlo) sum -= __ldg(Pd + 2 * (size_t)(ab.x - 1));
+    if (e.z > e.y) {
+        sum -= __ldg(Pm + 2 * (size_t)(e.z - 1));
+        if (e.y > e.x && __ldg(g.multi_t + e.y - 1) >= wlo) sum += __ldg(Pm + 2 * (size_t)(e.y - 1));
+    }
+    return sum;
+}
+
 // One side of tree node q (Claim 3.2): the product of the factors of q's
 // children that meet q at its tail (side 0) or head (side 1), for every edge
-// matched to q and both layers.  Threads walk the meeting vertex's own list
-// (out-list order for side 0, in-list order for side 1), so the lanes of a
-// warp share the vertex, its candidate lists and nearby positions in them.
-// Each child's range is galloped to from the parent edge's position in that
-// list (or its cross rank into the vertex's other list).  Both layers share
-// the unclipped range: e's windows of the two layers both contain t, so the
-// bound on the side of e itself is common and only the far bound is clipped,
-// in at most one layer, by a search inside the unclipped range.  The
-// excluded entries of Claim 3.1 are exactly the entries of the range whose
-// other endpoint is the parent's other endpoint: short ranges are scanned for
-// them in place (one pass serves both layers); long ones search the excluded
-// multi-edge list.
+// matched to q and both layers, in the order of the meeting vertex's lists.  A
+// child's factor is the sum of its weights over the kept range: a count for a
+// leaf, a difference of prefixes otherwise, minus the excluded entries'.
 // Results are written in this list order, or through `scatter` into another
 // order (a node whose parent scans the out-list order while its own DP runs
 // in in-list order writes through the in -> out map).  A root with children at both ends
@@ -65,236 +221,183 @@ constexpr int kScanStep = 8;          // independent loads per step (4 and 16 me
 // product through the out->in position map, and its pending-overflow bits
 // from two bit sets of m/32 words (one per layer; a warp of side 0 writes
 // the word of its 32 positions with a ballot), small enough to stay in L2.
-// Each child's ranges are also written out (8 bytes per edge, coalesced) for
-// the sampler, which would otherwise repeat the gallops and the search for
-// excluded entries, as one dependent load after another, for every sample.
-// The kernel is bound by the instructions it issues (about half of the issue
-// slots) and by occupancy, so empty ranges leave early, time bounds are 32-bit
-// compares and sides with leaf children only have a kernel without prefixes:
-// with these three and the ranges written 4.39 -> 4.21 ms for the three
-// launches of the 5-cycle + chord on 5e7 edges, 1,161 -> 1,125 us for the four
-// of a 6-path on 1e7 (without them the ranges cost 0.39 ms and 127 us).
 // Overflow rule: a factor >= 2^64, or an exact product >= 2^64 with no zero
 // factor.
-// LEAF: every child met on this side is a leaf, so no prefix sums are read and
-// the kernel needs few enough registers for 40 a thread almost without spills.
-#ifndef TM_DP_MINB
-#define TM_DP_MINB 6   // 40 registers, six blocks of 256 per SM (5 and 7 measured slower: 4355 and 4572 against 4206 us)
-#endif
-template <bool LEAF>
-__global__ void __launch_bounds__(256, TM_DP_MINB) k_dp(DevGraph g, DevPlan P, WinDiv wv, int q, int side, int first,
-                                                        int last, ChildPrefix cp, RangePtrs ranges,
-                                                        ulonglong2 *__restrict__ wout,
-                                                        const uint32_t *__restrict__ scatter,
-                                                        const ulonglong2 *__restrict__ in,
-                                                        const uint32_t *__restrict__ pin, uint32_t *__restrict__ pout,
-                                                        uint32_t *status)
+// LEAF: every child met on this side is a leaf, so no prefix sums are read.
+// The work per edge is a few loads and little else, so a thread takes K edges
+// (blockDim apart) whose loads are in flight together, and random accesses are
+// made for weights that are not zero only (a third of them): with one edge per
+// thread and every partial gathered, every weight scattered, the three launches
+// of the 5-cycle + chord on 5e7 edges took 3.25 ms, like this 1.5 (the four of
+// a 6-path on 1e7 edges 743 and 420 us).
+constexpr int kDpLeaf = 4, kDpInner = 2;   // K (four and five blocks per SM)
+template <bool LEAF, int K>
+__global__ void __launch_bounds__(256, LEAF ? 4 : 5)
+    k_dp(DevGraph g, const __grid_constant__ DevPlan P, WinDiv wv, int q, int side, int first, int last, ChildPrefix cp,
+         RangePtrs ranges, ulonglong2 *__restrict__ wout, const uint32_t *__restrict__ scatter,
+         uint32_t *__restrict__ nz, const ulonglong2 *__restrict__ in, const uint32_t *__restrict__ in_nz,
+         const uint32_t *__restrict__ pin, uint32_t *__restrict__ pout, uint32_t *status)
 {
-    const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
-    // whole warps stay for the pending-bit ballots of side 0
-    if (pos >= g.m && (last || (pos & ~31u) >= g.m)) return;
-    const bool live = pos < g.m;
-    uint32_t pend_bits = 0;
-    if (live) {
-        const uint32_t t = __ldg((side ? g.in_t : g.out_t) + pos);
-        const uint32_t z = __ldg((side ? g.in_dst : g.out_src) + pos);
-        // the parent's other endpoint; without Constraint 2 nothing is excluded
-        const uint32_t o = P.c2 ? __ldg((side ? g.in_nbr : g.out_nbr) + pos) : kNone;
-        const uint64_t d = (uint64_t)P.delta, wd = (uint64_t)wv.d;
-        const uint32_t qt = wv.quot(t);
-        // window bounds as 32-bit times: wlo <= t fits, whi is clamped to the
-        // largest t' (no time lies beyond it), which leaves every comparison
-        // below unchanged and keeps the bounds in half the registers
-        uint32_t wlo[2], whi[2];
-        uint64_t prod[2] = {1, 1};
-        bool zero[2], ovf[2] = {false, false};
+    const uint64_t pos0 = (uint64_t)blockIdx.x * (256 * K) + threadIdx.x;
+    auto at = [&](int k) { return (uint32_t)(pos0 + k * 256); };
+    auto live = [&](int k) { return pos0 + k * 256 < g.m; };
+    uint64_t prod[K][2];
+    uint32_t zero = 0, ovf = 0;   // bit 2 k + p: edge k's product in layer p is zero / wrapped
+    constexpr uint32_t kAll = (1u << (2 * K)) - 1u;
+    uint2 r[K];
+    int kind = -1;   // of the ranges in r
+    auto load_ranges = [&](int kd) {
+        kind = kd;
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-            const int64_t wi = WinDiv::win_of(qt, p);
-            zero[p] = wi < 0;
-            const uint64_t whi64 = ((uint64_t)wi + 2) * wd - 1;
-            wlo[p] = zero[p] ? 0u : (uint32_t)((uint64_t)wi * wd);
-            whi[p] = zero[p] ? 0u : (whi64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)whi64);
+        for (int k = 0; k < K; ++k)
+            if (((zero >> (2 * k)) & 3u) != 3u) r[k] = __ldg(ranges.base + (size_t)kind * ranges.stride + at(k));
+    };
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        prod[k][0] = prod[k][1] = 1;
+        r[k] = make_uint2(0, kRangeLong | (kRangeLong << 16));
+        if (!live(k)) zero |= 3u << (2 * k);
+    }
+    if (P.nchild[q] == 0) {   // a root without children: one for each window that holds the edge
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t t = live(k) ? __ldg(g.out_t + at(k)) : 0u;
+            zero |= ((wv.win(t, 0) < 0 ? 1u : 0u) | (wv.win(t, 1) < 0 ? 2u : 0u)) << (2 * k);
         }
-        if (!first) {
-            const uint32_t xp = __ldg(g.in_to_out + pos);   // side 1 reads side 0's partial (both layers)
-            const ulonglong2 pv = __ldg(in + xp);
-            const uint32_t words = (g.m + 31) >> 5;
-            const uint32_t pb = ((__ldg(pin + (xp >> 5)) >> (xp & 31)) & 1u) |
-                                (((__ldg(pin + words + (xp >> 5)) >> (xp & 31)) & 1u) << 1);
+    }
+    if (!first) {
+        // side 1 reads side 0's partial (both layers), a random access, where the
+        // range of this side's first child holds something and, by its bit set,
+        // the partial is not zero
+        if (ranges.base) {
+            int c = 0;
+            while (P.tzside[P.child[q][c]] != side) ++c;
+            load_ranges(P.tkind[P.child[q][c]]);
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                zero |= (((r[k].y & kRangeLong) == 0 ? 1u : 0u) | (((r[k].y >> 16) & kRangeLong) == 0 ? 2u : 0u)) << (2 * k);
+        }
+        uint32_t xp[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) xp[k] = live(k) ? __ldg(g.in_to_out + at(k)) : 0u;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (((zero >> (2 * k)) & 3u) != 3u && !((__ldg(in_nz + (xp[k] >> 5)) >> (xp[k] & 31)) & 1u)) zero |= 3u << (2 * k);
+        const uint32_t words = (g.m + 31) >> 5;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (((zero >> (2 * k)) & 3u) == 3u) continue;
+            const ulonglong2 pv = __ldg(in + xp[k]);
+            prod[k][0] = pv.x;
+            prod[k][1] = pv.y;
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (((zero >> (2 * k)) & 3u) == 3u) continue;
+            const uint32_t b0 = __ldg(pin + (xp[k] >> 5)) >> (xp[k] & 31), b1 = __ldg(pin + words + (xp[k] >> 5)) >> (xp[k] & 31);
+            ovf |= ((b0 & 1u) | ((b1 & 1u) << 1)) << (2 * k);
+            zero |= ((prod[k][0] == 0 ? 1u : 0u) | (prod[k][1] == 0 ? 2u : 0u)) << (2 * k);
+        }
+    }
+    for (int ci = 0; ci < P.nchild[q] && zero != kAll; ++ci) {
+        const int c = P.child[q][ci];
+        if (P.tzside[c] != side) continue;
+        const bool later = P.tlater[c] != 0, leaf = LEAF || P.tleaf[c] != 0;
+        if (ranges.base && P.tkind[c] != kind) load_ranges(P.tkind[c]);
+        // the range's weight with its excluded entries
+        uint64_t sum[K][2];
+        const uint64_t *Pd = leaf ? nullptr : (const uint64_t *)(cp.base + 2 * P.tslot[c] * cp.stride);
+        if (!LEAF && !leaf) {
+            uint32_t near[K];
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                near[k] = (r[k].y & kRangeFlags) && ((zero >> (2 * k)) & 3u) != 3u ? __ldg(&ranges.excl[r[k].x].x) : r[k].x;
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    const uint32_t half = (r[k].y >> (16 * p)) & 0xFFFFu, n = half & kRangeLong;
+                    const bool on = !((zero >> (2 * k + p)) & 1u) && n && n != kRangeLong;
+                    const uint32_t a = later ? near[k] : near[k] - n;
+                    sum[k][p] = on ? __ldg(Pd + 2 * (size_t)(a + n - 1) + p) : 0;
+                    if (on && (half & kRangeSame)) sum[k][p] -= __ldg(Pd + 2 * (size_t)(a - 1) + p);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                sum[k][0] = r[k].y & kRangeLong;
+                sum[k][1] = (r[k].y >> 16) & kRangeLong;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (((zero >> (2 * k)) & 3u) == 3u) continue;
+            uint4 ex = make_uint4(r[k].x, 0, 0, kExclBits);
+            if (r[k].y & kRangeFlags) ex = __ldg(ranges.excl + r[k].x);
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
-                if (zero[p]) continue;
-                prod[p] = lane_of(pv, p);
-                ovf[p] = (pb >> p) & 1u;
-                if (prod[p] == 0) zero[p] = true;
-            }
-        }
-        for (int ci = 0; ci < P.nchild[q] && !(zero[0] && zero[1]); ++ci) {
-            const int c = P.child[q][ci];
-            if (P.tzside[c] != side) continue;
-            const bool out = P.tout[c] != 0, later = P.tlater[c] != 0, leaf = LEAF || P.tleaf[c] != 0;
-            // no earlier time than 0, no later one than the largest t'
-            if ((!later && t == 0) || (later && t == 0xFFFFFFFFu)) { zero[0] = zero[1] = true; break; }
-            const uint32_t *off = out ? g.out_off : g.in_off;
-            const uint32_t *tarr = out ? g.out_t : g.in_t;
-            const uint32_t *nbr = out ? g.out_nbr : g.in_nbr;
-            const uint32_t beg = __ldg(off + z), end = __ldg(off + z + 1);
-            const uint32_t base = ((side == 0) == out) ? gallop_back(tarr, beg, pos, t)
-                                                       : __ldg((side == 0 ? g.out_xrank : g.in_xrank) + pos);
-            // per-layer ranges [a[p], b[p]) with times in [lo[p], hi[p]]
-            uint32_t a[2], b[2], lo[2], hi[2];
-            if (later) {
-                const uint64_t hu64 = (uint64_t)t + d;
-                const uint32_t l0 = t + 1, hu = hu64 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)hu64;
-                const uint32_t a0 = gallop_above(tarr, base, end, t);
-                const uint32_t bu = gallop_above(tarr, a0, end, hu);
-                if (bu == a0) { zero[0] = zero[1] = true; break; }
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    lo[p] = l0;
-                    hi[p] = hu < whi[p] ? hu : whi[p];
-                    a[p] = a0;
-                    b[p] = (zero[p] || hi[p] == hu) ? bu : above_idx(tarr, a0, bu, hi[p]);
-                    if (lo[p] > hi[p]) zero[p] = true;
-                }
-            } else {
-                const uint32_t h0 = t - 1, lu = (uint64_t)t >= d ? (uint32_t)((uint64_t)t - d) : 0u;
-                const uint32_t au = gallop_back(tarr, beg, base, lu);
-                if (au == base) { zero[0] = zero[1] = true; break; }
-#pragma unroll
-                for (int p = 0; p < 2; ++p) {
-                    hi[p] = h0;
-                    lo[p] = lu > wlo[p] ? lu : wlo[p];
-                    b[p] = base;
-                    a[p] = (zero[p] || lo[p] == lu) ? au : lower_idx(tarr, au, base, lo[p]);
-                    if (lo[p] > hi[p]) zero[p] = true;
-                }
-            }
-            if (zero[0] && zero[1]) break;
-            const ulonglong2 *Pd = leaf ? nullptr : cp.base + 2 * P.tslot[c] * cp.stride;
-            uint64_t excl[2] = {0, 0};
-            // the union of the live layers' ranges
-            uint32_t ua = 0xFFFFFFFFu, ub = 0;
-#pragma unroll
-            for (int p = 0; p < 2; ++p)
-                if (!zero[p]) { ua = min(ua, a[p]); ub = max(ub, b[p]); }
-            // an excluded entry x (other endpoint o) of the range: its weight,
-            // in each layer whose range holds it
-            // what the sampler is told of them: a bit each (short ranges), or
-            // their list positions and per-layer numbers
-            uint32_t ex_y = 0, ex_z = 0;
-            const bool scanned = ub <= ua || ub - ua <= kScanLimit;
-            auto add_excl = [&](uint32_t x) {
-                const uint32_t bit = later ? x - ua : ub - 1 - x;
-                if (bit < 32) ex_y |= 1u << bit; else ex_z |= 1u << (bit - 32);
-                ulonglong2 wx2 = make_ulonglong2(1, 1);
-                if (!leaf) {
-                    // the entry's weight: its prefix minus the previous entry's in
-                    // the same (vertex, window) segment
-                    const ulonglong2 px = __ldg(Pd + x);
-                    const ulonglong2 pp = x > beg ? __ldg(Pd + x - 1) : make_ulonglong2(0, 0);
-                    const uint32_t tp = x > beg ? __ldg(tarr + x - 1) : 0;
-                    wx2.x = px.x - ((x > beg && tp >= wlo[0]) ? pp.x : 0);
-                    wx2.y = px.y - ((x > beg && tp >= wlo[1]) ? pp.y : 0);
-                }
-#pragma unroll
-                for (int p = 0; p < 2; ++p)
-                    if (!zero[p] && x >= a[p] && x < b[p]) excl[p] += lane_of(wx2, p);
-            };
-            if (!P.c2) {
-                // without Constraint 2 nothing is excluded
-            } else if (scanned) {
-                for (uint32_t x0 = ua; x0 < ub; x0 += kScanStep) {
-                    uint32_t hit = 0;
-#pragma unroll
-                    for (int i = 0; i < kScanStep; ++i)
-                        hit |= (x0 + i < ub && __ldg(nbr + x0 + i) == o) ? 1u << i : 0u;
-                    while (hit) {
-                        add_excl(x0 + (uint32_t)__ffs((int)hit) - 1);
-                        hit &= hit - 1;
-                    }
-                }
-            } else {
-                // the excluded multi-edge list: z -> o for a child leaving z, o -> z
-                // for one entering it
-                const uint32_t pe = !P.c2 ? kNone : out ? pair_of(g, z, o) : pair_of(g, o, z);
-                if (pe != kNone) {
-                    const uint32_t xb = __ldg(g.pair_off + pe), xe = __ldg(g.pair_off + pe + 1);
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        if (zero[p]) continue;
-                        const uint32_t ea = lower_idx(g.multi_t, xb, xe, lo[p]);
-                        const uint32_t eb = gallop_idx(g.multi_t, ea, xe, (uint64_t)hi[p] + 1);
-                        if (eb <= ea) continue;
-                        // a later child's lists start together, an earlier one's end together
-                        ex_y = later ? ea : eb;
-                        ex_z |= min(eb - ea, kRangeLong) << (16 * p);
+                if ((zero >> (2 * k + p)) & 1u) continue;
+                const uint32_t half = (r[k].y >> (16 * p)) & 0xFFFFu, n = half & kRangeLong;
+                uint64_t &sm = sum[k][p];
+                if (n == kRangeLong) {
+                    sm = search_sum(g, P, wv, cp, c, at(k), p);
+                } else if (half & kRangeHasExcl) {
+                    const uint32_t a = later ? ex.x : ex.x - n;
+                    const uint32_t h = (ex.z >> (16 * p)) & 0xFFFFu, ne = h & kExclMany;   // of a list
+                    if (ex.w == kExclBits) {
+                        uint64_t bits = ((uint64_t)ex.y | ((uint64_t)ex.z << 32)) & (~0ull >> (64 - n));
                         if (leaf) {
-                            excl[p] = eb - ea;
+                            sm -= (uint32_t)__popcll((long long)bits);
                         } else {
-                            const ulonglong2 *Pm = cp.base + (2 * P.tslot[c] + 1) * cp.stride;
-                            const bool same = ea > xb && __ldg(g.multi_t + ea - 1) >= wlo[p];
-                            ex_z |= same ? 0x8000u << (16 * p) : 0u;
-                            excl[p] = lane_of(__ldg(Pm + eb - 1), p) - (same ? lane_of(__ldg(Pm + ea - 1), p) : 0);
+                            for (; bits; bits &= bits - 1) {
+                                // the entry's weight: its prefix minus the one before in its segment
+                                const uint32_t i = (uint32_t)__ffsll((long long)bits) - 1;
+                                const uint32_t x = later ? ex.x + i : ex.x - 1 - i;
+                                sm -= __ldg(Pd + 2 * (size_t)x + p);
+                                if (x > a || (half & kRangeSame)) sm += __ldg(Pd + 2 * (size_t)(x - 1) + p);
+                            }
                         }
-                    }
-                }
-            }
-            // the sampler draws this child from the same ranges
-            if (ranges.base) {
-                uint2 *rg = ranges.base + (size_t)(c - 1) * ranges.stride;
-                const uint32_t near = later ? a[0] : b[0];
-                uint32_t len0 = min(b[0] - a[0], kRangeLong), len1 = min(b[1] - a[1], kRangeLong);
-                uint2 rec = make_uint2(near, 0);
-                if (excl[0] | excl[1]) {
-                    const unsigned long long i = atomicAdd(ranges.excl_n, 1ull);
-                    if (i < ranges.excl_cap) {
-                        ranges.excl[i] = make_uint4(near, ex_y, ex_z, scanned ? kExclBits : kExclList);
-                        rec = make_uint2((uint32_t)i, (excl[0] ? 0x8000u : 0u) | (excl[1] ? 0x80000000u : 0u));
-                        if (!scanned) {   // more excluded entries than a half holds: searched
-                            if ((ex_z & kRangeLong) == kRangeLong) len0 = kRangeLong;
-                            if (((ex_z >> 16) & kRangeLong) == kRangeLong) len1 = kRangeLong;
-                        }
+                    } else if (leaf) {
+                        sm -= ne;
                     } else {
-                        len0 = len1 = kRangeLong;
+                        const uint64_t *Pm = (const uint64_t *)(cp.base + (2 * P.tslot[c] + 1) * cp.stride) + p;
+                        const uint32_t ea = later ? ex.y : ex.y - ne;
+                        sm -= __ldg(Pm + 2 * (size_t)(ea + ne - 1));
+                        if (h & 0x8000u) sm += __ldg(Pm + 2 * (size_t)(ea - 1));
                     }
                 }
-                rec.y |= len0 | (len1 << 16);
-                rg[pos] = rec;
+                bool o = false;
+                prod[k][p] = mul_chk(prod[k][p], sm, o);
+                ovf |= o ? 1u << (2 * k + p) : 0u;
+                zero |= sm == 0 ? 1u << (2 * k + p) : 0u;
             }
+        }
+    }
+    const uint32_t pend = ovf & ~zero;
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                if (zero[p]) continue;
-                uint64_t sum;
-                if (leaf) {
-                    sum = (uint64_t)(b[p] - a[p]) - excl[p];
-                } else if (b[p] > a[p]) {
-                    const uint64_t top = lane_of(__ldg(Pd + b[p] - 1), p);
-                    const uint64_t pbase = (a[p] > beg && __ldg(tarr + a[p] - 1) >= wlo[p])
-                                               ? lane_of(__ldg(Pd + a[p] - 1), p) : 0;
-                    sum = top - pbase - excl[p];
-                } else {
-                    sum = 0;
-                }
-                if (sum == 0) zero[p] = true;
-                else prod[p] = mul_chk(prod[p], sum, ovf[p]);
+    for (int k = 0; k < K; ++k) {
+        // both layers, one store; through the scatter map, where one is given,
+        // into an array of zeros
+        const bool some = ((zero >> (2 * k)) & 3u) != 3u;
+        if (live(k) && (some || !scatter))
+            wout[scatter ? __ldg(scatter + at(k)) : at(k)] =
+                make_ulonglong2((zero >> (2 * k)) & 1u ? 0 : prod[k][0], (zero >> (2 * k + 1)) & 1u ? 0 : prod[k][1]);
+        if (nz) {   // which weights are not zero, a bit each
+            const uint32_t w = __ballot_sync(0xffffffffu, some);
+            if ((threadIdx.x & 31) == 0 && live(k)) nz[at(k) >> 5] = w;
+        }
+        if (!last) {   // side 0: the warp's pending bits, one word per layer
+            const uint32_t b0 = __ballot_sync(0xffffffffu, (pend >> (2 * k)) & 1u);
+            const uint32_t b1 = __ballot_sync(0xffffffffu, (pend >> (2 * k + 1)) & 1u);
+            const uint32_t words = (g.m + 31) >> 5;
+            if ((threadIdx.x & 31) == 0 && live(k)) {
+                pout[at(k) >> 5] = b0;
+                pout[words + (at(k) >> 5)] = b1;
             }
         }
-        // both layers, one store; at the position scatter[pos] when a map is given
-        wout[scatter ? __ldg(scatter + pos) : pos] = make_ulonglong2(zero[0] ? 0 : prod[0], zero[1] ? 0 : prod[1]);
-        pend_bits = ((!zero[0] && ovf[0]) ? 1u : 0u) | ((!zero[1] && ovf[1]) ? 2u : 0u);
-        if (last && pend_bits) latch(status, ST_OVERFLOW);
     }
-    if (!last) {   // side 0: the warp's pending bits, one word per layer
-        const uint32_t b0 = __ballot_sync(0xffffffffu, pend_bits & 1u);
-        const uint32_t b1 = __ballot_sync(0xffffffffu, (pend_bits >> 1) & 1u);
-        if ((threadIdx.x & 31) == 0) {
-            const uint32_t words = (g.m + 31) >> 5;
-            pout[pos >> 5] = b0;
-            pout[words + (pos >> 5)] = b1;
-        }
-    }
+    if (last && pend) latch(status, ST_OVERFLOW);
 }
 
 // ---- scans over the three orders ----------------------------------------
@@ -336,20 +439,20 @@ struct RootHead {
 // one 16-byte gather; heads are per layer (bit p).
 struct DirScan2 {
     const ulonglong2 *w;        // (layer 0, layer 1) weights
+    const uint32_t *nz;         // bit set of the non-zero ones (null: none kept)
     const uint32_t *perm;       // scan position -> weight position (null: same order)
     const uint32_t *tarr;       // position -> t'
     const uint32_t *ownbits;    // bit set: position starts a new owner
     WinDiv wv;
-    __device__ ulonglong2 value2(uint64_t i) const { return __ldg(w + (perm ? __ldg(perm + i) : i)); }
     __device__ uint32_t owner_word(uint64_t w32) const { return __ldg(ownbits + w32); }
 };
 
 struct RootScan2 {
     const ulonglong2 *w;        // root weight pairs in list order
+    const uint32_t *nz;         // bit set of the non-zero ones
     const uint32_t *tarr;       // g_t
     WinDiv wv;
     const uint32_t *perm;       // gid -> weight position
-    __device__ ulonglong2 value2(uint64_t i) const { return __ldg(w + (perm ? __ldg(perm + i) : i)); }
     __device__ uint32_t owner_word(uint64_t) const { return 0u; }
 };
 
@@ -767,10 +870,10 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
                        al(guide_n(nwh[0]) * 4) + al(guide_n(nwh[1]) * 4) + al((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
         // the candidate ranges come last: a block this large that does not fit
         // with them is tried without (the sampler then searches the ranges)
-        // (room for excluded entries at a quarter of the edges per node: with
-        // bursts of repeated pairs a star's nodes have them at 0.2 - 0.3)
-        const size_t excl_cap = (size_t)(P.ntree - 1) * (mm / 4);
-        const size_t range_bytes = (size_t)(P.ntree - 1) * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl)) + al(8);
+        // (room for excluded entries at 0.3 of the edges per kind: with bursts of
+        // repeated pairs a star's ranges have them at 0.2 - 0.3)
+        const size_t excl_cap = (size_t)P.nkinds * (mm * 3 / 10);
+        const size_t range_bytes = (size_t)P.nkinds * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl)) + al(8);
         bool with_ranges = true;
         char *blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
         if (!blk && total >= ((size_t)4 << 30)) {
@@ -798,7 +901,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         mo->wguide = (uint32_t *)take((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
         if (with_ranges) {
             mo->range.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
-            mo->range.base = (uint2 *)take((size_t)(P.ntree - 1) * mo->range.stride * sizeof(uint2));
+            mo->range.base = (uint2 *)take((size_t)P.nkinds * mo->range.stride * sizeof(uint2));
             mo->range.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
             mo->range.excl_n = (unsigned long long *)take(8);
             mo->range.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
@@ -820,7 +923,9 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     ulonglong2 *w = nullptr, *pw = nullptr;   // (layer 0, layer 1) weight pairs
     uint32_t *pend = nullptr;                 // per layer a bit set: pending overflow of a side-0 partial
     w = (ulonglong2 *)salloc(ctx, (size_t)(m ? m : 1) * 16);
-    if (!w) return TM_E_NOMEM;
+    uint32_t *nz = (uint32_t *)salloc(ctx, ((size_t)m / 32 + 1) * 8);   // non-zero bits of w, then of pw
+    if (!w || !nz) return TM_E_NOMEM;
+    uint32_t *pw_nz = nz + (size_t)m / 32 + 1;
     const ChildPrefix cp{P.nslots ? mo->pref_dir[0] : nullptr, (size_t)((m ? m : 1) * (uint64_t)16 + 255) / 256 * 16};
     int maxh = 0;
     for (int q = 0; q < P.ntree; ++q) maxh = std::max(maxh, (int)P.height[q]);
@@ -829,6 +934,12 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         for (int q = P.ntree - 1; q >= 0; --q)
             if (P.height[q] == h) order.push_back(q);
     if (P.tleaf[0]) order.push_back(0);   // single-edge motif: the root is a leaf
+    if (mo->range.base && m) {
+        PhaseScope ph(ctx, TM_PH_DP);
+        for (int k = 0; k < P.nkinds; ++k)
+            launch(ctx, k_ranges, blocks_for(m, TB), TB, g, P.c2, P.delta, wv, P.kside[k], P.kout[k], P.klater[k],
+                   P.kinner[k], mo->range.base + (size_t)k * mo->range.stride, mo->range);
+    }
     for (int q : order) {
         // sides of q that children meet; the weights come out in the order of
         // the last side run (out-list order for side 0, in-list for side 1)
@@ -850,24 +961,28 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
             if (m) {
                 const uint32_t *none = nullptr;
                 const ulonglong2 *no_in = nullptr;
-                auto dp = [&](int side, int first, int last, ulonglong2 *wout, const uint32_t *scatter,
-                              const ulonglong2 *in, const uint32_t *pin, uint32_t *pout) {
-                    auto go = [&](auto kernel) {
-                        launch(ctx, kernel, blocks_for(m, TB), TB, g, P, wv, q, side, first, last, cp, mo->range, wout,
-                               scatter, in, pin, pout, ctx->status);
+                auto dp = [&](int side, int first, int last, ulonglong2 *wout, const uint32_t *scatter, uint32_t *out_nz,
+                              const ulonglong2 *in, const uint32_t *in_nz, const uint32_t *pin, uint32_t *pout) {
+                    auto go = [&](auto kernel, int per) {
+                        launch(ctx, kernel, blocks_for(m, TB * per), TB, g, P, wv, q, side, first, last, cp, mo->range,
+                               wout, scatter, out_nz, in, in_nz, pin, pout, ctx->status);
                     };
-                    if (inner[side]) go(k_dp<false>);
-                    else go(k_dp<true>);
+                    if (inner[side]) go(k_dp<false, kDpInner>, kDpInner);
+                    else go(k_dp<true, kDpLeaf>, kDpLeaf);
                 };
                 if (has[0] && has[1]) {
-                    dp(0, 1, 0, pw, none, no_in, none, pend);
-                    dp(1, 0, 1, w, none, pw, pend, nullptr);
+                    dp(0, 1, 0, pw, none, pw_nz, no_in, none, none, pend);
+                    dp(1, 0, 1, w, none, nz, pw, pw_nz, pend, nullptr);
                 } else {
                     // a non-root node leaving its parent's meeting vertex runs in
                     // in-list order and is scanned by its parent in out-list
                     // order: it writes through the in -> out map
                     const bool to_out = q != 0 && P.tout[q] != 0 && in_order;
-                    dp(in_order ? 1 : 0, 1, 1, w, to_out ? g.in_to_out : none, no_in, none, nullptr);
+                    // (only what is not zero: 5e7 random 16-byte writes are 1.3 ms,
+                    // clearing the array 0.13)
+                    if (to_out) cudaMemsetAsync(w, 0, (size_t)m * 16, st);
+                    dp(in_order ? 1 : 0, 1, 1, w, to_out ? g.in_to_out : none, to_out ? nullptr : nz, no_in, none, none,
+                       nullptr);
                 }
             }
         }
@@ -875,7 +990,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         if (rc) return rc;
         if (q == 0) {
             PhaseScope ph(ctx, TM_PH_ROOT);
-            RootScan2 f{w, g.g_t, wv, in_order ? g.in_pos : g.out_pos};
+            RootScan2 f{w, nz, g.g_t, wv, in_order ? g.in_pos : g.out_pos};
             rc = segmented_scan2_u64(ctx, f, m, mo->layer[0].root_cdf, mo->layer[1].root_cdf);
             if (rc) return rc;
         } else {
@@ -891,10 +1006,11 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
             // lists are grouped by source like the out-lists, so the multi-edge
             // prefix gathers, within each source's run, from the weights in
             // out-list order (w in both cases).
-            DirScan2 fd{w, out ? nullptr : g.in_to_out, out ? g.out_t : g.in_t, out ? ob.out : ob.in, wv};
+            const uint32_t *wnz = out && in_order ? nullptr : nz;   // (scattered weights have no bit set)
+            DirScan2 fd{w, wnz, out ? nullptr : g.in_to_out, out ? g.out_t : g.in_t, out ? ob.out : ob.in, wv};
             rc = segmented_scan2_u64(ctx, fd, m, nullptr, nullptr, mo->pref_dir[slot]);
             if (rc) return rc;
-            DirScan2 fm{w, g.multi_to_out, g.multi_t, ob.multi, wv};
+            DirScan2 fm{w, wnz, g.multi_to_out, g.multi_t, ob.multi, wv};
             rc = segmented_scan2_u64(ctx, fm, m, nullptr, nullptr, mo->pref_multi[slot]);
             if (rc) return rc;
         }
