@@ -1,7 +1,7 @@
 // Device-wide scans used by the CSR builder and the weight pass.
 //
 // * exclusive_scan_u32: reduce-then-scan over u32 counts (recursive over the
-//   tile totals), for compaction, pair ids and window offsets.
+//   tile totals), for compaction.
 // * segmented_scan2_u64: inclusive prefix sums that restart at segment heads,
 //   with every 64-bit addition inside a segment checked for wrap-around, in one
 //   pass with a bounded look-back between tiles.
@@ -363,22 +363,23 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
     if (ovf) latch(status, ST_OVERFLOW);
 }
 
+// Scratch of one scan (tile words and a ticket), to be cleared before it.
+inline size_t scan_state_bytes(uint64_t n)
+{
+    return ((n + kScan2Tile - 1) / kScan2Tile * sizeof(SegTile) + 64 + 255) / 256 * 256;
+}
+
 // Outputs: out0 / out1 (one array per layer), or outp (the (layer 0,
 // layer 1) pairs interleaved) when it is non-null.
 template <class F>
-int segmented_scan2_u64(tm_ctx *ctx, const F &f, uint64_t n, uint64_t *out0, uint64_t *out1,
+int segmented_scan2_u64(tm_ctx *ctx, const F &f, uint64_t n, char *state, uint64_t *out0, uint64_t *out1,
                         ulonglong2 *outp = nullptr)
 {
     if (n == 0) return TM_OK;
     const uint64_t tiles = (n + kScan2Tile - 1) / kScan2Tile;
-    ScratchScope scope(ctx);
     if (tiles >= 0xFFFFFFFFull) return set_err(ctx, TM_E_LIMIT, "scan of more than 2^32 tiles");
-    char *st = (char *)salloc(ctx, tiles * sizeof(SegTile) + 256);
-    if (!st) return TM_E_NOMEM;
-    uint32_t *counter = (uint32_t *)(st + tiles * sizeof(SegTile));
-    cudaMemsetAsync(st, 0, tiles * sizeof(SegTile) + 4, ctx->stream);
-    launch(ctx, k_segscan2_onepass<F>, (unsigned)tiles, SCAN_THREADS, f, n, (SegTile *)st, counter, out0, out1, outp,
-           ctx->status);
+    launch(ctx, k_segscan2_onepass<F>, (unsigned)tiles, SCAN_THREADS, f, n, (SegTile *)(state + 64), (uint32_t *)state,
+           out0, out1, outp, ctx->status);
     return check_cuda(ctx, cudaGetLastError(), "segmented scan");
 }
 

@@ -249,7 +249,8 @@ struct tm_ctx {
     timest::DevGraph g;
     std::vector<std::pair<void *, size_t>> graph_bufs;
     uint32_t *status = nullptr;          // device block, copied as a whole (kStatusBytes): [0] status bits,
-                                         // [1] the CSR build's pair count, [4] on: a call's small results
+                                         // [1] the CSR build's pair count, [2..3] a weight pass's window
+                                         // numbers, [4] on: a call's small results
     uint32_t *status_host = nullptr;     // its pinned mirror
     int num_sms = 0;
     // phase timing (cfg.profile)
@@ -306,7 +307,8 @@ int build_csr(tm_ctx *ctx);
 // guides = false leaves the samplers' guide tables to a later fill_guides (tree
 // selection needs them for the winner only)
 int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true);
-int fill_guides(tm_ctx *ctx, tm_motif *mo);
+// (nwin: the layers' window numbers on the device, null once the motif has them)
+int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin = nullptr);
 int export_weights(tm_ctx *ctx, tm_motif *mo, int q, int layer, uint64_t *host_out);
 
 // ---- sampler (sampler.cu) ----

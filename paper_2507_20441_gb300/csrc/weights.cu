@@ -37,8 +37,6 @@ struct ChildPrefix {
     size_t stride;
 };
 
-__device__ __forceinline__ uint64_t lane_of(const ulonglong2 v, int p) { return p ? v.y : v.x; }
-
 // Candidate ranges up to this many entries are scanned for the excluded
 // neighbour; longer ones search the excluded multi-edge list instead.
 constexpr uint32_t kScanLimit = 64;   // the bits of a RangeExcl
@@ -458,114 +456,107 @@ struct RootScan2 {
 
 // ---- windows of both layers (Constraint 3, Alg. 1) ------------------------
 // A window of layer p starts at GLOBAL position i when t'_i lies in a window
-// of layer p and t'_{i-1} does not lie in the same one.  Each thread takes
-// kWinItems consecutive positions; tile = one block's positions.
-constexpr int kWinItems = 8;
-constexpr int kWinTile = TB * kWinItems;
-
-// Head bits of position i (bit p: a window of layer p starts there) and the
-// window indices of both layers.
-__device__ __forceinline__ uint32_t win_heads_at(const uint32_t *__restrict__ t, uint32_t i, const WinDiv &wv,
-                                                 int64_t &w0, int64_t &w1)
-{
-    const uint32_t q = wv.quot(__ldg(t + i));
-    w0 = WinDiv::win_of(q, 0);
-    w1 = WinDiv::win_of(q, 1);
-    uint32_t h = (w0 >= 0 ? 1u : 0u) | (w1 >= 0 ? 2u : 0u);
-    if (i > 0) h &= win_change(wv, __ldg(t + i), __ldg(t + i - 1));
-    return h;
-}
-
-// Per tile: the number of window starts of each layer (counts[tile] for
-// layer 0, counts[ntile + tile] for layer 1).
-__global__ void __launch_bounds__(TB) k_win_count(const uint32_t *__restrict__ t, uint32_t m, WinDiv wv, uint32_t ntile,
-                                                  uint32_t *__restrict__ counts)
-{
-    __shared__ uint32_t s0[TB / 32], s1[TB / 32];
-    const uint32_t base = blockIdx.x * (uint32_t)kWinTile + threadIdx.x * kWinItems;
-    uint32_t c0 = 0, c1 = 0;
-#pragma unroll
-    for (int j = 0; j < kWinItems; ++j) {
-        const uint32_t i = base + j;
-        if (i >= m) break;
-        int64_t w0, w1;
-        const uint32_t h = win_heads_at(t, i, wv, w0, w1);
-        c0 += h & 1u;
-        c1 += h >> 1;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        c0 += __shfl_down_sync(0xffffffffu, c0, o);
-        c1 += __shfl_down_sync(0xffffffffu, c1, o);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) { s0[warp] = c0; s1[warp] = c1; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t a = 0, b = 0;
-        for (int w = 0; w < TB / 32; ++w) { a += s0[w]; b += s1[w]; }
-        counts[blockIdx.x] = a;
-        counts[ntile + blockIdx.x] = b;
-    }
-}
-
+// of layer p and t'_{i-1} does not lie in the same one.  One pass: starts are
+// counted over the rows of a warp, the warps of a tile and, by look-back, the
+// tiles before it (both layers' counts in one word, 31 bits each: there are at
+// most 2^31 windows of a layer), which gives each its place; then the windows'
+// first positions and indices, the end sentinels beg[nwin] = m and the numbers
+// of windows.  Nothing on the host waits for these numbers: the arrays are
+// sized by what T / delta allows (a count, its scan, the host's wait for it and
+// the fill were 250 us on 5e7 edges and 60 on 2e6).
 struct WinOut {
-    uint32_t *beg[2], *id[2];
-    uint32_t nwin[2];
+    uint32_t *beg[2], *id[2];   // null: only the numbers are wanted
+    uint32_t *nwin;             // [2]
 };
-
-// The windows' first positions and indices, written at the tile's scanned
-// offsets (offs[tile] for layer 0, offs[ntile + tile] - nw0 for layer 1),
-// plus the end sentinels beg[nwin] = m.
-__global__ void __launch_bounds__(TB) k_win_fill(const uint32_t *__restrict__ t, uint32_t m, WinDiv wv, uint32_t ntile,
-                                                 const uint32_t *__restrict__ offs, WinOut W)
+constexpr int kWinChunk = 8;    // rows whose loads are in flight together
+template <int ROWS>
+__global__ void __launch_bounds__(256) k_windows(const uint32_t *__restrict__ t, uint32_t m, WinDiv wv,
+                                                 unsigned long long *__restrict__ state, uint32_t *__restrict__ ticket,
+                                                 WinOut W, uint32_t *status)
 {
-    __shared__ uint32_t s0[TB / 32], s1[TB / 32];
-    const uint32_t base = blockIdx.x * (uint32_t)kWinTile + threadIdx.x * kWinItems;
-    uint32_t hb = 0, c0 = 0, c1 = 0;
-#pragma unroll
-    for (int j = 0; j < kWinItems; ++j) {
-        const uint32_t i = base + j;
-        if (i >= m) break;
-        int64_t w0, w1;
-        const uint32_t h = win_heads_at(t, i, wv, w0, w1);
-        hb |= h << (2 * j);
-        c0 += h & 1u;
-        c1 += h >> 1;
-    }
-    // exclusive ranks of this thread's starts inside the tile, per layer
+    __shared__ uint32_t s_h[2][8][ROWS], s_w[2][8], s_tile;
+    __shared__ unsigned long long s_before;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t i0 = c0, i1 = c1;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y0 = __shfl_up_sync(0xffffffffu, i0, o), y1 = __shfl_up_sync(0xffffffffu, i1, o);
-        if (lane >= o) { i0 += y0; i1 += y1; }
-    }
-    if (lane == 31) { s0[warp] = i0; s1[warp] = i1; }
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t r0 = 0, r1 = 0;
-        for (int w = 0; w < TB / 32; ++w) {
-            const uint32_t a = s0[w], b = s1[w];
-            s0[w] = r0; s1[w] = r1;
-            r0 += a; r1 += b;
+    const uint32_t tile = s_tile;
+    const uint64_t base = ((uint64_t)tile * 8 + warp) * (32 * ROWS);
+    uint32_t mine[2] = {0, 0};
+    for (int c = 0; c < ROWS; c += kWinChunk) {
+        const uint64_t x0 = base + c * 32;
+        uint32_t v[kWinChunk];
+#pragma unroll
+        for (int r = 0; r < kWinChunk; ++r) v[r] = x0 + r * 32 + lane < m ? __ldg(t + x0 + r * 32 + lane) : 0u;
+        uint32_t qb = wv.quot(x0 > 0 && x0 <= m ? __ldg(t + x0 - 1) : 0u);   // the quotient before the row
+#pragma unroll
+        for (int r = 0; r < kWinChunk; ++r) {
+            const uint64_t x = x0 + r * 32 + lane;
+            const uint32_t q = wv.quot(v[r]);
+            uint32_t qp = __shfl_up_sync(0xffffffffu, q, 1);
+            if (lane == 0) qp = qb;
+            qb = __shfl_sync(0xffffffffu, q, 31);
+            // the windows of q are those of q / 2 (layer 0) and (q + 1) / 2 (layer 1; none for q = 0)
+            const uint32_t h0 = __ballot_sync(0xffffffffu, x < m && (x == 0 || (q >> 1) != (qp >> 1)));
+            const uint32_t h1 = __ballot_sync(0xffffffffu, x < m && q > 0 && (x == 0 || ((q + 1) >> 1) != ((qp + 1) >> 1)));
+            mine[0] += __popc(h0);
+            mine[1] += __popc(h1);
+            if (lane == 0) { s_h[0][warp][c + r] = h0; s_h[1][warp][c + r] = h1; }
+        }
+    }
+    if (lane == 0) { s_w[0][warp] = mine[0]; s_w[1][warp] = mine[1]; }
+    __syncthreads();
+    constexpr unsigned long long kSum = 1ull << 62, kPrefix = 2ull << 62, kCounts = kSum - 1;
+    if (warp == 0) {
+        unsigned long long sum = 0;
+        for (int w = 0; w < 8; ++w) sum += s_w[0][w] | ((unsigned long long)s_w[1][w] << 31);
+        if (lane == 0) *(volatile unsigned long long *)(state + tile) = (tile == 0 ? kPrefix : kSum) | sum;
+        unsigned long long before = 0;
+        for (int64_t j = (int64_t)tile - 1 - lane; tile != 0; j -= 32) {   // lane i at the i-th tile before
+            unsigned long long x = 2ull << 62;
+            if (j >= 0) {
+                x = *(volatile unsigned long long *)(state + j);
+                for (int it = 0; (x >> 62) == 0 && it < kLookbackPolls; ++it) {
+                    __nanosleep(32);
+                    x = *(volatile unsigned long long *)(state + j);
+                }
+                if ((x >> 62) == 0) { latch(status, ST_TIMEOUT); x = 2ull << 62; }
+            }
+            const unsigned end = __ballot_sync(0xffffffffu, (x >> 62) == 2);
+            const int last = end ? __ffs((int)end) - 1 : 31;
+            unsigned long long c = lane <= last ? x & kCounts : 0;
+            for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+            before += c;
+            if (end) break;
+        }
+        if (lane == 0) {
+            if (tile != 0) *(volatile unsigned long long *)(state + tile) = kPrefix | (before + sum);
+            s_before = before;
         }
     }
     __syncthreads();
-    uint32_t k0 = offs[blockIdx.x] + s0[warp] + i0 - c0;
-    uint32_t k1 = offs[ntile + blockIdx.x] - W.nwin[0] + s1[warp] + i1 - c1;
+    uint32_t k[2] = {(uint32_t)(s_before & 0x7FFFFFFFu), (uint32_t)((s_before >> 31) & 0x7FFFFFFFu)};
+    for (int w = 0; w < warp; ++w) { k[0] += s_w[0][w]; k[1] += s_w[1][w]; }
+    for (int r = 0; r < ROWS; ++r) {
+        const uint64_t x = base + r * 32 + lane;
+        const uint32_t h[2] = {s_h[0][warp][r], s_h[1][warp][r]};
 #pragma unroll
-    for (int j = 0; j < kWinItems; ++j) {
-        const uint32_t h = (hb >> (2 * j)) & 3u;
-        if (!h) continue;
-        const uint32_t i = base + j;
-        const uint32_t q = wv.quot(__ldg(t + i));
-        if (h & 1u) { W.beg[0][k0] = i; W.id[0][k0] = (uint32_t)WinDiv::win_of(q, 0); ++k0; }
-        if (h & 2u) { W.beg[1][k1] = i; W.id[1][k1] = (uint32_t)WinDiv::win_of(q, 1); ++k1; }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        W.beg[0][W.nwin[0]] = m;
-        W.beg[1][W.nwin[1]] = m;
+        for (int p = 0; p < 2; ++p) {
+            const uint32_t at = k[p] + __popc(h[p] & ((1u << lane) - 1u)), mark = (h[p] >> lane) & 1u;
+            if (mark && W.beg[p]) {
+                W.beg[p][at] = (uint32_t)x;
+                W.id[p][at] = (uint32_t)wv.win(__ldg(t + x), p);
+            }
+            if (x == (uint64_t)m - 1) {
+                if (W.beg[p]) W.beg[p][at + mark] = m;
+                W.nwin[p] = at + mark;
+            }
+            k[p] += __popc(h[p]);
+        }
     }
 }
+// rows per warp: as the pair kernel's (a small array needs the blocks more than the fewer tiles)
+constexpr int kWinRowsSmall = 8, kWinRowsLarge = 64;
+constexpr uint32_t kWinSmall = 4000000;
 
 // ---- guide table of the root search --------------------------------------
 // Window kk of a layer gets about n/4 buckets of width 2^s over its draws
@@ -581,6 +572,8 @@ struct GuideLayer {
 };
 struct GuideArgs {
     GuideLayer L[2];
+    const uint32_t *nwin;   // on the device [2] (null: those of L)
+    __device__ __forceinline__ uint32_t windows(int p) const { return nwin ? __ldg(nwin + p) : p ? L[1].nwin : L[0].nwin; }
 };
 
 // Window totals W_i (last root-CDF entry of each window) and their 128-bit
@@ -597,7 +590,7 @@ __global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *_
     __shared__ u128 s_tot[32];
     __shared__ u128 s_carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t nw0 = A.L[0].nwin, nw1 = A.L[1].nwin;
+    const uint32_t nw0 = A.windows(0), nw1 = A.windows(1);
     const int b = blockIdx.x;
     const uint32_t n = b == 0 ? nw0 + nw1 : b == 1 ? nw0 : nw1;
     if (threadIdx.x == 0) s_carry = 0;
@@ -707,14 +700,15 @@ __global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m, cons
 {
     const int p = blockIdx.y;
     if (p == 2) {
-        const uint32_t nw = A.L[0].nwin + A.L[1].nwin;
+        const uint32_t nw = A.windows(0) + A.windows(1);
+        if (nw == 0) return;
         for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= 4 * (uint64_t)nw;
              j += (uint64_t)gridDim.x * blockDim.x)
             wguide_entry(wcum, nw, wguide, (uint32_t)j);
         return;
     }
     // per-field selects keep the parameter block out of local memory
-    const uint32_t nwin = p ? A.L[1].nwin : A.L[0].nwin;
+    const uint32_t nwin = A.windows(p);
     const uint64_t *__restrict__ cdf = p ? A.L[1].cdf : A.L[0].cdf;
     const uint32_t *__restrict__ win_beg = p ? A.L[1].win_beg : A.L[0].win_beg;
     const uint32_t *__restrict__ gshift = p ? A.L[1].gshift : A.L[0].gshift;
@@ -806,9 +800,10 @@ static void free_motif_weights(tm_ctx *ctx, tm_motif *mo)
 // Owner bit sets of the out-, in- and multi-edge orders (built with the graph).
 struct OwnerBits { const uint32_t *out, *in, *multi; };
 
-static GuideArgs guide_args(const tm_motif *mo)
+static GuideArgs guide_args(const tm_motif *mo, const uint32_t *nwin)
 {
     GuideArgs ga{};
+    ga.nwin = nwin;
     for (int p = 0; p < 2; ++p) {
         const LayerData &L = mo->layer[p];
         ga.L[p] = GuideLayer{L.root_cdf, L.win_beg, L.nwin, L.win_gshift, L.win_goff, L.guide};
@@ -816,12 +811,12 @@ static GuideArgs guide_args(const tm_motif *mo)
     return ga;
 }
 
-int fill_guides(tm_ctx *ctx, tm_motif *mo)
+int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin)
 {
     const uint64_t m = ctx->g.m;
-    if (m == 0 || mo->nwtot == 0) return TM_OK;
+    if (m == 0) return TM_OK;
     const uint64_t gwarps = (m + 32 * kGuideItems - 1) / (32 * kGuideItems);
-    launch(ctx, k_guide_fill, dim3(blocks_for(gwarps * 32, TB), 3), TB, guide_args(mo), (uint32_t)m,
+    launch(ctx, k_guide_fill, dim3(blocks_for(gwarps * 32, TB), 3), TB, guide_args(mo, nwin), (uint32_t)m,
            (const uint64_t *)mo->wcum, mo->wguide);
     return check_cuda(ctx, cudaGetLastError(), "guide tables");
 }
@@ -836,30 +831,38 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     const uint32_t m = g.m;
     const WinDiv wv = make_windiv(P.wdelta);   // window unit (delta, or one window without Constraint 3)
     int rc = TM_OK;
-    cudaMemsetAsync(ctx->status, 0, 4, st);
-    // ---- windows of each layer (K2): per tile the window starts of both
-    // layers, one scan over the tile counts, then one block for everything
-    // the motif keeps (windows, root CDF, prefix arrays, totals)
-    const uint32_t ntile = m ? (m + kWinTile - 1) / kWinTile : 0;
-    uint32_t *wcount = nullptr, *woffs = nullptr;
-    uint32_t nwh[2] = {0, 0};
-    {
+    cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
+    // cleared together: the windows' ticket and tile words, the number of kept
+    // excluded ranges, the tiles of every scan
+    const bool win_small = m <= kWinSmall;
+    const uint32_t win_tile = 256u * (win_small ? kWinRowsSmall : kWinRowsLarge), win_tiles = m ? (m - 1) / win_tile + 1 : 0;
+    const size_t win_bytes = ((size_t)win_tiles * 8 + 64 + 255) / 256 * 256, scan_bytes = scan_state_bytes(m);
+    const size_t clear_bytes = win_bytes + (2 * (size_t)P.nslots + 1) * scan_bytes;
+    char *clear = (char *)salloc(ctx, clear_bytes);
+    if (!clear) return TM_E_NOMEM;
+    cudaMemsetAsync(clear, 0, clear_bytes, st);
+    uint32_t *ticket = (uint32_t *)clear;   // [0] the windows' ticket, [2] the excluded ranges' number
+    unsigned long long *win_state = (unsigned long long *)(clear + 64);
+    char *scan_state = clear + win_bytes;
+    auto windows = [&](const WinOut &wo) {
+        launch(ctx, win_small ? k_windows<kWinRowsSmall> : k_windows<kWinRowsLarge>, win_tiles, 256, g.g_t, m, wv,
+               win_state, ticket, wo, ctx->status);
+    };
+    // ---- windows of each layer (K2): window indices go up to T / unit, the even
+    // ones in layer 0; one block for everything the motif keeps
+    const uint64_t qT = m ? (uint64_t)g.T / (uint64_t)P.wdelta : 0;
+    uint32_t nwh[2] = {(uint32_t)std::min<uint64_t>(m, qT / 2 + 1), (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2)};
+    if ((uint64_t)nwh[0] + nwh[1] > (uint64_t)m / 8 + 4096) {
+        // windows so short that most may be empty: counted before they take room
         PhaseScope ph(ctx, TM_PH_WINDOWS);
-        wcount = (uint32_t *)salloc(ctx, ((size_t)2 * ntile + 1) * 4);
-        woffs = (uint32_t *)salloc(ctx, ((size_t)2 * ntile + 2) * 4);
-        if (!wcount || !woffs) return TM_E_NOMEM;
-        if (m) {
-            launch(ctx, k_win_count, ntile, TB, g.g_t, m, wv, ntile, wcount);
-            rc = exclusive_scan_u32(ctx, wcount, woffs, 2 * (uint64_t)ntile, woffs + 2 * (size_t)ntile);
-            if (rc) return rc;
-            uint32_t *both = ctx->status_host + 4;   // pinned
-            copy_d2h(ctx, &both[0], woffs + ntile, 4);                  // layer 0's windows
-            copy_d2h(ctx, &both[1], woffs + 2 * (size_t)ntile, 4);      // all windows
-            rc = check_cuda(ctx, cudaStreamSynchronize(st), "window count");
-            if (rc) return rc;
-            nwh[0] = both[0];
-            nwh[1] = both[1] - both[0];
-        }
+        windows(WinOut{{nullptr, nullptr}, {nullptr, nullptr}, ctx->status + 2});
+        uint32_t bits = 0;
+        rc = read_status(ctx, &bits);
+        if (rc) return rc;
+        if (bits) return set_err(ctx, TM_E_CUDA, "device status error in the window count");
+        nwh[0] = ctx->status_host[2];
+        nwh[1] = ctx->status_host[3];
+        cudaMemsetAsync(clear, 0, win_bytes, st);
     }
     {
         auto al = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -873,7 +876,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         // (room for excluded entries at 0.3 of the edges per kind: with bursts of
         // repeated pairs a star's ranges have them at 0.2 - 0.3)
         const size_t excl_cap = (size_t)P.nkinds * (mm * 3 / 10);
-        const size_t range_bytes = (size_t)P.nkinds * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl)) + al(8);
+        const size_t range_bytes = (size_t)P.nkinds * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl));
         bool with_ranges = true;
         char *blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
         if (!blk && total >= ((size_t)4 << 30)) {
@@ -903,16 +906,15 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
             mo->range.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
             mo->range.base = (uint2 *)take((size_t)P.nkinds * mo->range.stride * sizeof(uint2));
             mo->range.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
-            mo->range.excl_n = (unsigned long long *)take(8);
+            mo->range.excl_n = (unsigned long long *)(ticket + 2);   // of this pass
             mo->range.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
-            cudaMemsetAsync(mo->range.excl_n, 0, 8, st);
         }
     }
     {
         PhaseScope ph(ctx, TM_PH_WINDOWS);
-        WinOut wo{{mo->layer[0].win_beg, mo->layer[1].win_beg}, {mo->layer[0].win_id, mo->layer[1].win_id},
-                  {nwh[0], nwh[1]}};
-        if (m) launch(ctx, k_win_fill, ntile, TB, g.g_t, m, wv, ntile, (const uint32_t *)woffs, wo);
+        if (m)
+            windows(WinOut{{mo->layer[0].win_beg, mo->layer[1].win_beg}, {mo->layer[0].win_id, mo->layer[1].win_id},
+                           ctx->status + 2});
         else {
             cudaMemsetAsync(mo->layer[0].win_beg, 0, 4, st);
             cudaMemsetAsync(mo->layer[1].win_beg, 0, 4, st);
@@ -991,7 +993,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         if (q == 0) {
             PhaseScope ph(ctx, TM_PH_ROOT);
             RootScan2 f{w, nz, g.g_t, wv, in_order ? g.in_pos : g.out_pos};
-            rc = segmented_scan2_u64(ctx, f, m, mo->layer[0].root_cdf, mo->layer[1].root_cdf);
+            rc = segmented_scan2_u64(ctx, f, m, scan_state, mo->layer[0].root_cdf, mo->layer[1].root_cdf);
             if (rc) return rc;
         } else {
             PhaseScope ph(ctx, TM_PH_PREFIX);
@@ -1008,21 +1010,19 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
             // out-list order (w in both cases).
             const uint32_t *wnz = out && in_order ? nullptr : nz;   // (scattered weights have no bit set)
             DirScan2 fd{w, wnz, out ? nullptr : g.in_to_out, out ? g.out_t : g.in_t, out ? ob.out : ob.in, wv};
-            rc = segmented_scan2_u64(ctx, fd, m, nullptr, nullptr, mo->pref_dir[slot]);
+            rc = segmented_scan2_u64(ctx, fd, m, scan_state + (1 + 2 * slot) * scan_bytes, nullptr, nullptr, mo->pref_dir[slot]);
             if (rc) return rc;
             DirScan2 fm{w, wnz, g.multi_to_out, g.multi_t, ob.multi, wv};
-            rc = segmented_scan2_u64(ctx, fm, m, nullptr, nullptr, mo->pref_multi[slot]);
+            rc = segmented_scan2_u64(ctx, fm, m, scan_state + (2 + 2 * slot) * scan_bytes, nullptr, nullptr, mo->pref_multi[slot]);
             if (rc) return rc;
         }
     }
     // ---- window totals and their 128-bit running sum (K5)
-    uint32_t nw0 = mo->layer[0].nwin, nw1 = mo->layer[1].nwin;
-    mo->nwtot = nw0 + nw1;
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
-        launch(ctx, k_window_totals, 3, 1024, guide_args(mo), mo->wcum, (uint64_t *)(ctx->status + 4));
+        launch(ctx, k_window_totals, 3, 1024, guide_args(mo, ctx->status + 2), mo->wcum, (uint64_t *)(ctx->status + 4));
         if (guides) {
-            rc = fill_guides(ctx, mo);
+            rc = fill_guides(ctx, mo, ctx->status + 2);
             if (rc) return rc;
         }
     }
@@ -1032,6 +1032,8 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a weight, prefix sum or window total exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "device status error in weight pass");
     memcpy(&mo->W, ctx->status_host + 4, 16);   // copied with the status
+    for (int p = 0; p < 2; ++p) mo->layer[p].nwin = ctx->status_host[2 + p];
+    mo->nwtot = mo->layer[0].nwin + mo->layer[1].nwin;
     mo->have_weights = true;
     mo->graph_epoch = ctx->epoch;
     return TM_OK;
