@@ -17,8 +17,7 @@
 // (read in GLOBAL order), which is the in -> out map, and the multi-edge
 // order is a stable re-sort of the IN order by source carrying t', the
 // destination and that map (-> multi_to_out).  The random accesses left are
-// the cross ranks, found by binary searches in the owner's other list (four
-// per thread in lockstep).
+// the cross ranks, found by searches in the owner's other list.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>
@@ -967,55 +966,54 @@ struct XR {
     const uint32_t *own_t, *owner, *other_off, *other_t;
     uint32_t *xrank;
 };
-// Two alternatives measured slower on 5e7 entries per list: letting the
-// first and last lanes of a warp whose entries share one owner search first
-// and the other lanes only the bracket those give (1.32 against 1.25 ms), and
-// merging each vertex's two lists along a merge path in chunks of 128 entries
-// per thread (1.44 ms: the chunk walk is one long chain of dependent loads).
-// The independent searches keep the most loads in flight.
-// Each thread runs TM_XR_ITEMS searches (entries i, i + stride, ...) in
-// lockstep, so that many independent probes are in flight per thread.
-#ifndef TM_XR_ITEMS
-#define TM_XR_ITEMS 4
-#endif
-__global__ void k_cross_rank(XR a, XR b, uint32_t m, uint32_t n)
+// A thread takes kXrItems consecutive entries: the first is searched for in the
+// whole of its owner's other list, the next ones of the same owner from there
+// on (their times do not fall), which takes a probe or two.
+// 5e7 edges: 797 us with four separate searches in lockstep per thread, 566 with
+// four consecutive entries, 481 with eight; 2e6 edges 34, 29 and 31.
+template <int kXrItems>
+__global__ void __launch_bounds__(256) k_cross_rank(XR a, XR b, uint32_t m, uint32_t n)
 {
-    constexpr int K = TM_XR_ITEMS;
     const bool s1 = blockIdx.y != 0;
-    const uint32_t *own_t = s1 ? b.own_t : a.own_t, *owner = s1 ? b.owner : a.owner;
-    const uint32_t *other_off = s1 ? b.other_off : a.other_off, *other_t = s1 ? b.other_t : a.other_t;
-    uint32_t *xrank = s1 ? b.xrank : a.xrank;
-    const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * K + threadIdx.x;
-    uint32_t lo[K], len[K], key[K];
+    const uint32_t *__restrict__ own_t = s1 ? b.own_t : a.own_t, *__restrict__ owner = s1 ? b.owner : a.owner;
+    const uint32_t *__restrict__ other_off = s1 ? b.other_off : a.other_off, *__restrict__ other_t = s1 ? b.other_t : a.other_t;
+    uint32_t *__restrict__ xrank = s1 ? b.xrank : a.xrank;
+    const uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * kXrItems;
+    if (i0 >= m) return;
+    uint32_t z[kXrItems], t[kXrItems], r[kXrItems];
+    const bool whole = i0 + kXrItems <= m;   // (the arrays are 256-byte aligned)
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const uint64_t i = i0 + (uint64_t)k * blockDim.x;
-        lo[k] = 0; len[k] = 0; key[k] = 0;
-        if (i < m) {
-            const uint32_t z = min(__ldg(owner + i), n - 1);   // (a sort whose wait ran out leaves anything here)
-            key[k] = __ldg(own_t + i);
-            lo[k] = __ldg(other_off + z);
-            len[k] = __ldg(other_off + z + 1) - lo[k];
-        }
-    }
-    // the binary search of lower_idx, all K at once
-    bool more = true;
-    while (more) {
-        more = false;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if (len[k] > 0) {
-                const uint32_t half = len[k] >> 1, mid = lo[k] + half;
-                if (__ldg(other_t + mid) < key[k]) { lo[k] = mid + 1; len[k] -= half + 1; }
-                else len[k] = half;
-                more |= len[k] > 0;
+    for (int k = 0; k < kXrItems; k += 4) {
+        if (whole) {
+            const uint4 vz = __ldg(reinterpret_cast<const uint4 *>(owner + i0 + k)), vt = __ldg(reinterpret_cast<const uint4 *>(own_t + i0 + k));
+            z[k] = vz.x; z[k + 1] = vz.y; z[k + 2] = vz.z; z[k + 3] = vz.w;
+            t[k] = vt.x; t[k + 1] = vt.y; t[k + 2] = vt.z; t[k + 3] = vt.w;
+        } else {
+            for (int j = k; j < k + 4; ++j) {
+                z[j] = __ldg(owner + min(i0 + j, (uint64_t)m - 1));
+                t[j] = __ldg(own_t + min(i0 + j, (uint64_t)m - 1));
             }
         }
     }
+    uint32_t lo = 0, hi = 0;
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const uint64_t i = i0 + (uint64_t)k * blockDim.x;
-        if (i < m) xrank[i] = lo[k];
+    for (int k = 0; k < kXrItems; ++k) {
+        if (k == 0 || z[k] != z[k - 1]) {
+            const uint32_t v = min(z[k], n - 1);   // (a sort whose wait ran out leaves anything here)
+            lo = __ldg(other_off + v);
+            hi = __ldg(other_off + v + 1);
+            lo = lower_idx(other_t, lo, hi, t[k]);
+        } else if (t[k] != t[k - 1]) {
+            lo = gallop_idx(other_t, lo, hi, t[k]);
+        }
+        r[k] = lo;
+    }
+#pragma unroll
+    for (int k = 0; k < kXrItems; k += 4) {
+        if (whole) *reinterpret_cast<uint4 *>(xrank + i0 + k) = make_uint4(r[k], r[k + 1], r[k + 2], r[k + 3]);
+        else
+            for (int j = k; j < k + 4; ++j)
+                if (i0 + j < m) xrank[i0 + j] = r[j];
     }
 }
 
@@ -1270,7 +1268,8 @@ int build_csr(tm_ctx *ctx)
                (const uint32_t *)key, (const uint32_t *)tmp, m, n, pair_state, hist + 3 * OS_HIST, g.pair_off,
                g.pair_dst, g.vpair_off, g.own_multi, ctx->status + 1, ctx->status);
         // cross ranks between a vertex's out- and in-lists
-        launch(ctx, k_cross_rank, dim3(blocks_for(((uint64_t)m + TM_XR_ITEMS - 1) / TM_XR_ITEMS, TB), 2), TB,
+        const int per = m <= kPairSmall ? 4 : 8;
+        launch(ctx, per == 4 ? k_cross_rank<4> : k_cross_rank<8>, dim3(blocks_for(((uint64_t)m + per - 1) / per, TB), 2), TB,
                XR{g.out_t, g.out_src, g.in_off, g.in_t, g.out_xrank},
                XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m, n);
     } else {
