@@ -577,87 +577,125 @@ struct GuideArgs {
 };
 
 // Window totals W_i (last root-CDF entry of each window) and their 128-bit
-// running sum over (layer 0 windows, layer 1 windows) by block 0, which also
-// puts their total at W; the guide
-// table's bucket width and offset of each window by block 1 + p for layer p.
-// A block takes kTotItems windows per thread at a time, whose loads are
-// independent (a contiguous run of windows per thread is one load after the
-// other: 82 + 38 us in two launches for 5.6e4 windows, 36 us like this).
-constexpr int kTotItems = 8;
-__global__ void __launch_bounds__(1024) k_window_totals(GuideArgs A, uint64_t *__restrict__ wcum,
-                                                        uint64_t *__restrict__ W)
+// running sum over (layer 0 windows, layer 1 windows) by the blocks of y = 0,
+// which also put their total at W; the guide table's bucket width and offset of
+// each window by y = 1 + p for layer p.  A tile of kTotTile windows is a block,
+// whose sum is looked back for as in the segmented scans: the number of windows
+// is known on the device alone, so the grid is for the most there can be and
+// the blocks past the last tile leave.  The loads of win_beg and of the CDF
+// behind it are what takes the time (random sectors): one block for each y,
+// eight windows per thread at a time, kept only three SMs' loads in flight.
+// 5.6e4 windows: 61 us like that, 14 so; 1.7e4: 24 and 12.
+constexpr int kTotItems = 4, kTotThreads = 256;
+constexpr uint32_t kTotTile = kTotThreads * kTotItems;
+__global__ void __launch_bounds__(kTotThreads) k_window_totals(GuideArgs A, uint64_t *__restrict__ wcum, uint64_t *__restrict__ W,
+                                                               SegTile *__restrict__ tiles, uint32_t *__restrict__ ticket,
+                                                               uint32_t *status)
 {
-    __shared__ u128 s_tot[32];
-    __shared__ u128 s_carry;
+    constexpr int kWarps = kTotThreads / 32;
+    __shared__ u128 s_tot[kWarps];
+    __shared__ u128 s_before;
+    __shared__ uint32_t s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nw0 = A.windows(0), nw1 = A.windows(1);
-    const int b = blockIdx.x;
-    const uint32_t n = b == 0 ? nw0 + nw1 : b == 1 ? nw0 : nw1;
-    if (threadIdx.x == 0) s_carry = 0;
-    for (uint32_t base = 0; base < n || base == 0; base += 1024 * kTotItems) {
-        const uint32_t k0 = base + threadIdx.x * kTotItems;
-        uint64_t v[kTotItems];
-        u128 sum = 0;
+    const int b = blockIdx.y;
+    const uint32_t n = b == 0 ? nw0 + nw1 : b == 1 ? nw0 : nw1, ntiles = n ? (n - 1) / kTotTile + 1 : 1;
+    if (blockIdx.x >= ntiles) return;   // (as many blocks stay as there are tiles)
+    tiles += (size_t)b * gridDim.x;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket + b, 1u);
+    __syncthreads();
+    const uint32_t tile = s_tile, k0 = tile * kTotTile + threadIdx.x * kTotItems;
+    uint64_t v[kTotItems];
+    u128 sum = 0;
 #pragma unroll
-        for (int j = 0; j < kTotItems; ++j) {
-            const uint32_t k = k0 + j;
-            v[j] = 0;
-            if (k < n) {
-                const bool second = b == 2 || (b == 0 && k >= nw0);
-                const uint32_t *win_beg = second ? A.L[1].win_beg : A.L[0].win_beg;
-                const uint32_t kk = b == 0 && second ? k - nw0 : k, wend = win_beg[kk + 1];
-                const uint64_t W = (second ? A.L[1].cdf : A.L[0].cdf)[wend - 1];
-                if (b == 0) {
-                    v[j] = W;
-                } else {
-                    // about n / 4 buckets of 2^sh draws each over the window's W
-                    const uint32_t ne = wend - win_beg[kk], target = ne >> 2 ? ne >> 2 : 1;
-                    uint32_t sh = 0;
-                    if (W) {
-                        const int d = __clz((int)target) - 32 + 64 - __clzll((long long)(W - 1));
-                        sh = d > 1 ? d - 1 : 0;   // not above the least width, then stepped up to it
-                        while (sh < 63 && ((W - 1) >> sh) + 1 > target) ++sh;
-                    }
-                    (second ? A.L[1].gshift : A.L[0].gshift)[kk] = sh;
-                    v[j] = (W ? ((W - 1) >> sh) + 1 : 0) + 1;
+    for (int j = 0; j < kTotItems; ++j) {
+        const uint32_t k = k0 + j;
+        v[j] = 0;
+        if (k < n) {
+            const bool second = b == 2 || (b == 0 && k >= nw0);
+            const uint32_t *win_beg = second ? A.L[1].win_beg : A.L[0].win_beg;
+            const uint32_t kk = b == 0 && second ? k - nw0 : k, wend = win_beg[kk + 1];
+            const uint64_t W = (second ? A.L[1].cdf : A.L[0].cdf)[wend - 1];
+            if (b == 0) {
+                v[j] = W;
+            } else {
+                // about n / 4 buckets of 2^sh draws each over the window's W
+                const uint32_t ne = wend - win_beg[kk], target = ne >> 2 ? ne >> 2 : 1;
+                uint32_t sh = 0;
+                if (W) {
+                    const int d = __clz((int)target) - 32 + 64 - __clzll((long long)(W - 1));
+                    sh = d > 1 ? d - 1 : 0;   // not above the least width, then stepped up to it
+                    while (sh < 63 && ((W - 1) >> sh) + 1 > target) ++sh;
                 }
+                (second ? A.L[1].gshift : A.L[0].gshift)[kk] = sh;
+                v[j] = (W ? ((W - 1) >> sh) + 1 : 0) + 1;
             }
-            sum += v[j];
         }
-        // exclusive scan of the threads' sums (128-bit) across the block
-        u128 incl = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint64_t yl = __shfl_up_sync(0xffffffffu, (uint64_t)incl, o);
-            const uint64_t yh = __shfl_up_sync(0xffffffffu, (uint64_t)(incl >> 64), o);
-            if (lane >= o) incl += (u128)yl | ((u128)yh << 64);
-        }
-        if (lane == 31) s_tot[warp] = incl;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            u128 run = s_carry;
-            for (int w = 0; w < 32; ++w) { const u128 c = s_tot[w]; s_tot[w] = run; run += c; }
-            s_carry = run;
-        }
-        __syncthreads();
-        u128 run = s_tot[warp] + incl - sum;
-#pragma unroll
-        for (int j = 0; j < kTotItems; ++j) {
-            const uint32_t k = k0 + j;
-            if (k < n) {
-                if (b == 0) {
-                    wcum[2 * (size_t)k] = (uint64_t)run;
-                    wcum[2 * (size_t)k + 1] = (uint64_t)(run >> 64);
-                } else {
-                    (b == 2 ? A.L[1].goff : A.L[0].goff)[k] = (uint32_t)run;
-                }
-            }
-            run += v[j];
-        }
-        __syncthreads();   // s_tot is written again
+        sum += v[j];
     }
-    if (b == 0 && threadIdx.x == 0) {
-        W[0] = wcum[2 * (size_t)n] = (uint64_t)s_carry;
-        W[1] = wcum[2 * (size_t)n + 1] = (uint64_t)(s_carry >> 64);
+    // exclusive scan of the threads' sums (128-bit) across the block
+    u128 incl = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t yl = __shfl_up_sync(0xffffffffu, (uint64_t)incl, o);
+        const uint64_t yh = __shfl_up_sync(0xffffffffu, (uint64_t)(incl >> 64), o);
+        if (lane >= o) incl += (u128)yl | ((u128)yh << 64);
+    }
+    if (lane == 31) s_tot[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        u128 T = 0, before = 0;
+        for (int w = 0; w < kWarps; ++w) T += s_tot[w];
+        if (lane == 0) seg_publish(tiles + tile, SegAgg2{(uint64_t)T, (uint64_t)(T >> 64), 0, 0}, tile == 0 ? 2u : 1u);
+        if (tile) {
+            for (int64_t jb = (int64_t)tile - 1;; jb -= 32) {   // 32 tiles at a time, the closest in lane 0
+                const int64_t j = jb - lane;
+                SegAgg2 x{0, 0, 0, 0};
+                uint32_t st = 2;
+                if (j >= 0) {
+                    st = seg_read(tiles + j, x);
+                    for (int it = 0; st == 0 && it < kLookbackPolls; ++it) {
+                        __nanosleep(64);
+                        st = seg_read(tiles + j, x);
+                    }
+                    if (st == 0) { latch(status, ST_TIMEOUT); x = SegAgg2{0, 0, 0, 0}; }
+                }
+                const unsigned stop = __ballot_sync(0xffffffffu, st != 1);
+                u128 y = !stop || lane < __ffs((int)stop) ? (u128)x.v0 | ((u128)x.v1 << 64) : 0;
+                for (int o = 16; o; o >>= 1) {
+                    const uint64_t yl = __shfl_xor_sync(0xffffffffu, (uint64_t)y, o);
+                    const uint64_t yh = __shfl_xor_sync(0xffffffffu, (uint64_t)(y >> 64), o);
+                    y += (u128)yl | ((u128)yh << 64);
+                }
+                before += y;
+                if (stop) break;
+            }
+            const u128 P = before + T;
+            if (lane == 0) seg_publish(tiles + tile, SegAgg2{(uint64_t)P, (uint64_t)(P >> 64), 0, 0}, 2);
+        }
+        if (lane == 0) {
+            s_before = before;
+            if (b == 0 && tile == ntiles - 1) {
+                const u128 all = before + T;
+                W[0] = wcum[2 * (size_t)n] = (uint64_t)all;
+                W[1] = wcum[2 * (size_t)n + 1] = (uint64_t)(all >> 64);
+            }
+        }
+    }
+    __syncthreads();
+    u128 run = s_before + incl - sum;
+    for (int w = 0; w < warp; ++w) run += s_tot[w];
+#pragma unroll
+    for (int j = 0; j < kTotItems; ++j) {
+        const uint32_t k = k0 + j;
+        if (k < n) {
+            if (b == 0) {
+                wcum[2 * (size_t)k] = (uint64_t)run;
+                wcum[2 * (size_t)k + 1] = (uint64_t)(run >> 64);
+            } else {
+                (b == 2 ? A.L[1].goff : A.L[0].goff)[k] = (uint32_t)run;
+            }
+        }
+        run += v[j];
     }
 }
 
@@ -832,26 +870,29 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     const WinDiv wv = make_windiv(P.wdelta);   // window unit (delta, or one window without Constraint 3)
     int rc = TM_OK;
     cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
-    // cleared together: the windows' ticket and tile words, the number of kept
-    // excluded ranges, the tiles of every scan
+    // window indices go up to T / unit, the even ones in layer 0
+    const uint64_t qT = m ? (uint64_t)g.T / (uint64_t)P.wdelta : 0;
+    uint32_t nwh[2] = {(uint32_t)std::min<uint64_t>(m, qT / 2 + 1), (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2)};
+    // cleared together: the tickets, the number of kept excluded ranges, the tile
+    // words of the windows, of their totals and of every scan
     const bool win_small = m <= kWinSmall;
     const uint32_t win_tile = 256u * (win_small ? kWinRowsSmall : kWinRowsLarge), win_tiles = m ? (m - 1) / win_tile + 1 : 0;
     const size_t win_bytes = ((size_t)win_tiles * 8 + 64 + 255) / 256 * 256, scan_bytes = scan_state_bytes(m);
-    const size_t clear_bytes = win_bytes + (2 * (size_t)P.nslots + 1) * scan_bytes;
+    const uint32_t tot_tiles = (uint32_t)(((uint64_t)nwh[0] + nwh[1]) / kTotTile) + 1;
+    const size_t tot_bytes = (3 * (size_t)tot_tiles * sizeof(SegTile) + 255) / 256 * 256;
+    const size_t clear_bytes = win_bytes + tot_bytes + (2 * (size_t)P.nslots + 1) * scan_bytes;
     char *clear = (char *)salloc(ctx, clear_bytes);
     if (!clear) return TM_E_NOMEM;
     cudaMemsetAsync(clear, 0, clear_bytes, st);
-    uint32_t *ticket = (uint32_t *)clear;   // [0] the windows' ticket, [2] the excluded ranges' number
+    uint32_t *ticket = (uint32_t *)clear;   // [0] the windows', [4..6] their totals'; [2] the excluded ranges' number
     unsigned long long *win_state = (unsigned long long *)(clear + 64);
-    char *scan_state = clear + win_bytes;
+    SegTile *tot_state = (SegTile *)(clear + win_bytes);
+    char *scan_state = clear + win_bytes + tot_bytes;
     auto windows = [&](const WinOut &wo) {
         launch(ctx, win_small ? k_windows<kWinRowsSmall> : k_windows<kWinRowsLarge>, win_tiles, 256, g.g_t, m, wv,
                win_state, ticket, wo, ctx->status);
     };
-    // ---- windows of each layer (K2): window indices go up to T / unit, the even
-    // ones in layer 0; one block for everything the motif keeps
-    const uint64_t qT = m ? (uint64_t)g.T / (uint64_t)P.wdelta : 0;
-    uint32_t nwh[2] = {(uint32_t)std::min<uint64_t>(m, qT / 2 + 1), (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2)};
+    // ---- windows of each layer (K2); one block for everything the motif keeps
     if ((uint64_t)nwh[0] + nwh[1] > (uint64_t)m / 8 + 4096) {
         // windows so short that most may be empty: counted before they take room
         PhaseScope ph(ctx, TM_PH_WINDOWS);
@@ -1020,7 +1061,9 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     // ---- window totals and their 128-bit running sum (K5)
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
-        launch(ctx, k_window_totals, 3, 1024, guide_args(mo, ctx->status + 2), mo->wcum, (uint64_t *)(ctx->status + 4));
+        const uint32_t tt = (uint32_t)(((uint64_t)nwh[0] + nwh[1]) / kTotTile) + 1;   // (not more than tot_tiles)
+        launch(ctx, k_window_totals, dim3(tt, 3), kTotThreads, guide_args(mo, ctx->status + 2), mo->wcum,
+               (uint64_t *)(ctx->status + 4), tot_state, ticket + 4, ctx->status);
         if (guides) {
             rc = fill_guides(ctx, mo, ctx->status + 2);
             if (rc) return rc;
