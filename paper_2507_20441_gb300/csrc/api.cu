@@ -404,6 +404,25 @@ static int parse_motif(uint32_t nv, uint32_t ne, const uint32_t *edges, const ui
     return TM_OK;
 }
 
+// A child's candidate ranges depend on the side it meets its parent at, its
+// direction and its pi relation to the parent alone.
+void assign_kinds(DevPlan &P)
+{
+    P.nkinds = 0;
+    P.tkind[0] = -1;
+    for (int q = 1; q < P.ntree; ++q) {
+        int k = 0;
+        while (k < P.nkinds && (P.kside[k] != P.tzside[q] || P.kout[k] != P.tout[q] || P.klater[k] != P.tlater[q])) ++k;
+        if (k == P.nkinds) {
+            ++P.nkinds;
+            P.kinner[k] = 0;
+            P.kside[k] = P.tzside[q]; P.kout[k] = P.tout[q]; P.klater[k] = P.tlater[q];
+        }
+        P.tkind[q] = k;
+        if (!P.tleaf[q]) P.kinner[k] = 1;
+    }
+}
+
 // Root the tree at `root` and lay it out in sampling order: breadth first;
 // children of the root at its tail, then at its head; a node's children in
 // increasing motif-edge index (the draw order of the counter-based streams).
@@ -457,18 +476,7 @@ static int compile_plan(const MotifDesc &M, const int *tree, int root, int64_t d
     }
     for (int q = 0; q < P.ntree; ++q) P.tslot[q] = (q > 0 && !P.tleaf[q]) ? slot++ : -1;
     P.nslots = slot;
-    P.nkinds = 0;
-    P.tkind[0] = -1;
-    for (int q = 1; q < P.ntree; ++q) {
-        int k = 0;
-        while (k < P.nkinds && (P.kside[k] != P.tzside[q] || P.kout[k] != P.tout[q] || P.klater[k] != P.tlater[q])) ++k;
-        if (k == P.nkinds) {
-            ++P.nkinds;
-            P.kside[k] = P.tzside[q]; P.kout[k] = P.tout[q]; P.klater[k] = P.tlater[q];
-        }
-        P.tkind[q] = k;
-        if (!P.tleaf[q]) P.kinner[k] = 1;
-    }
+    assign_kinds(P);
     // non-tree edges along pi and their neighbouring tree positions
     for (int e = 0; e < M.ne; ++e) P.tnode_of_edge[e] = -1;
     for (int q = 0; q < P.ntree; ++q) P.tnode_of_edge[P.tedge[q]] = q;
@@ -776,13 +784,66 @@ static bool u128_less(const tm_u128 &a, const tm_u128 &b) { return a.hi < b.hi |
 
 // tm_weights without the samplers' guide tables: a candidate is asked for its W
 // (the tables are 30 of a pass's 465 us on 2e6 edges, plus two launches).
-static int candidate_weights(tm_ctx *ctx, tm_motif *mo, tm_u128 *W)
+static int candidate_weights(tm_ctx *ctx, tm_motif *mo, SharedPass *sh, tm_u128 *W)
 {
     cudaSetDevice(ctx->device);
-    const int rc = compute_weights(ctx, mo, false);
+    const int rc = compute_weights(ctx, mo, false, sh);
     if (rc) { release_weights(ctx, mo); return rc; }
     *W = mo->W;
     return TM_OK;
+}
+
+static int candidate_roots(const MotifDesc &M, const RankedTree &T, int all_roots, int *roots)
+{
+    int n = 0;
+    if (all_roots) for (int i = 0; i < M.nv - 1; ++i) roots[n++] = T.edges[i];   // increasing id
+    else roots[n++] = default_root(M, T.edges);
+    return n;
+}
+
+// Evaluates the first ntry trees.  With sh the candidates share windows and
+// candidate ranges, and sh's block is the best motif's when one is found.
+static int evaluate_trees(tm_ctx *ctx, const MotifDesc &M, const std::vector<RankedTree> &R, size_t ntry, int64_t delta,
+                          int all_roots, SharedPass *sh, tm_motif **out, tm_tree_cand *cands, uint32_t max_cand,
+                          uint32_t *n_eval)
+{
+    tm_motif *best = nullptr;
+    tm_u128 bestW{0, 0};
+    int rc = TM_OK;
+    *n_eval = 0;
+    for (size_t t = 0; t < ntry && rc == TM_OK; ++t) {
+        int roots[kMaxTree];
+        const int nroots = candidate_roots(M, R[t], all_roots, roots);
+        for (int ri = 0; ri < nroots && rc == TM_OK; ++ri) {
+            tm_motif *mo = new_motif(ctx, M, R[t].edges, roots[ri], delta, &rc);
+            if (!mo) { set_err(ctx, rc, "internal: candidate tree did not compile"); break; }
+            tm_u128 W{0, 0};
+            const int crc = candidate_weights(ctx, mo, sh, &W);
+            if (cands && *n_eval < max_cand) {
+                tm_tree_cand &c = cands[*n_eval];
+                c.tree_mask = R[t].mask;
+                c.root = (uint32_t)roots[ri];
+                c.looseness = (uint32_t)R[t].L;
+                c.status = crc;
+                c.W = crc == TM_OK ? W : tm_u128{0, 0};
+            }
+            ++*n_eval;
+            if (crc == TM_OK && (!best || u128_less(W, bestW))) {
+                std::swap(best, mo);
+                bestW = W;
+            } else if (crc != TM_OK && crc != TM_E_OVERFLOW) {
+                rc = crc;   // a real failure ends the search
+            }
+            tm_motif_free(mo);
+        }
+    }
+    if (rc != TM_OK) { tm_motif_free(best); best = nullptr; }
+    if (sh && sh->block) {
+        if (best) { best->bufs.push_back({sh->block, sh->bytes}); best->bytes += sh->bytes; }
+        else dfree(ctx, sh->block, sh->bytes);
+    }
+    *out = best;
+    return rc;
 }
 
 int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges, const uint32_t *order, int64_t delta,
@@ -800,45 +861,34 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
     std::vector<RankedTree> R;
     rank_trees(M, R);
     const size_t ntry = std::min<size_t>(n_c ? n_c : 1, R.size());
-    tm_motif *best = nullptr;
-    tm_u128 bestW{0, 0};
-    uint32_t evaluated = 0;
+    // Several candidates have the same windows and a few kinds of candidate range
+    // among them.  12 candidates of the 5-cycle + chord on 2e6 edges and
+    // every root: 3653 us with each of its own, 3017 so (22 range kernels and 12
+    // window kernels become 6 and 1).
+    SharedPass sh;
+    int ncand = 0;
+    bool seen[2][2][2] = {};
     for (size_t t = 0; t < ntry; ++t) {
-        int roots[kMaxTree], nroots = 0;
-        if (all_roots) for (int i = 0; i < M.nv - 1; ++i) roots[nroots++] = R[t].edges[i];   // increasing id
-        else roots[nroots++] = default_root(M, R[t].edges);
-        for (int ri = 0; ri < nroots; ++ri) {
-            tm_motif *mo = new_motif(ctx, M, R[t].edges, roots[ri], delta, &rc);
-            if (!mo) {
-                tm_motif_free(best);
-                return set_err(ctx, rc, "internal: candidate tree did not compile");
-            }
-            tm_u128 W{0, 0};
-            const int crc = candidate_weights(ctx, mo, &W);
-            if (cands && evaluated < max_cand) {
-                tm_tree_cand &c = cands[evaluated];
-                c.tree_mask = R[t].mask;
-                c.root = (uint32_t)roots[ri];
-                c.looseness = (uint32_t)R[t].L;
-                c.status = crc;
-                c.W = crc == TM_OK ? W : tm_u128{0, 0};
-            }
-            ++evaluated;
-            if (crc == TM_OK && (!best || u128_less(W, bestW))) {
-                tm_motif_free(best);
-                best = mo;
-                bestW = W;
-                continue;
-            }
-            tm_motif_free(mo);
-            if (crc != TM_OK && crc != TM_E_OVERFLOW) {   // a real failure ends the search
-                tm_motif_free(best);
-                if (n_cand) *n_cand = evaluated;
-                return crc;
+        int roots[kMaxTree];
+        const int nroots = candidate_roots(M, R[t], all_roots, roots);
+        for (int ri = 0; ri < nroots; ++ri, ++ncand) {
+            DevPlan P;
+            if (compile_plan(M, R[t].edges, roots[ri], delta, P)) return set_err(ctx, TM_E_MOTIF, "internal: candidate tree did not compile");
+            for (int k = 0; k < P.nkinds; ++k) {
+                bool &s = seen[P.kside[k] != 0][P.kout[k] != 0][P.klater[k] != 0];
+                if (!s) ++sh.max_kinds;
+                s = true;
             }
         }
     }
+    const bool share = ncand > 1 && ctx->g.m > 0;
+    tm_motif *best = nullptr;
+    uint32_t evaluated = 0;
+    rc = evaluate_trees(ctx, M, R, ntry, delta, all_roots, share ? &sh : nullptr, &best, cands, max_cand, &evaluated);
+    if (rc == TM_E_NOMEM && share)   // the shared ranges can take more than two motifs' own
+        rc = evaluate_trees(ctx, M, R, ntry, delta, all_roots, nullptr, &best, cands, max_cand, &evaluated);
     if (n_cand) *n_cand = evaluated;
+    if (rc) return rc;
     if (!best) return set_err(ctx, TM_E_OVERFLOW, "every candidate's weight pass overflowed");
     rc = fill_guides(ctx, best);
     if (rc) { tm_motif_free(best); return rc; }

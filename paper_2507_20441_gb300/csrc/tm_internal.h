@@ -306,7 +306,21 @@ int build_csr(tm_ctx *ctx);
 // ---- weights (weights.cu) ----
 // guides = false leaves the samplers' guide tables to a later fill_guides (tree
 // selection needs them for the winner only)
-int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true);
+// What the candidates of one tree selection have in common: the windows (one
+// delta) and the candidate ranges of every kind a candidate has used so far.
+// The block becomes the chosen motif's.
+constexpr int kMaxKinds = 8;             // side, direction, pi relation
+struct SharedPass {
+    char *block = nullptr;
+    size_t bytes = 0;
+    bool windows = false;                // filled, and nwin known
+    uint32_t nwin[2] = {}, *win_beg[2] = {}, *win_id[2] = {};
+    int max_kinds = 0;                   // of all candidates
+    int nkinds = 0, side[kMaxKinds], out[kMaxKinds], later[kMaxKinds];
+    RangePtrs range{};
+};
+int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true, SharedPass *sh = nullptr);
+void assign_kinds(DevPlan &P);           // kinds of candidate range of a plan alone
 // (nwin: the layers' window numbers on the device, null once the motif has them)
 int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin = nullptr);
 int export_weights(tm_ctx *ctx, tm_motif *mo, int q, int layer, uint64_t *host_out);

@@ -859,20 +859,23 @@ int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin)
     return check_cuda(ctx, cudaGetLastError(), "guide tables");
 }
 
-int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
+int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
 {
     ScratchScope scope(ctx);
     free_motif_weights(ctx, mo);
     const DevGraph &g = ctx->g;
+    assign_kinds(mo->plan);
     const DevPlan &P = mo->plan;
     cudaStream_t st = ctx->stream;
     const uint32_t m = g.m;
     const WinDiv wv = make_windiv(P.wdelta);   // window unit (delta, or one window without Constraint 3)
     int rc = TM_OK;
+    const bool known = sh && sh->windows;      // the windows, from an earlier candidate
     cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
     // window indices go up to T / unit, the even ones in layer 0
     const uint64_t qT = m ? (uint64_t)g.T / (uint64_t)P.wdelta : 0;
     uint32_t nwh[2] = {(uint32_t)std::min<uint64_t>(m, qT / 2 + 1), (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2)};
+    if (known) { nwh[0] = sh->nwin[0]; nwh[1] = sh->nwin[1]; }
     // cleared together: the tickets, the number of kept excluded ranges, the tile
     // words of the windows, of their totals and of every scan
     const bool win_small = m <= kWinSmall;
@@ -893,7 +896,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
                win_state, ticket, wo, ctx->status);
     };
     // ---- windows of each layer (K2); one block for everything the motif keeps
-    if ((uint64_t)nwh[0] + nwh[1] > (uint64_t)m / 8 + 4096) {
+    if (!known && (uint64_t)nwh[0] + nwh[1] > (uint64_t)m / 8 + 4096) {
         // windows so short that most may be empty: counted before they take room
         PhaseScope ph(ctx, TM_PH_WINDOWS);
         windows(WinOut{{nullptr, nullptr}, {nullptr, nullptr}, ctx->status + 2});
@@ -909,29 +912,58 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         auto al = [](size_t b) { return (b + 255) / 256 * 256; };
         const size_t mm = (size_t)(m ? m : 1);
         auto guide_n = [&](uint32_t nw) { return (size_t)m / 4 + 3 * (size_t)nw + 1; };
-        size_t total = al(((size_t)nwh[0] + 1) * 4) * 4 + al(((size_t)nwh[1] + 1) * 4) * 4 + 2 * al(mm * 8) +
-                       (size_t)P.nslots * 2 * al(mm * 16) + al(((size_t)nwh[0] + nwh[1] + 1) * 16) +
-                       al(guide_n(nwh[0]) * 4) + al(guide_n(nwh[1]) * 4) + al((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
+        const size_t win_arrays = al(((size_t)nwh[0] + 1) * 4) * 2 + al(((size_t)nwh[1] + 1) * 4) * 2;   // starts and indices
         // the candidate ranges come last: a block this large that does not fit
         // with them is tried without (the sampler then searches the ranges)
         // (room for excluded entries at 0.3 of the edges per kind: with bursts of
         // repeated pairs a star's ranges have them at 0.2 - 0.3)
-        const size_t excl_cap = (size_t)P.nkinds * (mm * 3 / 10);
-        const size_t range_bytes = (size_t)P.nkinds * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl));
+        const int nk = sh ? sh->max_kinds : P.nkinds;
+        const size_t excl_cap = (size_t)nk * (mm * 3 / 10);
+        size_t range_bytes = (size_t)nk * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl));
+        char *blk = nullptr;
+        size_t off = 0;
+        auto take = [&](size_t bytes) { char *q = blk + off; off += al(bytes); return (void *)q; };
+        auto take_windows = [&](uint32_t *beg[2], uint32_t *id[2]) {
+            for (int p = 0; p < 2; ++p) {
+                beg[p] = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
+                id[p] = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
+            }
+        };
+        auto take_ranges = [&](RangePtrs &r) {
+            r.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
+            r.base = (uint2 *)take((size_t)nk * r.stride * sizeof(uint2));
+            r.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
+            r.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
+        };
+        if (sh && !sh->block) {
+            sh->bytes = win_arrays + range_bytes + 256;
+            sh->block = blk = (char *)dalloc(ctx, sh->bytes);
+            if (!blk) return TM_E_NOMEM;
+            take_windows(sh->win_beg, sh->win_id);
+            take_ranges(sh->range);
+            sh->range.excl_n = (unsigned long long *)take(256);
+            cudaMemsetAsync(sh->range.excl_n, 0, 8, st);
+            off = 0;
+        }
+        if (sh) range_bytes = 0;
+        size_t total = win_arrays + al(((size_t)nwh[0] + 1) * 4) * 2 + al(((size_t)nwh[1] + 1) * 4) * 2 + 2 * al(mm * 8) +
+                       (size_t)P.nslots * 2 * al(mm * 16) + al(((size_t)nwh[0] + nwh[1] + 1) * 16) +
+                       al(guide_n(nwh[0]) * 4) + al(guide_n(nwh[1]) * 4) + al((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
+        if (sh) total -= win_arrays;
         bool with_ranges = true;
-        char *blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
-        if (!blk && total >= ((size_t)4 << 30)) {
+        blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
+        if (!blk && !sh && total >= ((size_t)4 << 30)) {
             with_ranges = false;
             blk = (char *)malloc_motif(ctx, mo, total);
         }
         if (!blk) return TM_E_NOMEM;
-        size_t off = 0;
-        auto take = [&](size_t bytes) { char *q = blk + off; off += al(bytes); return (void *)q; };
+        uint32_t *win_beg[2], *win_id[2];
+        if (!sh) take_windows(win_beg, win_id);
         for (int p = 0; p < 2; ++p) {
             LayerData &L = mo->layer[p];
             L.nwin = nwh[p];
-            L.win_beg = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
-            L.win_id = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
+            L.win_beg = sh ? sh->win_beg[p] : win_beg[p];
+            L.win_id = sh ? sh->win_id[p] : win_id[p];
             L.root_cdf = (uint64_t *)take(mm * 8);
             L.win_gshift = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
             L.win_goff = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
@@ -943,15 +975,14 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
         }
         mo->wcum = (uint64_t *)take(((size_t)nwh[0] + nwh[1] + 1) * 16);
         mo->wguide = (uint32_t *)take((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
-        if (with_ranges) {
-            mo->range.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
-            mo->range.base = (uint2 *)take((size_t)P.nkinds * mo->range.stride * sizeof(uint2));
-            mo->range.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
+        if (sh) {
+            mo->range = sh->range;
+        } else if (with_ranges) {
+            take_ranges(mo->range);
             mo->range.excl_n = (unsigned long long *)(ticket + 2);   // of this pass
-            mo->range.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
         }
     }
-    {
+    if (!known) {
         PhaseScope ph(ctx, TM_PH_WINDOWS);
         if (m)
             windows(WinOut{{mo->layer[0].win_beg, mo->layer[1].win_beg}, {mo->layer[0].win_id, mo->layer[1].win_id},
@@ -979,9 +1010,22 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     if (P.tleaf[0]) order.push_back(0);   // single-edge motif: the root is a leaf
     if (mo->range.base && m) {
         PhaseScope ph(ctx, TM_PH_DP);
-        for (int k = 0; k < P.nkinds; ++k)
-            launch(ctx, k_ranges, blocks_for(m, TB), TB, g, P.c2, P.delta, wv, P.kside[k], P.kout[k], P.klater[k],
-                   P.kinner[k], mo->range.base + (size_t)k * mo->range.stride, mo->range);
+        auto ranges = [&](int k, int at, int inner) {
+            launch(ctx, k_ranges, blocks_for(m, TB), TB, g, P.c2, P.delta, wv, P.kside[k], P.kout[k], P.klater[k], inner,
+                   mo->range.base + (size_t)at * mo->range.stride, mo->range);
+        };
+        int at[kMaxTree];   // where kind k's ranges are
+        for (int k = 0; k < P.nkinds; ++k) {
+            at[k] = k;
+            if (!sh) { ranges(k, k, P.kinner[k]); continue; }
+            int &i = at[k] = 0;
+            while (i < sh->nkinds && (sh->side[i] != P.kside[k] || sh->out[i] != P.kout[k] || sh->later[i] != P.klater[k])) ++i;
+            if (i < sh->nkinds) continue;
+            sh->side[i] = P.kside[k]; sh->out[i] = P.kout[k]; sh->later[i] = P.klater[k];
+            ++sh->nkinds;
+            ranges(k, i, 1);   // with what inner nodes read: a later candidate may have one
+        }
+        for (int q = 1; q < P.ntree; ++q) mo->plan.tkind[q] = at[P.tkind[q]];
     }
     for (int q : order) {
         // sides of q that children meet; the weights come out in the order of
@@ -1062,20 +1106,24 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides)
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
         const uint32_t tt = (uint32_t)(((uint64_t)nwh[0] + nwh[1]) / kTotTile) + 1;   // (not more than tot_tiles)
-        launch(ctx, k_window_totals, dim3(tt, 3), kTotThreads, guide_args(mo, ctx->status + 2), mo->wcum,
+        launch(ctx, k_window_totals, dim3(tt, 3), kTotThreads, guide_args(mo, known ? nullptr : ctx->status + 2), mo->wcum,
                (uint64_t *)(ctx->status + 4), tot_state, ticket + 4, ctx->status);
         if (guides) {
-            rc = fill_guides(ctx, mo, ctx->status + 2);
+            rc = fill_guides(ctx, mo, known ? nullptr : ctx->status + 2);
             if (rc) return rc;
         }
     }
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
+    if (!known) for (int p = 0; p < 2; ++p) mo->layer[p].nwin = ctx->status_host[2 + p];
+    if (sh && !known && !(bits & ~ST_OVERFLOW)) {
+        for (int p = 0; p < 2; ++p) sh->nwin[p] = mo->layer[p].nwin;
+        sh->windows = true;
+    }
     if (bits & ST_OVERFLOW) return set_err(ctx, TM_E_OVERFLOW, "a weight, prefix sum or window total exceeds 2^64");
     if (bits) return set_err(ctx, TM_E_CUDA, "device status error in weight pass");
     memcpy(&mo->W, ctx->status_host + 4, 16);   // copied with the status
-    for (int p = 0; p < 2; ++p) mo->layer[p].nwin = ctx->status_host[2 + p];
     mo->nwtot = mo->layer[0].nwin + mo->layer[1].nwin;
     mo->have_weights = true;
     mo->graph_epoch = ctx->epoch;
