@@ -132,9 +132,8 @@ def measured_peaks():
 KERNEL_SOURCES = {
     "k_sample": ["sampler.cu", "tm_device.cuh", "tm_internal.h"],
     "k_dp": ["weights.cu", "tm_device.cuh", "tm_internal.h"],
-    "k_gather2_pair": ["csr.cu", "tm_internal.h"],
-    "k_gather2": ["csr.cu", "tm_internal.h"],
-    "k_rs_scatter": ["csr.cu", "tm_internal.h"],
+    "k_ranges": ["weights.cu", "tm_device.cuh", "tm_internal.h"],
+    "k_rs_sweep": ["csr.cu", "tm_internal.h"],
     "k_segscan2": ["scan.cuh", "weights.cu", "tm_device.cuh", "tm_internal.h"],
 }
 
@@ -174,19 +173,10 @@ def profiled_traffic(kernel, workload):
 # ------------------------------------------------ algorithmic byte models ----
 def dp_bytes_per_edge(plan_children):
     """Bytes one weight-DP launch must move per edge for a tree node with the
-    given children (list of leaf flags), both layers: the edge record (t,
-    src, dst, pair) and the reverse-pair id, read once; per layer and child
-    the two list bounds (2 x 4 B offsets) and, for a non-leaf child, the four
-    prefix values that bound the candidate range and its exclusion (4 x 8 B);
-    per layer the 8 B weight written."""
-    b = 16 + 4
-    for _ in range(2):
-        for leaf in plan_children:
-            b += 8
-            if not leaf:
-                b += 32
-        b += 8
-    return b
+    given children (list of leaf flags), both layers: per child the 8 B range
+    record and, for a non-leaf child, the two 16 B prefix pairs that bound the
+    range; the 16 B weight pair written."""
+    return 16 + sum(8 if leaf else 8 + 32 for leaf in plan_children)
 
 
 def tree_children(order, parent):
@@ -233,19 +223,19 @@ def sampler_bytes_per_sample(ntree, nontree, stats, nwin):
     """The per-sample effective-bytes model of the sampler, every probe of
     every search counted at 8 B: the window search over the window totals
     (16 B entries) and the root search over the root CDF, 16 B for the root
-    edge record; per non-root tree edge a 16 B record and five searches of the
-    meeting vertex's list (two window bounds, two exclusion bounds, the
-    inverse-CDF pick); per non-tree edge one search of its multi-edge list."""
+    edge record; per non-root tree edge a 16 B record, the 8 B range record and
+    the inverse-CDF pick in the meeting vertex's list; per non-tree edge one
+    search of its multi-edge list."""
     import math
     lg = lambda x: max(1, math.ceil(math.log2(max(x, 2.0))))
     b = lg(nwin) * 16 + lg(2 * stats["m"]) * 8 + 16
-    b += (ntree - 1) * (16 + lg(stats["list_len"]) * 8 * 5)
+    b += (ntree - 1) * (16 + 8 + lg(stats["list_len"]) * 8)
     b += nontree * lg(stats["pair_len"]) * 8
     return b
 
 
 def kernel_family(name):
-    for fam in ("k_sample", "k_dp", "k_gather2_pair", "k_gather2", "k_rs_scatter", "k_segscan2"):
+    for fam in ("k_sample", "k_dp", "k_ranges", "k_rs_sweep", "k_segscan2"):
         if name.startswith(fam):
             return fam
     return name.split("<")[0]
@@ -260,11 +250,12 @@ def kernel_model(name, launches_per_step, ctx_m, k, children, per_sample):
     if fam == "k_dp":
         per_step = sum(ctx_m * dp_bytes_per_edge([not children[c] for c in ch]) for ch in children.values() if ch)
         return per_step / max(launches_per_step, 1), \
-            "streamed edge record, list bounds, prefix reads and weight writes per edge (averaged over the DP launches)"
-    if fam == "k_gather2_pair":
-        return 40 * ctx_m, "two sets x (4 B index + two 4 B gathered reads + two 4 B writes) per edge"
-    if fam == "k_gather2":
-        return 20 * ctx_m, "4 B index + two 4 B gathered reads + two 4 B writes per edge"
+            "range record, prefix bounds and weight pair per edge (averaged over the DP launches)"
+    if fam == "k_ranges":
+        return 20 * ctx_m, "time, vertex and cross rank read, 8 B record written per edge"
+    if fam == "k_rs_sweep":
+        np_ = int(name.split("<")[1].split(",")[0])
+        return 8 * (1 + np_) * ctx_m, "key and payloads read and written once per edge"
     return None, None
 
 
