@@ -86,6 +86,7 @@ __device__ __forceinline__ void hist_flush(const uint32_t *__restrict__ h, int n
 __global__ void __launch_bounds__(OS_THREADS) k_rs_hist(const uint32_t *__restrict__ key, uint32_t n, DigitPlan D,
                                                         uint32_t *__restrict__ hist)
 {
+    grid_wait();
     __shared__ uint32_t h[OS_HIST];
     for (int i = threadIdx.x; i < OS_HIST; i += OS_THREADS) h[i] = 0;
     __syncthreads();
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
     k_rs_sweep(RsSet J, uint32_t n, int shift, int bits, const uint32_t *__restrict__ hist,
                unsigned long long *__restrict__ state, uint32_t *__restrict__ ticket, uint32_t *status)
 {
+    grid_wait();
     constexpr int TILE = OS_THREADS * ITEMS, WCHUNK = ITEMS * 32;
     static_assert(ITEMS % 2 == 0, "slots are kept two to a register");
     __shared__ uint32_t s_buf[TILE];                          // one array of the tile
@@ -323,6 +325,7 @@ __device__ __forceinline__ void os_block_scan512(uint32_t *vals /* smem [512] in
 constexpr int IB_MAXB = 512;
 __global__ void k_inv_cursor(uint32_t *__restrict__ cursor, uint32_t nb, int shift)
 {
+    grid_wait();
     const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b < nb) cursor[b] = b << shift;
 }
@@ -331,6 +334,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__
                                                                uint32_t nb, uint32_t *__restrict__ cursor,
                                                                uint32_t *__restrict__ tkey, uint32_t *__restrict__ tpos)
 {
+    grid_wait();
     __shared__ uint32_t s_cnt[IB_MAXB], s_base[IB_MAXB], s_wt[OS_WARPS];
     __shared__ uint32_t s_key[OS_TILE], s_pos[OS_TILE];
     const int t = threadIdx.x;
@@ -384,6 +388,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__
 __global__ void k_inv_fill(const uint32_t *__restrict__ tkey, const uint32_t *__restrict__ tpos, uint32_t n,
                            uint32_t *__restrict__ inv)
 {
+    grid_wait();
     const uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x * TM_INV_VECS + threadIdx.x;
     uint4 k[TM_INV_VECS], p[TM_INV_VECS];
 #pragma unroll
@@ -465,6 +470,7 @@ struct RsTo {
 
 __global__ void k_iota(uint32_t *__restrict__ a, uint32_t m)
 {
+    grid_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) a[i] = i;
 }
@@ -564,6 +570,7 @@ struct Stats {
 __global__ void k_input_stats(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst,
                               const int64_t *__restrict__ t, uint64_t m, uint32_t n, Stats *st)
 {
+    grid_wait();
     long long lo = LLONG_MAX, hi = LLONG_MIN;
     unsigned long long ns = 0, nb = 0;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -613,6 +620,7 @@ constexpr int kElemItems = TM_ELEM_ITEMS;
 __global__ void k_keep_nonself(const uint32_t *__restrict__ src, const uint32_t *__restrict__ dst, uint64_t m,
                                uint32_t *__restrict__ keep)
 {
+    grid_wait();
     uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) keep[i] = src[i] != dst[i] ? 1u : 0u;
 }
@@ -627,6 +635,7 @@ __global__ void __launch_bounds__(OS_THREADS)
                     uint32_t *__restrict__ ot, uint32_t *__restrict__ os, uint32_t *__restrict__ od, DigitPlan Dt,
                     DigitPlan Dv, uint32_t *__restrict__ hist)
 {
+    grid_wait();
     __shared__ uint32_t h[3 * OS_HIST];
     for (int i = threadIdx.x; i < 3 * OS_HIST; i += OS_THREADS) h[i] = 0;
     __syncthreads();
@@ -720,6 +729,7 @@ __global__ void k_order_runs(const uint32_t *__restrict__ t, uint32_t *__restric
                              uint32_t m, uint32_t *__restrict__ too_long, uint2 *__restrict__ long_runs,
                              uint32_t *__restrict__ n_long, unsigned long long *__restrict__ ndup)
 {
+    grid_wait();
     const uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
 #pragma unroll
     for (int k = 0; k < kElemItems; ++k) {
@@ -737,6 +747,7 @@ __global__ void __launch_bounds__(256) k_order_long_runs(uint32_t *__restrict__ 
                                                          const uint32_t *__restrict__ n_long,
                                                          unsigned long long *__restrict__ ndup)
 {
+    grid_wait();
     __shared__ uint64_t key[kBlockRunMax];
     const uint32_t nl = *n_long;
     for (uint32_t r = blockIdx.x; r < nl; r += gridDim.x) {
@@ -773,6 +784,7 @@ __global__ void k_flag_unique(const uint32_t *__restrict__ t, const uint32_t *__
                               const uint32_t *__restrict__ d, uint32_t m, uint32_t *__restrict__ keep,
                               unsigned long long *ndup)
 {
+    grid_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     bool dup = i > 0 && t[i] == t[i - 1] && s[i] == s[i - 1] && d[i] == d[i - 1];
@@ -785,6 +797,7 @@ __global__ void k_compact3(const uint32_t *__restrict__ a, const uint32_t *__res
                            const uint32_t *__restrict__ pos, uint32_t *__restrict__ oa, uint32_t *__restrict__ ob,
                            uint32_t *__restrict__ oc)
 {
+    grid_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m || !keep[i]) return;
     uint32_t p = pos[i];
@@ -811,6 +824,7 @@ __global__ void k_owners(const uint32_t *__restrict__ out_src, const uint32_t *_
                          uint32_t *__restrict__ own_out, uint32_t *__restrict__ own_in,
                          const uint32_t *__restrict__ status)
 {
+    grid_wait();
     if (*status & ST_TIMEOUT) return;   // a sort whose wait ran out: its keys are anything
     const int lane = threadIdx.x & 31;
     const uint64_t x0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
@@ -860,6 +874,7 @@ __global__ void __launch_bounds__(256) k_pairs(const uint32_t *__restrict__ msrc
                                                uint32_t *__restrict__ own_multi, uint32_t *__restrict__ npairs,
                                                uint32_t *status)
 {
+    grid_wait();
     __shared__ uint32_t s_w[8], s_tile, s_before, s_h[8][ROWS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0)   // a sort whose wait ran out: its keys are anything
@@ -974,6 +989,7 @@ struct XR {
 template <int kXrItems>
 __global__ void __launch_bounds__(256) k_cross_rank(XR a, XR b, uint32_t m, uint32_t n)
 {
+    grid_wait();
     const bool s1 = blockIdx.y != 0;
     const uint32_t *__restrict__ own_t = s1 ? b.own_t : a.own_t, *__restrict__ owner = s1 ? b.owner : a.owner;
     const uint32_t *__restrict__ other_off = s1 ? b.other_off : a.other_off, *__restrict__ other_t = s1 ? b.other_t : a.other_t;

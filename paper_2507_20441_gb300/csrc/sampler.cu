@@ -633,6 +633,7 @@ __global__ void __launch_bounds__(kSampleThreads, kTraceMinB) k_sample(DevGraph 
                                                               Acc *acc, uint32_t *status, uint32_t *tr_gid,
                                                               uint64_t *tr_contrib, int32_t *tr_reason)
 {
+    grid_wait();
     __shared__ DevPlan sp;
 #if TM_RECS_SMEM
     __shared__ uint32_t recs[kRecRows * kSampleThreads];
@@ -670,6 +671,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB) k_sample_reg(D
                                                               SampleJob J, uint64_t seed, uint64_t first, uint64_t k,
                                                               Acc *acc, uint32_t *status)
 {
+    grid_wait();
     __shared__ DevPlan sp;
     {
         const int *src = reinterpret_cast<const int *>(&plan);
@@ -759,6 +761,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
     k_list_count(DevGraph g, const DevPlan *__restrict__ plan, SampleJob J, uint64_t seed, uint64_t first, uint64_t k,
                  uint64_t *__restrict__ cnt_out, uint32_t *status)
 {
+    grid_wait();
     __shared__ DevPlan sp;
     {
         const int *src = reinterpret_cast<const int *>(plan);
@@ -814,6 +817,7 @@ __device__ __forceinline__ uint64_t list_block_scan(uint64_t v, uint64_t &total,
 __global__ void __launch_bounds__(kSampleThreads) k_list_sums(const uint64_t *__restrict__ cnt, uint64_t k,
                                                               uint64_t *__restrict__ sums, uint32_t *status)
 {
+    grid_wait();
     const uint64_t i0 = (uint64_t)blockIdx.x * kListTile + (uint64_t)threadIdx.x * kListItems;
     uint64_t s = 0, total;
     bool ovf = false;
@@ -827,6 +831,7 @@ __global__ void __launch_bounds__(kSampleThreads) k_list_sums(const uint64_t *__
 __global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums, uint64_t n, uint64_t *__restrict__ end,
                                                     uint64_t *__restrict__ total, uint32_t *status)
 {
+    grid_wait();
     uint64_t carry = 0;
     bool ovf = false;
     for (uint64_t b = 0; b < n; b += blockDim.x) {
@@ -843,6 +848,7 @@ __global__ void __launch_bounds__(1024) k_list_scan(uint64_t *__restrict__ sums,
 __global__ void __launch_bounds__(kSampleThreads) k_list_offsets(uint64_t *__restrict__ cnt, uint64_t k,
                                                                  const uint64_t *__restrict__ sums)
 {
+    grid_wait();
     const uint64_t i0 = (uint64_t)blockIdx.x * kListTile + (uint64_t)threadIdx.x * kListItems;
     uint64_t v[kListItems], s = 0, total;
     bool ovf = false;   // a wrap was latched by the sums
@@ -864,6 +870,7 @@ __global__ void __launch_bounds__(kSampleThreads, TM_SAMPLE_MINB)
                 const uint64_t *__restrict__ offs, uint64_t max_inst, uint32_t *__restrict__ inst_gids,
                 uint64_t *__restrict__ inst_sample, uint32_t *status)
 {
+    grid_wait();
     __shared__ DevPlan sp;
     {
         const int *src = reinterpret_cast<const int *>(plan);
@@ -903,6 +910,7 @@ __global__ void __launch_bounds__(kSampleThreads, kGroupMinB)
     k_sample_group(DevGraph g, const DevPlan *__restrict__ plans, SampleJob J, uint64_t seed, uint64_t first,
                    uint64_t k, Acc *acc, uint32_t *status)
 {
+    grid_wait();
     __shared__ DevPlan sp[NM];
     {
         const int *src = reinterpret_cast<const int *>(plans);
@@ -981,6 +989,7 @@ __global__ void __launch_bounds__(THREADS, kBatchThreads / THREADS) k_batch(DevG
                                                   const uint32_t *__restrict__ tile_base, uint32_t nq, uint32_t tile,
                                                   uint32_t *counter, Acc *accs, uint32_t *status)
 {
+    grid_wait();
     __shared__ BatchQuery sq;
     __shared__ uint32_t s_item;
     __shared__ int s_q;

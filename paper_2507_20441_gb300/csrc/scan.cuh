@@ -23,6 +23,7 @@ constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 // ---------------------------------------------------------------- u32 ----
 __global__ void k_tile_sum_u32(const uint32_t *__restrict__ in, uint64_t n, uint32_t *__restrict__ tile_sum)
 {
+    grid_wait();
     __shared__ uint32_t warp_sum[SCAN_THREADS / 32];
     uint64_t base = (uint64_t)blockIdx.x * SCAN_TILE;
     uint32_t s = 0;
@@ -51,6 +52,7 @@ __global__ void k_tile_scan_u32(const uint32_t *__restrict__ in, uint64_t n, con
                                 uint32_t *__restrict__ out, uint32_t *__restrict__ total,
                                 const uint32_t *__restrict__ tile_sums = nullptr)
 {
+    grid_wait();
     __shared__ uint32_t warp_tot[SCAN_THREADS / 32];
     __shared__ uint32_t s_carry;
     if (tile_sums) {
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(SCAN_THREADS, TM_SCAN_MINB) k_segscan2_onepass
                                                                    uint64_t *__restrict__ out1,
                                                                    ulonglong2 *__restrict__ outp, uint32_t *status)
 {
+    grid_wait();
     __shared__ SegAgg2 warp_agg[SCAN_THREADS / 32];
     __shared__ uint32_t s_tile;
     if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1u);

@@ -390,6 +390,33 @@ struct KernelTimer {
     ~KernelTimer();
 };
 
+#ifdef __CUDACC__
+// A kernel is set up while the one before it on the stream ends, which saves a
+// microsecond or more of each gap between two: an estimate on 2e4 edges (about 38
+// launches) 309 -> 264 us, on 2e6 1007 -> 951, a selection of 12 candidates 3030
+// -> 2854.  EVERY kernel begins with grid_wait, before any other statement: it
+// returns when the kernels before it have ended and what they wrote is seen.
+// (Letting the next kernel's blocks in as soon as this one's last block has
+// started gained 0 - 0.7 % more, and was left out.)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... KArgs>
+inline void launch_early(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, KArgs... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = &at;
+    c.numAttrs = stream == cudaStreamLegacy ? 0 : 1;
+    cudaLaunchKernelEx(&c, kernel, args...);
+}
+#endif
+
 // Every kernel of the library is launched through here (counted per context,
 // timed per kernel when cfg.profile >= 2).
 #ifdef __CUDACC__
@@ -398,7 +425,7 @@ inline void launch(tm_ctx *ctx, void (*kernel)(KArgs...), dim3 grid, dim3 block,
 {
     ++ctx->kernel_launches;
     KernelTimer kt(ctx, (const void *)kernel);
-    kernel<<<grid, block, 0, ctx->stream>>>(static_cast<KArgs>(args)...);
+    launch_early(kernel, grid, block, 0, ctx->stream, static_cast<KArgs>(args)...);
 }
 // The same with dynamic shared memory.
 template <typename... KArgs, typename... Args>
@@ -406,7 +433,7 @@ inline void launch_smem(tm_ctx *ctx, void (*kernel)(KArgs...), dim3 grid, dim3 b
 {
     ++ctx->kernel_launches;
     KernelTimer kt(ctx, (const void *)kernel);
-    kernel<<<grid, block, smem, ctx->stream>>>(static_cast<KArgs>(args)...);
+    launch_early(kernel, grid, block, smem, ctx->stream, static_cast<KArgs>(args)...);
 }
 #endif
 void prof_collect(tm_ctx *ctx);   // call after the stream is synchronized

@@ -62,6 +62,7 @@ constexpr int kScanStep = 8;          // independent loads per step (4 and 16 me
 __global__ void __launch_bounds__(256, 8) k_ranges(DevGraph g, int c2, int64_t delta, WinDiv wv, int side, int out,
                                                    int later, int inner, uint2 *__restrict__ rec, RangePtrs R)
 {
+    grid_wait();
     const uint32_t pos = blockIdx.x * blockDim.x + threadIdx.x;
     if (pos >= g.m) return;
     const uint32_t t = __ldg((side ? g.in_t : g.out_t) + pos);
@@ -236,6 +237,7 @@ __global__ void __launch_bounds__(256, LEAF ? 4 : 5)
          uint32_t *__restrict__ nz, const ulonglong2 *__restrict__ in, const uint32_t *__restrict__ in_nz,
          const uint32_t *__restrict__ pin, uint32_t *__restrict__ pout, uint32_t *status)
 {
+    grid_wait();
     const uint64_t pos0 = (uint64_t)blockIdx.x * (256 * K) + threadIdx.x;
     auto at = [&](int k) { return (uint32_t)(pos0 + k * 256); };
     auto live = [&](int k) { return pos0 + k * 256 < g.m; };
@@ -474,6 +476,7 @@ __global__ void __launch_bounds__(256) k_windows(const uint32_t *__restrict__ t,
                                                  unsigned long long *__restrict__ state, uint32_t *__restrict__ ticket,
                                                  WinOut W, uint32_t *status)
 {
+    grid_wait();
     __shared__ uint32_t s_h[2][8][ROWS], s_w[2][8], s_tile;
     __shared__ unsigned long long s_before;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -592,6 +595,7 @@ __global__ void __launch_bounds__(kTotThreads) k_window_totals(GuideArgs A, uint
                                                                SegTile *__restrict__ tiles, uint32_t *__restrict__ ticket,
                                                                uint32_t *status)
 {
+    grid_wait();
     constexpr int kWarps = kTotThreads / 32;
     __shared__ u128 s_tot[kWarps];
     __shared__ u128 s_before;
@@ -736,6 +740,7 @@ constexpr int kGuideItems = TM_GUIDE_ITEMS;
 __global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m, const uint64_t *__restrict__ wcum,
                                                    uint32_t *__restrict__ wguide)
 {
+    grid_wait();
     const int p = blockIdx.y;
     if (p == 2) {
         const uint32_t nw = A.windows(0) + A.windows(1);
@@ -801,6 +806,7 @@ template <class F>
 __global__ void k_unprefix(F f, const uint64_t *__restrict__ pref, int stride, const uint32_t *__restrict__ perm,
                            uint32_t m, uint64_t *__restrict__ out)
 {
+    grid_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= m) return;
     uint64_t w = pref[(size_t)i * stride] - (f.head(i) ? 0 : pref[(size_t)(i - 1) * stride]);
@@ -809,6 +815,7 @@ __global__ void k_unprefix(F f, const uint64_t *__restrict__ pref, int stride, c
 
 __global__ void k_leaf_weights(const uint32_t *__restrict__ t, uint32_t m, int p, WinDiv wv, uint64_t *__restrict__ out)
 {
+    grid_wait();
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < m) out[i] = wv.win(t[i], p) >= 0 ? 1 : 0;
 }
