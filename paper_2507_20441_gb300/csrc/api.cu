@@ -890,6 +890,7 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
     if (n_cand) *n_cand = evaluated;
     if (rc) return rc;
     if (!best) return set_err(ctx, TM_E_OVERFLOW, "every candidate's weight pass overflowed");
+    cudaMemsetAsync(ctx->status, 0, kStatusBytes, ctx->stream);   // (bits of a candidate that overflowed after the winner)
     rc = fill_guides(ctx, best);
     if (rc) { tm_motif_free(best); return rc; }
     *out = best;

@@ -321,7 +321,8 @@ struct SharedPass {
 };
 int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true, SharedPass *sh = nullptr);
 void assign_kinds(DevPlan &P);           // kinds of candidate range of a plan alone
-// (nwin: the layers' window numbers on the device, null once the motif has them)
+// (nwin: the layers' window numbers on the device, null once the motif has them;
+// nothing is filled when the status block holds a bit)
 int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin = nullptr);
 int export_weights(tm_ctx *ctx, tm_motif *mo, int q, int layer, uint64_t *host_out);
 

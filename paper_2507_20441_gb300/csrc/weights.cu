@@ -732,17 +732,21 @@ __device__ void wguide_entry(const uint64_t *__restrict__ wcum, uint32_t nw, uin
 // window of its first edge by a binary search over the window starts, and a
 // lane steps to the next window as its edges cross one, so a window of any
 // size is spread over many threads.  blockIdx.y = 2: the window pick's guide,
-// a bucket per thread.
+// a bucket per thread.  A pass that has latched anything by now fills nothing:
+// sums that wrapped 2^64 do not rise along a window, so their buckets need not
+// lie in the room that the window's last sum was given.
 #ifndef TM_GUIDE_ITEMS
 #define TM_GUIDE_ITEMS 32   // measured: 32 edges per lane beat 8 (1.77 against 1.81 ms for the root phase) and 2
 #endif
 constexpr int kGuideItems = TM_GUIDE_ITEMS;
 __global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m, const uint64_t *__restrict__ wcum,
-                                                   uint32_t *__restrict__ wguide)
+                                                   uint32_t *__restrict__ wguide, const uint32_t *status)
 {
     grid_wait();
+    const uint32_t bits = latched(status);   // (asked below, once the window is found)
     const int p = blockIdx.y;
     if (p == 2) {
+        if (bits) return;
         const uint32_t nw = A.windows(0) + A.windows(1);
         if (nw == 0) return;
         for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= 4 * (uint64_t)nw;
@@ -769,6 +773,7 @@ __global__ void __launch_bounds__(TB) k_guide_fill(GuideArgs A, uint32_t m, cons
         const uint32_t mid = (lo + hi) >> 1;
         if (win_beg[mid] <= x0) lo = mid + 1; else hi = mid;
     }
+    if (bits) return;
     int64_t kk = (int64_t)lo - 1;
     const uint64_t xe = min((uint64_t)m, (uint64_t)(xs + 32u * kGuideItems));
     // kGuideBatch edges' CDF pairs loaded before any is used (independent
@@ -862,7 +867,7 @@ int fill_guides(tm_ctx *ctx, tm_motif *mo, const uint32_t *nwin)
     if (m == 0) return TM_OK;
     const uint64_t gwarps = (m + 32 * kGuideItems - 1) / (32 * kGuideItems);
     launch(ctx, k_guide_fill, dim3(blocks_for(gwarps * 32, TB), 3), TB, guide_args(mo, nwin), (uint32_t)m,
-           (const uint64_t *)mo->wcum, mo->wguide);
+           (const uint64_t *)mo->wcum, mo->wguide, (const uint32_t *)ctx->status);
     return check_cuda(ctx, cudaGetLastError(), "guide tables");
 }
 
