@@ -111,7 +111,10 @@ constexpr int kLookback = 4;   // tiles read at a time when looking back (2 meas
 
 // One pass.  Tiles are taken from a counter, so every tile before this one has
 // been started and publishes its counts without waiting for anyone; waits for
-// them are bounded all the same (ST_TIMEOUT).  A warp ranks 32 keys at a time:
+// them are bounded all the same (ST_TIMEOUT).  After a wait that ran out the
+// pass's output has holes, and its keys no longer match the digit counts that
+// place them: from then on tiles publish an empty prefix and write nothing, in
+// this pass and in every later one.  A warp ranks 32 keys at a time:
 // each lane marks its bit in its digit's word of shared memory and reads the
 // word back, which gives the peers before it (a ballot per digit bit, which
 // this replaces, was most of the pass's instructions).  The tile is staged
@@ -136,12 +139,17 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
     __shared__ uint16_t s_wcnt[OS_WARPS * OS_MAXRADIX];       // [warp][digit] counts, then tile slots
     __shared__ uint32_t s_gpos[OS_MAXRADIX];                  // digit start in the output - in the tile
     __shared__ uint32_t s_wt[8];
-    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_tile, s_stop;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) s_tile = atomicAdd(ticket, 1u);
+    if (t == 32) s_stop = latched(status) & ST_TIMEOUT;   // (both on their way together)
     for (int i = t; i < OS_WARPS * OS_MAXRADIX; i += OS_THREADS) { s_wcnt[i] = 0; s_match[i] = 0; }
     __syncthreads();
     const uint32_t tile = s_tile;
+    if (s_stop) {
+        if (t < OS_MAXRADIX) *(volatile unsigned long long *)(state + (size_t)tile * OS_MAXRADIX + t) = kTilePrefix;
+        return;
+    }
     const uint32_t radix = 1u << bits, dmask = radix - 1u;
     const uint32_t base = tile * (uint32_t)TILE;
     const uint32_t tile_n = min((uint32_t)TILE, n - base);
@@ -330,11 +338,14 @@ __global__ void k_inv_cursor(uint32_t *__restrict__ cursor, uint32_t nb, int shi
     if (b < nb) cursor[b] = b << shift;
 }
 
+// (perm is no permutation when a wait of its sort ran out: nothing is written then)
 __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__restrict__ perm, uint32_t n, int shift,
                                                                uint32_t nb, uint32_t *__restrict__ cursor,
-                                                               uint32_t *__restrict__ tkey, uint32_t *__restrict__ tpos)
+                                                               uint32_t *__restrict__ tkey, uint32_t *__restrict__ tpos,
+                                                               const uint32_t *status)
 {
     grid_wait();
+    const uint32_t stop = latched(status) & ST_TIMEOUT;
     __shared__ uint32_t s_cnt[IB_MAXB], s_base[IB_MAXB], s_wt[OS_WARPS];
     __shared__ uint32_t s_key[OS_TILE], s_pos[OS_TILE];
     const int t = threadIdx.x;
@@ -347,12 +358,12 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__
         const uint32_t i = base + j * OS_THREADS + t;
         v[j] = i < n ? __ldg(perm + i) : 0u;
     }
+    if (stop) return;
     __syncthreads();
     uint32_t r[OS_ITEMS];   // rank inside the tile's bucket (shared atomics: any order)
 #pragma unroll
     for (int j = 0; j < OS_ITEMS; ++j) {
         const uint32_t i = base + j * OS_THREADS + t;
-        v[j] = min(v[j], n - 1);   // (a sort whose wait ran out leaves anything here)
         r[j] = i < n ? atomicAdd(&s_cnt[v[j] >> shift], 1u) : 0u;
     }
     __syncthreads();
@@ -386,9 +397,10 @@ __global__ void __launch_bounds__(OS_THREADS, 4) k_inv_bucket(const uint32_t *__
 #define TM_INV_VECS 1   // 2 and 4 measured no faster
 #endif
 __global__ void k_inv_fill(const uint32_t *__restrict__ tkey, const uint32_t *__restrict__ tpos, uint32_t n,
-                           uint32_t *__restrict__ inv)
+                           uint32_t *__restrict__ inv, const uint32_t *status)
 {
     grid_wait();
+    const uint32_t stop = latched(status) & ST_TIMEOUT;   // the pairs were not written
     const uint64_t v0 = (uint64_t)blockIdx.x * blockDim.x * TM_INV_VECS + threadIdx.x;
     uint4 k[TM_INV_VECS], p[TM_INV_VECS];
 #pragma unroll
@@ -399,6 +411,7 @@ __global__ void k_inv_fill(const uint32_t *__restrict__ tkey, const uint32_t *__
             p[r] = __ldg(reinterpret_cast<const uint4 *>(tpos + i));
         }
     }
+    if (stop) return;
 #pragma unroll
     for (int r = 0; r < TM_INV_VECS; ++r) {
         const uint64_t i = (v0 + (uint64_t)r * blockDim.x) * 4;
@@ -444,9 +457,10 @@ static int inverse_perm(tm_ctx *ctx, const uint32_t *perm, uint32_t n, uint32_t 
     while (((uint64_t)(n - 1) >> shift) >= (uint64_t)IB_MAXB) ++shift;
     const uint32_t nb = (uint32_t)(((uint64_t)(n - 1) >> shift) + 1);
     launch(ctx, k_inv_cursor, 1, IB_MAXB, cursor, nb, shift);
-    launch(ctx, k_inv_bucket, (n + OS_TILE - 1) / OS_TILE, OS_THREADS, perm, n, shift, nb, cursor, tkey, tpos);
+    launch(ctx, k_inv_bucket, (n + OS_TILE - 1) / OS_TILE, OS_THREADS, perm, n, shift, nb, cursor, tkey, tpos,
+           (const uint32_t *)ctx->status);
     launch(ctx, k_inv_fill, (unsigned)(((uint64_t)n + 1024 * TM_INV_VECS - 1) / (1024 * TM_INV_VECS)), 256,
-           (const uint32_t *)tkey, (const uint32_t *)tpos, n, inv);
+           (const uint32_t *)tkey, (const uint32_t *)tpos, n, inv, (const uint32_t *)ctx->status);
     return check_cuda(ctx, cudaGetLastError(), "inverse permutation");
 }
 // Up to here the last pass writes the inverse itself, a random 4-byte store per
@@ -825,7 +839,7 @@ __global__ void k_owners(const uint32_t *__restrict__ out_src, const uint32_t *_
                          const uint32_t *__restrict__ status)
 {
     grid_wait();
-    if (*status & ST_TIMEOUT) return;   // a sort whose wait ran out: its keys are anything
+    if (latched(status) & ST_TIMEOUT) return;   // a sort whose wait ran out: its keys are anything
     const int lane = threadIdx.x & 31;
     const uint64_t x0 = (uint64_t)blockIdx.x * blockDim.x * kElemItems + threadIdx.x;
     uint32_t k[2][kElemItems], kp[2][kElemItems];
@@ -878,7 +892,7 @@ __global__ void __launch_bounds__(256) k_pairs(const uint32_t *__restrict__ msrc
     __shared__ uint32_t s_w[8], s_tile, s_before, s_h[8][ROWS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0)   // a sort whose wait ran out: its keys are anything
-        s_tile = (*(volatile uint32_t *)status & ST_TIMEOUT) ? 0xFFFFFFFFu : atomicAdd(ticket, 1u);
+        s_tile = (latched(status) & ST_TIMEOUT) ? 0xFFFFFFFFu : atomicAdd(ticket, 1u);
     __syncthreads();
     const uint32_t tile = s_tile;
     if (tile == 0xFFFFFFFFu) return;
@@ -987,9 +1001,10 @@ struct XR {
 // 5e7 edges: 797 us with four separate searches in lockstep per thread, 566 with
 // four consecutive entries, 481 with eight; 2e6 edges 34, 29 and 31.
 template <int kXrItems>
-__global__ void __launch_bounds__(256) k_cross_rank(XR a, XR b, uint32_t m, uint32_t n)
+__global__ void __launch_bounds__(256) k_cross_rank(XR a, XR b, uint32_t m, const uint32_t *status)
 {
     grid_wait();
+    const uint32_t stop = latched(status) & ST_TIMEOUT;   // the list offsets were not written
     const bool s1 = blockIdx.y != 0;
     const uint32_t *__restrict__ own_t = s1 ? b.own_t : a.own_t, *__restrict__ owner = s1 ? b.owner : a.owner;
     const uint32_t *__restrict__ other_off = s1 ? b.other_off : a.other_off, *__restrict__ other_t = s1 ? b.other_t : a.other_t;
@@ -1011,13 +1026,13 @@ __global__ void __launch_bounds__(256) k_cross_rank(XR a, XR b, uint32_t m, uint
             }
         }
     }
+    if (stop) return;
     uint32_t lo = 0, hi = 0;
 #pragma unroll
     for (int k = 0; k < kXrItems; ++k) {
         if (k == 0 || z[k] != z[k - 1]) {
-            const uint32_t v = min(z[k], n - 1);   // (a sort whose wait ran out leaves anything here)
-            lo = __ldg(other_off + v);
-            hi = __ldg(other_off + v + 1);
+            lo = __ldg(other_off + z[k]);
+            hi = __ldg(other_off + z[k] + 1);
             lo = lower_idx(other_t, lo, hi, t[k]);
         } else if (t[k] != t[k - 1]) {
             lo = gallop_idx(other_t, lo, hi, t[k]);
@@ -1062,6 +1077,13 @@ static uint32_t *gtake(GraphBlock &b, size_t count)
     uint32_t *p = (uint32_t *)(b.base + b.off);
     b.off += bytes;
     return p;
+}
+
+// The build's status as last copied.
+static int build_status(tm_ctx *ctx)
+{
+    const uint32_t bits = *ctx->status_host;
+    return bits ? set_err(ctx, TM_E_CUDA, "CSR build: device status " + std::to_string(bits)) : TM_OK;
 }
 
 int build_csr(tm_ctx *ctx)
@@ -1171,7 +1193,7 @@ int build_csr(tm_ctx *ctx)
         unsigned long long hnd[2] = {0, 0};
         copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
         rc = check_cuda(ctx, cudaStreamSynchronize(st), "duplicate scan");
-        if (rc) return rc;
+        if (rc || (rc = build_status(ctx))) return rc;
         memcpy(hnd, ctx->status_host + 4, 16);
         if (hnd[1]) {
             // (the work arrays hold the same tuples in input order)
@@ -1185,7 +1207,7 @@ int build_csr(tm_ctx *ctx)
             launch(ctx, k_flag_unique, blocks_for(m, TB), TB, g.g_t, g.g_src, g.g_dst, m, keep, nd);
             copy_d2h(ctx, ctx->status_host, ctx->status, kStatusBytes);
             rc = check_cuda(ctx, cudaStreamSynchronize(st), "duplicate scan");
-            if (rc) return rc;
+            if (rc || (rc = build_status(ctx))) return rc;
             memcpy(hnd, ctx->status_host + 4, 8);
         }
         const unsigned long long ndup = hnd[0];
@@ -1287,7 +1309,7 @@ int build_csr(tm_ctx *ctx)
         const int per = m <= kPairSmall ? 4 : 8;
         launch(ctx, per == 4 ? k_cross_rank<4> : k_cross_rank<8>, dim3(blocks_for(((uint64_t)m + per - 1) / per, TB), 2), TB,
                XR{g.out_t, g.out_src, g.in_off, g.in_t, g.out_xrank},
-               XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m, n);
+               XR{g.in_t, g.in_dst, g.out_off, g.out_t, g.in_xrank}, m, (const uint32_t *)ctx->status);
     } else {
         GraphBlock pbk;
         if (!gblock_open(ctx, pbk, 3 * 256)) return TM_E_NOMEM;
@@ -1301,8 +1323,7 @@ int build_csr(tm_ctx *ctx)
     if (rc2) return rc2;
     if (m) np = ctx->status_host[1];   // copied with the status
     g.npairs = np;
-    if (bits) return set_err(ctx, TM_E_CUDA, "CSR build: device status " + std::to_string(bits));
-    return TM_OK;
+    return build_status(ctx);
 }
 
 }  // namespace timest

@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(kTotThreads) k_window_totals(GuideArgs A, uint
     constexpr int kWarps = kTotThreads / 32;
     __shared__ u128 s_tot[kWarps];
     __shared__ u128 s_before;
-    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_tile, s_stop;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t nw0 = A.windows(0), nw1 = A.windows(1);
     const int b = blockIdx.y;
@@ -607,7 +607,12 @@ __global__ void __launch_bounds__(kTotThreads) k_window_totals(GuideArgs A, uint
     if (blockIdx.x >= ntiles) return;   // (as many blocks stay as there are tiles)
     tiles += (size_t)b * gridDim.x;
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket + b, 1u);
+    if (threadIdx.x == 32) s_stop = latched(status) & ST_TIMEOUT;
     __syncthreads();
+    if (s_stop) {   // a wait ran out: win_beg may have holes; no tile waits for this one
+        if (threadIdx.x == 0) seg_publish(tiles + s_tile, SegAgg2{0, 0, 0, 0}, 2);
+        return;
+    }
     const uint32_t tile = s_tile, k0 = tile * kTotTile + threadIdx.x * kTotItems;
     uint64_t v[kTotItems];
     u128 sum = 0;

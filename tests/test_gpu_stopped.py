@@ -1,0 +1,124 @@
+"""A wait between tiles that ran out: the stages behind it, whose input then has
+holes, do nothing and the call returns an error, after which the context is as
+good as new.  No wait is made to run out: the allocator hook latches the status
+bit on the context's stream at an allocation inside the build or the weight pass
+(the status block is the first that a context asks for)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ST_TIMEOUT = 4
+PATTERN = 0xA5
+
+
+class Latch:
+    """Allocator hooks that fill every block with a pattern and latch
+    ST_TIMEOUT at the request whose 1-based number is `at`."""
+
+    def __init__(self):
+        import torch
+        import paper_2507_20441_gb300 as tg
+        self.calls, self.at, self.sizes = 0, 0, []
+        self.live, self.status, self.block, self.untouched = {}, None, None, None
+
+        def _alloc(nbytes, stream, user):
+            self.calls += 1
+            self.sizes.append(nbytes)
+            s = torch.cuda.ExternalStream(stream)
+            with torch.cuda.stream(s):
+                t = torch.full((nbytes,), PATTERN, dtype=torch.uint8, device="cuda")
+                if self.status is None:
+                    self.status = t.view(torch.int32)
+                if self.calls == self.at:
+                    self.status[0:1].fill_(ST_TIMEOUT)
+                    self.block = t.data_ptr()
+            self.live[t.data_ptr()] = t
+            return t.data_ptr()
+
+        def _free(ptr, nbytes, stream, user):
+            torch.cuda.synchronize()
+            t = self.live.pop(ptr)
+            if ptr == self.block:
+                self.untouched = bool((t == PATTERN).all())
+                self.block = None
+
+        self.hooks = (tg.ALLOC_FN(_alloc), tg.FREE_FN(_free))
+
+    def arm(self, after):
+        """At the after-th request from now on."""
+        self.calls, self.sizes, self.at, self.block, self.untouched = 0, [], after, None, None
+
+
+def _edges(n, m):
+    rng = np.random.default_rng(m)
+    s = rng.integers(0, n, m).astype(np.uint32)
+    d = ((s + 1 + rng.integers(0, n - 1, m)) % n).astype(np.uint32)
+    return s, d, rng.permutation(m).astype(np.int64)
+
+
+def _arrays(ctx):
+    return [ctx.csr(a) for a in ("out_off", "in_off", "out_pos", "in_pos", "in_xrank", "multi_to_out", "pair_off")]
+
+
+# small and large tiles of the sorts, and inverses that go through buckets
+@pytest.mark.parametrize("n,m", [(300, 20_000), (5000, 700_001), (70_001, 16_100_001)])
+def test_build_behind_a_stopped_sort(n, m):
+    import paper_2507_20441_gb300 as tg
+    tg.build()
+    edges = _edges(n, m)
+    hook = Latch()
+    ctx = tg.Context(alloc_hooks=hook.hooks)
+    hook.arm(0)
+    ctx.load_graph(n, *edges)
+    calls = hook.calls
+    up = lambda words: (4 * words + 255) // 256 * 256
+    graph = 1 + hook.sizes.index(20 * up(m) + 256 + 3 * up(n + 1) + 3 * up(m // 32 + 1))   # every array of the graph
+    want = _arrays(ctx)
+    ctx.close()
+    failed = set()
+    for at in range(1, calls + 1):
+        hook = Latch()
+        ctx = tg.Context(alloc_hooks=hook.hooks)
+        hook.arm(at)
+        try:
+            ctx.load_graph(n, *edges)
+        except tg.TimestError as e:
+            assert e.code == tg.TM_E_CUDA and "device status 4" in str(e), (at, e)
+            failed.add(at)
+            if at == graph:       # latched before the first sort: no array of the graph was written
+                assert hook.untouched
+            hook.arm(0)
+            ctx.load_graph(n, *edges)
+        assert all(np.array_equal(a, b) for a, b in zip(_arrays(ctx), want)), at
+        ctx.close()
+    assert graph in failed
+    if m > 16_000_000:            # scratch grows inside the later sorts too
+        assert len(failed) >= 4, failed
+
+
+@pytest.mark.parametrize("m,delta", [(20_001, 300), (400_003, 5000)])
+def test_weights_behind_a_stopped_wait(m, delta):
+    import paper_2507_20441_gb300 as tg
+    tg.build()
+    n = 500
+    hook = Latch()
+    ctx = tg.Context(alloc_hooks=hook.hooks)
+    ctx.load_graph(n, *_edges(n, m))
+    args = (4, [(0, 1), (1, 2), (2, 3), (3, 0)], [0, 1, 2, 3], delta)
+    mo = ctx.motif(*args).set_tree([0, 1, 2], 0)      # a path from its end: one inner node
+    W = mo.weights()
+    want = mo.sample(20_000, 5)
+    hook.arm(1)
+    other = ctx.motif(*args).set_tree([0, 1, 2], 0)
+    with pytest.raises(tg.TimestError) as e:
+        other.weights()
+    assert e.value.code == tg.TM_E_CUDA
+    assert hook.calls >= 1
+    hook.arm(0)
+    assert other.weights() == W
+    for x in (mo, other):
+        r = x.sample(20_000, 5)
+        assert (r.W, r.hits2, r.valid, r.rej_vertex, r.rej_delta, r.rej_order) == \
+               (want.W, want.hits2, want.valid, want.rej_vertex, want.rej_delta, want.rej_order)
+    ctx.close()
