@@ -383,8 +383,8 @@ int tm_serve_poll(tm_ctx *ctx, uint64_t ticket, tm_result *out, int timeout_ms);
 /* Counters, cache behaviour and latency percentiles since tm_serve_start. */
 int tm_serve_stats(tm_ctx *ctx, tm_serve_stats_t *out);
 
-/* Stop serving: queries being sampled finish their rounds, queued ones are
- * dropped, cached weights are freed. */
+/* Stop serving: queries being sampled finish their rounds (a round whose wait
+ * ran out too), queued ones are dropped, cached weights are freed. */
 int tm_serve_stop(tm_ctx *ctx);
 
 /* Phases timed when cfg.profile = 1 (CUDA events on the context stream). */

@@ -24,6 +24,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -90,6 +91,7 @@ struct Server {
     uint64_t use_clock = 0;
     uint64_t next_ticket = 1;
     bool stop = false;
+    std::atomic<bool> late{false};   // a round ran out of its wait and may still be running
     std::thread admit_thr, sched_thr;
     // statistics
     uint64_t submitted = 0, completed = 0, failed = 0, hits = 0, misses = 0, evictions = 0, rounds = 0;
@@ -131,6 +133,19 @@ size_t estimate_bytes(const tm_motif *mo, uint64_t m, uint64_t T)
     // slot, 12 B per kind of candidate range
     const uint64_t ranges = (uint64_t)mo->plan.nkinds;
     return (size_t)((18 + 32 * slots + 12 * ranges) * std::max<uint64_t>(m, 1) + 96 * nwin + 4096);
+}
+
+// Waits for a round that ran out of its wait: its kernel reads the plans and
+// weights of queries that have been told so and hold them no longer.
+void wait_late(Server *S)
+{
+    if (S->late.exchange(false)) cudaStreamSynchronize(S->main->stream);
+}
+
+void free_weights(Server *S, tm_motif *mo)
+{
+    wait_late(S);
+    tm_motif_free(mo);
 }
 
 void finish_locked(Server *S, Request *r)
@@ -213,7 +228,7 @@ void admit_loop(Server *S)
                 S->cache.erase(victim);
                 S->evictions++;
                 lk.unlock();
-                tm_motif_free(vm);
+                free_weights(S, vm);
                 lk.lock();
                 continue;
             }
@@ -241,7 +256,7 @@ void admit_loop(Server *S)
                 }
             }
             lk.unlock();
-            for (tm_motif *vm : freed) tm_motif_free(vm);
+            for (tm_motif *vm : freed) free_weights(S, vm);
             lk.lock();
             S->cv_admit.wait_for(lk, std::chrono::milliseconds(kNoMemWaitMs));
             lk.unlock();
@@ -316,6 +331,7 @@ void sched_loop(Server *S)
             accs.assign(items.size(), SampleAcc{0, 0, 0, 0, 0, 0});
             rc = run_batch_items(ctx, items.data(), (uint32_t)items.size(), tile, accs.data(), S->cfg.poll_timeout_ms);
         }
+        if (rc == TM_E_TIMEOUT) S->late = true;   // before its queries let go of their weights
         lk.lock();
         S->rounds++;
         std::vector<Request *> still;
@@ -511,7 +527,8 @@ int tm_serve_stop(tm_ctx *ctx)
     for (Request *r : S->ready) delete r;
     for (Request *r : S->active) delete r;
     for (auto &d : S->done) delete d.second;
-    for (auto &c : S->cache) tm_motif_free(c.second.mo);
+    for (auto &c : S->cache) free_weights(S, c.second.mo);
+    wait_late(S);
     tm_destroy(S->shadow);
     ctx->server = nullptr;
     delete S;
