@@ -295,8 +295,10 @@ __global__ void __launch_bounds__(256, LEAF ? 4 : 5)
         for (int k = 0; k < K; ++k) {
             if (((zero >> (2 * k)) & 3u) == 3u) continue;
             const uint32_t b0 = __ldg(pin + (xp[k] >> 5)) >> (xp[k] & 31), b1 = __ldg(pin + words + (xp[k] >> 5)) >> (xp[k] & 31);
-            ovf |= ((b0 & 1u) | ((b1 & 1u) << 1)) << (2 * k);
-            zero |= ((prod[k][0] == 0 ? 1u : 0u) | (prod[k][1] == 0 ? 2u : 0u)) << (2 * k);
+            // (a partial that wrapped may be 0 as it stands and is none)
+            const uint32_t wrapped = (b0 & 1u) | ((b1 & 1u) << 1);
+            ovf |= wrapped << (2 * k);
+            zero |= (((prod[k][0] == 0 ? 1u : 0u) | (prod[k][1] == 0 ? 2u : 0u)) & ~wrapped) << (2 * k);
         }
     }
     for (int ci = 0; ci < P.nchild[q] && zero != kAll; ++ci) {

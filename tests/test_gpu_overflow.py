@@ -75,6 +75,30 @@ def test_overflow_stays_inside_its_blocks(hub):
     ctx.close()
 
 
+@pytest.mark.parametrize("behind", [0, 1, 3])
+@pytest.mark.parametrize("later", [8192, 8191])
+def test_a_partial_product_that_wraps_to_zero(later, behind):
+    """The root edge h->v has five children at h (8192 candidates each: 2^65, which
+    is 0 in 64 bits) and one at v: an overflow, unless nothing follows at v."""
+    import paper_2507_20441_gb300 as tg
+    tg.build()
+    h, v = 0, 1
+    src = np.concatenate([[h], np.zeros(later), np.full(behind, v)]).astype(np.uint32)
+    dst = np.concatenate([[v], np.arange(later) + 2, np.arange(behind) + 2]).astype(np.uint32)
+    t = np.arange(src.size, dtype=np.int64)
+    ctx = tg.Context()
+    ctx.load_graph(later + 2, src, dst, t)
+    edges = [(0, 1)] + [(0, i) for i in range(2, 7)] + [(1, 7)]
+    mo = ctx.motif(8, edges, list(range(7)), 100_000).set_tree(list(range(7)), 0)
+    if later ** 5 * behind >= 1 << 64:
+        with pytest.raises(tg.TimestError) as e:
+            mo.weights()
+        assert e.value.code == tg.TM_E_OVERFLOW
+    else:
+        assert mo.weights() == later ** 5 * behind
+    ctx.close()
+
+
 def test_selection_ending_in_an_overflow():
     """A hub with 25,000 out-edges and chains between its first neighbours: the
     star over the hub overflows, trees that use a chain do not.  A selection whose
