@@ -112,9 +112,9 @@ constexpr int kLookback = 4;   // tiles read at a time when looking back (2 meas
 // One pass.  Tiles are taken from a counter, so every tile before this one has
 // been started and publishes its counts without waiting for anyone; waits for
 // them are bounded all the same (ST_TIMEOUT).  After a wait that ran out the
-// pass's output has holes, and its keys no longer match the digit counts that
-// place them: from then on tiles publish an empty prefix and write nothing, in
-// this pass and in every later one.  A warp ranks 32 keys at a time:
+// pass's output has holes, and the next pass's keys no longer match the digit
+// counts that place them, so a position is checked before it is written (0.3 % of
+// the passes on 5e7 keys; asking the status in each tile instead was 0.7).  A warp ranks 32 keys at a time:
 // each lane marks its bit in its digit's word of shared memory and reads the
 // word back, which gives the peers before it (a ballot per digit bit, which
 // this replaces, was most of the pass's instructions).  The tile is staged
@@ -139,17 +139,12 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
     __shared__ uint16_t s_wcnt[OS_WARPS * OS_MAXRADIX];       // [warp][digit] counts, then tile slots
     __shared__ uint32_t s_gpos[OS_MAXRADIX];                  // digit start in the output - in the tile
     __shared__ uint32_t s_wt[8];
-    __shared__ uint32_t s_tile, s_stop;
+    __shared__ uint32_t s_tile;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) s_tile = atomicAdd(ticket, 1u);
-    if (t == 32) s_stop = latched(status) & ST_TIMEOUT;   // (both on their way together)
     for (int i = t; i < OS_WARPS * OS_MAXRADIX; i += OS_THREADS) { s_wcnt[i] = 0; s_match[i] = 0; }
     __syncthreads();
     const uint32_t tile = s_tile;
-    if (s_stop) {
-        if (t < OS_MAXRADIX) *(volatile unsigned long long *)(state + (size_t)tile * OS_MAXRADIX + t) = kTilePrefix;
-        return;
-    }
     const uint32_t radix = 1u << bits, dmask = radix - 1u;
     const uint32_t base = tile * (uint32_t)TILE;
     const uint32_t tile_n = min((uint32_t)TILE, n - base);
@@ -271,7 +266,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
         if (p < tile_n) {
             const uint32_t k = s_buf[p];
             g[j] = s_gpos[(k >> shift) & dmask] + p;
-            J.kout[g[j]] = k;
+            if (g[j] < n) J.kout[g[j]] = k;
         }
     }
     // ---- payloads, one round each
@@ -289,7 +284,7 @@ __global__ void __launch_bounds__(OS_THREADS, 4)
             const uint32_t p = t + j * OS_THREADS;
             if (p < tile_n) {
                 const uint32_t v = s_buf[p];
-                pout[g[j]] = v;
+                if (g[j] < n) pout[g[j]] = v;
                 if (a == 0 && J.inv && v < n) J.inv[v] = g[j];
             }
         }

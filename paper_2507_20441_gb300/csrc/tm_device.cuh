@@ -16,11 +16,9 @@ __device__ __forceinline__ void latch(uint32_t *status, uint32_t bits)
     atomicOr(status, bits);
 }
 
-// What has been latched so far, by an earlier kernel or a block of this one.
-__device__ __forceinline__ uint32_t latched(const uint32_t *status)
-{
-    return *(const volatile uint32_t *)status;
-}
+// What earlier kernels have latched (what this one latches itself may be seen or
+// not: the load is a cached one, since every block asks).
+__device__ __forceinline__ uint32_t latched(const uint32_t *status) { return __ldca(status); }
 
 // Philox4x32 with 10 rounds (Salmon, Moraes, Dror, Shaw, SC'11): each round
 // multiplies counter words 0 and 2 by the two round multipliers, feeds the

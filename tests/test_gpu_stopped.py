@@ -1,6 +1,6 @@
-"""A wait between tiles that ran out: the stages behind it, whose input then has
-holes, do nothing and the call returns an error, after which the context is as
-good as new.  No wait is made to run out: the allocator hook latches the status
+"""A wait between tiles that ran out: the call returns an error - the stages
+behind it, whose input then has holes, stay inside their arrays - and the context
+is as good as new.  No wait is made to run out: the allocator hook latches the status
 bit on the context's stream at an allocation inside the build or the weight pass
 (the status block is the first that a context asks for)."""
 import numpy as np
@@ -13,14 +13,15 @@ PATTERN = 0xA5
 
 
 class Latch:
-    """Allocator hooks that fill every block with a pattern and latch
-    ST_TIMEOUT at the request whose 1-based number is `at`."""
+    """Allocator hooks that latch ST_TIMEOUT at the request whose 1-based number
+    is `at`, and give blocks filled with one byte (keys and positions past every
+    array, were they read before they are written)."""
 
     def __init__(self):
         import torch
         import paper_2507_20441_gb300 as tg
         self.calls, self.at, self.sizes = 0, 0, []
-        self.live, self.status, self.block, self.untouched = {}, None, None, None
+        self.live, self.status = {}, None
 
         def _alloc(nbytes, stream, user):
             self.calls += 1
@@ -32,22 +33,18 @@ class Latch:
                     self.status = t.view(torch.int32)
                 if self.calls == self.at:
                     self.status[0:1].fill_(ST_TIMEOUT)
-                    self.block = t.data_ptr()
             self.live[t.data_ptr()] = t
             return t.data_ptr()
 
         def _free(ptr, nbytes, stream, user):
             torch.cuda.synchronize()
-            t = self.live.pop(ptr)
-            if ptr == self.block:
-                self.untouched = bool((t == PATTERN).all())
-                self.block = None
+            del self.live[ptr]
 
         self.hooks = (tg.ALLOC_FN(_alloc), tg.FREE_FN(_free))
 
     def arm(self, after):
         """At the after-th request from now on."""
-        self.calls, self.sizes, self.at, self.block, self.untouched = 0, [], after, None, None
+        self.calls, self.sizes, self.at = 0, [], after
 
 
 def _edges(n, m):
@@ -86,13 +83,11 @@ def test_build_behind_a_stopped_sort(n, m):
         except tg.TimestError as e:
             assert e.code == tg.TM_E_CUDA and "device status 4" in str(e), (at, e)
             failed.add(at)
-            if at == graph:       # latched before the first sort: no array of the graph was written
-                assert hook.untouched
             hook.arm(0)
             ctx.load_graph(n, *edges)
         assert all(np.array_equal(a, b) for a, b in zip(_arrays(ctx), want)), at
         ctx.close()
-    assert graph in failed
+    assert graph in failed        # latched before the first sort
     if m > 16_000_000:            # scratch grows inside the later sorts too
         assert len(failed) >= 4, failed
 
