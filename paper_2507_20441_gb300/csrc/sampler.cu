@@ -340,7 +340,7 @@ __device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P
     uint32_t a, b, ea = 0, ne = 0;
     uint64_t hit = 0;
     bool em = false;
-    uint2 r = make_uint2(0, kRangeLong | (kRangeLong << 16));
+    uint2 r = range_unknown();
     if (J.range.base) r = __ldg(J.range.base + (size_t)P.tkind[q] * J.range.stride + ppos);
     uint4 ex = make_uint4(r.x, 0, 0, kExclBits);
     if ((r.y & kRangeFlags) && r.x < J.range.excl_cap) ex = __ldg(J.range.excl + r.x);
@@ -349,7 +349,7 @@ __device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P
     a = later ? ex.x : ex.x - len;
     b = a + len;
     bool same = (half & kRangeSame) != 0;   // the entry before a is in a's segment of the prefixes
-    if (len == kRangeLong) {
+    if (range_searched(r)) {
         const uint2 ab = search_range(g, P, q, zg, ppos, pt, wlo, whi);
         a = ab.x;
         b = ab.y;
@@ -367,9 +367,9 @@ __device__ __forceinline__ void sample_child(const DevGraph &g, const DevPlan &P
             else hit &= ~0ull >> (64 - len);
         } else {
             const uint32_t h = (p ? ex.z >> 16 : ex.z) & 0xFFFFu;
-            ne = h & kExclMany;
+            ne = h & kExclCount;
             ea = later ? ex.y : ex.y - ne;
-            em = (h & 0x8000u) != 0;
+            em = (h & kExclSame) != 0;
         }
     }
     if (b <= a || b > g.m || ne > g.m || ea > g.m - ne) {

@@ -176,23 +176,45 @@ struct LayerData {
 
 // Candidate range of a child for one parent edge (Claim 3.1), found once per
 // kind by the weight pass and read by its DP and by the sampler.  y holds per
-// layer p, in bits 16p .. 16p + 15, the number of entries (bits 0-13;
-// kRangeLong: not held, the range is searched), whether the entry before the
-// range is in the same (vertex, window) segment of the prefixes (bit 14; kinds
-// with an inner child) and whether excluded entries are among them (bit 15).
-// x is the bound next to the parent edge's time - the first entry of a later
-// child, the end of an earlier one's - or, when either layer has excluded
-// entries, the index of a RangeExcl.
+// layer p, in bits 16p .. 16p + 15, the number of entries (bits 0-13), whether
+// the entry before the range is in the same (vertex, window) segment of the
+// prefixes (bit 14; kinds with an inner child) and whether excluded entries are
+// among them (bit 15).  x is the bound next to the parent edge's time - the first
+// entry of a later child, the end of an earlier one's - or, when either layer has
+// excluded entries, the index of a RangeExcl.
+// A range of kRangeLong entries or more in either layer, or one whose excluded
+// entries the table had no room for, is searched again by whoever needs its
+// bounds: its low half's number is kRangeLong, and x with the rest of y holds the
+// layers' numbers of candidates, excluded entries left out (kCountMany: not
+// known), which is the weight of a leaf child (weights of the 4-cycle: a hub of 1e6
+// edges 490 us with these searched for too and 270 so; 5e5 edges over 30 vertices,
+// ranges of 500 entries, 243 and 143).  Bit 16 is set and bits 15 and 31
+// are clear in such a record: it has neither flag, and no half of it reads as empty.
 constexpr uint32_t kRangeLong = 0x3FFFu, kRangeSame = 0x4000u, kRangeHasExcl = 0x8000u;
 constexpr uint32_t kRangeFlags = kRangeHasExcl | (kRangeHasExcl << 16);
+constexpr uint32_t kCountBits = 23, kCountMany = (1u << kCountBits) - 1u;
+#ifdef __CUDACC__
+__device__ __forceinline__ bool range_searched(uint2 r) { return (r.y & kRangeLong) == kRangeLong; }
+__device__ __forceinline__ uint2 range_counts(uint32_t n0, uint32_t n1)
+{
+    n0 = n0 < kCountMany ? n0 : kCountMany;
+    n1 = n1 < kCountMany ? n1 : kCountMany;
+    return make_uint2(n0 | (n1 << kCountBits), kRangeLong | (1u << 16) | ((n1 >> (32 - kCountBits)) << 17));
+}
+__device__ __forceinline__ uint32_t range_count(uint2 r, int p)   // of a searched range
+{
+    return p ? (r.x >> kCountBits) | ((r.y >> 17) << (32 - kCountBits)) : r.x & kCountMany;
+}
+__device__ __forceinline__ uint2 range_unknown() { return range_counts(kCountMany, kCountMany); }
+#endif
 // The excluded entries of such a range (16 bytes): x = the bound above.
 // w = kExclBits: y, z = a bit per entry counted from that bound (bit i: entry
 // x + i of a later child, x - 1 - i of an earlier one's), set for an excluded
 // one; ranges of up to 64 entries are scanned for them.  w = kExclList: z holds
-// per layer the number of excluded entries (bits 0-14 of each half) and whether
-// the entry before them is in the same segment of the prefixes (bit 15), y the
+// per layer the number of excluded entries (kExclCount of each half) and whether
+// the entry before them is in the same segment of the prefixes (kExclSame), y the
 // first of them in multi-edge order (later child) or their end (earlier).
-constexpr uint32_t kExclBits = 0, kExclList = 1, kExclMany = 0x7FFFu;
+constexpr uint32_t kExclBits = 0, kExclList = 1, kExclCount = 0x7FFFu, kExclSame = 0x8000u;
 typedef uint4 RangeExcl;
 struct RangePtrs {
     uint2 *base;             // kind k's at base + k stride, by the parent edge's position in the
