@@ -859,6 +859,11 @@ static void free_motif_weights(tm_ctx *ctx, tm_motif *mo)
     mo->have_weights = false;
 }
 
+// A block of this size or more that is refused with candidate ranges is asked for
+// without them.  A smaller one is reported as any other: scratch is taken in
+// chunks of at least 64 MiB, so where 4 MiB are refused there is nothing to run with.
+constexpr size_t kRangesOptional = (size_t)4 << 20;
+
 // Owner bit sets of the out-, in- and multi-edge orders (built with the graph).
 struct OwnerBits { const uint32_t *out, *in, *multi; };
 
@@ -937,8 +942,8 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
         const size_t mm = (size_t)(m ? m : 1);
         auto guide_n = [&](uint32_t nw) { return (size_t)m / 4 + 3 * (size_t)nw + 1; };
         const size_t win_arrays = al(((size_t)nwh[0] + 1) * 4) * 2 + al(((size_t)nwh[1] + 1) * 4) * 2;   // starts and indices
-        // the candidate ranges come last: a block this large that does not fit
-        // with them is tried without (the sampler then searches the ranges)
+        // the candidate ranges come last: a block that does not fit with them is
+        // tried without (the DP and the samplers then search the ranges)
         // (room for excluded entries at 0.3 of the edges per kind: with bursts of
         // repeated pairs a star's ranges have them at 0.2 - 0.3)
         const int nk = sh ? sh->max_kinds : P.nkinds;
@@ -976,7 +981,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
         if (sh) total -= win_arrays;
         bool with_ranges = true;
         blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
-        if (!blk && !sh && total >= ((size_t)4 << 30)) {
+        if (!blk && !sh && total + range_bytes >= kRangesOptional) {
             with_ranges = false;
             blk = (char *)malloc_motif(ctx, mo, total);
         }
