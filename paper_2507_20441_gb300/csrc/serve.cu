@@ -122,19 +122,6 @@ std::string make_key(uint32_t nv, uint32_t ne, const uint32_t *edges, const uint
     return s;
 }
 
-// Device bytes a motif's resident weights will need (root CDF and its guide
-// table, prefix slots, candidate ranges, window lists), before they are computed.
-size_t estimate_bytes(const tm_motif *mo, uint64_t m, uint64_t T)
-{
-    uint64_t slots = (uint64_t)mo->plan.nslots;
-    uint64_t nwin = T / (uint64_t)std::max<int64_t>(1, mo->plan.wdelta) + 2;
-    nwin = std::min<uint64_t>(nwin, m + 2);
-    // root CDF 16 B and root-search guide about 2 B per edge, 32 B per prefix
-    // slot, 12 B per kind of candidate range
-    const uint64_t ranges = (uint64_t)mo->plan.nkinds;
-    return (size_t)((18 + 32 * slots + 12 * ranges) * std::max<uint64_t>(m, 1) + 96 * nwin + 4096);
-}
-
 // Waits for a round that ran out of its wait: its kernel reads the plans and
 // weights of queries that have been told so and hold them no longer.
 void wait_late(Server *S)
@@ -213,7 +200,7 @@ void admit_loop(Server *S)
             finish_locked(S, r);
             continue;
         }
-        size_t need = estimate_bytes(mo, S->shadow->g.m, S->shadow->g.T);
+        const size_t need = weights_bytes(mo->plan, S->shadow->g.m, S->shadow->g.T);
         for (;;) {
             if (S->stop) { lk.unlock(); tm_motif_free(mo); lk.lock(); return; }
             if (S->resident + need <= S->cfg.weight_budget) break;

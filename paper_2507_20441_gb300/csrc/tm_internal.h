@@ -342,6 +342,7 @@ struct SharedPass {
     RangePtrs range{};
 };
 int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides = true, SharedPass *sh = nullptr);
+size_t weights_bytes(const DevPlan &P, uint64_t m, uint64_t T);   // of a motif's block, or somewhat more
 void assign_kinds(DevPlan &P);           // kinds of candidate range of a plan alone
 // (nwin: the layers' window numbers on the device, null once the motif has them;
 // nothing is filled when the status block holds a bit)

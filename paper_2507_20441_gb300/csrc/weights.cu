@@ -864,6 +864,44 @@ static void free_motif_weights(tm_ctx *ctx, tm_motif *mo)
 // chunks of at least 64 MiB, so where 4 MiB are refused there is nothing to run with.
 constexpr size_t kRangesOptional = (size_t)4 << 20;
 
+// Sizes of the arrays that a motif keeps, each at a multiple of 256 bytes.
+static size_t aligned(size_t b) { return (b + 255) / 256 * 256; }
+static size_t guide_entries(uint64_t m, uint32_t nw) { return (size_t)m / 4 + 3 * (size_t)nw + 1; }
+// window starts and indices of both layers
+static size_t window_bytes(const uint32_t nw[2])
+{
+    return aligned(((size_t)nw[0] + 1) * 4) * 2 + aligned(((size_t)nw[1] + 1) * 4) * 2;
+}
+// room for excluded entries at 0.3 of the edges per kind: with bursts of repeated
+// pairs a star's ranges have them at 0.2 - 0.3
+static size_t excl_entries(uint64_t m, int kinds) { return (size_t)kinds * ((size_t)m * 3 / 10); }
+static size_t range_bytes_of(uint64_t m, int kinds)
+{
+    return (size_t)kinds * aligned((size_t)m * sizeof(uint2)) + aligned(excl_entries(m, kinds) * sizeof(RangeExcl));
+}
+static size_t block_bytes(const DevPlan &P, uint64_t m, const uint32_t nw[2])   // without the ranges
+{
+    const size_t both = (size_t)nw[0] + nw[1];
+    return 2 * window_bytes(nw) + 2 * aligned((size_t)m * 8) + (size_t)P.nslots * 2 * aligned((size_t)m * 16) +
+           aligned((both + 1) * 16) + aligned(guide_entries(m, nw[0]) * 4) + aligned(guide_entries(m, nw[1]) * 4) +
+           aligned((4 * both + 2) * 4);
+}
+// The most windows there can be: their indices go up to T / unit, the even ones in layer 0.
+static void window_bounds(const DevPlan &P, uint64_t m, uint64_t T, uint32_t nw[2])
+{
+    const uint64_t qT = m ? T / (uint64_t)P.wdelta : 0;
+    nw[0] = (uint32_t)std::min<uint64_t>(m, qT / 2 + 1);
+    nw[1] = (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2);
+}
+
+size_t weights_bytes(const DevPlan &P, uint64_t m, uint64_t T)
+{
+    uint32_t nw[2];
+    window_bounds(P, m, T, nw);
+    const uint64_t mm = m ? m : 1;
+    return block_bytes(P, mm, nw) + range_bytes_of(mm, P.nkinds);
+}
+
 // Owner bit sets of the out-, in- and multi-edge orders (built with the graph).
 struct OwnerBits { const uint32_t *out, *in, *multi; };
 
@@ -901,9 +939,8 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
     int rc = TM_OK;
     const bool known = sh && sh->windows;      // the windows, from an earlier candidate
     cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
-    // window indices go up to T / unit, the even ones in layer 0
-    const uint64_t qT = m ? (uint64_t)g.T / (uint64_t)P.wdelta : 0;
-    uint32_t nwh[2] = {(uint32_t)std::min<uint64_t>(m, qT / 2 + 1), (uint32_t)std::min<uint64_t>(m, (qT + 1) / 2)};
+    uint32_t nwh[2];
+    window_bounds(P, m, g.T, nwh);
     if (known) { nwh[0] = sh->nwin[0]; nwh[1] = sh->nwin[1]; }
     // cleared together: the tickets, the number of kept excluded ranges, the tile
     // words of the windows, of their totals and of every scan
@@ -938,20 +975,15 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
         cudaMemsetAsync(clear, 0, win_bytes, st);
     }
     {
-        auto al = [](size_t b) { return (b + 255) / 256 * 256; };
         const size_t mm = (size_t)(m ? m : 1);
-        auto guide_n = [&](uint32_t nw) { return (size_t)m / 4 + 3 * (size_t)nw + 1; };
-        const size_t win_arrays = al(((size_t)nwh[0] + 1) * 4) * 2 + al(((size_t)nwh[1] + 1) * 4) * 2;   // starts and indices
         // the candidate ranges come last: a block that does not fit with them is
         // tried without (the DP and the samplers then search the ranges)
-        // (room for excluded entries at 0.3 of the edges per kind: with bursts of
-        // repeated pairs a star's ranges have them at 0.2 - 0.3)
         const int nk = sh ? sh->max_kinds : P.nkinds;
-        const size_t excl_cap = (size_t)nk * (mm * 3 / 10);
-        size_t range_bytes = (size_t)nk * al(mm * sizeof(uint2)) + al(excl_cap * sizeof(RangeExcl));
+        const size_t excl_cap = excl_entries(mm, nk), win_arrays = window_bytes(nwh);
+        size_t range_bytes = range_bytes_of(mm, nk);
         char *blk = nullptr;
         size_t off = 0;
-        auto take = [&](size_t bytes) { char *q = blk + off; off += al(bytes); return (void *)q; };
+        auto take = [&](size_t bytes) { char *q = blk + off; off += aligned(bytes); return (void *)q; };
         auto take_windows = [&](uint32_t *beg[2], uint32_t *id[2]) {
             for (int p = 0; p < 2; ++p) {
                 beg[p] = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
@@ -959,7 +991,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
             }
         };
         auto take_ranges = [&](RangePtrs &r) {
-            r.stride = al(mm * sizeof(uint2)) / sizeof(uint2);
+            r.stride = aligned(mm * sizeof(uint2)) / sizeof(uint2);
             r.base = (uint2 *)take((size_t)nk * r.stride * sizeof(uint2));
             r.excl = (RangeExcl *)take(excl_cap * sizeof(RangeExcl));
             r.excl_cap = (uint32_t)std::min<size_t>(excl_cap, 0xFFFFFFFFu);
@@ -975,9 +1007,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
             off = 0;
         }
         if (sh) range_bytes = 0;
-        size_t total = win_arrays + al(((size_t)nwh[0] + 1) * 4) * 2 + al(((size_t)nwh[1] + 1) * 4) * 2 + 2 * al(mm * 8) +
-                       (size_t)P.nslots * 2 * al(mm * 16) + al(((size_t)nwh[0] + nwh[1] + 1) * 16) +
-                       al(guide_n(nwh[0]) * 4) + al(guide_n(nwh[1]) * 4) + al((4 * ((size_t)nwh[0] + nwh[1]) + 2) * 4);
+        size_t total = block_bytes(P, mm, nwh);
         if (sh) total -= win_arrays;
         bool with_ranges = true;
         blk = (char *)malloc_motif(ctx, mo, total + range_bytes);
@@ -996,7 +1026,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
             L.root_cdf = (uint64_t *)take(mm * 8);
             L.win_gshift = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
             L.win_goff = (uint32_t *)take(((size_t)nwh[p] + 1) * 4);
-            L.guide = (uint32_t *)take(guide_n(nwh[p]) * 4);
+            L.guide = (uint32_t *)take(guide_entries(m, nwh[p]) * 4);
         }
         for (int sl = 0; sl < P.nslots; ++sl) {   // one after the other (ChildPrefix)
             mo->pref_dir[sl] = (ulonglong2 *)take(mm * 16);
