@@ -891,8 +891,13 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
     if (rc) return rc;
     if (!best) return set_err(ctx, TM_E_OVERFLOW, "every candidate's weight pass overflowed");
     cudaMemsetAsync(ctx->status, 0, kStatusBytes, ctx->stream);   // (bits of a candidate that overflowed after the winner)
-    rc = fill_guides(ctx, best);
-    if (rc) { tm_motif_free(best); return rc; }
+    {
+        PhaseScope ph(ctx, TM_PH_ROOT);
+        rc = fill_guides(ctx, best);
+    }
+    uint32_t bits = 0;
+    const int rc2 = read_status(ctx, &bits);   // the tables are filled when the call returns
+    if (rc || rc2) { tm_motif_free(best); return rc ? rc : rc2; }
     *out = best;
     return TM_OK;
 }
