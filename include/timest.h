@@ -303,9 +303,9 @@ int tm_sample_trace(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64
  * cannot afford an allocator call).  The paper has no counterpart: it is an
  * interface choice of this library.  Results are bit-identical to tm_sample
  * with the same arguments.  The call allocates nothing: its scratch (the
- * result accumulators, behind room for the motif plan, which goes with the
- * launch) is a fixed 4096-byte array that every device loading the library
- * holds until the process exits; a plan that does not fit returns TM_E_LIMIT.  The first
+ * result accumulators; the motif plan goes with the launch) is a fixed
+ * 4096-byte array that every device loading the library holds until the
+ * process exits (device ordinals from 64 on return TM_E_LIMIT).  The first
  * call on a device looks up the array's device address (once per device,
  * with that device current), so make that first call before any stream
  * capture.  The accumulators are cleared at the start of every call, but all

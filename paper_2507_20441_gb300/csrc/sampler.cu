@@ -1081,9 +1081,8 @@ __global__ void __launch_bounds__(THREADS, kBatchThreads / THREADS) k_batch(DevG
 
 }  // namespace
 
-void fill_job(tm_motif *mo, SampleJob &J, const DevPlan *dplan)
+void fill_job(tm_motif *mo, SampleJob &J)
 {
-    J.plan = dplan;
     J.wcum = mo->wcum;
     J.wguide = mo->wguide;
     J.wshift = wguide_shift(mo->W.lo, mo->W.hi, mo->nwtot);
@@ -1158,7 +1157,7 @@ int run_samples(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t f
     Acc *dacc = (Acc *)(ctx->status + 4);
     cudaMemsetAsync(ctx->status, 0, kStatusBytes, st);
     SampleJob J;
-    fill_job(mo, J, nullptr);
+    fill_job(mo, J);
     const int threads = kSampleThreads;
     uint64_t want = (k + threads - 1) / threads;
     const bool local = trace || !reg_plan(mo->plan);   // records in local memory: k_sample
@@ -1218,7 +1217,7 @@ int run_list(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t seed, uint64_t firs
     copy_h2d(ctx, dplan, &mo->plan, sizeof(DevPlan));
     cudaMemsetAsync(ctx->status, 0, 4, st);
     SampleJob J;
-    fill_job(mo, J, dplan);
+    fill_job(mo, J);
     const uint64_t want = (k + kSampleThreads - 1) / kSampleThreads;
     const unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)ctx->num_sms * 16));
     {
@@ -1319,7 +1318,7 @@ int run_group(tm_ctx *ctx, tm_motif *const *motifs, uint32_t nm, uint64_t k, uin
     cudaMemsetAsync(dacc, 0, acc_bytes, st);
     cudaMemsetAsync(ctx->status, 0, 4, st);
     SampleJob J;
-    fill_job(m0, J, dplans);
+    fill_job(m0, J);
     const uint64_t want = (k + kSampleThreads - 1) / kSampleThreads;
     const unsigned blocks = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)ctx->num_sms * 16));
     {
@@ -1426,7 +1425,7 @@ int run_batch_items(tm_ctx *ctx, const BatchItem *items, uint32_t n, uint32_t ti
     uint32_t *dbase = (uint32_t *)(buf + ((qbytes + 255) / 256) * 256);
     Acc *dacc = (Acc *)((char *)dbase + ((bbytes + 255) / 256) * 256);
     uint32_t *dcounter = (uint32_t *)((char *)dacc + ((abytes + 255) / 256) * 256);
-    for (uint32_t q = 0; q < n; ++q) fill_job(items[q].mo, hq[q].job, &dq[q].plan);
+    for (uint32_t q = 0; q < n; ++q) fill_job(items[q].mo, hq[q].job);
     copy_h2d(ctx, dq, hq.data(), qbytes);
     copy_h2d(ctx, dbase, base.data(), bbytes);
     cudaMemsetAsync(dacc, 0, abytes, st);
@@ -1493,13 +1492,14 @@ int run_batch(tm_ctx *ctx, uint32_t nq, tm_motif *const *motifs, const uint64_t 
 // or a latency-bound loop that cannot afford an allocator call (which may
 // synchronise the device).  tm_sample_noalloc runs the same sampling kernel
 // as tm_sample (the motif plan goes with the launch), but its scratch -- the
-// result accumulators behind room for a plan -- lives in the fixed array below
-// instead of memory obtained from the allocator.
+// result accumulators -- lives in the fixed array below instead of memory
+// obtained from the allocator.
 // ---------------------------------------------------------------------------
 namespace timest {
 namespace {
 
-constexpr size_t kNoAllocScratchBytes = 4096;   // plan copy + accumulators
+constexpr size_t kNoAllocScratchBytes = 4096;
+static_assert(sizeof(Acc) <= kNoAllocScratchBytes, "the accumulators fit the scratch");
 constexpr int kNoAllocMaxDevices = 64;
 
 // One array per device that loads the library, held until the process exits.
@@ -1536,11 +1536,6 @@ extern "C" int tm_sample_noalloc(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t
     if (!ctx || !mo || mo->ctx != ctx || !out) return TM_E_ARG;
     if (!mo->have_weights || mo->graph_epoch != ctx->epoch || !ctx->preprocessed)
         return set_err(ctx, TM_E_STATE, "weights not computed for the current graph");
-    const size_t plan_bytes = ((sizeof(DevPlan) + 15) / 16) * 16;
-    const size_t need = plan_bytes + sizeof(Acc);
-    if (need > kNoAllocScratchBytes)
-        return set_err(ctx, TM_E_LIMIT, "motif plan (" + std::to_string(need) + " bytes) exceeds the " +
-                                            std::to_string(kNoAllocScratchBytes) + "-byte allocation-free scratch");
     int rc = check_cuda(ctx, cudaSetDevice(ctx->device), "cudaSetDevice");
     if (rc) return rc;
     unsigned char *scratch = nullptr;
@@ -1551,12 +1546,12 @@ extern "C" int tm_sample_noalloc(tm_ctx *ctx, tm_motif *mo, uint64_t k, uint64_t
         finish_result(mo, k, zero, out);
         return TM_OK;
     }
-    Acc *dacc = (Acc *)(scratch + plan_bytes);
+    Acc *dacc = (Acc *)scratch;
     cudaStream_t st = ctx->stream;
     cudaMemsetAsync(dacc, 0, sizeof(Acc), st);   // the array keeps the previous call's sums
     cudaMemsetAsync(ctx->status, 0, 4, st);
     SampleJob J;
-    fill_job(mo, J, nullptr);
+    fill_job(mo, J);
     const int threads = kSampleThreads;
     uint64_t want = (k + threads - 1) / threads;
     uint64_t cap = (uint64_t)ctx->num_sms * 16;

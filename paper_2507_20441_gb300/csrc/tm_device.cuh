@@ -339,12 +339,4 @@ __device__ __forceinline__ uint64_t mul_chk(uint64_t a, uint64_t b, bool &ovf)
     return a * b;
 }
 
-// Window of layer p holding t' (windows [i*d, (i+2)*d), i = p mod 2), or -1.
-__device__ __forceinline__ int64_t layer_window(uint32_t t, int p, int64_t d)
-{
-    int64_t tt = (int64_t)t;
-    if (tt < p * d) return -1;
-    return p + 2 * ((tt - p * d) / (2 * d));
-}
-
 }  // namespace timest

@@ -220,7 +220,7 @@ struct RangePtrs {
     uint2 *base;             // kind k's at base + k stride, by the parent edge's position in the
     size_t stride;           // meeting vertex's list; null: ranges not kept
     RangeExcl *excl;         // shared by the kinds, in no order
-    unsigned long long *excl_n;   // entries asked for (beyond the capacity: such ranges are searched)
+    unsigned long long *excl_n;   // entries asked for (beyond the capacity: such ranges are searched); null after the pass
     uint32_t excl_cap;
 };
 
@@ -351,7 +351,6 @@ int export_weights(tm_ctx *ctx, tm_motif *mo, int q, int layer, uint64_t *host_o
 
 // ---- sampler (sampler.cu) ----
 struct SampleJob {
-    const DevPlan *plan;                 // device pointer
     const uint64_t *wcum;                // u128 pairs
     const uint32_t *wguide;              // guide table of the window pick (shift wshift)
     uint32_t wshift;
@@ -470,6 +469,6 @@ void copy_d2h(tm_ctx *ctx, void *dst, const void *src, size_t bytes);
 int check_cuda(tm_ctx *ctx, cudaError_t e, const char *what);
 int set_err(tm_ctx *ctx, int code, const std::string &msg);
 int read_status(tm_ctx *ctx, uint32_t *bits);   // syncs the stream
-void fill_job(tm_motif *mo, SampleJob &job, const DevPlan *dplan);
+void fill_job(tm_motif *mo, SampleJob &job);
 
 }  // namespace timest

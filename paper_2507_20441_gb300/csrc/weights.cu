@@ -1172,6 +1172,7 @@ int compute_weights(tm_ctx *ctx, tm_motif *mo, bool guides, SharedPass *sh)
             if (rc) return rc;
         }
     }
+    mo->range.excl_n = nullptr;   // (of the pass, or of the selection)
     uint32_t bits = 0;
     rc = read_status(ctx, &bits);
     if (rc) return rc;
