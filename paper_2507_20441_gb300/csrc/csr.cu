@@ -43,7 +43,8 @@ namespace {
 // input, which reads the keys anyway), and a pass is one kernel: a tile of
 // keys is ranked stably, the tile finds where its digits start in the output
 // by looking back over the counts that the tiles before it have published, and
-// writes its digit runs out.
+// writes its digit runs out (Adinets and Merrill, "Onesweep: A Faster Least
+// Significant Digit Radix Sort for GPUs", 2022).
 #ifndef TM_RS_ITEMS
 #define TM_RS_ITEMS 16   // keys per thread (8 and 12 measured slower)
 #endif

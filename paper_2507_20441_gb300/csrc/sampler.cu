@@ -622,9 +622,11 @@ constexpr int kSampleThreads = TM_SAMPLE_THREADS;
 #define TM_RECS_SMEM 0   // per-sample records in local memory: L1 stays large for the searches
 #endif
 
-// Blocks per SM of the samplers with their records in local memory: the trace
-// measured 122 us at five against 134 at four and 136 at six (5e5 samples, 2e6
-// edges), a group of five motifs 431 at six against 466 at four (1e6 samples).
+// Blocks per SM of the samplers with their records in local memory, 1e6 samples
+// on 2e6 edges at 4 / 5 / 6 blocks, us a call: the general DeriveCnt 285 / 264 /
+// 281, tm_sample_noalloc 254 / 259 / 255 (the trace's kernel, 5e5 samples: 134 /
+// 122 / 136); groups of 1, 3, 5 and 8 motifs 268 / 267 / 264, 408 / 402 / 373, 523
+// / 505 / 481 and 673 / 661 / 623.
 constexpr int kTraceMinB = 5, kGroupMinB = 6;
 
 template <bool TRACE>

@@ -165,6 +165,8 @@ __device__ __forceinline__ SegAgg2 seg_combine2(SegAgg2 a, SegAgg2 b, bool &ovf)
 }
 
 // ---- one pass with decoupled look-back -------------------------------
+// (Merrill and Garland, "Single-pass Parallel Prefix Scan with Decoupled
+// Look-back", NVIDIA NVR-2016-002, 2016)
 // Each block takes the next tile from a counter (so every tile before it has
 // been started), scans it, publishes its aggregate, then its first warp walks
 // back over the tiles before it, 32 at a time, combining their aggregates
@@ -184,7 +186,11 @@ struct alignas(32) SegTile {
     unsigned long long w[4];
 };
 
-constexpr int kLookbackPolls = 1 << 22;   // with a 64 ns sleep each: a limit of at least a quarter second
+// Polls before a look-back gives up (ST_TIMEOUT), with __nanosleep(64) between
+// them, or (32) in the radix passes, the pair tables and the windows.  The sleep
+// is a hint with an upper bound of twice its argument and no lower one, so this
+// bounds the number of polls alone.
+constexpr int kLookbackPolls = 1 << 22;
 
 __device__ __forceinline__ void seg_publish(SegTile *t, const SegAgg2 &v, uint32_t st)   // st 1: aggregate, 2: prefix
 {

@@ -415,8 +415,8 @@ struct KernelTimer {
 
 #ifdef __CUDACC__
 // A kernel is set up while the one before it on the stream ends, which saves a
-// microsecond or more of each gap between two: an estimate on 2e4 edges (about 38
-// launches) 309 -> 264 us, on 2e6 1007 -> 951, a selection of 12 candidates 3030
+// microsecond or more of each gap between two: an estimate on 2e4 edges (23
+// kernels, 15 clears and copies) 309 -> 264 us, on 2e6 1007 -> 951, a selection of 12 candidates 3030
 // -> 2854.  EVERY kernel begins with grid_wait, before any other statement: it
 // returns when the kernels before it have ended and what they wrote is seen.
 // (Letting the next kernel's blocks in as soon as this one's last block has
