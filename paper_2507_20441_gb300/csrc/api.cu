@@ -890,13 +890,14 @@ int tm_select_tree(tm_ctx *ctx, uint32_t nv, uint32_t ne, const uint32_t *edges,
     if (n_cand) *n_cand = evaluated;
     if (rc) return rc;
     if (!best) return set_err(ctx, TM_E_OVERFLOW, "every candidate's weight pass overflowed");
-    cudaMemsetAsync(ctx->status, 0, kStatusBytes, ctx->stream);   // (bits of a candidate that overflowed after the winner)
+    // (the bits last read are the last candidate's, which may have overflowed)
+    if (*ctx->status_host) cudaMemsetAsync(ctx->status, 0, kStatusBytes, ctx->stream);
     {
         PhaseScope ph(ctx, TM_PH_ROOT);
         rc = fill_guides(ctx, best);
     }
-    uint32_t bits = 0;
-    const int rc2 = read_status(ctx, &bits);   // the tables are filled when the call returns
+    const int rc2 = check_cuda(ctx, cudaStreamSynchronize(ctx->stream), "guide tables");   // filled when the call returns
+    prof_collect(ctx);
     if (rc || rc2) { tm_motif_free(best); return rc ? rc : rc2; }
     *out = best;
     return TM_OK;
